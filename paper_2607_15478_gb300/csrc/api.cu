@@ -140,32 +140,17 @@ cudaError_t pardtw::launch_plan(const DpPlan& plan, const DpArgs& a, int dp, int
     }
 }
 
-// Which way to sweep a pair.  The persistent warp-pair DP runs its strip
-// groups in waves of one group per SM: a CTA sweeps all columns of a group
-// before it takes the next, and the next group in the chain starts a few
-// blocks behind the one above.  So the time is about
-//   ceil(groups / SMs) x columns  +  strips x (lag of one strip, ~18 columns)
-// column steps; the transposed sweep (B's frames as rows) wins when that is
-// smaller for (Lb rows, La columns), e.g. a pair that fits one wave with B
-// longer: its chain then runs over La columns instead of Lb.  Only the
-// warp-pair DP at 3 rows per lane has the transposed tie order.
-namespace {
-double sweep_estimate(int rows, int cols, int dp, const dtw_options& o, int num_sms) {
-    const DpPlan p = choose_plan(rows, dp, o, num_sms);
-    const int rps = strip_rows(p.R);
-    const long long strips = (rows + rps - 1) / rps;
-    const long long groups = (strips + p.spg - 1) / p.spg;
-    const long long waves = num_sms > 0 ? (groups + num_sms - 1) / num_sms : 1;
-    return (double)waves * cols + 18.0 * (double)strips;
-}
-}  // namespace
-
+// Which way to sweep a pair.  The strips form one chain: its time is about
+//   columns + strips x (lag of one strip, ~18 columns)
+// column steps, and the cells swept (those a path can cross) are the same in
+// either direction, so the sweep runs over the shorter sequence's frames.
+// Only the warp-pair DP at 3 rows per lane has the transposed tie order.
 bool pardtw::transpose_pair(int La, int Lb, int dp, const dtw_options& o, int num_sms) {
     if (o.transpose == DTW_TRANSPOSE_NEVER) return false;
     const DpPlan pt = choose_plan(Lb, dp, o, num_sms);  // the plan the transposed pair gets
     if (pt.kind != 2 || pt.R != 3) return false;
     if (o.transpose == DTW_TRANSPOSE_ALWAYS) return true;
-    return sweep_estimate(Lb, La, dp, o, num_sms) < sweep_estimate(La, Lb, dp, o, num_sms);
+    return Lb > La;
 }
 
 namespace {

@@ -116,6 +116,20 @@ struct DpArgs {
                                     // La-1 at every column (nchunk * 16 floats), else null
 };
 
+// Columns of row i that a path can cross, [path_lo, path_hi]: with steps of
+// slope 1/2 to 2, the cells reachable from (0, 0) that can still reach
+// (La-1, Lb-1).  Both bounds grow with i, and every predecessor a path can
+// take lies inside them, so cells outside (two thirds of a square matrix)
+// never change a path, a total or a field that a path reads.
+__host__ __device__ inline int path_lo(int i, int La, int Lb) {
+    const int a = (i + 1) / 2, b = Lb - 1 - 2 * (La - 1 - i);
+    return a > b ? a : b;
+}
+__host__ __device__ inline int path_hi(int i, int La, int Lb) {
+    const int a = 2 * i, b = Lb - 1 - (La - i) / 2;
+    return a < b ? a : b;
+}
+
 // Backpointer word address of cell (i, j): strip-major, then 16-column chunk,
 // then row within the strip.  A strip of rps rows stores wpb >= rps words
 // per chunk (32 per warp and row of a lane: the ghost lane's words are
