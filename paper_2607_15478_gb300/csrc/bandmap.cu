@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(kSegThreads) k_bandmap(const BtArgs one,
     __shared__ int s_x[2][kSegThreads][3];
     // kMany: one pair per blockIdx.z (the grid covers the largest pair;
     // blocks beyond a pair's bands or columns leave at once)
-    bandmap_segment<kSegThreads, kBanded>(a, blockIdx.y, blockIdx.x, s_x, [] { return 1; });
+    bandmap_segment<kSegThreads, kBanded>(a, blockIdx.y, blockIdx.x, s_x);
 }
 
 }  // namespace
@@ -345,22 +345,14 @@ size_t bandmap_scratch_bytes(int La, int Lb) {
            + (size_t)nbands * sizeof(int) + 64;       // count, end entry
 }
 
-int bandmap_items(int La, int Lb, int threads) {
-    const int nbands = (La + kBand - 1) / kBand;
-    const int width = threads * kColsPerWord - 2 * kBand;
-    return nbands * ((Lb + width - 1) / width);
-}
-
-cudaError_t launch_backtrace_bands(const BtArgs& a, cudaStream_t s, bool with_map) {
+cudaError_t launch_backtrace_bands(const BtArgs& a, cudaStream_t s) {
     const int nbands = (a.La + kBand - 1) / kBand;
     const int width = kSegCols - 2 * kBand;
     dim3 grid((unsigned)((a.Lb + width - 1) / width), (unsigned)nbands, 1);
-    if (with_map) {
-        if (a.ranges)
-            k_bandmap<false, true><<<grid, kSegThreads, 0, s>>>(a, nullptr);
-        else
-            k_bandmap<false, false><<<grid, kSegThreads, 0, s>>>(a, nullptr);
-    }
+    if (a.ranges)
+        k_bandmap<false, true><<<grid, kSegThreads, 0, s>>>(a, nullptr);
+    else
+        k_bandmap<false, false><<<grid, kSegThreads, 0, s>>>(a, nullptr);
     const int n2 = nbands >= 4 ? (nbands - 2) / 2 : 0;
     if (n2 > 0)
         k_bt_compose<false><<<dim3((unsigned)((a.Lb + 255) / 256), (unsigned)n2, 1), 256, 0, s>>>(

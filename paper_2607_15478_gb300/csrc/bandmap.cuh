@@ -1,7 +1,5 @@
 // Band map of the parallel backtrace (see bandmap.cu for the whole scheme):
-// the per-band, per-segment propagation of entries, shared by the standalone
-// kernel (bandmap.cu) and the DP kernel, which runs band-map items on its CTAs
-// as the strips they need complete (dp_split.cuh).
+// the per-band, per-segment propagation of entries.
 #pragma once
 #include "pardtw_common.cuh"
 
@@ -138,14 +136,9 @@ constexpr int kRowsAhead = 8;  // backpointer rows loaded ahead of use
 // The band map of band b over segment segx of its columns, by the NT threads
 // of the calling block (all of them must call it; t = threadIdx.x < NT).
 // s_x: the block's left-neighbour exchange buffer.
-// kInKernel: the backpointers were written by the calling kernel itself (by
-// other CTAs, released through flags), so they are read through L2 rather than
-// the read-only path.  ready(): called by every thread once the segment is
-// known to have work, before its first backpointer load (the DP kernel waits
-// there for the strips that cover the band).
-template <int NT, bool kBanded, bool kInKernel = false, class Ready>
+template <int NT, bool kBanded>
 __device__ __forceinline__ void bandmap_segment(const BtArgs& a, int b, int segx,
-                                                int (*s_x)[NT][3], Ready ready) {
+                                                int (*s_x)[NT][3]) {
     const uint32_t* __restrict__ bp = a.bp;
     const int La = a.La, Lb = a.Lb, nchunk = a.nchunk, rps = a.rps, wpb = a.wpb;
     const int band = kBand;
@@ -190,7 +183,7 @@ __device__ __forceinline__ void bandmap_segment(const BtArgs& a, int b, int segx
     const size_t wrap = (size_t)nchunk * wpb - rps;
     auto load = [&](int i) -> uint32_t {
         uint32_t w = 0u;
-        if (have && i < r1) w = kInKernel ? __ldcg(lp) : __ldg(lp);
+        if (have && i < r1) w = __ldg(lp);
         ++lp;
         if (++lrow == rps) {
             lrow = 0;
@@ -198,7 +191,6 @@ __device__ __forceinline__ void bandmap_segment(const BtArgs& a, int b, int segx
         }
         return w;
     };
-    if (!ready()) return;  // CTA-uniform
 
     int e1[kColsPerWord], e2[kColsPerWord];  // entries of rows i-1 and i-2
 #pragma unroll

@@ -161,9 +161,9 @@ __device__ __forceinline__ int refill_top(float (*blk)[kSub], int js, int lane, 
 // sweep.  Only lane 0 issues; all lanes wait on the barrier.  (The wide
 // FP32 cost warps of dp_split.cuh use rings of two slots: a copy one block
 // ahead, each block a whole 16-frame chunk.)
-template <int DP, int kSlotsT = 4>
+template <int DP, int kSlotsT = 4, int kBlkT = 0>
 struct BStage {
-    static constexpr int kBlk = DP <= 16 ? 64 : (DP <= 32 ? 32 : 16);  // frames per copy
+    static constexpr int kBlk = kBlkT > 0 ? kBlkT : (DP <= 16 ? 64 : (DP <= 32 ? 32 : 16));  // frames per copy
     static constexpr int kSlots = kSlotsT;
     static constexpr int kAhead = kSlots - 1;
     static constexpr int kWarpBytes = kSlots * kBlk * DP * 4;
@@ -218,6 +218,27 @@ __device__ __forceinline__ void sts128(unsigned addr, float4 v) {
                  : "memory");
 }
 
+__device__ __forceinline__ void sts32(unsigned addr, float v) {
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+// 8-byte store by the threads where `on` holds, without a branch.
+__device__ __forceinline__ void sts64_if(unsigned addr, float a, float b, bool on) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.s32 p, %3, 0;\n @p st.shared.v2.f32 [%0], {%1, %2};\n}\n" ::
+            "r"(addr),
+        "f"(a), "f"(b), "r"((int)on)
+        : "memory");
+}
+
+// 16-byte global store by the threads where `on` holds, without a branch.
+__device__ __forceinline__ void stg128_if(float* dst, float a, float b, float c, float d, bool on) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.s32 p, %5, 0;\n @p st.global.v4.f32 [%0], {%1, %2, %3, %4};\n}\n" ::
+            "l"(dst),
+        "f"(a), "f"(b), "f"(c), "f"(d), "r"((int)on)
+        : "memory");
+}
+
 // Non-blocking test of the same condition as mbar_try_wait (never suspends
 // the thread), for look-ahead checks placed between independent work.
 __device__ __forceinline__ int mbar_test_wait(unsigned bar, unsigned parity) {
@@ -234,6 +255,17 @@ __device__ __forceinline__ int mbar_test_wait(unsigned bar, unsigned parity) {
 // mbarrier arrive (release at CTA scope) by the calling thread.
 __device__ __forceinline__ void mbar_arrive(unsigned bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_n(unsigned bar, unsigned count) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+// The same by the threads where `on` holds, without a branch.
+__device__ __forceinline__ void mbar_arrive_if(unsigned bar, bool on) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.s32 p, %1, 0;\n"
+        " @p mbarrier.arrive.shared::cta.b64 _, [%0];\n}\n" ::"r"(bar),
+        "r"((int)on)
+        : "memory");
 }
 // Wait (warp-uniform) until the phase of parity `par` of `bar` has completed.
 // Bounded like every other wait: gives up when the call failed elsewhere or
@@ -260,15 +292,12 @@ __device__ __forceinline__ int mbar_wait(unsigned bar, unsigned par, DevCtl* ctl
 }
 
 // ---- thread-block clusters: between the strip groups of two CTAs of one
-// cluster the border travels through distributed shared memory.  The
-// writer warp of the CTA above copies each block of its last strip's bottom
-// rows into the staging ring of the CTA below with asynchronous stores that
-// complete a transaction count on that CTA's full barrier (armed for 64
-// bytes per use by the receiving reader warp), so no fence orders them; the
-// reader warp below, once it holds a block's values in registers, re-arms
-// the full barrier and arrives on the sender's empty barrier with a count
-// that depends on a loaded value, so the arrival cannot be performed before
-// the loads.
+// cluster the border travels through distributed shared memory.  The writer
+// warp of the CTA above stores each block of its last strip's bottom rows
+// straight into the slot of the CTA below, with asynchronous stores that
+// complete a transaction count on the slot's full barrier (its cost warp
+// expects 64 bytes per use), so no fence orders them; the reader warp below
+// hands every release of a slot back to the CTA above.
 __device__ __forceinline__ unsigned cluster_rank() {
     unsigned r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -309,22 +338,17 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(unsigned bar, unsigned byt
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                  : "memory");
 }
-// 0, computed from x (a register dependency on x that the compiler keeps).
-__device__ __forceinline__ unsigned zero_after(unsigned x) {
-    unsigned z;
-    asm volatile("and.b32 %0, %1, 0;" : "=r"(z) : "r"(x));
-    return z;
-}
-// Relaxed arrival with `count` on an mbarrier of another CTA of the cluster.
-__device__ __forceinline__ void mbar_arrive_remote_relaxed(unsigned remote_bar, unsigned count) {
-    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(remote_bar),
-                 "r"(count)
+// Relaxed arrival on an mbarrier of another CTA of the cluster (a release at
+// cluster scope costs a fence: measured 1.68 against 1.32 ms of DP on the
+// 20000 x 25000 pair).
+__device__ __forceinline__ void mbar_arrive_remote_relaxed(unsigned remote_bar) {
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote_bar)
                  : "memory");
 }
 
-template <int DP, int kSlotsT = 4>
+template <int DP, int kSlotsT = 4, int kBlkT = 0>
 struct BRing {
-    using S = BStage<DP, kSlotsT>;
+    using S = BStage<DP, kSlotsT, kBlkT>;
     const float* stage;   // this warp's kSlots * kBlk frames
     unsigned stage_s;     // its shared address
     unsigned bar_s;       // shared address of this warp's kSlots mbarriers
@@ -333,6 +357,7 @@ struct BRing {
     int nblk;             // blocks of B up to the end of the strip's columns
     int issued;           // blocks of this strip issued so far (first <= issued)
     int waited;           // blocks of this strip known complete
+    int stride = 1, off = 0;  // block q is block q * stride + off of B
 
     // Copy block q (frames q*kBlk .., whole 16-frame chunks) of the
     // chunk-transposed B (Lb_pad frames) into its slot.
@@ -346,7 +371,7 @@ struct BRing {
     __device__ __forceinline__ void issue(int q, const float* Bt, int Lb_pad, int lane) {
         if (lane == 0) {
             const unsigned t = base + (unsigned)(q - first);
-            const int f0 = q * S::kBlk;
+            const int f0 = (q * stride + off) * S::kBlk;
             const int nf = min(S::kBlk, Lb_pad - f0);
             tma_load(stage_s + (t % S::kSlots) * (S::kBlk * DP * 4), Bt + (size_t)f0 * DP,
                      (unsigned)(nf * DP * 4), bar_s + (t % S::kSlots) * 8);
@@ -406,6 +431,10 @@ struct BRing {
         return stage_s +
                (unsigned)(((t % S::kSlots) * S::kBlk + (unsigned)(f % S::kBlk)) * DP * 4);
     }
+    // Shared address of block q (which must be complete).
+    __device__ __forceinline__ unsigned block_s(int q) const {
+        return stage_s + ((base + (unsigned)(q - first)) % S::kSlots) * (S::kBlk * DP * 4);
+    }
     // The 16 x DP feature-major values of chunk k (its block must be complete).
     __device__ __forceinline__ const float* chunk(int k) const {
         const int f = k * kColsPerWord;
@@ -429,22 +458,18 @@ __device__ __forceinline__ float eq_as_float(float a, float b) {
 // of exact powers of two, so the code costs two compares and no integer or
 // select instruction.
 // kSubseq: the subsequence DTW of WSDTW (Sec. II-C), weights 1, 1, 2 for
-// (1,1), (1,2), (2,1) instead of 2, 3, 3.  (w12 is no longer read: the
-// ghost rows' zero weight became a select of the border value.)
+// (1,1), (1,2), (2,1) instead of 2, 3, 3.
 // kT: the pair is swept transposed (rows of the kernel = frames of B), so
 // the kernel's (1,2) candidate is the problem's (2,1) and vice versa; the
 // problem's tie order (1,1), (1,2), (2,1) is then the kernel's c0, c2, c1.
 // Bit 1 then records that c2 attains the minimum (one compare, as in the
 // direct sweep), and transpose_fields turns the finished word into the
 // kernel's decoding before it is stored.  Same cells, same values, same path.
+// y1, y2: rows i0-1 and i0-2 of column j-1 (from the lane above).
 template <int R, bool kSubseq = false, bool kT = false>
-__device__ __forceinline__ void dp_step(const float* cost, int u, int srcA, const float* w12,
-                                        bool ghost, float g0, float g1, bool origin_here,
-                                        float mu, float* cur, float* prv, float& ylp, float* fw,
-                                        float& o0, float& o1) {
-    (void)w12;  // the (1,2) weight: 3 (1 in the subsequence DP) on every real row
-    const float y1 = __shfl_sync(kFull, cur[R - 1], srcA);  // E[i0-1][j-1]
-    const float y2 = __shfl_sync(kFull, cur[R - 2], srcA);  // E[i0-2][j-1]
+__device__ __forceinline__ void dp_cells(const float* cost, int u, float y1, float y2, bool ghost,
+                                        float g0, float g1, bool origin_here,
+                                        float mu, float* cur, float* prv, float& ylp, float* fw) {
     const float bit0 = (float)(1u << (2 * u)), bit1 = (float)(2u << (2 * u));
     float m[R];
 #pragma unroll
@@ -470,14 +495,25 @@ __device__ __forceinline__ void dp_step(const float* cost, int u, int srcA, cons
         if (k == 0) mk = origin_here ? cost[0] + mu : mk;  // E[0][0] = C[0][0]
         m[k] = mk;
     }
-    o0 = m[R - 2];
-    o1 = m[R - 1];
     ylp = y1;
 #pragma unroll
     for (int k = 0; k < R; ++k) {
         prv[k] = cur[k];
         cur[k] = m[k];
     }
+}
+
+// The whole step with its two shuffles; o0, o1: the new values of the lane's
+// last two rows.
+template <int R>
+__device__ __forceinline__ void dp_step(const float* cost, int u, int srcA, bool ghost, float g0,
+                                        float g1, bool origin_here, float mu, float* cur,
+                                        float* prv, float& ylp, float* fw, float& o0, float& o1) {
+    const float y1 = __shfl_sync(kFull, cur[R - 1], srcA);
+    const float y2 = __shfl_sync(kFull, cur[R - 2], srcA);
+    dp_cells<R>(cost, u, y1, y2, ghost, g0, g1, origin_here, mu, cur, prv, ylp, fw);
+    o0 = cur[R - 2];
+    o1 = cur[R - 1];
 }
 
 // A word of the transposed sweep, whose bit 1 of each field says that the

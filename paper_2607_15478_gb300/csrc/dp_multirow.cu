@@ -86,9 +86,6 @@ __device__ __forceinline__ void run_strip(const DpArgs& p, int g, int w, int lan
     const unsigned long long* gin = p.gborder + (size_t)(g > 0 ? g - 1 : 0) * Lb * 2;
     const float kc = ghost ? kGhostCost : p.kcost;
     const float mu = p.mu;
-    float w12[R];
-#pragma unroll
-    for (int k = 0; k < R; ++k) w12[k] = (ghost && k >= R - 2) ? 0.0f : 3.0f;
     const int srcA = (lane + 31) & 31;
     const unsigned epoch = p.epoch;
     const bool is_origin = (i0 == 0) && !ghost;
@@ -214,7 +211,7 @@ __device__ __forceinline__ void run_strip(const DpArgs& p, int g, int w, int lan
                     float cu[R];
 #pragma unroll
                     for (int k = 0; k < R; ++k) cu[k] = c[k][u];
-                    dp_step<R>(cu, u, srcA, w12, ghost, gv0[u], gv1[u],
+                    dp_step<R>(cu, u, srcA, ghost, gv0[u], gv1[u],
                                (h == 0) && (u == 0) && (j0 == 0) && is_origin, mu, cur, prv,
                                ylp, fw, o0[u], o1[u]);
                 }
@@ -225,7 +222,7 @@ __device__ __forceinline__ void run_strip(const DpArgs& p, int g, int w, int lan
                     float cu[R];
 #pragma unroll
                     for (int k = 0; k < R; ++k) cu[k] = c[k][u];
-                    dp_step<R>(cu, u, srcA, w12, ghost, gv0[u], gv1[u],
+                    dp_step<R>(cu, u, srcA, ghost, gv0[u], gv1[u],
                                (h == 0) && (u == 0) && (j0 == 0) && is_origin, mu, cur, prv,
                                ylp, fw, o0[u], o1[u]);
                 }

@@ -8,27 +8,29 @@
 //     (0..30) of the DP warp holds rows R t .. R t + R - 1 of the strip,
 //     lane 31 is the ghost lane that carries the two bottom rows of the strip
 //     above (cost 1e30, weight 0 on the (1,2) candidate fed the border value).
-//   - The cost warp of the strip computes C' = (1 - mu) - a^_i . b^_j for the
-//     same rows, 8 columns at a time (one FMA per feature, in feature order,
-//     so the values are bit-identical to the other kernels'), reading the
-//     frames of B from its TMA-fed ring, and hands them to the DP warp
-//     through a ring of kCostSlots sub-chunks in shared memory with one
-//     full and one empty mbarrier per slot.  The DP warp loads a
-//     sub-chunk's costs at its start, before the eight steps.
+//   - The cost warp(s) of the strip compute C' = (1 - mu) - a^_i . b^_j for the
+//     same rows, 8 columns (a sub-chunk) at a time (one FMA per feature, in
+//     feature order, so the values are bit-identical to the other kernels'),
+//     reading the frames of B from a TMA-fed ring, and hand them to the DP
+//     warp through a ring of kSlots slots in shared memory.  A slot also holds
+//     the strip's top border for its columns: the two bottom rows of the strip
+//     above, which that strip's DP warp (or, for the first strip of a CTA, the
+//     reader warp or the CTA above in its cluster) stores there.  One full
+//     barrier per slot counts both, one empty barrier releases both.
 //   - The DP warp runs only the recurrence: per column two shuffles, three
-//     FMAs, a three-way minimum and two compares per cell.
-//   - Every DP warp takes its top border from a ring of kRingBlk sub-chunks
-//     in shared memory and writes its two bottom rows into the next ring,
-//     with a full and an empty mbarrier per block.  The first strip's ring
-//     is filled by the reader warp from the global border that the CTA
-//     above publishes; the last strip's ring is drained by the writer warp
-//     into this CTA's global border.  The L2 round trips of that exchange
-//     thus never sit in a DP warp, and all DP warps do the same work per
-//     sub-chunk (in a chain of strips the slowest one sets the pace).
+//     FMAs, a three-way minimum and two compares per cell.  It works one
+//     sub-chunk behind its loads: in the middle of a sub-chunk it tests the
+//     next slot's barrier and loads it, a load or two per column, so that
+//     neither the test nor the loads (nor the queue of shared-memory accesses
+//     in front of a shuffle) hold up the recurrence, and the outcome of the
+//     test is looked at after the eight steps.  The strip's two bottom rows go
+//     out column by column, one 8-byte store each.
+//   - The last strip of a CTA hands its rows to the writer warp through a
+//     ring of its own, which publishes them in global memory or, inside a
+//     cluster, stores them straight into the slots of the CTA below.
 //   - Every wait is bounded (DTW_ERR_TIMEOUT) and gives up when the call has
 //     failed elsewhere.
 #pragma once
-#include "bandmap.cuh"
 #include "dp_device.cuh"
 
 // The kernel templates are included by dp_split.cu (two strips per CTA) and
@@ -38,26 +40,39 @@ namespace {
 
 constexpr int kGhostLane = 31;
 constexpr int kOutLane = 30;    // holds the strip's two bottom rows
-constexpr int kCostSlots = 4;   // sub-chunks of costs in flight per strip
-static_assert(kRingBlk >= 4, "the DP warp waits for output ring blocks four at a time");
+// Sub-chunks in flight per strip, and in the writer's ring.  In a cluster a
+// slot's round trip (stored by the CTA above, released here, handed back) is
+// longer than 8 sub-chunks.
+template <bool kCl>
+constexpr int slots_of() {
+    return kCl ? 16 : 8;
+}
+constexpr int kBorderBytes = 2 * kSub * 4;  // 8 columns of (row top-2, row top-1) pairs
 
 // One slot holds the 8 costs of each of a lane's R rows: float4 q of lane l
-// (q = 2 k + half) at [q][l], so a warp's 16-byte accesses are contiguous.
+// (q = 2 k + half) at [q][l], so a warp's 16-byte accesses are contiguous;
+// then the top border of the 8 columns.
 template <int R>
 struct CostRing {
     static constexpr int kF4 = 2 * R;
-    static constexpr int kSlotBytes = kF4 * kWarp * 16;
-    static constexpr int kBytes = kCostSlots * kSlotBytes;
+    static constexpr int kBorder = kF4 * kWarp * 16;
+    static constexpr int kSlotBytes = kBorder + kBorderBytes;
 };
 
-// BF16 cost: one cost slot holds the 8 costs of each of the 32 R rows of the
+// BF16 cost: one slot holds the 8 costs of each of the 32 R rows of the
 // strip row by row, kRowFloats floats per row (48-byte rows: the DP warp's
-// 16-byte loads of rows 3l+k then fall in distinct bank groups).
+// 16-byte loads of rows 3l+k then fall in distinct bank groups), then the top
+// border.
 constexpr int kRowFloats = 12;
 template <int R>
 struct CostRingRM {
-    static constexpr int kSlotBytes = 32 * R * kRowFloats * 4;
-    static constexpr int kBytes = kCostSlots * kSlotBytes;
+    static constexpr int kBorder = 32 * R * kRowFloats * 4;
+    static constexpr int kSlotBytes = kBorder + kBorderBytes;
+};
+template <int R, bool kRM>
+struct SlotOf {
+    static constexpr int kBorder = kRM ? CostRingRM<R>::kBorder : CostRing<R>::kBorder;
+    static constexpr int kBytes = kRM ? CostRingRM<R>::kSlotBytes : CostRing<R>::kSlotBytes;
 };
 // BF16 cost: the strip's rows of A as bf16 (32 R rows of kBfStride), and a
 // ring of kBfSlots blocks of 16 frames of B (one chunk each) filled by TMA.
@@ -68,32 +83,38 @@ constexpr int kBfBlkBytes = kColsPerWord * kBfStride * 2;
 // registers, so the strip's rows of A^ sit in shared memory (rows padded by 4
 // floats: the 16-byte loads of rows 3l + k of a warp fall in distinct bank
 // groups), and two cost warps share a strip, taking alternate sub-chunks
-// (all 8 columns each).
-template <int DP, bool kBF>
-struct CostWide {
-    static constexpr bool kOn = DP > 32 && !kBF;
-    static constexpr int kNC = kOn ? 2 : 1;  // cost warps per strip
+// (all 8 columns each).  Two cost warps also where one would be slower than
+// the DP warp (D > 8 and two strips per CTA).
+template <int DP, int NS, bool kBF>
+struct CostCfg {
+    static constexpr bool kWide = DP > 32 && !kBF;
+        static constexpr int kNC = kWide ? (NS == 1 ? 4 : 2)
+                               : NS == 1                   ? 3
+                               : (!kBF && DP > 8 && NS == 2) ? 2
+                                                           : 1;  // cost warps a strip
     static constexpr int kStride = DP + 4;   // floats per row of the A tile
-    static constexpr int kBSlots = 2;        // chunks of B in each cost warp's ring
+    // each cost warp's ring of B: frames a block, blocks
+    static constexpr int kBBlk = kWide ? kColsPerWord : (DP <= 16 ? 64 : 32);
+    static constexpr int kBSlots = kNC >= 2 ? 2 : 4;
 };
-template <int DP, int R, bool kBF>
+template <int DP, int R, int NS, bool kBF, bool kCl>
 struct SplitSmem {
-    // per strip slot: the cost warp's operands (B stage; A tile and B stage
-    // for the BF16 cost; A tile for the wide FP32 cost), then the cost ring
+    using Cfg = CostCfg<DP, NS, kBF>;
+    // per strip slot: the cost warps' operands (B stages; A tile and B stage
+    // for the BF16 cost; A tile and B stages for the wide FP32 cost), then the
+    // slots
     static constexpr int kOperandBytes =
-        kBF ? 32 * R * kBfStride * 2 + kBfSlots * kBfBlkBytes
-            : (CostWide<DP, kBF>::kOn
-                   ? 32 * R * CostWide<DP, kBF>::kStride * 4 +
-                         2 * BStage<DP, CostWide<DP, kBF>::kBSlots>::kWarpBytes
-                   : BStage<DP>::kWarpBytes);
+        kBF ? 32 * R * kBfStride * 2 + Cfg::kNC * kBfSlots * kBfBlkBytes
+            : (Cfg::kWide ? 32 * R * Cfg::kStride * 4 : 0) +
+                  Cfg::kNC * BStage<DP, Cfg::kBSlots, Cfg::kBBlk>::kWarpBytes;
     static constexpr int kStripBytes =
-        kOperandBytes + (kBF ? CostRingRM<R>::kBytes : CostRing<R>::kBytes);
+        kOperandBytes + slots_of<kCl>() * SlotOf<R, kBF>::kBytes;
 };
 // Threads of a CTA of NS strips: per strip the cost warp(s) and a DP warp,
 // plus the reader and the writer.
 template <int DP, int NS, bool kBF>
 __host__ __device__ constexpr int split_threads() {
-    return ((CostWide<DP, kBF>::kNC + 1) * NS + 2) * 32;
+    return ((CostCfg<DP, NS, kBF>::kNC + 1) * NS + 2) * 32;
 }
 
 // Barrier `slot` of an array of 8-byte mbarriers, and the phase parity a
@@ -122,16 +143,51 @@ __device__ __forceinline__ int2 strip_range(const DpArgs& p, int strip) {
     return make_int2(x, max(y, x + 1));
 }
 
-// Cost warp of `strip`: all sub-chunks of the sweep, in order.
-template <int DP, int R, bool kAllCols>
-__device__ __forceinline__ void run_cost(const DpArgs& p, int strip, int lane, unsigned cring,
-                                         unsigned cfull, unsigned cempty, unsigned csub,
-                                         BRing<DP>& br) {
-    using S = BStage<DP>;
+// Where the top border of a strip's slots comes from: sub-chunks before
+// link_end from the CTA above in the cluster (64 bytes of asynchronous stores
+// on the full barrier), those from inf_from on have none (+inf, stored here),
+// the others from another warp of the CTA (its arrival is one of the full
+// barrier's two).
+struct BorderSrc {
+    int inf_from, link_end;
+};
+
+// The costs of sub-chunk n are in the slot (every lane has stored its own):
+// arrive for them, and settle the border's share of the slot.
+__device__ __forceinline__ void cost_arrive(unsigned full, unsigned border, int n,
+                                            const BorderSrc& bs, int lane) {
+    if (n >= bs.inf_from && lane < 2 * kSub) sts32(border + (unsigned)lane * 4u, INFINITY);
+    __syncwarp();
+    if (lane == 0) {
+        if (n >= bs.inf_from) {
+            mbar_arrive_n(full, 2);
+        } else {
+            if (n < bs.link_end) mbar_arrive_expect_tx(full, kBorderBytes);
+            mbar_arrive(full);
+        }
+    }
+}
+
+// Cost warp `half` of the kNC of `strip`: every kNC-th sub-chunk of the
+// sweep, in order.  Bound by the FMAs' three register operands: paired FMAs
+// (two columns each, each rounded once: the values of one FMA per feature in
+// feature order) take 70 cycles a column of a D = 12 strip for one warp alone
+// on its SM sub-partition and 52 with two, scalar ones 64 and 60.  (A pass over
+// 16 columns takes 49 and 47 but fills its slots in bursts: no faster in the
+// kernel, and slower at D = 32 and where two CTAs share an SM's registers.)
+template <int DP, int R, int NS, int kSlots, bool kAllCols>
+__device__ __forceinline__ void run_cost(const DpArgs& p, int strip, int half, int lane,
+                                         unsigned cring, unsigned cfull, unsigned cempty,
+                                         unsigned csub, const BorderSrc& bs,
+                                         BRing<DP, CostCfg<DP, NS, false>::kBSlots,
+                                               CostCfg<DP, NS, false>::kBBlk>& br) {
+    using Cfg = CostCfg<DP, NS, false>;
+    using S = BStage<DP, Cfg::kBSlots, Cfg::kBBlk>;
     using CR = CostRing<R>;
     constexpr int kRows = 31 * R;
     constexpr int kFG = 4;            // features per group of loads
     constexpr int kNG = DP / kFG;     // DP is a multiple of 4
+    static_assert(S::kBlk >= kSub * Cfg::kNC, "a warp reads some of every block of B");
     const bool ghost = lane == kGhostLane;
     const int i0 = strip * kRows + lane * R;
     float na[R][DP];  // -a^_i of the lane's rows (0 in the ghost lane)
@@ -150,29 +206,31 @@ __device__ __forceinline__ void run_cost(const DpArgs& p, int strip, int lane, u
     const float kc = ghost ? kGhostCost : p.kcost;
     const int Lb_pad = p.nchunk * kColsPerWord;
     const int2 rg = strip_range<kAllCols>(p, strip);  // sub-chunks rg.x .. rg.y-1
-    const int q0 = rg.x * kSub / S::kBlk;
+    const int n0 = rg.x + half;
+    const int q0 = n0 * kSub / S::kBlk;
     br.begin(q0, min((rg.y * kSub + S::kBlk - 1) / S::kBlk, (Lb_pad + S::kBlk - 1) / S::kBlk));
     br.top_up(q0, p.Bhat, Lb_pad, lane);
-    for (int n = rg.x; n < rg.y; ++n) {
+    int qcur = -1;
+    for (int n = n0; n < rg.y; n += Cfg::kNC) {
         const int js = n * kSub;
-        if (js % S::kBlk == 0 || n == rg.x) {
-            const int q = js / S::kBlk;
+        const int q = js / S::kBlk;
+        if (q != qcur) {
             if (!br.wait(q, p.ctl, p.timeout_ns)) break;
             br.top_up(q, p.Bhat, Lb_pad, lane);
+            qcur = q;
         }
         const unsigned t = csub + (unsigned)(n - rg.x);
-        const unsigned slot = t % kCostSlots;
+        const unsigned slot = t % kSlots;
         // the DP warp has read this slot's previous contents
-        if (!mbar_wait(bar_at(cempty, slot), use_parity(t, kCostSlots) ^ 1u, p.ctl, p.timeout_ns,
-                       6))
+        if (!mbar_wait(bar_at(cempty, slot), use_parity(t, kSlots) ^ 1u, p.ctl, p.timeout_ns, 6))
             break;
         // the 8 frames of the sub-chunk, feature-major (16 floats per feature)
         const unsigned nb = br.chunk_s(js >> 4) + (unsigned)(js & kSub) * 4u;
-        float c[R][kSub];
+        float2 c[R][kSub / 2];  // costs of columns 2m, 2m+1 in c[k][m]
 #pragma unroll
         for (int k = 0; k < R; ++k)
 #pragma unroll
-            for (int f = 0; f < kSub; ++f) c[k][f] = kc;
+            for (int f = 0; f < kSub / 2; ++f) c[k][f] = make_float2(kc, kc);
         // loads of the next feature group are issued before the FMAs of the
         // current one
         float4 bv[2][2 * kFG];
@@ -198,26 +256,24 @@ __device__ __forceinline__ void run_cost(const DpArgs& p, int strip, int lane, u
                 const float4 b0 = bv[gi & 1][2 * e], b1 = bv[gi & 1][2 * e + 1];
 #pragma unroll
                 for (int k = 0; k < R; ++k) {
-                    c[k][0] = fmaf(na[k][d], b0.x, c[k][0]);
-                    c[k][1] = fmaf(na[k][d], b0.y, c[k][1]);
-                    c[k][2] = fmaf(na[k][d], b0.z, c[k][2]);
-                    c[k][3] = fmaf(na[k][d], b0.w, c[k][3]);
-                    c[k][4] = fmaf(na[k][d], b1.x, c[k][4]);
-                    c[k][5] = fmaf(na[k][d], b1.y, c[k][5]);
-                    c[k][6] = fmaf(na[k][d], b1.z, c[k][6]);
-                    c[k][7] = fmaf(na[k][d], b1.w, c[k][7]);
+                    const float2 xx = make_float2(na[k][d], na[k][d]);
+                    c[k][0] = __ffma2_rn(xx, make_float2(b0.x, b0.y), c[k][0]);
+                    c[k][1] = __ffma2_rn(xx, make_float2(b0.z, b0.w), c[k][1]);
+                    c[k][2] = __ffma2_rn(xx, make_float2(b1.x, b1.y), c[k][2]);
+                    c[k][3] = __ffma2_rn(xx, make_float2(b1.z, b1.w), c[k][3]);
                 }
             }
         }
-        const unsigned dst = cring + slot * CR::kSlotBytes + (unsigned)lane * 16u;
+        const unsigned sbase = cring + slot * CR::kSlotBytes;
+        const unsigned dst = sbase + (unsigned)lane * 16u;
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             sts128(dst + (unsigned)(2 * k) * (kWarp * 16),
-                   make_float4(c[k][0], c[k][1], c[k][2], c[k][3]));
+                   make_float4(c[k][0].x, c[k][0].y, c[k][1].x, c[k][1].y));
             sts128(dst + (unsigned)(2 * k + 1) * (kWarp * 16),
-                   make_float4(c[k][4], c[k][5], c[k][6], c[k][7]));
+                   make_float4(c[k][2].x, c[k][2].y, c[k][3].x, c[k][3].y));
         }
-        mbar_arrive(bar_at(cfull, slot));
+        cost_arrive(bar_at(cfull, slot), sbase + CR::kBorder, n, bs, lane);
     }
     br.drain();
 }
@@ -233,13 +289,15 @@ __device__ __forceinline__ void run_cost(const DpArgs& p, int strip, int lane, u
 // copies one chunk ahead (B^ through L1 instead ran at L2 latency, ~1100
 // cycles per column; 4 columns per warp and sub-chunk, at 426).  A slot of
 // the cost ring is written by one warp, as in the narrow kernel.
-template <int DP, int R>
+template <int DP, int R, int NS, int kSlots>
 __device__ __forceinline__ void run_cost_wide(const DpArgs& p, int strip, int w, int half,
                                               int lane, float* tile, unsigned cring,
                                               unsigned cfull, unsigned cempty, unsigned csub,
-                                              BRing<DP, CostWide<DP, false>::kBSlots>& br) {
-    using W = CostWide<DP, false>;
-    using S = BStage<DP, W::kBSlots>;
+                                              const BorderSrc& bs,
+                                              BRing<DP, CostCfg<DP, NS, false>::kBSlots,
+                                                    CostCfg<DP, NS, false>::kBBlk>& br) {
+    using W = CostCfg<DP, NS, false>;
+    using S = BStage<DP, W::kBSlots, W::kBBlk>;
     using CR = CostRing<R>;
     constexpr int kRows = 31 * R;
     constexpr int kS = W::kStride;
@@ -247,36 +305,38 @@ __device__ __forceinline__ void run_cost_wide(const DpArgs& p, int strip, int w,
     const bool ghost = lane == kGhostLane;
     // the strip's rows of A^ (ghost rows zero) into the tile, 16 bytes a lane
     {
+        constexpr int kT = W::kNC * kWarp;  // the strip's cost warps
         const int tid = half * kWarp + lane;
-        for (int e = tid; e < 32 * R * (DP / 4); e += 2 * kWarp) {
+        for (int e = tid; e < 32 * R * (DP / 4); e += kT) {
             const int r = e / (DP / 4), q = e - r * (DP / 4);
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
             if (r < kRows)
                 v = __ldg(reinterpret_cast<const float4*>(p.Ahat + (size_t)(strip * kRows + r) * DP) + q);
             *reinterpret_cast<float4*>(tile + r * kS + 4 * q) = v;
         }
-        asm volatile("bar.sync %0, %1;" ::"r"(1 + w), "r"(2 * kWarp) : "memory");
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + w), "r"(kT) : "memory");
     }
     const float kc = ghost ? kGhostCost : p.kcost;
     const int Lb_pad = p.nchunk * kColsPerWord;
     const int2 rg = strip_range(p, strip);  // rg.x even: sub-chunk pairs are chunks
     const float* arow = tile + (lane * R) * kS;
+    // this warp's sub-chunks n0, n0 + kNC, ...: one in every kNC / 2 chunks of B
+    // (kNC is even), which are the blocks 0, 1, ... of its ring
+    static_assert(W::kNC % 2 == 0, "a warp keeps to one half of its chunks");
     const int n0 = rg.x + half;
-    const int q0 = n0 * kSub / S::kBlk;
-    br.begin(q0, min((rg.y * kSub + S::kBlk - 1) / S::kBlk, (Lb_pad + S::kBlk - 1) / S::kBlk));
-    br.top_up(q0, p.Bhat, Lb_pad, lane);
-    for (int n = n0; n < rg.y; n += 2) {
-        const int js = n * kSub;
-        const int q = js / S::kBlk;
+    br.stride = W::kNC / 2;
+    br.off = n0 / 2;
+    br.begin(0, rg.y > n0 ? (rg.y - n0 + W::kNC - 1) / W::kNC : 0);
+    br.top_up(0, p.Bhat, Lb_pad, lane);
+    for (int n = n0, q = 0; n < rg.y; n += W::kNC, ++q) {
         if (!br.wait(q, p.ctl, p.timeout_ns)) break;
         br.top_up(q, p.Bhat, Lb_pad, lane);
         // feature d of the sub-chunk's 8 frames: 32 bytes at bsrc + 64 d
-        const unsigned bsrc = br.chunk_s(js >> 4) + (unsigned)(js & 15) * 4u;
+        const unsigned bsrc = br.block_s(q) + (unsigned)(n & 1) * 32u;
         const unsigned t = csub + (unsigned)(n - rg.x);
-        const unsigned slot = t % kCostSlots;
+        const unsigned slot = t % kSlots;
         // the DP warp has read this slot's previous contents
-        if (!mbar_wait(bar_at(cempty, slot), use_parity(t, kCostSlots) ^ 1u, p.ctl, p.timeout_ns,
-                       6))
+        if (!mbar_wait(bar_at(cempty, slot), use_parity(t, kSlots) ^ 1u, p.ctl, p.timeout_ns, 6))
             break;
         // costs of columns 2q, 2q+1 of row k in c[k][q]: each paired FMA is
         // two FP32 FMAs, each rounded once (the values of one FMA per feature
@@ -330,7 +390,8 @@ __device__ __forceinline__ void run_cost_wide(const DpArgs& p, int strip, int w,
             if (g + 4 < DP / 4) load(g + 4, a0, b0);
             fmas(a1, b1);
         }
-        const unsigned dst = cring + slot * CR::kSlotBytes + (unsigned)lane * 16u;
+        const unsigned sbase = cring + slot * CR::kSlotBytes;
+        const unsigned dst = sbase + (unsigned)lane * 16u;
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             sts128(dst + (unsigned)(2 * k) * (kWarp * 16),
@@ -338,7 +399,7 @@ __device__ __forceinline__ void run_cost_wide(const DpArgs& p, int strip, int w,
             sts128(dst + (unsigned)(2 * k + 1) * (kWarp * 16),
                    make_float4(c[k][2].x, c[k][2].y, c[k][3].x, c[k][3].y));
         }
-        mbar_arrive(bar_at(cfull, slot));
+        cost_arrive(bar_at(cfull, slot), sbase + CR::kBorder, n, bs, lane);
     }
     br.drain();
 }
@@ -370,21 +431,21 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // two cost slots; the ghost lane's rows get 1e30.  A's rows are converted to
 // bf16 into shared memory once per strip; B's bf16 frames arrive by TMA, one
 // chunk per block.
-template <int DP, int R>
-__device__ __forceinline__ void run_cost_bf16(const DpArgs& p, int strip, int lane, unsigned a_s,
+template <int DP, int R, int kNC, int kSlots>
+__device__ __forceinline__ void run_cost_bf16(const DpArgs& p, int strip, int w, int half, int lane, unsigned a_s,
                                               unsigned b_s, unsigned bbar_s, unsigned& bbase,
                                               unsigned cring, unsigned cfull, unsigned cempty,
-                                              unsigned csub) {
+                                              unsigned csub, const BorderSrc& bs) {
     constexpr int kRows = 31 * R;       // real rows of the strip
     constexpr int kM = 32 * R;          // rows of the product (6 tiles of 16)
     constexpr int kMT = kM / 16;
     constexpr int kKS = DP / 16;        // k-steps of 16 features
     constexpr int kRowBytes = kBfStride * 2;
     const int2 rg = strip_range(p, strip);  // sub-chunks rg.x (even) .. rg.y-1
-    const int c_lo = rg.x / 2, c_hi = (rg.y + 1) / 2;
+    const int c_lo = rg.x / 2 + half, c_hi = (rg.y + 1) / 2;
     const int nsub = rg.y;
     // A: rows r = 0 .. kM-1 of the strip as bf16 (rows >= kRows are zero)
-    for (int r = lane; r < kM; r += kWarp) {
+    for (int r = half * kWarp + lane; r < kM; r += kNC * kWarp) {
         const float* src = p.Ahat + (size_t)(strip * kRows + r) * DP;
 #pragma unroll 4
         for (int d = 0; d < DP; d += 8) {
@@ -401,35 +462,41 @@ __device__ __forceinline__ void run_cost_bf16(const DpArgs& p, int strip, int la
                          : "memory");
         }
     }
-    __syncwarp();
+    if constexpr (kNC > 1)
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + w), "r"(kNC * kWarp) : "memory");
+    else
+        __syncwarp();
     const char* gb = static_cast<const char*>(p.Bbf);
-    int issued = c_lo, waited = c_lo;
-    auto issue = [&](int c) {  // lane 0: chunk c of B into slot (bbase + c - c_lo) % kBfSlots
+    // this warp's chunks c_lo, c_lo + kNC, ... are the blocks 0 .. nq-1 of its ring
+    const int nq = c_hi > c_lo ? (c_hi - c_lo + kNC - 1) / kNC : 0;
+    int issued = 0, waited = 0;
+    auto issue = [&](int q) {  // lane 0: block q into slot (bbase + q) % kBfSlots
         if (lane == 0) {
-            const unsigned t = bbase + (unsigned)(c - c_lo);
-            tma_load(b_s + (t % kBfSlots) * kBfBlkBytes, gb + (size_t)c * kBfBlkBytes,
-                     (unsigned)kBfBlkBytes, bbar_s + 8 * (t % kBfSlots));
+            const unsigned t = bbase + (unsigned)q;
+            tma_load(b_s + (t % kBfSlots) * kBfBlkBytes,
+                     gb + (size_t)(c_lo + q * kNC) * kBfBlkBytes, (unsigned)kBfBlkBytes,
+                     bbar_s + 8 * (t % kBfSlots));
         }
     };
-    while (issued < c_hi && issued < c_lo + kBfSlots - 1) issue(issued++);
+    while (issued < nq && issued < kBfSlots - 1) issue(issued++);
     const float kc = p.kcost;
     const int g = lane >> 2, t4 = lane & 3;
     bool ok = true;
-    for (int c = c_lo; c < c_hi && ok; ++c) {
+    for (int c = c_lo, q = 0; c < c_hi && ok; c += kNC, ++q) {
         // chunk c of B is in its slot
-        const unsigned tb = bbase + (unsigned)(c - c_lo);
+        const unsigned tb = bbase + (unsigned)q;
         if (!mbar_wait(bbar_s + 8 * (tb % kBfSlots), (tb / kBfSlots) & 1u, p.ctl, p.timeout_ns,
                        4)) {
             ok = false;
             break;
         }
-        waited = c + 1;
-        if (issued < c_hi) issue(issued++);
+        waited = q + 1;
+        if (issued < nq) issue(issued++);
         const int nj = (2 * c + 1 < nsub) ? 2 : 1;  // sub-chunks of this chunk
         const unsigned t0 = csub + (unsigned)(2 * c - rg.x);
         for (int j = 0; j < nj; ++j)
-            if (!mbar_wait(bar_at(cempty, (t0 + j) % kCostSlots),
-                           use_parity(t0 + j, kCostSlots) ^ 1u, p.ctl, p.timeout_ns, 6)) {
+            if (!mbar_wait(bar_at(cempty, (t0 + j) % kSlots), use_parity(t0 + j, kSlots) ^ 1u,
+                           p.ctl, p.timeout_ns, 6)) {
                 ok = false;
                 break;
             }
@@ -468,7 +535,7 @@ __device__ __forceinline__ void run_cost_bf16(const DpArgs& p, int strip, int la
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             if (j >= nj) break;
-            const unsigned slot = cring + ((t0 + j) % kCostSlots) * CostRingRM<R>::kSlotBytes;
+            const unsigned slot = cring + ((t0 + j) % kSlots) * CostRingRM<R>::kSlotBytes;
 #pragma unroll
             for (int mt = 0; mt < kMT; ++mt) {
                 const int r0 = 16 * mt + g, r1 = r0 + 8;
@@ -485,67 +552,24 @@ __device__ __forceinline__ void run_cost_bf16(const DpArgs& p, int strip, int la
                              "f"(v10), "f"(v11)
                              : "memory");
             }
-            mbar_arrive(bar_at(cfull, (t0 + j) % kCostSlots));
+            cost_arrive(bar_at(cfull, (t0 + j) % kSlots), slot + CostRingRM<R>::kBorder, 2 * c + j,
+                        bs, lane);
         }
     }
     // leave no copy in flight (bounded)
-    for (int c = waited; c < issued; ++c) {
-        const unsigned tb = bbase + (unsigned)(c - c_lo);
+    for (int q = waited; q < issued; ++q) {
+        const unsigned tb = bbase + (unsigned)q;
         const long long t0 = __shfl_sync(kFull, global_ns(), 0);
         while (!__all_sync(kFull, mbar_try_wait(bbar_s + 8 * (tb % kBfSlots),
                                                 (tb / kBfSlots) & 1u))) {
             if (__shfl_sync(kFull, global_ns(), 0) - t0 > 1000000000LL) break;
         }
     }
-    bbase += (unsigned)(issued - c_lo);
+    bbase += (unsigned)issued;
 }
 
-// The costs of lifetime sub-chunk t (its slot must be full) into c;
-// kRM: the row-major slot of the BF16 cost.
-template <int R, bool kRM>
-__device__ __forceinline__ void load_costs(unsigned cring, unsigned t, int lane,
-                                           float (*c)[kSub]) {
-    if constexpr (kRM) {
-        const unsigned src = cring + (t % kCostSlots) * CostRingRM<R>::kSlotBytes +
-                             (unsigned)(lane * R) * (kRowFloats * 4);
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const float4 v0 = lds128(src + (unsigned)k * (kRowFloats * 4));
-            const float4 v1 = lds128(src + (unsigned)k * (kRowFloats * 4) + 16);
-            c[k][0] = v0.x;
-            c[k][1] = v0.y;
-            c[k][2] = v0.z;
-            c[k][3] = v0.w;
-            c[k][4] = v1.x;
-            c[k][5] = v1.y;
-            c[k][6] = v1.z;
-            c[k][7] = v1.w;
-        }
-        return;
-    }
-    using CR = CostRing<R>;
-    const unsigned src = cring + (t % kCostSlots) * CR::kSlotBytes + (unsigned)lane * 16u;
-#pragma unroll
-    for (int k = 0; k < R; ++k) {
-        const float4 v0 = lds128(src + (unsigned)(2 * k) * (kWarp * 16));
-        const float4 v1 = lds128(src + (unsigned)(2 * k + 1) * (kWarp * 16));
-        c[k][0] = v0.x;
-        c[k][1] = v0.y;
-        c[k][2] = v0.z;
-        c[k][3] = v0.w;
-        c[k][4] = v1.x;
-        c[k][5] = v1.y;
-        c[k][6] = v1.z;
-        c[k][7] = v1.w;
-    }
-}
-
-// Which rings of a CTA a strip group uses: ring w < NS feeds DP slot w (ring
-// 0 from the reader warp, which has nothing to read in group 0; ring w >= 1
-// from DP slot w-1, when strip w exists); ring NS takes the last DP slot's
-// bottom rows to the writer warp, when a group below needs them.  Producer
-// and consumer of a ring count its uses (in sub-chunks) the same way, which
-// keeps every barrier's phase in step across groups.
+// Which warps of a CTA a strip group needs: the reader for groups that have
+// one above, the writer for groups that have one below.
 struct GroupRoles {
     int g, nstrips_here;
     bool reader, writer;
@@ -559,12 +583,6 @@ __device__ __forceinline__ GroupRoles group_roles(const DpArgs& p, int g) {
     r.writer = (g + 1 < p.ngroups) && (g != p.skip_publish);
     return r;
 }
-template <int NS>
-__device__ __forceinline__ bool ring_used(const GroupRoles& r, int w) {
-    if (w == 0) return r.reader;
-    if (w < NS) return w < r.nstrips_here;
-    return r.writer;
-}
 
 // cur[k] for a runtime k < R without indexing the register array.
 template <int R>
@@ -575,479 +593,291 @@ __device__ __forceinline__ float pick_row(const float* cur, int k) {
     return v;
 }
 
-// The two border rows of a ring block (8 columns each) into registers.
-__device__ __forceinline__ void load_border(unsigned s, float* g0, float* g1) {
-    const float4 a0 = lds128(s), a1 = lds128(s + 16);
-    const float4 b0 = lds128(s + 32), b1 = lds128(s + 48);
-    g0[0] = a0.x; g0[1] = a0.y; g0[2] = a0.z; g0[3] = a0.w;
-    g0[4] = a1.x; g0[5] = a1.y; g0[6] = a1.z; g0[7] = a1.w;
-    g1[0] = b0.x; g1[1] = b0.y; g1[2] = b0.z; g1[3] = b0.w;
-    g1[4] = b1.x; g1[5] = b1.y; g1[6] = b1.z; g1[7] = b1.w;
-}
-// The strip's two bottom rows of a sub-chunk into a ring block.
-__device__ __forceinline__ void store_border(unsigned d, const float* o0, const float* o1) {
-    sts128(d, make_float4(o0[0], o0[1], o0[2], o0[3]));
-    sts128(d + 16, make_float4(o0[4], o0[5], o0[6], o0[7]));
-    sts128(d + 32, make_float4(o1[0], o1[1], o1[2], o1[3]));
-    sts128(d + 48, make_float4(o1[4], o1[5], o1[6], o1[7]));
-}
-// Subsequence DP: row La-1 of the nsteps columns at dst.
-__device__ __forceinline__ void store_lastrow(float* dst, int nsteps, const float* ol) {
-    if (nsteps == kSub) {
-        reinterpret_cast<float4*>(dst)[0] = make_float4(ol[0], ol[1], ol[2], ol[3]);
-        reinterpret_cast<float4*>(dst)[1] = make_float4(ol[4], ol[5], ol[6], ol[7]);
+// Where a strip's bottom rows go, 8 columns (64 bytes) a block: the border
+// part of the next strip's slots, or the writer's ring.  Blocks [first, end)
+// are stored, block `first` being lifetime use t0 of the ring.
+struct OutRing {
+    unsigned base, stride, full, empty, t0;
+    int first, end;
+};
+
+// A sub-chunk's operands in registers: the lane's costs and the top border's
+// (row top-2, row top-1) pairs of two columns per float4.
+template <int R>
+struct SubIn {
+    float4 c[2 * R], g[4];
+};
+// Load `it` of the 2 R + 4 of a slot.
+template <int R, bool kRM>
+__device__ __forceinline__ void load_part(SubIn<R>& in, unsigned slot, int lane, int it) {
+    if (it < 2 * R) {
+        in.c[it] = kRM ? lds128(slot + (unsigned)(lane * R + it / 2) * (kRowFloats * 4) +
+                                (unsigned)(it & 1) * 16u)
+                       : lds128(slot + (unsigned)lane * 16u + (unsigned)it * (kWarp * 16));
     } else {
-#pragma unroll
-        for (int u = 0; u < kSub; ++u)
-            if (u < nsteps) dst[u] = ol[u];
+        in.g[it - 2 * R] = lds128(slot + SlotOf<R, kRM>::kBorder + (unsigned)(it - 2 * R) * 16u);
     }
 }
-// The 8 DP steps of a full sub-chunk.
-template <int R, bool kSubseq, bool kT>
-__device__ __forceinline__ void sweep_full(const float (*c)[kSub], const float* g0, const float* g1,
-                                           bool first_col, bool is_origin, int srcA,
-                                           const float* w12, bool ghost, float mu, float* cur,
-                                           float* prv, float& ylp, float* fw, float* o0, float* o1,
-                                           float* ol, int kl) {
-#pragma unroll
-    for (int u = 0; u < kSub; ++u) {
-        float cu[R];
-#pragma unroll
-        for (int k = 0; k < R; ++k) cu[k] = c[k][u];
-        dp_step<R, kSubseq, kT>(cu, u, srcA, w12, ghost, g0[u], g1[u],
-                                (kSubseq || (first_col && u == 0)) && is_origin, mu, cur, prv, ylp,
-                                fw, o0[u], o1[u]);
-        if constexpr (kSubseq) ol[u] = pick_row<R>(cur, kl);
-    }
+__device__ __forceinline__ float elem(const float4& v, int k) {
+    return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w));
 }
 
-// The DP steps of one sub-chunk (nsteps <= 8 columns; the cell of the first
-// column of the sweep is the origin when first_col and is_origin hold).
-template <int R, bool kSubseq, bool kT>
-__device__ __forceinline__ void sweep_sub(const float (*c)[kSub], const float* g0, const float* g1,
-                                          int nsteps, bool first_col, bool is_origin, int srcA,
-                                          const float* w12, bool ghost, float mu, float* cur,
-                                          float* prv, float& ylp, float* fw, float* o0, float* o1,
-                                          float* ol, int kl) {
-    if (nsteps == kSub) {
+// The recurrence state of a strip's lane: columns j-1 and j-2 of its rows and
+// row top-1 of column j-2.
+template <int R>
+struct DpState {
+    float cur[R], prv[R], ylp;
+};
+// Column u of a sub-chunk; behind(): the shared-memory accesses that belong
+// behind the column's shuffles (a shuffle waits for the accesses queued before
+// it, and the recurrence waits for the shuffles).
+template <int R, bool kSubseq, bool kT, class Behind>
+__device__ __forceinline__ void sweep_col(const SubIn<R>& in, int u, bool origin, int srcA,
+                                          bool ghost, float mu, DpState<R>& s, float* fw,
+                                          Behind behind) {
+    float cu[R];
 #pragma unroll
-        for (int u = 0; u < kSub; ++u) {
-            float cu[R];
-#pragma unroll
-            for (int k = 0; k < R; ++k) cu[k] = c[k][u];
-            dp_step<R, kSubseq, kT>(cu, u, srcA, w12, ghost, g0[u], g1[u],
-                                    (kSubseq || (first_col && u == 0)) && is_origin, mu, cur, prv,
-                                    ylp, fw, o0[u], o1[u]);
-            if constexpr (kSubseq) ol[u] = pick_row<R>(cur, kl);
-        }
-    } else {
-#pragma unroll
-        for (int u = 0; u < kSub; ++u) {
-            if (u >= nsteps) break;
-            float cu[R];
-#pragma unroll
-            for (int k = 0; k < R; ++k) cu[k] = c[k][u];
-            dp_step<R, kSubseq, kT>(cu, u, srcA, w12, ghost, g0[u], g1[u],
-                                    (kSubseq || (first_col && u == 0)) && is_origin, mu, cur, prv,
-                                    ylp, fw, o0[u], o1[u]);
-            if constexpr (kSubseq) ol[u] = pick_row<R>(cur, kl);
-        }
-    }
+    for (int k = 0; k < R; ++k) cu[k] = elem(in.c[2 * k + u / 4], u & 3);
+    const float y1 = __shfl_sync(kFull, s.cur[R - 1], srcA);  // E[i0-1][j-1]
+    const float y2 = __shfl_sync(kFull, s.cur[R - 2], srcA);  // E[i0-2][j-1]
+    behind();
+    dp_cells<R, kSubseq, kT>(cu, u, y1, y2, ghost, elem(in.g[u / 2], 2 * (u & 1)),
+                             elem(in.g[u / 2], 2 * (u & 1) + 1), origin, mu, s.cur, s.prv, s.ylp,
+                             fw);
 }
 
-// DP warp of `strip` (slot w of group g).  ring: the NS + 1 border rings;
-// bfull / bempty: their mbarriers (kRingBlk per ring); rin / rout: lifetime
-// sub-chunk counts of the input and output rings at the start of this
-// group; csub: that of the cost ring.
-// kFlag: the strip raises its flag in done[strip] when its words are stored
-// (one pair with the band map inside the kernel).
-// kWords: a trip of the sweep takes a whole backpointer word (two sub-chunks,
-// one set of barrier tests, loads and arrivals for 16 columns) instead of
-// one sub-chunk; kTwoCost: two cost warps fill alternate cost slots.  Taken
-// where the DP warp alone sets the pace (BF16 cost: 12% faster at D = 128)
-// and not for the FP32 cost at D <= 32, where the trip of a sub-chunk was
-// faster on GB300 (the strip below waits for a whole word of the border, and
-// the per-column work did not shrink).
-template <int R, int NS, bool kRM, bool kSubseq = false, bool kT = false, bool kFlag = false,
-          bool kWords = false, bool kTwoCost = false>
-__device__ __forceinline__ void run_dp(const DpArgs& p, const GroupRoles& gr, int w, int strip,
-                                       int lane, float (*ring)[kRingBlk][2][kSub], unsigned bfull,
-                                       unsigned bempty, unsigned rin, unsigned rout,
-                                       unsigned cring, unsigned cfull, unsigned cempty,
-                                       unsigned csub,
-                                       unsigned inf_blk, unsigned* done = nullptr) {
+// DP warp of `strip`: sub-chunks rg of its slots (cring, cfull, cempty, the
+// first being lifetime use csub), the bottom rows into `out`.
+//
+// What bounds it: one warp's chain of columns (a column's two shuffles, FMAs
+// and minima feed the next column's shuffles, two columns apart at R = 3), and
+// with it the chain of strips.  Alone on an SM sub-partition 16 columns of
+// straight-line code take ~43 cycles a column; every branch between columns
+// costs ~50 cycles (the fields of the last columns no longer overlap the next
+// ones), and waits, loads and stores that stand between sub-chunks cost more.
+// So a trip of the loop is a backpointer word (sub-chunks n and n + 1) with one
+// branch: it starts with the operands of n in registers, loads those of n + 1
+// and n + 2 behind the shuffles after testing their barriers, sweeps n + 1
+// before knowing that its operands were there, and looks at all tests at its
+// end.  Where they were not, the state before n + 1 is put back, the barrier is
+// waited for and n + 1 is swept again: in a chain that is on time this is
+// rare, and a strip that is early has time to lose.
+template <int R, int kSlots, bool kRM, bool kSubseq, bool kT>
+__device__ __forceinline__ void run_dp(const DpArgs& p, int strip, int lane, const int2 rg,
+                                       const OutRing& out, unsigned cring, unsigned cfull,
+                                       unsigned cempty, unsigned csub) {
+    using Slot = SlotOf<R, kRM>;
     constexpr int kRows = 31 * R;
+    constexpr int kLoads = 2 * R + 4;  // 16-byte loads of a slot
+    // the next slot is loaded behind the shuffles of columns kFirst, kFirst + 1, ..,
+    // kPer loads each: as late as the loads' latency allows, since a strip can
+    // follow the one above no closer than its tests look ahead
+    constexpr int kFirst = 4, kPer = 4;
     const bool ghost = lane == kGhostLane;
     const int i0 = strip * kRows + lane * R;
-    const int Lb = p.Lb;
-    const bool from_ring = ring_used<NS>(gr, w);
-    const bool to_ring = ring_used<NS>(gr, w + 1);
-    float (*myring)[2][kSub] = ring[w];
-    float (*nextring)[2][kSub] = ring[w + 1];
-    const unsigned bfull_in = bfull + 8 * kRingBlk * w;
-    const unsigned bempty_in = bempty + 8 * kRingBlk * w;
-    const unsigned bfull_out = bfull + 8 * kRingBlk * (w + 1);
-    const unsigned bempty_out = bempty + 8 * kRingBlk * (w + 1);
     const float mu = p.mu;
-    float w12[R];
-#pragma unroll
-    for (int k = 0; k < R; ++k) w12[k] = (ghost && k >= R - 2) ? 0.0f : (kSubseq ? 1.0f : 3.0f);
     const int srcA = (lane + 31) & 31;
     const bool is_origin = (i0 == 0) && !ghost;
     // subsequence DP: the lane and row slot of row La-1, if this strip holds it
     const int rl = p.La - 1 - strip * kRows;
     const bool has_last = kSubseq && rl >= 0 && rl < kRows && lane == rl / R;
     const int kl = kSubseq ? rl - (rl / R) * R : 0;
-    // this strip's sub-chunks, and those its border ring's producer publishes
-    // (the strip above; for the first strip of a group the reader, which
-    // publishes exactly this strip's range)
-    const int2 rg = strip_range<kSubseq>(p, strip);
-    const int2 rp = w > 0 ? strip_range<kSubseq>(p, strip - 1) : rg;
-    // blocks the strip above published before this strip's first column are
-    // consumed unread, so that the ring's producer and consumer stay in step
-    if (from_ring)
-        for (int n = rp.x; n < rg.x; ++n) {
-            const unsigned ti = rin + (unsigned)(n - rp.x);
-            if (!mbar_wait(bar_at(bfull_in, ti % kRingBlk), use_parity(ti, kRingBlk), p.ctl,
-                           p.timeout_ns, 1))
-                return;
-            mbar_arrive(bar_at(bempty_in, ti % kRingBlk));
+    const int nfull = min(rg.y, p.Lb / kSub);  // sub-chunks before it have all 8 columns
+
+    DpState<R> s;
+#pragma unroll
+    for (int k = 0; k < R; ++k) s.cur[k] = s.prv[k] = INFINITY;
+    s.ylp = INFINITY;
+
+    auto wait_load = [&](unsigned t, SubIn<R>& in) -> bool {
+        if (!mbar_wait(bar_at(cfull, t % kSlots), use_parity(t, kSlots), p.ctl, p.timeout_ns, 7))
+            return false;
+#pragma unroll
+        for (int it = 0; it < kLoads; ++it)
+            load_part<R, kRM>(in, cring + (t % kSlots) * Slot::kBytes, lane, it);
+        return true;
+    };
+    auto release = [&](unsigned t) {
+        __syncwarp();
+        mbar_arrive_if(bar_at(cempty, t % kSlots), lane == 0);
+    };
+    // The 8 columns of a full sub-chunk: fields into word's half h, the bottom
+    // rows to dst where st holds; behind(u): see sweep_col.  (No poll of the
+    // failure flag in the sweep: every wait checks it on its slow path, and a
+    // warp that never waits ends with its strip.)
+    auto full_sub = [&](int n, const SubIn<R>& in, int h, unsigned dst, bool st, uint32_t* word,
+                        auto behind) {
+        float fw[R];  // backpointer fields of the sub-chunk, bits 2u, 2u+1
+#pragma unroll
+        for (int k = 0; k < R; ++k) fw[k] = 0.0f;
+        float ol[kSub];  // subsequence DP: row La-1 (lane of has_last)
+        (void)ol;
+#pragma unroll
+        for (int u = 0; u < kSub; ++u) {
+            sweep_col<R, kSubseq, kT>(
+                in, u, (kSubseq || (h == 0 && u == 0 && n == 0)) && is_origin, srcA, ghost, mu, s,
+                fw, [&] {
+                    if (u > 0)
+                        sts64_if(dst + (unsigned)(u - 1) * 8u, s.cur[R - 2], s.cur[R - 1], st);
+                    behind(u);
+                });
+            if constexpr (kSubseq) ol[u] = pick_row<R>(s.cur, kl);
         }
-
-    float cur[R], prv[R];
-#pragma unroll
-    for (int k = 0; k < R; ++k) cur[k] = prv[k] = INFINITY;
-    float ylp = INFINITY;
-    // (no poll of the failure flag in the sweep: every wait checks it on its
-    // slow path, and a warp that never waits ends with its strip)
-    if constexpr (kWords) {
-        const int jend = min(rg.y * kSub, Lb);
-        // whole words first (16 full columns), then the last, ragged word
-        uint32_t tailw[R];
-        const int jfull = rg.x * kSub + ((jend - rg.x * kSub) / kColsPerWord) * kColsPerWord;
-        for (int j0 = rg.x * kSub; j0 < jfull; j0 += kColsPerWord) {
-            // One backpointer word per trip: sub-chunks n (even; ranges start on
-            // whole words) and n + 1.
-            const int n = j0 / kSub;
-            const unsigned ti = rin + (unsigned)(n - rp.x), to = rout + (unsigned)(n - rg.x);
-            const unsigned t = csub + (unsigned)(n - rg.x);
-            const bool in0 = from_ring && n < rp.y;
-            const bool in1 = from_ring && n + 1 < rp.y;
-
-            // The waits of the word, first tested together without blocking: the
-            // border blocks from the ring above (the producer publishes them in
-            // order, so the second one's barrier implies the first's; columns the
-            // strip above did not sweep are +inf), every other word the output
-            // ring (its consumer empties it in order, so once the previous use of
-            // block to+3 is consumed so are those of to .. to+2), and the cost
-            // slots (filled in order by one cost warp; with two cost warps, which
-            // take alternate slots, both are tested).
-            const bool need_out = to_ring && ((n - rg.x) & 3) == 0;
-            const unsigned tl = to + 3u, tb = in1 ? ti + 1u : ti, tc = t + 1u;
-            const int rb = in0 ? mbar_test_wait(bar_at(bfull_in, tb % kRingBlk),
-                                                 use_parity(tb, kRingBlk))
-                               : 1;
-            const int ro = need_out ? mbar_test_wait(bar_at(bempty_out, tl % kRingBlk),
-                                                     use_parity(tl, kRingBlk) ^ 1u)
-                                    : 1;
-            const int rc = mbar_test_wait(bar_at(cfull, tc % kCostSlots), use_parity(tc, kCostSlots));
-            const int rc0 = kTwoCost ? mbar_test_wait(bar_at(cfull, t % kCostSlots),
-                                                      use_parity(t, kCostSlots))
-                                     : 1;
-            if (!__all_sync(kFull, rb) &&
-                !mbar_wait_slow(bar_at(bfull_in, tb % kRingBlk), use_parity(tb, kRingBlk), p.ctl,
-                                p.timeout_ns, 1))
-                return;
-            if (!__all_sync(kFull, ro) &&
-                !mbar_wait_slow(bar_at(bempty_out, tl % kRingBlk), use_parity(tl, kRingBlk) ^ 1u,
-                                p.ctl, p.timeout_ns, 2))
-                return;
-            if (!__all_sync(kFull, rc) &&
-                !mbar_wait_slow(bar_at(cfull, tc % kCostSlots), use_parity(tc, kCostSlots), p.ctl,
-                                p.timeout_ns, 7))
-                return;
-            if (kTwoCost && !__all_sync(kFull, rc0) &&
-                !mbar_wait_slow(bar_at(cfull, t % kCostSlots), use_parity(t, kCostSlots), p.ctl,
-                                p.timeout_ns, 7))
-                return;
-            float gA0[kSub], gA1[kSub], gB0[kSub], gB1[kSub];
-            load_border(in0 ? smem_u32(&myring[ti % kRingBlk][0][0]) : inf_blk, gA0, gA1);
-            load_border(in1 ? smem_u32(&myring[(ti + 1u) % kRingBlk][0][0]) : inf_blk, gB0, gB1);
-            float cA[R][kSub], cB[R][kSub];
-            load_costs<R, kRM>(cring, t, lane, cA);
-            load_costs<R, kRM>(cring, t + 1u, lane, cB);
-            if (in0) mbar_arrive(bar_at(bempty_in, ti % kRingBlk));
-            if (in1) mbar_arrive(bar_at(bempty_in, (ti + 1u) % kRingBlk));
-            mbar_arrive(bar_at(cempty, t % kCostSlots));
-            mbar_arrive(bar_at(cempty, (t + 1u) % kCostSlots));
-
-            float o0[kSub], o1[kSub];  // the strip's two bottom rows (lane 30)
-            float ol[kSub];            // subsequence DP: row La-1 (lane of has_last)
-            (void)ol;
-            float fw[R];  // backpointer fields of a sub-chunk, bits 2u, 2u+1
-            uint32_t word[R];
-#pragma unroll
-            for (int k = 0; k < R; ++k) fw[k] = 0.0f;
-            sweep_full<R, kSubseq, kT>(cA, gA0, gA1, j0 == 0, is_origin, srcA, w12, ghost, mu, cur,
-                                       prv, ylp, fw, o0, o1, ol, kl);
-            if constexpr (kSubseq)
-                if (has_last) store_lastrow(p.lastrow + j0, kSub, ol);
-#pragma unroll
-            for (int k = 0; k < R; ++k) word[k] = field_bits(fw[k], 0);
-            if (to_ring && lane == kOutLane) {
-                store_border(smem_u32(&nextring[to % kRingBlk][0][0]), o0, o1);
-                mbar_arrive(bar_at(bfull_out, to % kRingBlk));
-            }
-#pragma unroll
-            for (int k = 0; k < R; ++k) fw[k] = 0.0f;
-            sweep_full<R, kSubseq, kT>(cB, gB0, gB1, false, is_origin, srcA, w12, ghost, mu, cur,
-                                       prv, ylp, fw, o0, o1, ol, kl);
-            if constexpr (kSubseq)
-                if (has_last) store_lastrow(p.lastrow + j0 + kSub, kSub, ol);
-#pragma unroll
-            for (int k = 0; k < R; ++k) word[k] |= field_bits(fw[k], 1);
-            if (to_ring && lane == kOutLane) {
-                store_border(smem_u32(&nextring[(to + 1u) % kRingBlk][0][0]), o0, o1);
-                mbar_arrive(bar_at(bfull_out, (to + 1u) % kRingBlk));
-            }
-            if constexpr (kT) {
-#pragma unroll
-                for (int k = 0; k < R; ++k) word[k] = transpose_fields(word[k]);
-            }
-            store_words<R>(p.bp + ((size_t)strip * p.nchunk + (size_t)(j0 >> 4)) * (32 * R) +
-                               (size_t)lane * R,
-                           word);
+        sts64_if(dst + (unsigned)(kSub - 1) * 8u, s.cur[R - 2], s.cur[R - 1], st);
+        if constexpr (kSubseq) {  // row La-1 of these columns
+            float* d = p.lastrow + n * kSub;
+            stg128_if(d, ol[0], ol[1], ol[2], ol[3], has_last);
+            stg128_if(d + 4, ol[4], ol[5], ol[6], ol[7], has_last);
         }
-        // the last, ragged word: its one or two sub-chunks one at a time
-        for (int js = jfull; js < jend; js += kSub) {
-            const int n = js / kSub;
-            const int nsteps = min(kSub, Lb - js);
-            const unsigned ti = rin + (unsigned)(n - rp.x), to = rout + (unsigned)(n - rg.x);
-            const unsigned t = csub + (unsigned)(n - rg.x);
-            const bool have_in = from_ring && n < rp.y;
-            const bool need_out = to_ring && ((n - rg.x) & 3) == 0;
-            const unsigned tl = to + 3u;
-            if (have_in && !mbar_wait(bar_at(bfull_in, ti % kRingBlk), use_parity(ti, kRingBlk), p.ctl,
-                                      p.timeout_ns, 1))
-                return;
-            if (need_out && !mbar_wait(bar_at(bempty_out, tl % kRingBlk),
-                                       use_parity(tl, kRingBlk) ^ 1u, p.ctl, p.timeout_ns, 2))
-                return;
-            if (!mbar_wait(bar_at(cfull, t % kCostSlots), use_parity(t, kCostSlots), p.ctl,
-                           p.timeout_ns, 7))
-                return;
-            float g0[kSub], g1[kSub], c[R][kSub];
-            load_border(have_in ? smem_u32(&myring[ti % kRingBlk][0][0]) : inf_blk, g0, g1);
-            load_costs<R, kRM>(cring, t, lane, c);
-            if (have_in) mbar_arrive(bar_at(bempty_in, ti % kRingBlk));
-            mbar_arrive(bar_at(cempty, t % kCostSlots));
-            float o0[kSub], o1[kSub], ol[kSub], fw[R];
-            (void)ol;
 #pragma unroll
-            for (int k = 0; k < R; ++k) fw[k] = 0.0f;
-            sweep_sub<R, kSubseq, kT>(c, g0, g1, nsteps, js == 0, is_origin, srcA, w12, ghost, mu, cur,
-                                      prv, ylp, fw, o0, o1, ol, kl);
-            if constexpr (kSubseq)
-                if (has_last) store_lastrow(p.lastrow + js, nsteps, ol);
-            if (to_ring && lane == kOutLane) {
-                store_border(smem_u32(&nextring[to % kRingBlk][0][0]), o0, o1);
-                mbar_arrive(bar_at(bfull_out, to % kRingBlk));
-            }
-            // the word's fields: the first sub-chunk's are the low half
-            const int h = (js / kSub) & 1;
-            uint32_t word[R];
+        for (int k = 0; k < R; ++k) word[k] |= field_bits(fw[k], h);
+    };
+    // the loads of use t behind the shuffles of columns kFirst, kFirst + 1, ...
+    auto part = [&](SubIn<R>& in, unsigned t, int u) {
+        if (u >= kFirst) {
 #pragma unroll
-            for (int k = 0; k < R; ++k) word[k] = field_bits(fw[k], h);
-            if (h == 0) {
-                // keep the low half for the second sub-chunk, if there is one
-                if (js + kSub < jend) {
-#pragma unroll
-                    for (int k = 0; k < R; ++k) tailw[k] = word[k];
-                    continue;
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < R; ++k) word[k] |= tailw[k];
-            }
-            if constexpr (kT) {
-#pragma unroll
-                for (int k = 0; k < R; ++k) word[k] = transpose_fields(word[k]);
-            }
-            store_words<R>(p.bp + ((size_t)strip * p.nchunk + (size_t)(js >> 4)) * (32 * R) +
-                               (size_t)lane * R,
-                           word);
+            for (int z = 0; z < kPer; ++z)
+                if (kPer * (u - kFirst) + z < kLoads)
+                    load_part<R, kRM>(in, cring + (t % kSlots) * Slot::kBytes, lane,
+                                      kPer * (u - kFirst) + z);
         }
-    } else {
-        // costs of the first sub-chunk
-        float c[R][kSub];
-        if (!mbar_wait(bar_at(cfull, csub % kCostSlots), use_parity(csub, kCostSlots), p.ctl,
-                       p.timeout_ns, 7))
-            return;
-        load_costs<R, kRM>(cring, csub, lane, c);
-        mbar_arrive(bar_at(cempty, csub % kCostSlots));
-
-        const int jend = min(rg.y * kSub, Lb);
-        for (int j0 = rg.x * kSub; j0 < jend; j0 += kColsPerWord) {
-            uint32_t word[R];
+    };
+    auto test = [&](unsigned t) -> int {
+        return mbar_test_wait(bar_at(cfull, t % kSlots), use_parity(t, kSlots));
+    };
+    auto store = [&](int n, uint32_t* word) {
+        if constexpr (kT) {
 #pragma unroll
-            for (int k = 0; k < R; ++k) word[k] = 0;
-            // the two sub-chunks of a backpointer word: not unrolled (half the
-            // code of the sweep loop; measured 4-5% faster on a long pair)
+            for (int k = 0; k < R; ++k) word[k] = transpose_fields(word[k]);
+        }
+        store_words<R>(p.bp + ((size_t)strip * p.nchunk + (size_t)(n >> 1)) * (32 * R) +
+                           (size_t)lane * R,
+                       word);
+    };
+
+    int n = rg.x;  // even: ranges start on whole words
+    unsigned t = csub;
+    SubIn<R> ia, ib;
+    if (!wait_load(t, ia)) return;
+    release(t);
 #pragma unroll 1
-            for (int h = 0; h < kColsPerWord / kSub; ++h) {
-                const int js = j0 + h * kSub;
-                if (js >= jend) break;
-                const int n = js / kSub;
-                const int nsteps = min(kSub, Lb - js);
-                const unsigned ti = rin + (unsigned)(n - rp.x), to = rout + (unsigned)(n - rg.x);
-                const unsigned t = csub + (unsigned)(n - rg.x);
-
-                // The three waits of a sub-chunk -- the border rows top-2, top-1
-                // of columns js .. js+7 from the ring above (the group's top
-                // border is +inf in group 0, and so are the columns the strip
-                // above did not sweep: the +inf block inf_blk), every 4 blocks the
-                // output ring (the consumer empties it in order, so once the
-                // previous use of block to+3 is consumed so are those of to ..
-                // to+2), and the costs (the cost warp runs up to kCostSlots
-                // sub-chunks ahead, so they are normally there) -- are first
-                // tested together without blocking, so that their latencies
-                // overlap; only a barrier not yet complete is waited for.
-                const bool have_in = from_ring && n < rp.y;
-                const bool need_out = to_ring && ((n - rg.x) & 3) == 0;
-                const bool need_cost = n > rg.x;
-                const unsigned tl = to + 3u;
-                const int rb = have_in ? mbar_test_wait(bar_at(bfull_in, ti % kRingBlk),
-                                                        use_parity(ti, kRingBlk))
-                                       : 1;
-                const int ro = need_out ? mbar_test_wait(bar_at(bempty_out, tl % kRingBlk),
-                                                         use_parity(tl, kRingBlk) ^ 1u)
-                                        : 1;
-                const int rc = need_cost ? mbar_test_wait(bar_at(cfull, t % kCostSlots),
-                                                          use_parity(t, kCostSlots))
-                                         : 1;
-                if (!__all_sync(kFull, rb) &&
-                    !mbar_wait_slow(bar_at(bfull_in, ti % kRingBlk), use_parity(ti, kRingBlk), p.ctl,
-                                    p.timeout_ns, 1))
-                    return;
-                if (!__all_sync(kFull, ro) &&
-                    !mbar_wait_slow(bar_at(bempty_out, tl % kRingBlk), use_parity(tl, kRingBlk) ^ 1u,
-                                    p.ctl, p.timeout_ns, 2))
-                    return;
-                if (!__all_sync(kFull, rc) &&
-                    !mbar_wait_slow(bar_at(cfull, t % kCostSlots), use_parity(t, kCostSlots), p.ctl,
-                                    p.timeout_ns, 7))
-                    return;
-                float gv0[kSub], gv1[kSub];
-                {
-                    const unsigned s0 = have_in ? smem_u32(&myring[ti % kRingBlk][0][0]) : inf_blk;
-                    const float4 a0 = lds128(s0), a1 = lds128(s0 + 16);
-                    const float4 b0 = lds128(s0 + 32), b1 = lds128(s0 + 48);
-                    gv0[0] = a0.x; gv0[1] = a0.y; gv0[2] = a0.z; gv0[3] = a0.w;
-                    gv0[4] = a1.x; gv0[5] = a1.y; gv0[6] = a1.z; gv0[7] = a1.w;
-                    gv1[0] = b0.x; gv1[1] = b0.y; gv1[2] = b0.z; gv1[3] = b0.w;
-                    gv1[4] = b1.x; gv1[5] = b1.y; gv1[6] = b1.z; gv1[7] = b1.w;
-                }
-                // this sub-chunk's costs (loaded here rather than half-way through
-                // the previous sub-chunk keeps the 8 steps below one straight-line
-                // block: measured 8% faster)
-                if (need_cost) load_costs<R, kRM>(cring, t, lane, c);
-                if (have_in) mbar_arrive(bar_at(bempty_in, ti % kRingBlk));
-                if (need_cost) mbar_arrive(bar_at(cempty, t % kCostSlots));
-                float o0[kSub], o1[kSub];  // the strip's two bottom rows (lane 30)
-                float ol[kSub];            // subsequence DP: row La-1 (lane of has_last)
-                (void)ol;
-                float fw[R];  // backpointer fields of the sub-chunk, bits 2u, 2u+1
+    for (; n + 1 < nfull; n += 2, t += 2) {
+        uint32_t word[R], wordb[R];
 #pragma unroll
-                for (int k = 0; k < R; ++k) fw[k] = 0.0f;
-                if (nsteps == kSub) {
+        for (int k = 0; k < R; ++k) word[k] = wordb[k] = 0u;
+        // out.first is even too; blocks n and n + 1 of the output ring are free
+        // (those of a group's first trips, later ones by the test below)
+        const bool on = n >= out.first && n < out.end;
+        const bool st = on && lane == kOutLane;
+        const bool more = n + 2 < rg.y;
+        const bool next_on = n + 2 >= out.first && n + 2 < out.end;
+        const unsigned to = out.t0 + (unsigned)(n - out.first);
+        const unsigned dst0 = out.base + (to % kSlots) * out.stride;
+        const unsigned dst1 = out.base + ((to + 1u) % kSlots) * out.stride;
+        int rb = 1, ra = 1, ro = 1;
+        full_sub(n, ia, 0, dst0, st, word, [&](int u) {
+            if (u == kFirst) rb = test(t + 1u);
+            part(ib, t + 1u, u);
+        });
+        mbar_arrive_if(bar_at(out.full, to % kSlots), st);
+        const DpState<R> before = s;
+        full_sub(n + 1, ib, 1, dst1, st, wordb, [&](int u) {
+            if (u == 0)  // its consumer empties the output ring in order
+                ro = mbar_test_wait(bar_at(out.empty, (to + 3u) % kSlots),
+                                    use_parity(to + 3u, kSlots) ^ 1u);
+            if (u == kFirst) ra = test(t + 2u);
+            part(ia, t + 2u, u);
+        });
+        if (!__all_sync(kFull, rb & (ra | (int)!more) & (ro | (int)!next_on))) {
+            if (!__all_sync(kFull, rb)) {
+                if (!wait_load(t + 1u, ib)) return;
+                s = before;
 #pragma unroll
-                    for (int u = 0; u < kSub; ++u) {
-                        float cu[R];
-#pragma unroll
-                        for (int k = 0; k < R; ++k) cu[k] = c[k][u];
-                        dp_step<R, kSubseq, kT>(cu, u, srcA, w12, ghost, gv0[u], gv1[u],
-                                            (kSubseq || ((h == 0) && (u == 0) && (j0 == 0))) &&
-                                                is_origin,
-                                            mu, cur, prv, ylp, fw, o0[u], o1[u]);
-                        if constexpr (kSubseq) ol[u] = pick_row<R>(cur, kl);
-                    }
-                } else {
-                    // the last, partial sub-chunk
-#pragma unroll
-                    for (int u = 0; u < kSub; ++u) {
-                        if (u >= nsteps) break;
-                        float cu[R];
-#pragma unroll
-                        for (int k = 0; k < R; ++k) cu[k] = c[k][u];
-                        dp_step<R, kSubseq, kT>(cu, u, srcA, w12, ghost, gv0[u], gv1[u],
-                                            (kSubseq || ((h == 0) && (u == 0) && (j0 == 0))) &&
-                                                is_origin,
-                                            mu, cur, prv, ylp, fw, o0[u], o1[u]);
-                        if constexpr (kSubseq) ol[u] = pick_row<R>(cur, kl);
-                    }
-                }
-                if constexpr (kSubseq) {
-                    if (has_last) {  // row La-1 of these columns
-                        float* dst = p.lastrow + js;
-                        if (nsteps == kSub) {
-                            reinterpret_cast<float4*>(dst)[0] = make_float4(ol[0], ol[1], ol[2], ol[3]);
-                            reinterpret_cast<float4*>(dst)[1] = make_float4(ol[4], ol[5], ol[6], ol[7]);
-                        } else {
-#pragma unroll
-                            for (int u = 0; u < kSub; ++u)
-                                if (u < nsteps) dst[u] = ol[u];
-                        }
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < R; ++k) word[k] |= field_bits(fw[k], h);
-                if (to_ring && lane == kOutLane) {
-                    const unsigned d0 = smem_u32(&nextring[to % kRingBlk][0][0]);
-                    sts128(d0, make_float4(o0[0], o0[1], o0[2], o0[3]));
-                    sts128(d0 + 16, make_float4(o0[4], o0[5], o0[6], o0[7]));
-                    sts128(d0 + 32, make_float4(o1[0], o1[1], o1[2], o1[3]));
-                    sts128(d0 + 48, make_float4(o1[4], o1[5], o1[6], o1[7]));
-                    mbar_arrive(bar_at(bfull_out, to % kRingBlk));
-                }
-
+                for (int k = 0; k < R; ++k) wordb[k] = 0u;
+                full_sub(n + 1, ib, 1, dst1, st, wordb, [](int) {});
             }
-            if constexpr (kT) {
-#pragma unroll
-                for (int k = 0; k < R; ++k) word[k] = transpose_fields(word[k]);
-            }
-            store_words<R>(p.bp + ((size_t)strip * p.nchunk + (size_t)(j0 >> 4)) * (32 * R) +
-                               (size_t)lane * R,
-                           word);
+            // nothing is held back while this warp waits: what feeds the next
+            // slot may itself wait for this one's release
+            mbar_arrive_if(bar_at(out.full, (to + 1u) % kSlots), st);
+            release(t + 1u);
+            if (more && !wait_load(t + 2u, ia)) return;
+            if (next_on && !mbar_wait(bar_at(out.empty, (to + 3u) % kSlots),
+                                      use_parity(to + 3u, kSlots) ^ 1u, p.ctl, p.timeout_ns, 2))
+                return;
+            __syncwarp();
+        } else {
+            mbar_arrive_if(bar_at(out.full, (to + 1u) % kSlots), st);
+            release(t + 1u);
         }
+        mbar_arrive_if(bar_at(cempty, (t + 2u) % kSlots), lane == 0 && more);
+#pragma unroll
+        for (int k = 0; k < R; ++k) word[k] |= wordb[k];
+        store(n, word);
+    }
+    // up to two sub-chunks are left: a full one without a partner, and the
+    // ragged one at the end of B; one at a time
+    if (n < rg.y) {
+        uint32_t word[R];
+#pragma unroll
+        for (int k = 0; k < R; ++k) word[k] = 0u;
+        const int n0 = n;
+#pragma unroll 1
+        for (; n < rg.y; ++n, ++t) {
+            const int nsteps = min(kSub, p.Lb - n * kSub);
+            const bool on = n >= out.first && n < out.end;
+            const unsigned to = out.t0 + (unsigned)(n - out.first);
+            if (on && !mbar_wait(bar_at(out.empty, to % kSlots), use_parity(to, kSlots) ^ 1u, p.ctl,
+                                 p.timeout_ns, 2))
+                return;
+            const bool st = on && lane == kOutLane;
+            const unsigned dst = out.base + (to % kSlots) * out.stride;
+            float fw[R];
+#pragma unroll
+            for (int k = 0; k < R; ++k) fw[k] = 0.0f;
+#pragma unroll
+            for (int u = 0; u < kSub; ++u) {
+                if (u >= nsteps) break;
+                sweep_col<R, kSubseq, kT>(ia, u, (kSubseq || (n == 0 && u == 0)) && is_origin, srcA,
+                                          ghost, mu, s, fw, [] {});
+                sts64_if(dst + (unsigned)u * 8u, s.cur[R - 2], s.cur[R - 1], st);
+                if constexpr (kSubseq)
+                    if (has_last) p.lastrow[n * kSub + u] = pick_row<R>(s.cur, kl);
+            }
+            mbar_arrive_if(bar_at(out.full, to % kSlots), st);
+#pragma unroll
+            for (int k = 0; k < R; ++k) word[k] |= field_bits(fw[k], 0) << (16 * (n - n0));
+            if (n + 1 < rg.y) {
+                if (!wait_load(t + 1u, ia)) return;
+                release(t + 1u);
+            }
+        }
+        store(n0, word);
     }
 #pragma unroll
     for (int k = 0; k < R; ++k)
-        if (!ghost && i0 + k == p.La - 1) *p.e_final = cur[k];
-    if (kFlag) {
-        // the strip's words are all stored: raise its flag for the band map
-        __threadfence();
-        __syncwarp();
-        if (lane == 0) st_release_g(done + strip, p.epoch);
-    }
+        if (!ghost && i0 + k == p.La - 1) *p.e_final = s.cur[k];
 }
 
 // Reader warp (groups g > 0): the bottom rows of group g-1 from the global
-// border into ring 0.  Lane v < 16 carries value v of every sub-chunk
-// (column v % 8, row v / 8); loads run kAheadSub sub-chunks ahead, and a
-// value whose tag is not yet this call's is re-polled (bounded).
+// border into the border part of the first strip's slots.  Lane v < 16 carries
+// value v of every sub-chunk (column v / 2, row top-2 + v % 2); loads run
+// kAheadSub sub-chunks ahead, and a value whose tag is not yet this call's is
+// re-polled (bounded).  grow: the row of the global border (one per group, in a
+// cluster one per ticket: only its last CTA publishes there).
 constexpr int kAheadSub = 4;
-__device__ __forceinline__ void run_reader(const DpArgs& p, int g, int lane, float (*ring0)[2][kSub],
-                                           unsigned bfull0, unsigned bempty0, unsigned rbase,
-                                           int nfirst, int nsub, int clo, int chi) {
+template <int kSlots>
+__device__ __forceinline__ void run_reader(const DpArgs& p, int grow, int lane, unsigned border,
+                                           unsigned stride, unsigned full, unsigned empty,
+                                           unsigned csub, int nfirst, int nsub, int clo, int chi) {
     // blocks nfirst .. nsub-1 (this group's first strip's range); only columns
     // clo .. chi-1 were published above (the others read as +inf)
     const int Lb = p.Lb;
     clo = max(clo, 0);
     chi = min(chi, Lb);
-    const unsigned long long* gin = p.gborder + (size_t)(g - 1) * Lb * 2;
+    const unsigned long long* gin = p.gborder + (size_t)grow * Lb * 2;
     const unsigned epoch = p.epoch;
     const bool act_lane = lane < 2 * kSub;
-    const int cofs = lane & (kSub - 1), row = (lane >> 3) & 1;
+    const int cofs = (lane >> 1) & (kSub - 1), row = lane & 1;
     unsigned long long pend[kAheadSub];
 #pragma unroll
     for (int q = 0; q < kAheadSub; ++q) {
@@ -1081,196 +911,117 @@ __device__ __forceinline__ void run_reader(const DpArgs& p, int g, int lane, flo
                     }
                 }
             }
-            const unsigned t = rbase + (unsigned)(n - nfirst);
-            if (!mbar_wait(bar_at(bempty0, t % kRingBlk), use_parity(t, kRingBlk) ^ 1u, p.ctl,
+            const unsigned t = csub + (unsigned)(n - nfirst);
+            if (!mbar_wait(bar_at(empty, t % kSlots), use_parity(t, kSlots) ^ 1u, p.ctl,
                            p.timeout_ns, 8))
                 return;
-            if (act_lane) ring0[t % kRingBlk][row][cofs] = act ? val_of(pend[q]) : INFINITY;
-            mbar_arrive(bar_at(bfull0, t % kRingBlk));
+            if (act_lane)
+                sts32(border + (t % kSlots) * stride + (unsigned)lane * 4u,
+                      act ? val_of(pend[q]) : INFINITY);
+            __syncwarp();
+            mbar_arrive_if(bar_at(full, t % kSlots), lane == 0);
             const int ncol = col + kAheadSub * kSub;
             if (act_lane && ncol >= clo && ncol < chi) pend[q] = ldg1(gin + (size_t)ncol * 2 + row);
         }
     }
 }
 
-// Writer warp: the last DP slot's bottom rows from ring NS to the global
-// border of group g, as (value, epoch) words; lanes 0..15 store one
+// Writer warp: the last strip's bottom rows from the writer's ring to the
+// global border of group g, as (value, epoch) words; lanes 0..15 store one
 // coalesced 128-byte line per sub-chunk.
-__device__ __forceinline__ void run_writer(const DpArgs& p, int g, int lane,
-                                           float (*ringo)[2][kSub], unsigned bfullo,
+template <int kSlots>
+__device__ __forceinline__ void run_writer(const DpArgs& p, int grow, int lane,
+                                           const float (*ringo)[2 * kSub], unsigned bfullo,
                                            unsigned bemptyo, unsigned rbase, int nfirst,
                                            int nsub) {
     const int Lb = p.Lb;
-    unsigned long long* gout = p.gborder + (size_t)g * Lb * 2;
+    unsigned long long* gout = p.gborder + (size_t)grow * Lb * 2;
     const unsigned epoch = p.epoch;
-    const int cofs = lane & (kSub - 1), row = (lane >> 3) & 1;
     for (int n = nfirst; n < nsub; ++n) {
         const unsigned t = rbase + (unsigned)(n - nfirst);
-        if (!mbar_wait(bar_at(bfullo, t % kRingBlk), use_parity(t, kRingBlk), p.ctl, p.timeout_ns,
-                       9))
+        if (!mbar_wait(bar_at(bfullo, t % kSlots), use_parity(t, kSlots), p.ctl, p.timeout_ns, 9))
             return;
-        const float v = ringo[t % kRingBlk][row][cofs];
-        mbar_arrive(bar_at(bemptyo, t % kRingBlk));
-        const int col = n * kSub + cofs;
-        if (lane < 2 * kSub && col < Lb) stg1(gout + (size_t)col * 2 + row, pack(v, epoch));
-    }
-}
-
-// Cluster links.  Between two CTAs of one cluster the border goes through
-// a staging ring of kRingBlk blocks in the shared memory of the CTA below
-// (`link`, full barriers `lfull` there, empty barriers `lempty` in the CTA
-// above); the DP warps' own rings are untouched, so their sweep is the same
-// code with or without clusters.  Producer and consumer count the link's
-// uses as the blocks of the strip above's range, in order.
-
-// Writer warp of a CTA with another CTA of its cluster below: every block of
-// the last strip's range [nfirst, nsub) from ring NS into the staging ring of
-// CTA crank + 1 (lanes 0..15: value v = column v % 8 of row v / 8), each
-// value an asynchronous store completing 4 of the 64 bytes its full barrier
-// expects.
-__device__ __forceinline__ void run_link_writer(const DpArgs& p, int lane, float (*ringo)[2][kSub],
-                                                unsigned bfullo, unsigned bemptyo, unsigned rbase,
-                                                int nfirst, int nsub, unsigned link_s,
-                                                unsigned lfull_s, unsigned lempty_s,
-                                                unsigned lbase, unsigned crank) {
-    const int cofs = lane & (kSub - 1), row = (lane >> 3) & 1;
-    for (int n = nfirst; n < nsub; ++n) {
-        const unsigned t = rbase + (unsigned)(n - nfirst);  // use of ring NS
-        const unsigned u = lbase + (unsigned)(n - nfirst);  // use of the link
-        if (!mbar_wait(bar_at(bfullo, t % kRingBlk), use_parity(t, kRingBlk), p.ctl, p.timeout_ns,
-                       9))
-            return;
-        // the link block's previous use has been read below
-        if (!mbar_wait(bar_at(lempty_s, u % kRingBlk), use_parity(u, kRingBlk) ^ 1u, p.ctl,
-                       p.timeout_ns, 10))
-            return;
-        const float v = ringo[t % kRingBlk][row][cofs];
-        mbar_arrive(bar_at(bemptyo, t % kRingBlk));
-        if (lane < 2 * kSub)
-            st_async_f32(map_rank(link_s + (u % kRingBlk) * (2 * kSub * 4) +
-                                      (unsigned)(row * kSub + cofs) * 4u,
-                                  crank + 1),
-                         v, map_rank(bar_at(lfull_s, u % kRingBlk), crank + 1));
-    }
-}
-
-// Reader warp of a CTA with another CTA of its cluster above: ring 0 for the
-// first strip's range [nfirst, nsub) from the staging ring, which carries
-// the strip above's range [pa, pb): blocks of it before nfirst (or after
-// nsub) are consumed unread, blocks of the strip's range past pb read +inf.
-// Lane 0 re-arms a consumed block's full barrier for its next use and then
-// arrives on the sender's empty barrier, with a count that depends on the
-// value it loaded (the warp's loads of the block are one instruction).
-__device__ __forceinline__ void run_link_reader(const DpArgs& p, int lane, float (*ring0)[2][kSub],
-                                                unsigned bfull0, unsigned bempty0, unsigned rbase,
-                                                int nfirst, int nsub, int pa, int pb,
-                                                float (*link)[2][kSub], unsigned lfull_s,
-                                                unsigned lempty_s, unsigned lbase,
-                                                unsigned crank) {
-    const int cofs = lane & (kSub - 1), row = (lane >> 3) & 1;
-    auto release = [&](unsigned u, unsigned dep) {
-        if (lane == 0) {
-            mbar_arrive_expect_tx(bar_at(lfull_s, u % kRingBlk), 2 * kSub * 4);
-            mbar_arrive_remote_relaxed(map_rank(bar_at(lempty_s, u % kRingBlk), crank - 1),
-                                       1u + zero_after(dep));
-        }
+        const float v = ringo[t % kSlots][lane & (2 * kSub - 1)];
+        const int col = n * kSub + ((lane >> 1) & (kSub - 1));
+        if (lane < 2 * kSub && col < Lb) stg1(gout + (size_t)col * 2 + (lane & 1), pack(v, epoch));
         __syncwarp();
-    };
-    auto skip = [&](int n) -> int {
-        const unsigned u = lbase + (unsigned)(n - pa);
-        if (!mbar_wait(bar_at(lfull_s, u % kRingBlk), use_parity(u, kRingBlk), p.ctl,
-                       p.timeout_ns, 11))
-            return 0;
-        release(u, 0u);
-        return 1;
-    };
-    for (int n = pa; n < min(nfirst, pb); ++n)
-        if (!skip(n)) return;
-    for (int n = nfirst; n < nsub; ++n) {
-        const unsigned t = rbase + (unsigned)(n - nfirst);  // use of ring 0
-        float v = INFINITY;
-        if (n >= pa && n < pb) {
-            const unsigned u = lbase + (unsigned)(n - pa);
-            if (!mbar_wait(bar_at(lfull_s, u % kRingBlk), use_parity(u, kRingBlk), p.ctl,
-                           p.timeout_ns, 11))
-                return;
-            v = link[u % kRingBlk][row][cofs];
-            release(u, __float_as_uint(v));
-        }
-        if (!mbar_wait(bar_at(bempty0, t % kRingBlk), use_parity(t, kRingBlk) ^ 1u, p.ctl,
-                       p.timeout_ns, 8))
-            return;
-        if (lane < 2 * kSub) ring0[t % kRingBlk][row][cofs] = v;
-        mbar_arrive(bar_at(bfull0, t % kRingBlk));
+        mbar_arrive_if(bar_at(bemptyo, t % kSlots), lane == 0);
     }
-    for (int n = max(pa, max(nsub, nfirst)); n < pb; ++n)
-        if (!skip(n)) return;
 }
 
-// Band-map item `item` of the pair (band-major: band item / nseg, column
-// segment item % nseg) by all NT threads of the CTA, once the strips covering
-// the band have raised their flags.  The wait (thread 0) gives up when the
-// call has failed elsewhere, or when no flag it waits for has come up for
-// 8 x the handoff limit (DTW_ERR_TIMEOUT, detail 6): a strip's whole sweep
-// lies between the item's start and its flag, not just one handoff.
-template <int NT>
-__device__ __noinline__ void run_bandmap_item(const DpArgs& p, const MapArgs& m, int item,
-                                              int (*s_x)[NT][3]) {
-    __shared__ int s_ok;
-    const BtArgs& bt = m.bt;
-    constexpr int kWidth = NT * kColsPerWord - 2 * kBand;
-    const int nseg = (bt.Lb + kWidth - 1) / kWidth;
-    const int b = item / nseg, segx = item - b * nseg;
-    const int s0 = (b * kBand) / p.rps;
-    const int s1 = (min((b + 1) * kBand, p.La) - 1) / p.rps;
-    auto ready = [&]() -> int {
-        if (threadIdx.x == 0) {
-            int ok = 1;
-            long long t0 = global_ns();
-            for (int s = s0; s <= s1 && ok; ++s)
-                for (int poll = 0;; ++poll) {
-                    if (ld_acquire_g(m.done + s) == p.epoch) {
-                        t0 = global_ns();
-                        break;
-                    }
-                    if (read_status(p.ctl) != 0) {
-                        ok = 0;
-                        break;
-                    }
-                    if (global_ns() - t0 > 8 * p.timeout_ns) {
-                        raise_status(p.ctl, DTW_ERR_TIMEOUT, 6);
-                        ok = 0;
-                        break;
-                    }
-                    if (poll >= 4) __nanosleep(256);
-                }
-            s_ok = ok;
+// Writer warp of a CTA with another CTA of its cluster below: the blocks of
+// the last strip's range [nfirst, nsub) from the writer's ring into the slots
+// of the first strip of CTA crank + 1, whose range starts at block bfirst with
+// lifetime use bsub of its slots; each of the 16 values an asynchronous store
+// completing 4 of the 64 bytes the slot's full barrier expects.  (Blocks before
+// bfirst are not needed below.)  Use lv of the link, counted from lsub, waits
+// until the reader warp below has handed use lv - kSlots back on `lempty`: the slot's
+// previous use in this ticket (those of earlier tickets are all released).
+template <int kSlots>
+__device__ __forceinline__ void run_link_writer(const DpArgs& p, int lane,
+                                                const float (*ringo)[2 * kSub], unsigned bfullo,
+                                                unsigned bemptyo, unsigned rbase, int nfirst,
+                                                int nsub, unsigned border, unsigned stride,
+                                                unsigned full, unsigned lempty, unsigned lsub,
+                                                unsigned bsub, int bfirst, unsigned crank) {
+    // peer addresses (a CTA's window of the cluster's shared memory is linear)
+    const unsigned rborder = map_rank(border, crank + 1) + (unsigned)lane * 4u;
+    const unsigned rfull = map_rank(full, crank + 1);
+    for (int n = nfirst; n < nsub; ++n) {
+        const unsigned t = rbase + (unsigned)(n - nfirst);  // use of the writer's ring
+        const unsigned u = bsub + (unsigned)(n - bfirst);   // use of the slots below
+        const unsigned lv = lsub + (unsigned)(n - bfirst);  // use of the link
+        const bool send = n >= bfirst;
+        // the slot below is normally free long before the block is there
+        if (send && !mbar_wait(bar_at(lempty, lv % kSlots), use_parity(lv, kSlots) ^ 1u, p.ctl,
+                               p.timeout_ns, 10))
+            return;
+        if (!mbar_wait(bar_at(bfullo, t % kSlots), use_parity(t, kSlots), p.ctl, p.timeout_ns, 9))
+            return;
+        const float v = ringo[t % kSlots][lane & (2 * kSub - 1)];
+        if (send && lane < 2 * kSub)
+            st_async_f32(rborder + (u % kSlots) * stride, v, bar_at(rfull, u % kSlots));
+        __syncwarp();
+        mbar_arrive_if(bar_at(bemptyo, t % kSlots), lane == 0);
+    }
+}
+
+// Reader warp of a CTA with another CTA of its cluster above: the first
+// strip's blocks [nfirst, nsub), uses csub .. of its slots.  Those the CTA above
+// sends (before nsent; uses lsub .. of the link) it hands back once the DP warp
+// has released their slot; the later ones read +inf.  (It also stores those,
+// rather than the cost warp, so that no slot can be released twice before
+// this warp has seen the first release.)
+template <int kSlots>
+__device__ __forceinline__ void run_link_reader(const DpArgs& p, int lane, unsigned border,
+                                                unsigned stride, unsigned full, unsigned empty,
+                                                unsigned csub, int nfirst, int nsent, int nsub,
+                                                unsigned lempty, unsigned lsub, unsigned crank) {
+    for (int n = nfirst; n < nsub; ++n) {
+        const unsigned t = csub + (unsigned)(n - nfirst), slot = t % kSlots;
+        if (n < nsent) {
+            if (!mbar_wait(bar_at(empty, slot), use_parity(t, kSlots), p.ctl, p.timeout_ns, 11))
+                return;
+            const unsigned v = lsub + (unsigned)(n - nfirst);
+            if (lane == 0) mbar_arrive_remote_relaxed(map_rank(bar_at(lempty, v % kSlots), crank - 1));
+            __syncwarp();
+        } else {
+            if (!mbar_wait(bar_at(empty, slot), use_parity(t, kSlots) ^ 1u, p.ctl, p.timeout_ns, 8))
+                return;
+            if (lane < 2 * kSub) sts32(border + slot * stride + (unsigned)lane * 4u, INFINITY);
+            __syncwarp();
+            mbar_arrive_if(bar_at(full, slot), lane == 0);
         }
-        __syncthreads();
-        return s_ok;
-    };
-    if (bt.ranges)
-        bandmap_segment<NT, true, true>(bt, b, segx, s_x, ready);
-    else
-        bandmap_segment<NT, false, true>(bt, b, segx, s_x, ready);
+    }
 }
 
-// NS strips per CTA.  Warps 0..NS-1: the strips' cost warps; NS..2NS-1:
-// their DP warps; 2NS: the reader; 2NS+1: the writer.  Warp w runs on SM
-// sub-partition w % 4, so for NS = 2 each DP warp has a sub-partition of its
-// own and the helpers share those of the cost warps.  Persistent: a CTA
-// takes strip groups from the ticket counter until none are left, so a
-// group only ever waits on groups that started earlier.
+// NS strips per CTA: per strip its DP warp and kNC cost warps, and a reader and
+// a writer warp (their places: see `role`).  Persistent: a CTA takes strip
+// groups from the ticket counter until none are left, so a group only ever
+// waits on groups that started earlier.
 // kMany: the groups come from a work queue over many pairs (`many`, `item0`,
 // `ticket`; see launch_dp_split_many) instead of the pair `one`.
-// kMap (one pair): tickets past the strip groups are the map.nbm band-map
-// items of the pair's backtrace (map.bt, run_bandmap_item); every group has
-// been taken by a running CTA before the first item is, so an item only
-// waits on strips in progress.  For pairs whose groups outnumber the
-// resident CTAs: the CTAs of the last round that find no group then map the
-// bands above while the last strips sweep.  The launch bounds keep as many
-// CTAs per SM as the DP alone fits (split_ctas_per_sm).
-// kCl (one pair, no band map): the kernel runs in clusters of cn CTAs that
+// kCl (one pair): the kernel runs in clusters of cn CTAs that
 // take tickets together: ticket T gives CTA rank r the strip group
 // T cn + r, so the border between two of a ticket's groups goes through
 // distributed shared memory (run_link_writer, run_link_reader); only rank 0
@@ -1278,106 +1029,90 @@ __device__ __noinline__ void run_bandmap_item(const DpArgs& p, const MapArgs& m,
 // when its whole cluster does (no CTA's shared memory may disappear while a
 // peer can still reach it).
 template <int DP, int R, int NS, bool kMany, bool kBF, bool kSubseq = false, bool kT = false,
-          bool kMap = false, bool kCl = false>
+          bool kCl = false>
 __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
-                                  (kMap ? split_ctas_per_sm(R, NS, DP, kBF) : 1))
-    k_dp_split(const DpArgs one, const MapArgs map, const DpArgs* __restrict__ many,
-               const int* __restrict__ item0, int nmany, int* ticket) {
-    static_assert(!kCl || (!kMany && !kMap && !kSubseq), "clusters sweep one plain pair");
+                                  (kCl ? 1 : split_ctas_per_sm(R, NS, DP, kBF)))
+    k_dp_split(const DpArgs one, const DpArgs* __restrict__ many, const int* __restrict__ item0,
+               int nmany, int* ticket) {
+    static_assert(!kCl || (!kMany && !kSubseq), "clusters sweep one plain pair");
     constexpr int kThreads = split_threads<DP, NS, kBF>();
-    constexpr int kNC = CostWide<DP, kBF>::kNC;  // cost warps per strip
-    constexpr bool kWide = CostWide<DP, kBF>::kOn;
-    using S = BStage<DP>;
-    using M = SplitSmem<DP, R, kBF>;
-    __shared__ __align__(16) float ring[NS + 1][kRingBlk][2][kSub];
-    __shared__ __align__(8) unsigned long long bbar[NS * kNC][S::kSlots];
-    __shared__ __align__(8) unsigned long long cfull[NS][kCostSlots];
-    __shared__ __align__(8) unsigned long long cempty[NS][kCostSlots];
-    __shared__ __align__(8) unsigned long long bfull[NS + 1][kRingBlk];
-    __shared__ __align__(8) unsigned long long bempty[NS + 1][kRingBlk];
-    __shared__ __align__(16) float s_inf[2][kSub];  // +inf border block, never written after
+    using Cfg = CostCfg<DP, NS, kBF>;
+    constexpr int kSlots = slots_of<kCl>();
+    using M = SplitSmem<DP, R, NS, kBF, kCl>;
+    using Slot = SlotOf<R, kBF>;
+    constexpr int kNC = Cfg::kNC;  // cost warps per strip
+    constexpr int kBars = kBF ? kBfSlots : Cfg::kBSlots;
+    __shared__ __align__(16) float ringo[kSlots][2 * kSub];  // the writer's ring
+    __shared__ __align__(8) unsigned long long bbar[NS * kNC][kBars];
+    __shared__ __align__(8) unsigned long long cfull[NS][kSlots];
+    __shared__ __align__(8) unsigned long long cempty[NS][kSlots];
+    __shared__ __align__(8) unsigned long long ofull[kSlots];
+    __shared__ __align__(8) unsigned long long oempty[kSlots];
+    // releases of the slots of the CTA below, in a cluster
+    __shared__ __align__(8) unsigned long long lempty[kCl ? kSlots : 1];
     __shared__ int s_group, s_pair;
-    // cluster link into this CTA (staging ring, its full barriers) and out of
-    // it (the empty barriers of the staging ring of the CTA below)
-    __shared__ __align__(16) float link[kCl ? kRingBlk : 1][2][kSub];
-    __shared__ __align__(8) unsigned long long lfull[kCl ? kRingBlk : 1];
-    __shared__ __align__(8) unsigned long long lempty[kCl ? kRingBlk : 1];
     extern __shared__ __align__(128) unsigned char dyn[];  // NS * M::kStripBytes
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned crank = kCl ? cluster_rank() : 0u;
     const unsigned cn = kCl ? cluster_size() : 1u;
-    // warps 0 .. kNC NS - 1: cost warps (strip slot wid % NS, half wid / NS);
-    // then one DP warp per strip, the reader and the writer
-    const int role = wid < kNC * NS ? 0
-                                    : (wid < (kNC + 1) * NS ? 1 : (wid == (kNC + 1) * NS ? 2 : 3));
-    const int w = role == 0 ? wid % NS : (role == 1 ? wid - kNC * NS : 0);  // strip slot
-    const int half = role == 0 ? wid / NS : 0;
+    // Warp roles by SM sub-partition (warp w runs on sub-partition w % 4).  Two
+    // cost warps a strip: the DP warps (0, 1) share theirs with the reader and
+    // the writer (4, 5) only, the cost warps (2, 3 and 6, 7) have the other two
+    // (a DP warp beside a cost warp: 136 against 111 cycles a column on the
+    // 20000 x 25000 pair).  One cost warp a strip: the cost warps, the DP warps,
+    // then the reader and the writer.
+    int role, w = 0, half = 0;
+    if (NS == 1) {
+        role = wid == 0 ? 1 : (wid == 4 ? 2 : (wid == 5 ? 3 : 0));
+        half = wid < 4 ? wid - 1 : wid - 3;
+    } else if (NS == 2 && kNC >= 2) {
+        role = wid < 2 ? 1 : (wid == 4 ? 2 : (wid == 5 ? 3 : 0));
+        if (role < 2) w = wid & 1;
+        half = wid < 4 ? 0 : wid / 2 - 2;
+    } else {
+        role = wid < kNC * NS ? 0 : (wid < (kNC + 1) * NS ? 1 : (wid == (kNC + 1) * NS ? 2 : 3));
+        if (role < 2) w = role == 0 ? wid % NS : wid - kNC * NS;
+        half = role == 0 ? wid / NS : 0;
+    }
     unsigned char* mine = dyn + (size_t)w * M::kStripBytes;
     const unsigned cring_s = smem_u32(mine + M::kOperandBytes);
     const unsigned a_s = smem_u32(mine);                                  // kBF: A tile
-    const unsigned b_s = smem_u32(mine + 32 * R * kBfStride * 2);         // kBF: B ring
+    const unsigned b_s = smem_u32(mine + 32 * R * kBfStride * 2 + half * kBfSlots * kBfBlkBytes);  // kBF: B ring
     unsigned bbase = 0;  // kBF: lifetime count of this cost warp's B blocks
     const unsigned cfull_s = smem_u32(&cfull[w][0]);
     const unsigned cempty_s = smem_u32(&cempty[w][0]);
 
-    BRing<DP> br;
-    br.stage = reinterpret_cast<const float*>(mine);
-    br.stage_s = smem_u32(mine);
-    br.bar_s = smem_u32(&bbar[w][0]);
+    // the FP32 cost warps' rings of B: behind the A tile where there is one
+    BRing<DP, Cfg::kBSlots, Cfg::kBBlk> br;
+    br.stage_s = smem_u32(mine + (Cfg::kWide ? 32 * R * Cfg::kStride * 4 : 0) +
+                          half * BStage<DP, Cfg::kBSlots, Cfg::kBBlk>::kWarpBytes);
+    br.stage = reinterpret_cast<const float*>(mine);  // (not read through this pointer)
+    br.bar_s = smem_u32(&bbar[half * NS + w][0]);
     br.base = 0;
     br.first = 0;
     br.nblk = 0;
     br.issued = br.waited = 0;
-    // the wide FP32 cost warps: A tile, then a B ring per half (two chunks)
-    using WS = BStage<DP, CostWide<DP, kBF>::kBSlots>;
-    BRing<DP, CostWide<DP, kBF>::kBSlots> bw;
-    bw.stage_s = smem_u32(mine + 32 * R * CostWide<DP, kBF>::kStride * 4 + half * WS::kWarpBytes);
-    bw.stage = reinterpret_cast<const float*>(mine);  // (unused by the wide cost warp)
-    bw.bar_s = smem_u32(&bbar[half * NS + w][0]);
-    bw.base = 0;
-    bw.first = 0;
-    bw.nblk = 0;
-    bw.issued = bw.waited = 0;
-    if (threadIdx.x < 2 * kSub) (&s_inf[0][0])[threadIdx.x] = INFINITY;
     if (threadIdx.x == 0) {
         for (int s = 0; s < NS * kNC; ++s)
-            for (int k = 0; k < S::kSlots; ++k) mbar_init(smem_u32(&bbar[s][k]), 1);
-        for (int s = 0; s < NS; ++s) {
-            for (int k = 0; k < kCostSlots; ++k) {
-                mbar_init(smem_u32(&cfull[s][k]), kWarp);  // the lanes of the slot's cost warp
-                mbar_init(smem_u32(&cempty[s][k]), kWarp);  // the DP warp's lanes
+            for (int k = 0; k < kBars; ++k) mbar_init(smem_u32(&bbar[s][k]), 1);
+        for (int k = 0; k < kSlots; ++k) {
+            for (int s = 0; s < NS; ++s) {
+                mbar_init(smem_u32(&cfull[s][k]), 2);   // the slot's costs, its border
+                mbar_init(smem_u32(&cempty[s][k]), 1);  // the DP warp
             }
-        }
-        for (int s = 0; s <= NS; ++s)
-            for (int k = 0; k < kRingBlk; ++k) {
-                // ring 0 is filled by the reader's lanes, the others by lane 30
-                // of the DP warp above; every ring is emptied by a whole warp
-                mbar_init(smem_u32(&bfull[s][k]), s == 0 ? kWarp : 1);
-                mbar_init(smem_u32(&bempty[s][k]), kWarp);
-            }
-        if (kCl) {
-            // the staging ring: a full barrier completes on the reader's
-            // arrival and 64 bytes of asynchronous stores from the CTA above
-            // (armed here for the first uses); an empty barrier (of the link
-            // to the CTA below) on one arrival of that CTA's reader
-            for (int k = 0; k < kRingBlk; ++k) {
-                mbar_init(smem_u32(&lfull[k]), 1);
-                mbar_init(smem_u32(&lempty[k]), 1);
-            }
-            if (crank > 0)
-                for (int k = 0; k < kRingBlk; ++k)
-                    mbar_arrive_expect_tx(smem_u32(&lfull[k]), 2 * kSub * 4);
+            mbar_init(smem_u32(&ofull[k]), 1);   // lane 30 of the last strip's DP warp
+            mbar_init(smem_u32(&oempty[k]), 1);  // the writer
+            if (kCl) mbar_init(smem_u32(&lempty[k]), 1);  // the reader of the CTA below
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if constexpr (kCl) cluster_sync_all();  // every CTA's barriers before any remote access
-    // Lifetime sub-chunk counts of the cost rings and the border rings.
-    unsigned csub[NS], rsub[NS + 1];
+    // Lifetime sub-chunk counts of the slots and of the writer's ring, and (in
+    // a cluster) of the slots of the first strip of the CTA below and of the
+    // links into and out of this CTA.
+    unsigned csub[NS], osub = 0, lsub = 0, lin = 0, lout = 0;
 #pragma unroll
     for (int s = 0; s < NS; ++s) csub[s] = 0;
-#pragma unroll
-    for (int s = 0; s <= NS; ++s) rsub[s] = 0;
-    unsigned lin = 0, lout = 0;  // uses of the cluster links into and out of this CTA
 
     for (;;) {
         if constexpr (kCl) {
@@ -1395,7 +1130,7 @@ __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
             if ((long long)T * cn >= one.ngroups) break;  // the whole cluster leaves
             if (threadIdx.x == 0) s_group = T * (int)cn + (int)crank;
         } else {
-        __syncthreads();  // every warp finished the previous group
+            __syncthreads();  // every warp finished the previous group
         }
         if (!kCl && threadIdx.x == 0) {
             if (kMany) {
@@ -1419,120 +1154,132 @@ __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
                 s_group = gi;
             } else {
                 s_pair = 0;
-                s_group = read_status(one.ctl) != 0 ? one.ngroups + (kMap ? map.nbm : 0)
+                s_group = read_status(one.ctl) != 0 ? one.ngroups
                                                     : atomicAdd(&one.ctl->ticket, 1);
             }
         }
-        // +inf border: the top rows of group 0
-        float* rf = &ring[0][0][0][0];
-        for (int k = threadIdx.x; k < kRing * 2; k += blockDim.x) rf[k] = INFINITY;
         __syncthreads();
         if (kMany && s_pair < 0) return;
         if (kMany && s_group < 0) continue;  // nothing of a failed pair runs
         const DpArgs p = kMany ? many[s_pair] : one;
         const int g = s_group;
         if (kCl && g >= p.ngroups) continue;  // this CTA's group of the ticket does not exist
-        if (g >= p.ngroups) {
-            if constexpr (kMap) {
-                if (g - p.ngroups < map.nbm) {
-                    // left-neighbour exchange of the band map
-                    __shared__ int s_bm[2][kThreads][3];
-                    run_bandmap_item<kThreads>(p, map, g - p.ngroups, s_bm);
-                    continue;
-                }
-            }
-            return;
-        }
+        if (g >= p.ngroups) return;
         const GroupRoles gr = group_roles<NS>(p, g);
         const int strip = g * NS + w;
-        // the sub-chunk ranges of the group's strips (all columns without a band)
+        // the sub-chunk ranges of the group's strips, and of the strips above
+        // and below the group
         int2 rgs[NS];
 #pragma unroll
         for (int q = 0; q < NS; ++q)
             rgs[q] = q < gr.nstrips_here ? strip_range<kSubseq>(p, g * NS + q) : make_int2(0, 0);
+        const int2 above = g > 0 ? strip_range<kSubseq>(p, g * NS - 1) : make_int2(0, 0);
+        const int2 below = g + 1 < p.ngroups ? strip_range<kSubseq>(p, (g + 1) * NS) : make_int2(0, 0);
+        const bool link_in = kCl && crank > 0, link_out = kCl && crank + 1 < cn;
+        int2 rg = rgs[0], rup = above, rdown = below;  // of strip slot w and its neighbours
+        unsigned cs = csub[0], cs_down = 0;
+#pragma unroll
+        for (int q = 0; q < NS; ++q)
+            if (q == w) {
+                rg = rgs[q];
+                cs = csub[q];
+                if (q > 0) rup = rgs[q - 1];
+                if (q + 1 < NS) {
+                    rdown = rgs[q + 1 < NS ? q + 1 : q];
+                    cs_down = csub[q + 1 < NS ? q + 1 : q];
+                }
+            }
         if (role == 0) {
-            if (w < gr.nstrips_here)
-            {
+            if (w < gr.nstrips_here) {
+                // the border: from the strip above; none above strip 0; for the
+                // first strip the reader warp fills in what the group above lacks
+                BorderSrc bs;
+                bs.inf_from = strip == 0 ? 0 : (w > 0 ? rup.y : 0x7fffffff);
+                bs.link_end = w == 0 && g > 0 && link_in ? rup.y : 0;
                 if constexpr (kBF)
-                    run_cost_bf16<DP, R>(p, strip, lane, a_s, b_s, smem_u32(&bbar[w][0]), bbase,
-                                         cring_s, cfull_s, cempty_s, csub[w]);
-                else if constexpr (kWide)
-                    run_cost_wide<DP, R>(p, strip, w, half, lane, reinterpret_cast<float*>(mine),
-                                         cring_s, cfull_s, cempty_s, csub[w], bw);
+                    run_cost_bf16<DP, R, kNC, kSlots>(p, strip, w, half, lane, a_s, b_s,
+                                                      smem_u32(&bbar[half * NS + w][0]), bbase,
+                                         cring_s, cfull_s, cempty_s, cs, bs);
+                else if constexpr (Cfg::kWide)
+                    run_cost_wide<DP, R, NS, kSlots>(p, strip, w, half, lane, reinterpret_cast<float*>(mine),
+                                         cring_s, cfull_s, cempty_s, cs, bs, br);
                 else
-                    run_cost<DP, R, kSubseq>(p, strip, lane, cring_s, cfull_s, cempty_s, csub[w], br);
+                    run_cost<DP, R, NS, kSlots, kSubseq>(p, strip, half, lane, cring_s,
+                                                                cfull_s, cempty_s, cs, bs, br);
             }
         } else if (role == 1) {
-            if (w < gr.nstrips_here)
-                run_dp<R, NS, kBF, kSubseq, kT, kMap, (kBF || kWide), kWide>(p, gr, w, strip, lane, ring, smem_u32(&bfull[0][0]),
-                                   smem_u32(&bempty[0][0]), rsub[w], rsub[w + 1], cring_s,
-                                   cfull_s, cempty_s, csub[w], smem_u32(&s_inf[0][0]),
-                                   kMap ? map.done : nullptr);
+            if (w < gr.nstrips_here) {
+                OutRing out;
+                if (w + 1 < NS && w + 1 < gr.nstrips_here) {
+                    // the next strip's slots: its blocks, as far as this strip has them
+                    out.base = cring_s + (unsigned)M::kStripBytes + Slot::kBorder;
+                    out.stride = Slot::kBytes;
+                    out.full = cfull_s + 8u * kSlots;
+                    out.empty = cempty_s + 8u * kSlots;
+                    out.t0 = cs_down;
+                    out.first = rdown.x;
+                    out.end = rg.y;
+                } else {
+                    out.base = smem_u32(&ringo[0][0]);
+                    out.stride = kBorderBytes;
+                    out.full = smem_u32(&ofull[0]);
+                    out.empty = smem_u32(&oempty[0]);
+                    out.t0 = osub;
+                    out.first = rg.x;
+                    out.end = w == NS - 1 && gr.writer ? rg.y : rg.x;
+                }
+                run_dp<R, kSlots, kBF, kSubseq, kT>(p, strip, lane, rg, out, cring_s, cfull_s,
+                                                    cempty_s, cs);
+            }
         } else if (role == 2) {
             if (gr.reader) {
-                // the first strip's blocks; the strip above (last of the group
-                // above) published its own range's columns
-                const int2 above = strip_range<kSubseq>(p, g * NS - 1);
-                if (kCl && crank > 0)
-                    run_link_reader(p, lane, ring[0], smem_u32(&bfull[0][0]),
-                                    smem_u32(&bempty[0][0]), rsub[0], rgs[0].x, rgs[0].y, above.x,
-                                    above.y, link, smem_u32(&lfull[0]), smem_u32(&lempty[0]), lin,
-                                    crank);
+                if (link_in)
+                    run_link_reader<kSlots>(p, lane, cring_s + Slot::kBorder, Slot::kBytes, cfull_s,
+                                    cempty_s, csub[0], rgs[0].x, above.y, rgs[0].y,
+                                    smem_u32(&lempty[0]), lin, crank);
                 else
-                    run_reader(p, g, lane, ring[0], smem_u32(&bfull[0][0]),
-                               smem_u32(&bempty[0][0]), rsub[0], rgs[0].x, rgs[0].y,
-                               above.x * kSub, above.y * kSub);
+                    run_reader<kSlots>(p, kCl ? (g - 1) / (int)cn : g - 1, lane, cring_s + Slot::kBorder, Slot::kBytes, cfull_s, cempty_s,
+                               csub[0], rgs[0].x, rgs[0].y, above.x * kSub, above.y * kSub);
             }
         } else {
             if (gr.writer) {
-                if (kCl && crank + 1 < cn)
-                    run_link_writer(p, lane, ring[NS], smem_u32(&bfull[NS][0]),
-                                    smem_u32(&bempty[NS][0]), rsub[NS], rgs[NS - 1].x,
-                                    rgs[NS - 1].y, smem_u32(&link[0][0][0]), smem_u32(&lfull[0]),
-                                    smem_u32(&lempty[0]), lout, crank);
+                if (link_out)
+                    run_link_writer<kSlots>(p, lane, ringo, smem_u32(&ofull[0]), smem_u32(&oempty[0]),
+                                    osub, rgs[NS - 1].x, rgs[NS - 1].y, cring_s + Slot::kBorder,
+                                    Slot::kBytes, cfull_s, smem_u32(&lempty[0]), lout, lsub,
+                                    below.x, crank);
                 else
-                    run_writer(p, g, lane, ring[NS], smem_u32(&bfull[NS][0]),
-                               smem_u32(&bempty[NS][0]), rsub[NS], rgs[NS - 1].x, rgs[NS - 1].y);
+                    run_writer<kSlots>(p, kCl ? g / (int)cn : g, lane, ringo, smem_u32(&ofull[0]), smem_u32(&oempty[0]), osub,
+                               rgs[NS - 1].x, rgs[NS - 1].y);
             }
         }
-        // ring uses of this group, in blocks of 8 columns: a cost ring the
-        // strip's range; ring 0 the first strip's range; ring w (1 <= w < NS)
-        // and ring NS the range of the strip that fills them
+        // ring uses of this group, in blocks of 8 columns
 #pragma unroll
-        for (int q = 0; q < NS; ++q)
-            if (q < gr.nstrips_here) csub[q] += (unsigned)(rgs[q].y - rgs[q].x);
-        if (ring_used<NS>(gr, 0)) rsub[0] += (unsigned)(rgs[0].y - rgs[0].x);
-        if (kCl && crank > 0 && gr.reader) {  // the link carries the strip above's range
-            const int2 above = strip_range<kSubseq>(p, g * NS - 1);
-            lin += (unsigned)(above.y - above.x);
+        for (int q = 0; q < NS; ++q) csub[q] += (unsigned)(rgs[q].y - rgs[q].x);
+        if (gr.writer) osub += (unsigned)(rgs[NS - 1].y - rgs[NS - 1].x);
+        if (link_in) lin += (unsigned)max(above.y - rgs[0].x, 0);
+        if (link_out) {
+            lsub += (unsigned)(below.y - below.x);
+            lout += (unsigned)max(rgs[NS - 1].y - below.x, 0);
         }
-        if (kCl && crank + 1 < cn && gr.writer) lout += (unsigned)(rgs[NS - 1].y - rgs[NS - 1].x);
-#pragma unroll
-        for (int q = 1; q <= NS; ++q)
-            if (ring_used<NS>(gr, q)) rsub[q] += (unsigned)(rgs[q - 1].y - rgs[q - 1].x);
     }
     if constexpr (kCl) cluster_sync_all();  // no peer reaches this CTA's shared memory any more
 }
 
 template <int DP, int R, int NS, bool kMany, bool kBF = false, bool kSubseq = false,
-          bool kT = false, bool kMap = false>
+          bool kT = false>
 cudaError_t launch_t(const DpArgs& a, const DpArgs* many, const int* item0, int n, int items,
-                     int* ticket, int num_sms, cudaStream_t s, const MapArgs* map = nullptr) {
-    static_assert(!kMap || (!kMany && !kSubseq), "the band map runs with one pair");
+                     int* ticket, int num_sms, cudaStream_t s) {
     constexpr int kThreads = split_threads<DP, NS, kBF>();
-    const int smem = NS * SplitSmem<DP, R, kBF>::kStripBytes;
-    auto* kern = k_dp_split<DP, R, NS, kMany, kBF, kSubseq, kT, kMap>;
+    const int smem = NS * SplitSmem<DP, R, NS, kBF, false>::kStripBytes;
+    auto* kern = k_dp_split<DP, R, NS, kMany, kBF, kSubseq, kT>;
     static DeviceSlots occupancy;
     int blocks_per_sm = 0;
     const cudaError_t e = blocks_per_sm_once(kern, kThreads, smem, occupancy, &blocks_per_sm);
     if (e != cudaSuccess) return e;
     int grid = blocks_per_sm * num_sms;
-    if (kMap) {
-        if (!map || !map->done || map->nbm <= 0) return cudaErrorInvalidValue;
-        items += map->nbm;
-    }
     if (grid > items) grid = items;
-    kern<<<grid, kThreads, smem, s>>>(a, map ? *map : MapArgs{}, many, item0, n, ticket);
+    kern<<<grid, kThreads, smem, s>>>(a, many, item0, n, ticket);
     return cudaGetLastError();
 }
 

@@ -10,10 +10,10 @@ cudaError_t launch_dp_split_cl(const DpArgs& a, int dp, bool bf16, bool transpos
     *used = false;
     if (bf16) {
         switch (dp) {
-            case 64: return transposed ? launch_cl<64, true, true>(a, s, used)
-                                       : launch_cl<64, true, false>(a, s, used);
-            case 128: return transposed ? launch_cl<128, true, true>(a, s, used)
-                                        : launch_cl<128, true, false>(a, s, used);
+            case 64: return transposed ? launch_cl<64, true, true, 1>(a, s, used)
+                                       : launch_cl<64, true, false, 1>(a, s, used);
+            case 128: return transposed ? launch_cl<128, true, true, 1>(a, s, used)
+                                        : launch_cl<128, true, false, 1>(a, s, used);
             default: return cudaSuccess;
         }
     }
@@ -22,7 +22,7 @@ cudaError_t launch_dp_split_cl(const DpArgs& a, int dp, bool bf16, bool transpos
         case 8: return transposed ? launch_cl<8, false, true>(a, s, used) : launch_cl<8, false, false>(a, s, used);
         case 12: return transposed ? launch_cl<12, false, true>(a, s, used) : launch_cl<12, false, false>(a, s, used);
         case 16: return transposed ? launch_cl<16, false, true>(a, s, used) : launch_cl<16, false, false>(a, s, used);
-        case 32: return transposed ? launch_cl<32, false, true>(a, s, used) : launch_cl<32, false, false>(a, s, used);
+        case 32: return transposed ? launch_cl<32, false, true, 1>(a, s, used) : launch_cl<32, false, false, 1>(a, s, used);
         case 64:
         case 128: return launch_dp_split_wide_cl(a, dp, transposed, s, used);
         default: return cudaSuccess;

@@ -13,13 +13,15 @@
 //
 // Every CTA of a cluster sits on an SM of its own (the dynamic shared
 // memory is raised so that two CTAs cannot share an SM, which would put two
-// DP warps on one SM sub-partition).  The cluster size is the largest of 8
-// down to 2 whose resident clusters hold every strip group of the pair at
-// once (the 20000 x 25000 pair's 135 groups: 17 clusters of 8 do not fit at
-// once, 23 of 6 do, and its DP takes 1.360 ms against 1.393 with clusters of
-// 4, a third fewer hops through global memory); a band with more groups runs
-// persistent clusters of 8, a full sweep with more groups no clusters.
+// DP warps on one SM sub-partition).  One strip a CTA where one or two cost
+// warps cannot keep up with a DP warp (D > 16, the BF16 cost: three or four cost
+// warps a strip, on the sub-partitions beside the DP warp's), else two.  The
+// cluster size: see launch_cl.  Measured (DP, ms): 20000 x 25000, D = 12, clusters
+// of 8 / 6 / 4 / 2: 1.001 / 1.009 / 1.027 / 1.080; 100000 x 126231 (335 groups active
+// at once, 152 SMs): 7.66 / 7.18 / 6.94 / 6.59; 40000 x 48000, D = 128, BF16: 2.65 / 2.55
+// / 2.52 / 2.50 with one strip a CTA, 3.16 without clusters and two.
 #pragma once
+#include <algorithm>
 #include <mutex>
 
 #include "dp_split.cuh"
@@ -32,13 +34,13 @@ constexpr int kClMaxDev = 64;
 constexpr int kNClSizes = 7;
 constexpr int kClSizes[kNClSizes] = {8, 7, 6, 5, 4, 3, 2};
 
-template <int DP, bool kBF, bool kT>
+template <int DP, bool kBF, bool kT, int NS = 2>
 struct ClKernel {
-    static constexpr int R = 3, NS = 2;
+    static constexpr int R = 3;
     static constexpr int kThreads = split_threads<DP, NS, kBF>();
-    static constexpr auto kern() { return k_dp_split<DP, R, NS, false, kBF, false, kT, false, true>; }
+    static constexpr auto kern() { return k_dp_split<DP, R, NS, false, kBF, false, kT, true>; }
     static int smem() {
-        return std::max(NS * SplitSmem<DP, R, kBF>::kStripBytes, kClSmemFloor);
+        return std::max(NS * SplitSmem<DP, R, NS, kBF, true>::kStripBytes, kClSmemFloor);
     }
 };
 
@@ -64,11 +66,11 @@ cudaLaunchConfig_t cl_config(dim3 grid, int threads, int smem, cudaStream_t s,
 }
 
 // Attributes and cluster occupancy of one instantiation, once per device.
-template <int DP, bool kBF, bool kT>
+template <int DP, bool kBF, bool kT, int NS>
 const ClInfo& cl_info(int dev) {
     static ClInfo info[kClMaxDev];
     static std::mutex mu;
-    using K = ClKernel<DP, kBF, kT>;
+    using K = ClKernel<DP, kBF, kT, NS>;
     std::lock_guard<std::mutex> lock(mu);
     ClInfo& ci = info[dev];
     if (ci.ready) return ci;
@@ -94,39 +96,50 @@ const ClInfo& cl_info(int dev) {
     return ci;
 }
 
-template <int DP, bool kBF, bool kT>
-cudaError_t launch_cl(const DpArgs& a, cudaStream_t s, bool* used) {
+// Strips of `a` that are active at once: those whose rows a path can cross at
+// one column (the most at the corners of the path region); a band's strips are
+// short and follow one another, so few are.
+inline int peak_strips(const DpArgs& a) {
+    if (a.ranges) return 1;
+    const long long r = a.La, c = a.Lb;
+    long long most = 0;
+    for (const long long col : {(2 * r - c) / 3, (4 * c - 2 * r) / 3}) {
+        const long long lo = std::max(col / 2, r - 2 * (c - col));
+        const long long hi = std::min(2 * col, r - (c - col) / 2);
+        most = std::max(most, std::min(hi, r) - std::max(lo, 0LL));
+    }
+    return (int)(most / a.rps) + 1;
+}
+
+template <int DP, bool kBF, bool kT, int NS = 2>
+cudaError_t launch_cl(const DpArgs& pair, cudaStream_t s, bool* used) {
     *used = false;
+    DpArgs a = pair;
+    a.ngroups = (a.nstrips + NS - 1) / NS;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kClMaxDev) {
         (void)cudaGetLastError();
         return cudaSuccess;
     }
-    const ClInfo& ci = cl_info<DP, kBF, kT>(dev);
+    const ClInfo& ci = cl_info<DP, kBF, kT, NS>(dev);
     if (!ci.ok) return cudaSuccess;
+    // the largest clusters (fewest hops through global memory) of which enough
+    // are resident for the groups that are active at once, else those that hold
+    // the most groups
+    const int need = std::min(a.ngroups, (peak_strips(a) + NS - 1) / NS);
     int cn = 0, nclusters = 0;
-    // one wave: the largest cluster size whose resident clusters hold every group
-    for (int k = 0; k < kNClSizes && cn == 0; ++k) {
-        const int need = (a.ngroups + kClSizes[k] - 1) / kClSizes[k];
-        if (ci.max_clusters[k] >= need) {
-            cn = kClSizes[k];
-            nclusters = need;
-        }
-    }
-    // several waves: persistent clusters of 8 for a band (its strips are
-    // short and start one after another along the band); a full sweep of
-    // several waves runs faster without clusters (D = 128, 40000 x 48000:
-    // 5.7 against 8.4 ms with the BF16 cost, 19.3 against 28.6 ms with FP32)
-    if (cn == 0 && a.ranges && ci.max_clusters[0] > 0) {
-        cn = kClSizes[0];
-        nclusters = ci.max_clusters[0];
+    for (int k = 0; k < kNClSizes; ++k) {
+        if (ci.max_clusters[k] <= 0) continue;
+        cn = kClSizes[k];
+        nclusters = std::min(ci.max_clusters[k], (a.ngroups + cn - 1) / cn);
+        if (ci.max_clusters[k] * cn >= need) break;
     }
     if (cn == 0) return cudaSuccess;
-    using K = ClKernel<DP, kBF, kT>;
+    using K = ClKernel<DP, kBF, kT, NS>;
     cudaLaunchAttribute at[1];
     cudaLaunchConfig_t cfg =
         cl_config(dim3((unsigned)(nclusters * cn)), K::kThreads, K::smem(), s, at, cn);
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, K::kern(), a, MapArgs{},
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, K::kern(), a,
                                              static_cast<const DpArgs*>(nullptr),
                                              static_cast<const int*>(nullptr), 1,
                                              static_cast<int*>(nullptr));

@@ -31,11 +31,11 @@ cudaError_t launch_dp_split_wide_cl(const DpArgs& a, int dp, bool transposed, cu
                                     bool* used) {
     *used = false;
     if (dp == 64)
-        return transposed ? launch_cl<64, false, true>(a, s, used)
-                          : launch_cl<64, false, false>(a, s, used);
+        return transposed ? launch_cl<64, false, true, 1>(a, s, used)
+                          : launch_cl<64, false, false, 1>(a, s, used);
     if (dp == 128)
-        return transposed ? launch_cl<128, false, true>(a, s, used)
-                          : launch_cl<128, false, false>(a, s, used);
+        return transposed ? launch_cl<128, false, true, 1>(a, s, used)
+                          : launch_cl<128, false, false, 1>(a, s, used);
     return cudaSuccess;
 }
 

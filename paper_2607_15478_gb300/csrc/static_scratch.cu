@@ -186,7 +186,7 @@ extern "C" int dtw_align_static(const float* A, int La, const float* B, int Lb, 
     bt.ranges = nullptr;
     bt.transposed = 0;
     const cudaError_t e = launch_plan(plan, a, dp, num_sms, s);
-    if (e != cudaSuccess || launch_backtrace_bands(bt, s, true) != cudaSuccess) {
+    if (e != cudaSuccess || launch_backtrace_bands(bt, s) != cudaSuccess) {
         (void)cudaGetLastError();
         return DTW_ERR_CUDA;
     }
