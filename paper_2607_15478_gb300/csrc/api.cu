@@ -995,11 +995,11 @@ EncSeq enc_seq(size_t base, int Lc, int D) {
     q.total = o;
     return q;
 }
-// Both sequences, then the per-row training data of A: targets (int), the
-// sums behind them (u64, int), width targets, width-logit gradients.
+// Both sequences, then the per-row training data of A: targets (int), width
+// targets, width-logit gradients.
 struct EncBuf {
     EncSeq a, b;
-    size_t tgt, jsum, cnt, wt, dS, total;
+    size_t tgt, wt, dS, total;
 };
 EncBuf enc_buf(int Lac, int Lbc, int D) {
     EncBuf e;
@@ -1007,8 +1007,6 @@ EncBuf enc_buf(int Lac, int Lbc, int D) {
     e.b = enc_seq(e.a.total, Lbc, D);
     size_t o = e.b.total;
     e.tgt = o; o = align256(o + (size_t)Lac * sizeof(int));
-    e.jsum = o; o = align256(o + (size_t)Lac * sizeof(unsigned long long));
-    e.cnt = o; o = align256(o + (size_t)Lac * sizeof(int));
     e.wt = o; o = align256(o + (size_t)Lac * sizeof(float));
     e.dS = o; o = align256(o + (size_t)Lac * sizeof(float));
     e.total = o;
@@ -1017,45 +1015,81 @@ EncBuf enc_buf(int Lac, int Lbc, int D) {
 
 float* ef(dtw_handle* h, size_t off) { return reinterpret_cast<float*>(h->enc + off); }
 
-// Encoder forward of one sequence X (L fine frames): pooled input, the three
-// conv layers and the heads, into the buffers of q.
-int enc_forward(dtw_handle* h, const float* P, const EncLayout& pl, int D, const float* X, int L,
-                int ds, int bf16, const EncSeq& q) {
+// One of the sequences an encoder pass runs over: its fine frames and buffers.
+struct EncIn {
+    const float* X;
+    int L;  // fine frames
+    EncSeq q;
+};
+
+// Encoder forward of n (1 or 2) sequences: pooled input, the three conv layers
+// and the heads, into the buffers of each.  train: also zeroes the embedding
+// gradients.
+int enc_forward(dtw_handle* h, const float* P, const EncLayout& pl, int D, const EncIn* in, int n,
+                int ds, int bf16, bool train) {
     cudaStream_t s = h->stream;
-    const int Lc = (L + ds - 1) / ds;
-    CU(launch_pool_norm(X, L, D, ds, ef(h, q.X), s));
-    CU(launch_conv(ef(h, q.X), nullptr, Lc, D, P + pl.W1, P + pl.b1, 1, 0, bf16, ef(h, q.H1), s));
-    CU(launch_conv(ef(h, q.H1), nullptr, Lc, kEncChannels, P + pl.W2, P + pl.b2, 1, 0, bf16,
-                   ef(h, q.H2), s));
-    CU(launch_conv(ef(h, q.H2), nullptr, Lc, kEncChannels, P + pl.W3, P + pl.b3, 1, 0, bf16,
-                   ef(h, q.H3), s));
-    CU(launch_embed(ef(h, q.H3), Lc, P, pl, bf16, (float)DTW_BAND_WMIN, (float)DTW_BAND_WMAX,
-                    ef(h, q.E), ef(h, q.invn), ef(h, q.S), ef(h, q.HW), s));
+    EncRows2 r{};
+    auto rows = [&](size_t EncSeq::*x, size_t EncSeq::*y) {
+        for (int k = 0; k < n; ++k)
+            r.s[k] = {ef(h, in[k].q.*x), nullptr, ef(h, in[k].q.*y), (in[k].L + ds - 1) / ds};
+    };
+    for (int k = 0; k < n; ++k) r.s[k] = {in[k].X, nullptr, ef(h, in[k].q.X), in[k].L};
+    CU(launch_pool_norm(r, n, D, ds, s));
+    rows(&EncSeq::X, &EncSeq::H1);
+    CU(launch_conv(r, n, D, P + pl.W1, P + pl.b1, 1, 0, bf16, s));
+    rows(&EncSeq::H1, &EncSeq::H2);
+    CU(launch_conv(r, n, kEncChannels, P + pl.W2, P + pl.b2, 1, 0, bf16, s));
+    rows(&EncSeq::H2, &EncSeq::H3);
+    CU(launch_conv(r, n, kEncChannels, P + pl.W3, P + pl.b3, 1, 0, bf16, s));
+    EncEmbed2 e{};
+    for (int k = 0; k < n; ++k) {
+        const EncSeq& q = in[k].q;
+        e.s[k] = {ef(h, q.H3), ef(h, q.E),  ef(h, q.invn),                 ef(h, q.S),
+                  ef(h, q.HW), train ? ef(h, q.G) : nullptr, nullptr, (in[k].L + ds - 1) / ds};
+    }
+    CU(launch_embed(e, n, P, pl, bf16, (float)DTW_BAND_WMIN, (float)DTW_BAND_WMAX, s));
     return DTW_OK;
 }
 
-// Backward of the trunk and the embedding head of one sequence, from the
-// gradient of the loss with respect to its embeddings (in q.G).
-int enc_backward(dtw_handle* h, const float* P, const EncLayout& pl, int D, int Lc,
-                 const EncSeq& q, float* grad) {
+// Backward of the trunk and the embedding head of both sequences, from the
+// gradients of the loss with respect to their embeddings (in q.G).
+int enc_backward(dtw_handle* h, const float* P, const EncLayout& pl, int D, const EncIn* in, int n,
+                 int ds, float* grad) {
     cudaStream_t s = h->stream;
     constexpr int C = kEncChannels;
-    CU(launch_embed_bwd(ef(h, q.E), ef(h, q.invn), Lc, P + pl.W4, ef(h, q.G), ef(h, q.dHa), s));
-    CU(launch_outer(ef(h, q.G), kEncEmbed, ef(h, q.H3), C, Lc, grad + pl.W4, s));
-    CU(launch_outer(ef(h, q.G), kEncEmbed, nullptr, 1, Lc, grad + pl.b4, s));
-    // layer 3: dH3 in dHa (masked by H3 inside)
-    CU(launch_conv_wgrad(ef(h, q.H2), Lc, C, ef(h, q.dHa), ef(h, q.H3), grad + pl.W3,
-                         grad + pl.b3, s));
-    CU(launch_conv(ef(h, q.dHa), ef(h, q.H3), Lc, C, P + pl.W3, nullptr, 0, 1, 0, ef(h, q.dHb),
-                   s));
+    auto Lc = [&](int k) { return (in[k].L + ds - 1) / ds; };
+    EncEmbed2 e{};
+    EncHead2 hd{};
+    for (int k = 0; k < n; ++k) {
+        const EncSeq& q = in[k].q;
+        e.s[k] = {nullptr, ef(h, q.E), ef(h, q.invn), nullptr, nullptr, ef(h, q.G), ef(h, q.dHa), Lc(k)};
+        hd.s[k] = {ef(h, q.G), ef(h, q.H3), Lc(k)};
+    }
+    CU(launch_embed_bwd(e, n, P + pl.W4, s));
+    CU(launch_head_grad(hd, n, kEncEmbed, grad + pl.W4, grad + pl.b4, s));
+    // a layer's weight gradient from dY (masked by its output inside), and the
+    // gradient of its input
+    auto wgrad = [&](size_t EncSeq::*x, size_t EncSeq::*dy, size_t EncSeq::*yout, int Cin, size_t W,
+                     size_t b) {
+        EncGrad2 g{};
+        for (int k = 0; k < n; ++k)
+            g.s[k] = {ef(h, in[k].q.*x), ef(h, in[k].q.*dy), ef(h, in[k].q.*yout), Lc(k)};
+        return launch_conv_wgrad(g, n, Cin, grad + W, grad + b, s);
+    };
+    auto dgrad = [&](size_t EncSeq::*dy, size_t EncSeq::*yout, size_t EncSeq::*dx, size_t W) {
+        EncRows2 r{};
+        for (int k = 0; k < n; ++k)
+            r.s[k] = {ef(h, in[k].q.*dy), ef(h, in[k].q.*yout), ef(h, in[k].q.*dx), Lc(k)};
+        return launch_conv(r, n, C, P + W, nullptr, 0, 1, 0, s);
+    };
+    // layer 3: dH3 in dHa
+    CU(wgrad(&EncSeq::H2, &EncSeq::dHa, &EncSeq::H3, C, pl.W3, pl.b3));
+    CU(dgrad(&EncSeq::dHa, &EncSeq::H3, &EncSeq::dHb, pl.W3));
     // layer 2: dH2 in dHb
-    CU(launch_conv_wgrad(ef(h, q.H1), Lc, C, ef(h, q.dHb), ef(h, q.H2), grad + pl.W2,
-                         grad + pl.b2, s));
-    CU(launch_conv(ef(h, q.dHb), ef(h, q.H2), Lc, C, P + pl.W2, nullptr, 0, 1, 0, ef(h, q.dHa),
-                   s));
+    CU(wgrad(&EncSeq::H1, &EncSeq::dHb, &EncSeq::H2, C, pl.W2, pl.b2));
+    CU(dgrad(&EncSeq::dHb, &EncSeq::H2, &EncSeq::dHa, pl.W2));
     // layer 1: dH1 in dHa
-    CU(launch_conv_wgrad(ef(h, q.X), Lc, D, ef(h, q.dHa), ef(h, q.H1), grad + pl.W1,
-                         grad + pl.b1, s));
+    CU(wgrad(&EncSeq::X, &EncSeq::dHa, &EncSeq::H1, D, pl.W1, pl.b1));
     return DTW_OK;
 }
 
@@ -1111,7 +1145,8 @@ int dtw_encode(dtw_handle* h, const float* params, int D, const float* X, int L,
     int rc = grow(h, &h->enc, &h->enc_cap, q.total);
     if (rc != DTW_OK) return rc;
     const EncLayout pl = enc_layout(D);
-    rc = enc_forward(h, params, pl, D, X, L, downsample, bf16 != 0, q);
+    const EncIn in = {X, L, q};
+    rc = enc_forward(h, params, pl, D, &in, 1, downsample, bf16 != 0, false);
     if (rc != DTW_OK) return rc;
     CU(cudaMemcpyAsync(emb, ef(h, q.E), sizeof(float) * (size_t)Lc * kEncEmbed,
                        cudaMemcpyDeviceToDevice, h->stream));
@@ -1141,19 +1176,15 @@ int dtw_encoder_grad(dtw_handle* h, const float* params, int D, int downsample, 
     int rc = grow(h, &h->enc, &h->enc_cap, eb.total);
     if (rc != DTW_OK) return rc;
     const EncLayout pl = enc_layout(D);
-    rc = enc_forward(h, params, pl, D, A, La, downsample, 0, eb.a);
-    if (rc == DTW_OK) rc = enc_forward(h, params, pl, D, B, Lb, downsample, 0, eb.b);
+    const EncIn in[2] = {{A, La, eb.a}, {B, Lb, eb.b}};
+    rc = enc_forward(h, params, pl, D, in, 2, downsample, 0, mode == 0);
     if (rc != DTW_OK) return rc;
     if (mode == 0) {
         int* tgt = reinterpret_cast<int*>(h->enc + eb.tgt);
-        CU(launch_targets(path, path_len, std::min(La, Lb), downsample, Lac, Lbc,
-                          reinterpret_cast<unsigned long long*>(h->enc + eb.jsum),
-                          reinterpret_cast<int*>(h->enc + eb.cnt), tgt, s));
+        CU(launch_targets(path, path_len, std::min(La, Lb), downsample, Lac, Lbc, tgt, s));
         CU(launch_loss_emb(ef(h, eb.a.E), Lac, ef(h, eb.b.E), Lbc, tgt, ef(h, eb.a.G),
                            ef(h, eb.b.G), loss, s));
-        rc = enc_backward(h, params, pl, D, Lac, eb.a, grad);
-        if (rc == DTW_OK) rc = enc_backward(h, params, pl, D, Lbc, eb.b, grad);
-        return rc;
+        return enc_backward(h, params, pl, D, in, 2, downsample, grad);
     }
     // mode 1: the coarse path on the current embeddings, the half-width each
     // coarse row of A needs, and the width head's gradient (trunk frozen)
@@ -1168,8 +1199,9 @@ int dtw_encoder_grad(dtw_handle* h, const float* params, int D, int downsample, 
     CU(launch_width_target(cpath, clen, path, path_len, downsample, Lac, (float)DTW_BAND_WMIN,
                            (float)DTW_BAND_WMAX, ef(h, eb.wt), s));
     CU(launch_loss_width(ef(h, eb.a.S), ef(h, eb.wt), Lac, ef(h, eb.dS), loss, s));
-    CU(launch_outer(ef(h, eb.dS), 1, ef(h, eb.a.H3), kEncChannels, Lac, grad + pl.W5, s));
-    CU(launch_outer(ef(h, eb.dS), 1, nullptr, 1, Lac, grad + pl.b5, s));
+    EncHead2 hd{};
+    hd.s[0] = {ef(h, eb.dS), ef(h, eb.a.H3), Lac};
+    CU(launch_head_grad(hd, 1, 1, grad + pl.W5, grad + pl.b5, s));
     return DTW_OK;
 }
 
@@ -1210,8 +1242,8 @@ int dtw_align_learned(dtw_handle* h, const float* A, int La, const float* B, int
     rc = grow(h, &h->band, &h->band_cap, bb.total);
     if (rc != DTW_OK) return rc;
     const EncLayout pl = enc_layout(D);
-    rc = enc_forward(h, params, pl, D, A, La, downsample, bf16 != 0, eb.a);
-    if (rc == DTW_OK) rc = enc_forward(h, params, pl, D, B, Lb, downsample, bf16 != 0, eb.b);
+    const EncIn in[2] = {{A, La, eb.a}, {B, Lb, eb.b}};
+    rc = enc_forward(h, params, pl, D, in, 2, downsample, bf16 != 0, false);
     if (rc != DTW_OK) return rc;
     return band_align(h, A, La, B, Lb, D, o, downsample, ef(h, eb.a.E), Lac, ef(h, eb.b.E), Lbc,
                       kEncEmbed, 0, ef(h, eb.a.HW), ef(h, eb.b.HW), bb, path, path_len,

@@ -26,9 +26,13 @@
 // the caller's gradient array with atomics.
 //
 // Kernels: k_pool_norm, k_conv (forward, and backward-data with transposed
-// flipped weights), k_conv_wgrad, k_embed, k_embed_bwd, k_outer (reductions
-// sum_l u[l][a] v[l][b] for the head weights), k_targets*, k_loss_emb,
-// k_width_target, k_loss_width, k_adam.
+// flipped weights), k_conv_wgrad, k_embed, k_embed_bwd, k_head_grad (the head
+// weights' gradients), k_targets, k_loss_emb, k_width_target, k_loss_width,
+// k_adam.  The layers of both sequences run in one launch each (EncRows2:
+// blockIdx.z is the sequence): a coarse sequence of a training pair has one to
+// three thousand rows, so a launch of its own and tiles of 64 rows and 64
+// channels left most SMs idle (a training step of 12000 x 14500 frames took 1.31 ms
+// that way, 0.84 of it in k_conv_wgrad on 12 of the 152 SMs; 0.14 ms now).
 #include "pardtw_common.cuh"
 
 #include <cuda_bf16.h>
@@ -51,26 +55,39 @@ __device__ __forceinline__ float round_bf16(float x) {
 }
 
 // Mean of each window of ds frames (the last may be shorter), L2-normalised
-// (a zero mean stays zero).  One thread per pooled frame.
-__global__ void k_pool_norm(const float* __restrict__ X, int L, int D, int ds,
-                            float* __restrict__ Y) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    const int Lc = (L + ds - 1) / ds;
-    if (c >= Lc) return;
-    const int f0 = c * ds, f1 = min(f0 + ds, L);
+// (a zero mean stays zero).  kG lanes per pooled frame, one (two for D > 32)
+// feature(s) a lane; the sum of squares runs over the features in order.
+template <int kG>
+__global__ void __launch_bounds__(128) k_pool_norm(const EncRows2 q, int D, int ds) {
+    const EncRows a = blockIdx.z ? q.s[1] : q.s[0];
+    const int L = a.L, Lc = (L + ds - 1) / ds;
+    const int c = (blockIdx.x * blockDim.x + threadIdx.x) / kG;
+    const int g = threadIdx.x % kG;
+    const int f0 = min(c, Lc - 1) * ds, f1 = min(f0 + ds, L);
+    float v[2] = {0.f, 0.f};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int d = g + h * kG;
+        if (d < D) {
+            float acc = 0.f;
+#pragma unroll 8
+            for (int f = f0; f < f1; ++f) acc += __ldg(a.X + (size_t)f * D + d);
+            v[h] = acc / (float)(f1 - f0);
+        }
+    }
     float ss = 0.f;
     for (int d = 0; d < D; ++d) {
-        float acc = 0.f;
-        for (int f = f0; f < f1; ++f) acc += X[(size_t)f * D + d];
-        acc /= (float)(f1 - f0);
-        Y[(size_t)c * D + d] = acc;
-        ss = fmaf(acc, acc, ss);
+        const float x = __shfl_sync(0xffffffffu, d < kG ? v[0] : v[1], d % kG, kG);
+        ss = fmaf(x, x, ss);
     }
     const float r = ss > 0.f ? rsqrtf(ss) : 0.f;
-    for (int d = 0; d < D; ++d) Y[(size_t)c * D + d] *= r;
+    if (c >= Lc) return;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (g + h * kG < D) a.Y[(size_t)c * D + g + h * kG] = v[h] * r;
 }
 
-// Generic conv5 over kTL rows per block, all kC output channels:
+// Generic conv5 over kTL rows and kCO output channels per block:
 //   Y[l][co] = bias[co] + sum_{ci < Cin, t} Wt(ci, t, co) * Xm[l + t - 2][ci]
 // Xm = X masked by (mask > 0) where mask is given (the relu derivative of
 // the layer whose gradient X is).  Wt(ci, t, co) = W[co][ci][t] (forward,
@@ -78,50 +95,123 @@ __global__ void k_pool_norm(const float* __restrict__ X, int L, int D, int ds,
 // forward weight [Cin_b = kC][Cout_b][kK] read transposed and flipped).
 // kBF16: inputs and weights rounded to bf16 (products exact in FP32, FP32
 // accumulation).
-// Thread t computes rows 4 (t / 16) .. + 3 and channels 4 (t % 16) .. + 3 of
-// the tile, each output by the same FMAs in the same order (input channel
-// outer, tap inner) as one thread per output would: per input channel 8 rows
-// of X and 5 x 4 weights from shared memory feed 80 FMAs (one thread per
-// channel and 16 rows read 17 values for 16; measured 52 us a layer of 15779
-// rows at Cin = 64).
+// Thread t computes rows 4 (t / 8) .. + 3 and channels 2 (t % 8), + 1 of the
+// tile, each output by the same FMAs in the same order (input channel outer,
+// tap inner) as one thread per output would: per input channel 8 rows of X and
+// 5 x 2 weights from shared memory feed 40 FMAs.  A block has a quarter of the
+// channels: the weights it stages (20 KB at Cin = 64) are read from global
+// memory in order, and 1500 rows make 96 blocks instead of 24 (28 us a layer of
+// 1500 rows at Cin = 64 with all 64 channels a block, 10 us for both sequences of
+// a pair now; bound by the staging and 64 dependent channel steps of few warps).
 constexpr int kTL = 64;
-constexpr int kConvThreads = 256;
+constexpr int kCO = 16;
+constexpr int kWS = kCO + 2;         // floats per (ci, t) row of staged weights
+constexpr int kConvThreads = 128;
 constexpr int kXS = kTL + 2 * kPad;  // rows of X per input channel in shared memory
-static_assert(kTL == 64 && kC == 64 && kConvThreads == 256, "4 x 4 outputs a thread");
+static_assert(kConvThreads == (kTL / 4) * (kCO / 2), "4 rows x 2 channels a thread");
 
-template <bool kBwd, bool kBF16>
+// kCin: the input channels (64: loads of 16 bytes, all in flight before the
+// first is stored), 0: Cin of them, one value at a time.
+template <int kCin, bool kBwd, bool kBF16>
 __global__ void __launch_bounds__(kConvThreads)
-    k_conv(const float* __restrict__ X, const float* __restrict__ mask, int L, int Cin,
-           const float* __restrict__ W, const float* __restrict__ bias, int relu,
-           float* __restrict__ Y) {
+    k_conv(const EncRows2 q, int Cin, const float* __restrict__ W, const float* __restrict__ bias,
+           int relu) {
+    static_assert(kCin == 0 || kCin == kC, "whole rows of 16-byte words");
+    if (kCin > 0) Cin = kCin;
     extern __shared__ __align__(16) float sm[];
-    float* Ws = sm;                       // [Cin * kK][kC]
-    float* Xs = sm + Cin * kK * kC;       // [Cin][kXS]
-    const int l0 = blockIdx.x * kTL;
+    float* Xs = sm;                       // [Cin][kXS]
+    float* Ws = sm + Cin * kXS;           // [Cin * kK][kWS]
+    const EncRows a = blockIdx.z ? q.s[1] : q.s[0];
+    const int L = a.L;
+    const int l0 = blockIdx.x * kTL, co0 = blockIdx.y * kCO;
+    if (l0 >= L) return;
+    const float* __restrict__ X = a.X;
+    const float* __restrict__ mask = a.M;
     const int tid = threadIdx.x;
-    for (int k = tid; k < Cin * kK * kC; k += kConvThreads) {
-        const int co = k % kC, ct = k / kC, ci = ct / kK, t = ct % kK;
-        float w = kBwd ? W[((size_t)ci * kC + co) * kK + (kK - 1 - t)]
-                       : W[((size_t)co * Cin + ci) * kK + t];
-        Ws[k] = kBF16 ? round_bf16(w) : w;
-    }
-    for (int k = tid; k < kXS * Cin; k += kConvThreads) {
-        const int r = k / Cin, ci = k % Cin;
-        const int l = l0 + r - kPad;
-        float v = 0.f;
-        if (l >= 0 && l < L) {
-            v = X[(size_t)l * Cin + ci];
-            if (mask && !(mask[(size_t)l * Cin + ci] > 0.f)) v = 0.f;
+    auto put_w = [&](int k, float w) {  // value k of the block's weights
+        int co, ct;
+        if (kBwd) {  // per ci, kCO x kK consecutive values
+            const int ci = k / (kCO * kK), r = k - ci * (kCO * kK);
+            co = r / kK;
+            ct = ci * kK + (kK - 1 - (r - co * kK));
+        } else {  // per channel, Cin x kK consecutive values
+            co = k / (Cin * kK);
+            ct = k - co * (Cin * kK);
         }
-        Xs[ci * kXS + r] = kBF16 ? round_bf16(v) : v;
+        Ws[ct * kWS + co] = kBF16 ? round_bf16(w) : w;
+    };
+    auto w_index = [&](int k) -> size_t {
+        if (!kBwd) return (size_t)co0 * Cin * kK + k;
+        const int ci = k / (kCO * kK);
+        return ((size_t)ci * kC + co0) * kK + (k - ci * (kCO * kK));
+    };
+    auto put_x = [&](int r, int ci, float v) { Xs[ci * kXS + r] = kBF16 ? round_bf16(v) : v; };
+    if constexpr (kCin > 0) {
+        constexpr int kWV = kCin * kK * kCO / 4, kXV = kXS * kCin / 4;
+        constexpr int kNW = kWV / kConvThreads, kNX = (kXV + kConvThreads - 1) / kConvThreads;
+        static_assert(kWV % kConvThreads == 0, "whole batches of weights");
+        float4 w[kNW], x[kNX];
+#pragma unroll
+        for (int u = 0; u < kNW; ++u) {
+            const float* src = W + w_index(4 * (tid + u * kConvThreads));
+            // a segment starts on a 16-byte boundary only where W does
+            w[u] = make_float4(__ldg(src), __ldg(src + 1), __ldg(src + 2), __ldg(src + 3));
+        }
+#pragma unroll
+        for (int u = 0; u < kNX; ++u) {
+            const int k = tid + u * kConvThreads;
+            const int l = l0 + k / (kCin / 4) - kPad;
+            x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (k < kXV && l >= 0 && l < L) {
+                const size_t o = (size_t)l * (kCin / 4) + k % (kCin / 4);
+                x[u] = __ldg(reinterpret_cast<const float4*>(X) + o);
+                if (kBwd && mask) {
+                    const float4 m = __ldg(reinterpret_cast<const float4*>(mask) + o);
+                    if (!(m.x > 0.f)) x[u].x = 0.f;
+                    if (!(m.y > 0.f)) x[u].y = 0.f;
+                    if (!(m.z > 0.f)) x[u].z = 0.f;
+                    if (!(m.w > 0.f)) x[u].w = 0.f;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kNW; ++u) {
+            const int k = 4 * (tid + u * kConvThreads);
+            put_w(k, w[u].x);
+            put_w(k + 1, w[u].y);
+            put_w(k + 2, w[u].z);
+            put_w(k + 3, w[u].w);
+        }
+#pragma unroll
+        for (int u = 0; u < kNX; ++u) {
+            const int k = tid + u * kConvThreads;
+            if (k < kXV) {
+                const int r = k / (kCin / 4), ci = 4 * (k % (kCin / 4));
+                put_x(r, ci, x[u].x);
+                put_x(r, ci + 1, x[u].y);
+                put_x(r, ci + 2, x[u].z);
+                put_x(r, ci + 3, x[u].w);
+            }
+        }
+    } else {
+        for (int k = tid; k < Cin * kK * kCO; k += kConvThreads) put_w(k, W[w_index(k)]);
+        for (int k = tid; k < kXS * Cin; k += kConvThreads) {
+            const int r = k / Cin, ci = k % Cin;
+            const int l = l0 + r - kPad;
+            float v = 0.f;
+            if (l >= 0 && l < L) {
+                v = X[(size_t)l * Cin + ci];
+                if (mask && !(mask[(size_t)l * Cin + ci] > 0.f)) v = 0.f;
+            }
+            put_x(r, ci, v);
+        }
     }
     __syncthreads();
-    const int cg = tid % 16, rg = tid / 16;  // channels 4 cg .., rows 4 rg ..
-    float acc[4][4];
+    const int cg = tid % (kCO / 2), rg = tid / (kCO / 2);  // channels 2 cg, +1, rows 4 rg ..
+    float acc[4][2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = 0.f;
+#pragma unroll 4
     for (int ci = 0; ci < Cin; ++ci) {
         // rows 4 rg .. 4 rg + 7 of the tile (with the halo): the taps' inputs
         const float4 xa = *reinterpret_cast<const float4*>(Xs + ci * kXS + 4 * rg);
@@ -129,113 +219,147 @@ __global__ void __launch_bounds__(kConvThreads)
         const float x[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
 #pragma unroll
         for (int t = 0; t < kK; ++t) {
-            const float4 w4 = *reinterpret_cast<const float4*>(Ws + (ci * kK + t) * kC + 4 * cg);
-            const float w[4] = {w4.x, w4.y, w4.z, w4.w};
+            const float2 w = *reinterpret_cast<const float2*>(Ws + (ci * kK + t) * kWS + 2 * cg);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(w[j], x[i + t], acc[i][j]);
+            for (int i = 0; i < 4; ++i) {
+                acc[i][0] = fmaf(w.x, x[i + t], acc[i][0]);
+                acc[i][1] = fmaf(w.y, x[i + t], acc[i][1]);
+            }
         }
     }
-    float b[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) b[j] = bias ? bias[4 * cg + j] : 0.f;
+    const int co = co0 + 2 * cg;
+    const float b0 = bias ? bias[co] : 0.f, b1 = bias ? bias[co + 1] : 0.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int l = l0 + 4 * rg + i;
         if (l < L) {
-            float y[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                y[j] = acc[i][j] + b[j];
-                if (relu) y[j] = fmaxf(y[j], 0.f);
+            float y0 = acc[i][0] + b0, y1 = acc[i][1] + b1;
+            if (relu) {
+                y0 = fmaxf(y0, 0.f);
+                y1 = fmaxf(y1, 0.f);
             }
-            *reinterpret_cast<float4*>(Y + (size_t)l * kC + 4 * cg) =
-                make_float4(y[0], y[1], y[2], y[3]);
+            *reinterpret_cast<float2*>(a.Y + (size_t)l * kC + co) = make_float2(y0, y1);
         }
     }
 }
 
-// Weight gradient of a conv5 layer over a tile of kTW rows:
+// Weight gradient of a conv5 layer over a tile of kTW rows and kCI input
+// channels:
 //   dW[co][ci][t] += sum_l dYm[l][co] X[l + t - 2][ci],  db[co] += sum_l dYm[l][co]
-// dYm = dY masked by (Yout > 0) (the layer's relu).  Thread (co, cg) owns the
-// input channels ci = cg, cg + 4, ... (up to kCPT of them) for all t.
-constexpr int kTW = 128;
-template <int kCPT>
-__global__ void __launch_bounds__(kConvThreads)
-    k_conv_wgrad(const float* __restrict__ X, int L, int Cin, const float* __restrict__ dY,
-                 const float* __restrict__ Yout, float* __restrict__ dW, float* __restrict__ db) {
-    extern __shared__ float sm[];
-    float* Gs = sm;                       // [kTW][kC]
-    float* Xs = sm + kTW * kC;            // [kTW + 2 kPad][Cin]
-    const int l0 = blockIdx.x * kTW;
+// dYm = dY masked by (Yout > 0) (the layer's relu).  Thread (co, cg) owns two
+// input channels for all t, whose rows it keeps in a sliding window.  (128 rows
+// and every input channel a block left 12 blocks on 1500 rows: 210 us a layer at
+// Cin = 64.)  Bound by the atomics of its sums: 20 us a layer for both sequences
+// of a pair with one tile a block, a training step 152, 140, 146, 145 us with 1, 2,
+// 3, 4 tiles.
+constexpr int kTW = 64;     // rows staged at a time
+constexpr int kTiles = 2;   // of which a block takes so many: its sums go out by atomics once
+constexpr int kCI = 8;
+constexpr int kWgThreads = kC * (kCI / 2);
+__global__ void __launch_bounds__(kWgThreads)
+    k_conv_wgrad(const EncGrad2 q, int Cin, float* __restrict__ dW, float* __restrict__ db) {
+    __shared__ __align__(16) float Gs[kTW][kC];
+    __shared__ __align__(8) float Xs[kTW + 2 * kPad][kCI];
+    const EncGrad a = blockIdx.z ? q.s[1] : q.s[0];
+    const int L = a.L;
+    const int l0b = blockIdx.x * (kTW * kTiles), ci0 = blockIdx.y * kCI;
+    if (l0b >= L) return;
     const int tid = threadIdx.x;
-    for (int k = tid; k < kTW * kC; k += kConvThreads) {
-        const int r = k / kC, co = k % kC;
-        const int l = l0 + r;
-        float g = 0.f;
-        if (l < L) {
-            const size_t o = (size_t)l * kC + co;
-            g = Yout[o] > 0.f ? dY[o] : 0.f;
-        }
-        Gs[k] = g;
-    }
-    for (int k = tid; k < (kTW + 2 * kPad) * Cin; k += kConvThreads) {
-        const int r = k / Cin, ci = k % Cin;
-        const int l = l0 + r - kPad;
-        Xs[k] = (l >= 0 && l < L) ? X[(size_t)l * Cin + ci] : 0.f;
-    }
-    __syncthreads();
     const int co = tid % kC, cg = tid / kC;
-    float acc[kCPT][kK];
+    float acc[2][kK];
     float bacc = 0.f;
 #pragma unroll
-    for (int q = 0; q < kCPT; ++q)
+    for (int t = 0; t < kK; ++t) acc[0][t] = acc[1][t] = 0.f;
+    for (int l0 = l0b; l0 < min(l0b + kTW * kTiles, L); l0 += kTW) {
+        __syncthreads();  // the previous tile has been read
+        constexpr int kNG = kTW * kC / 4 / kWgThreads;  // 16-byte words per thread
+        float4 gv[kNG], yv[kNG];
 #pragma unroll
-        for (int t = 0; t < kK; ++t) acc[q][t] = 0.f;
-    for (int r = 0; r < kTW; ++r) {
-        const float g = Gs[r * kC + co];
-        bacc += g;
-#pragma unroll
-        for (int q = 0; q < kCPT; ++q) {
-            const int ci = cg + 4 * q;
-            if (ci < Cin) {
-#pragma unroll
-                for (int t = 0; t < kK; ++t) acc[q][t] = fmaf(g, Xs[(r + t) * Cin + ci], acc[q][t]);
+        for (int u = 0; u < kNG; ++u) {
+            const int k = tid + u * kWgThreads;
+            const int l = l0 + k / (kC / 4);
+            gv[u] = yv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (l < L) {
+                const size_t o = (size_t)l * (kC / 4) + k % (kC / 4);
+                gv[u] = __ldg(reinterpret_cast<const float4*>(a.dY) + o);
+                yv[u] = __ldg(reinterpret_cast<const float4*>(a.Yout) + o);
             }
+        }
+#pragma unroll
+        for (int u = 0; u < kNG; ++u) {
+            const int k = tid + u * kWgThreads;
+            *reinterpret_cast<float4*>(&Gs[k / (kC / 4)][4 * (k % (kC / 4))]) =
+                make_float4(yv[u].x > 0.f ? gv[u].x : 0.f, yv[u].y > 0.f ? gv[u].y : 0.f,
+                            yv[u].z > 0.f ? gv[u].z : 0.f, yv[u].w > 0.f ? gv[u].w : 0.f);
+        }
+#pragma unroll
+        for (int k = tid; k < (kTW + 2 * kPad) * kCI; k += kWgThreads) {
+            const int r = k / kCI, ci = ci0 + k % kCI;
+            const int l = l0 + r - kPad;
+            Xs[r][k % kCI] = (l >= 0 && l < L && ci < Cin) ? a.X[(size_t)l * Cin + ci] : 0.f;
+        }
+        __syncthreads();
+        constexpr int kU = 8;
+        float2 x[kU + 2 * kPad];  // rows r .. r + kU + 3 of the two channels
+#pragma unroll
+        for (int t = 0; t < 2 * kPad; ++t) x[t] = *reinterpret_cast<const float2*>(&Xs[t][2 * cg]);
+        for (int r = 0; r < kTW; r += kU) {
+            float g[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                x[2 * kPad + u] = *reinterpret_cast<const float2*>(&Xs[r + 2 * kPad + u][2 * cg]);
+                g[u] = Gs[r + u][co];
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                bacc += g[u];
+#pragma unroll
+                for (int t = 0; t < kK; ++t) {
+                    acc[0][t] = fmaf(g[u], x[u + t].x, acc[0][t]);
+                    acc[1][t] = fmaf(g[u], x[u + t].y, acc[1][t]);
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < 2 * kPad; ++t) x[t] = x[kU + t];
         }
     }
 #pragma unroll
-    for (int q = 0; q < kCPT; ++q) {
-        const int ci = cg + 4 * q;
+    for (int h = 0; h < 2; ++h) {
+        const int ci = ci0 + 2 * cg + h;
         if (ci < Cin)
 #pragma unroll
-            for (int t = 0; t < kK; ++t) atomicAdd(&dW[((size_t)co * Cin + ci) * kK + t], acc[q][t]);
+            for (int t = 0; t < kK; ++t) atomicAdd(&dW[((size_t)co * Cin + ci) * kK + t], acc[h][t]);
     }
-    if (cg == 0) atomicAdd(&db[co], bacc);
+    if (blockIdx.y == 0 && cg == 0) atomicAdd(&db[co], bacc);
 }
 
-// Heads, one thread per row: z = W4 h3 + b4, e = z / |z| (invn = 1/|z|, 0
-// for z = 0), s = W5 . h3 + b5 and the half-width in fine frames.
-__global__ void k_embed(const float* __restrict__ H, int L, const float* __restrict__ W4,
+// Heads, four threads per row (four embedding components each): z = W4 h3 + b4,
+// e = z / |z| (invn = 1/|z|, 0 for z = 0), s = W5 . h3 + b5 and the half-width in
+// fine frames.  Sums run over the channels, and the norm over the components,
+// in order.  G (may be null): zeroed, the embedding gradient of a training step.
+__global__ void __launch_bounds__(128) k_embed(const EncEmbed2 q, const float* __restrict__ W4,
                         const float* __restrict__ b4, const float* __restrict__ W5,
-                        const float* __restrict__ b5, int bf16, float wmin, float wmax,
-                        float* __restrict__ Emb, float* __restrict__ invn, float* __restrict__ S,
-                        float* __restrict__ HW) {
-    __shared__ float w4[kE * kC], w5[kC], bb[kE + 1];
-    for (int k = threadIdx.x; k < kE * kC; k += blockDim.x)
-        w4[k] = bf16 ? round_bf16(W4[k]) : W4[k];
+                        const float* __restrict__ b5, int bf16, float wmin, float wmax) {
+    __shared__ __align__(16) float w4[kC * kE];  // [c][e]
+    __shared__ float w5[kC], bb[kE + 1];
+    const EncEmbed a = blockIdx.z ? q.s[1] : q.s[0];
+    const int L = a.L;
+    if (blockIdx.x * 32 >= L) return;
+#pragma unroll
+    for (int k = threadIdx.x; k < kE * kC; k += 128) {
+        const float w = W4[k];
+        w4[(k % kC) * kE + k / kC] = bf16 ? round_bf16(w) : w;
+    }
     for (int k = threadIdx.x; k < kC; k += blockDim.x) w5[k] = W5[k];
     if (threadIdx.x < kE) bb[threadIdx.x] = b4[threadIdx.x];
     if (threadIdx.x == 0) bb[kE] = b5[0];
     __syncthreads();
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= L) return;
-    float z[kE];
-#pragma unroll
-    for (int e = 0; e < kE; ++e) z[e] = 0.f;
+    const int l = blockIdx.x * 32 + threadIdx.x / 4, eg = threadIdx.x % 4;
+    const int lr = min(l, L - 1);  // every lane takes part in the shuffles
+    float z[4] = {0.f, 0.f, 0.f, 0.f};
     float s = 0.f;
-    const float4* h4 = reinterpret_cast<const float4*>(H + (size_t)l * kC);
+    const float4* h4 = reinterpret_cast<const float4*>(a.H + (size_t)lr * kC);
+#pragma unroll 4
     for (int c4 = 0; c4 < kC / 4; ++c4) {
         const float4 v = h4[c4];
         const float hv[4] = {v.x, v.y, v.z, v.w};
@@ -243,158 +367,230 @@ __global__ void k_embed(const float* __restrict__ H, int L, const float* __restr
         for (int u = 0; u < 4; ++u) {
             const int c = 4 * c4 + u;
             const float hc = bf16 ? round_bf16(hv[u]) : hv[u];
-#pragma unroll
-            for (int e = 0; e < kE; ++e) z[e] = fmaf(w4[e * kC + c], hc, z[e]);
+            const float4 w = *reinterpret_cast<const float4*>(w4 + c * kE + 4 * eg);
+            z[0] = fmaf(w.x, hc, z[0]);
+            z[1] = fmaf(w.y, hc, z[1]);
+            z[2] = fmaf(w.z, hc, z[2]);
+            z[3] = fmaf(w.w, hc, z[3]);
             s = fmaf(w5[c], hv[u], s);
         }
     }
     float ss = 0.f;
 #pragma unroll
-    for (int e = 0; e < kE; ++e) {
-        z[e] += bb[e];
-        ss = fmaf(z[e], z[e], ss);
+    for (int k = 0; k < 4; ++k) z[k] += bb[4 * eg + k];
+#pragma unroll
+    for (int step = 0; step < 4; ++step) {
+        float mine = ss;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mine = fmaf(z[k], z[k], mine);
+        ss = __shfl_sync(0xffffffffu, mine, step, 4);
     }
     const float r = ss > 0.f ? rsqrtf(ss) : 0.f;
-#pragma unroll
-    for (int e = 0; e < kE; ++e) Emb[(size_t)l * kE + e] = z[e] * r;
-    if (invn) invn[l] = r;
+    if (l >= L) return;
+    reinterpret_cast<float4*>(a.Emb + (size_t)l * kE)[eg] =
+        make_float4(z[0] * r, z[1] * r, z[2] * r, z[3] * r);
+    if (a.G) reinterpret_cast<float4*>(a.G + (size_t)l * kE)[eg] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (eg != 0) return;
+    if (a.invn) a.invn[l] = r;
     s += bb[kE];
-    if (S) S[l] = s;
-    if (HW) {
+    if (a.S) a.S[l] = s;
+    if (a.HW) {
         const float sg = 1.f / (1.f + expf(-s));
-        HW[l] = wmin * exp2f(sg * log2f(wmax / wmin));
+        a.HW[l] = wmin * exp2f(sg * log2f(wmax / wmin));
     }
 }
 
-// Backward of the embedding head for one row: ge = dL/de -> dz = (ge - e (e.ge))
-// * invn, stored in place of ge; dH[l][c] = sum_e W4[e][c] dz[e].
-__global__ void k_embed_bwd(const float* __restrict__ Emb, const float* __restrict__ invn, int L,
-                            const float* __restrict__ W4, float* __restrict__ G,
-                            float* __restrict__ dH) {
+// Backward of the embedding head, kBwdRows rows per block: ge = dL/de -> dz =
+// (ge - e (e.ge)) * invn, stored in place of ge; dH[l][c] = sum_e W4[e][c] dz[e].
+// Thread (row slot, c): a row's 64 channels are written side by side.
+constexpr int kBwdRows = 16;
+__global__ void __launch_bounds__(256) k_embed_bwd(const EncEmbed2 q, const float* __restrict__ W4) {
     __shared__ float w4[kE * kC];
+    __shared__ float es[kBwdRows][kE], gs[kBwdRows][kE];
+    const EncEmbed a = blockIdx.z ? q.s[1] : q.s[0];
+    const int L = a.L;
+    const int l0 = blockIdx.x * kBwdRows;
+    if (l0 >= L) return;
     for (int k = threadIdx.x; k < kE * kC; k += blockDim.x) w4[k] = W4[k];
+    const int r = threadIdx.x / kE, k = threadIdx.x % kE;  // 16 rows x 16 components
+    const int l = l0 + r;
+    if (l < L) {
+        es[r][k] = a.Emb[(size_t)l * kE + k];
+        gs[r][k] = a.G[(size_t)l * kE + k];
+    }
     __syncthreads();
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= L) return;
-    float e[kE], g[kE], dot = 0.f;
+    float dz = 0.f;
+    if (l < L) {
+        float dot = 0.f;
 #pragma unroll
-    for (int k = 0; k < kE; ++k) {
-        e[k] = Emb[(size_t)l * kE + k];
-        g[k] = G[(size_t)l * kE + k];
-        dot = fmaf(e[k], g[k], dot);
+        for (int e = 0; e < kE; ++e) dot = fmaf(es[r][e], gs[r][e], dot);
+        dz = (gs[r][k] - es[r][k] * dot) * a.invn[l];
+        a.G[(size_t)l * kE + k] = dz;
     }
-    const float r = invn[l];
-#pragma unroll
-    for (int k = 0; k < kE; ++k) {
-        g[k] = (g[k] - e[k] * dot) * r;
-        G[(size_t)l * kE + k] = g[k];
-    }
-    for (int c = 0; c < kC; ++c) {
+    __syncthreads();
+    gs[r][k] = dz;
+    __syncthreads();
+    const int c = threadIdx.x % kC;
+    for (int row = threadIdx.x / kC; row < kBwdRows && l0 + row < L; row += 256 / kC) {
         float acc = 0.f;
 #pragma unroll
-        for (int k = 0; k < kE; ++k) acc = fmaf(w4[k * kC + c], g[k], acc);
-        dH[(size_t)l * kC + c] = acc;
+        for (int e = 0; e < kE; ++e) acc = fmaf(w4[e * kC + c], gs[row][e], acc);
+        a.dH[(size_t)(l0 + row) * kC + c] = acc;
     }
 }
 
-// out[a][b] += sum_l U[l][a] V[l][b] for a < na, b < nb (V = null: all ones,
-// i.e. column sums of U), over a tile of 256 rows per block.  na * nb <= 1024.
-__global__ void k_outer(const float* __restrict__ U, int na, const float* __restrict__ V, int nb,
-                        int L, float* __restrict__ out) {
-    __shared__ float us[64][kE], vs[64][kC];
-    const int l0 = blockIdx.x * 256;
-    const int n = na * nb;
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int r0 = l0; r0 < min(l0 + 256, L); r0 += 64) {
-        __syncthreads();
-        for (int k = threadIdx.x; k < 64 * na; k += blockDim.x) {
-            const int r = k / na, a = k % na;
-            us[r][a] = (r0 + r < L) ? U[(size_t)(r0 + r) * na + a] : 0.f;
-        }
-        for (int k = threadIdx.x; k < 64 * nb; k += blockDim.x) {
-            const int r = k / nb, b = k % nb;
-            vs[r][b] = (r0 + r < L) ? (V ? V[(size_t)(r0 + r) * nb + b] : 1.f) : 0.f;
-        }
-        __syncthreads();
-        for (int q = 0; q < 4; ++q) {
-            const int o = threadIdx.x + q * blockDim.x;
-            if (o < n) {
-                const int a = o / nb, b = o % nb;
-                for (int r = 0; r < 64; ++r) acc[q] = fmaf(us[r][a], vs[r][b], acc[q]);
-            }
+// Gradients of a head over a tile of kHeadRows rows: dWh[e][c] += sum_l U[l][e]
+// H[l][c], dbh[e] += sum_l U[l][e], for kN = 16 (embedding) or 1 (half-width)
+// outputs.  Thread (c, eg) owns channel c of kN / 4 (or all) outputs.
+constexpr int kHeadRows = 32;
+template <int kN>
+__global__ void __launch_bounds__(256) k_head_grad(const EncHead2 q, float* __restrict__ dWh,
+                                                   float* __restrict__ dbh) {
+    constexpr int kPer = kN >= 4 ? kN / 4 : 1;
+    __shared__ __align__(16) float us[kHeadRows][kN];
+    const EncHead a = blockIdx.z ? q.s[1] : q.s[0];
+    const int l0 = blockIdx.x * kHeadRows;
+    if (l0 >= a.L) return;
+    const int n = min(kHeadRows, a.L - l0);
+    for (int k = threadIdx.x; k < n * kN; k += blockDim.x) us[k / kN][k % kN] = a.U[(size_t)l0 * kN + k];
+    __syncthreads();
+    const int c = threadIdx.x % kC, eg = threadIdx.x / kC;
+    if (kPer * eg >= kN) return;
+    float acc[kPer], bacc[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) acc[k] = bacc[k] = 0.f;
+#pragma unroll 8
+    for (int r = 0; r < n; ++r) {
+        const float h = a.H[(size_t)(l0 + r) * kC + c];
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            const float u = us[r][kPer * eg + k];
+            acc[k] = fmaf(u, h, acc[k]);
+            bacc[k] += u;
         }
     }
-    for (int q = 0; q < 4; ++q) {
-        const int o = threadIdx.x + q * blockDim.x;
-        if (o < n) atomicAdd(&out[o], acc[q]);
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        atomicAdd(&dWh[(kPer * eg + k) * kC + c], acc[k]);
+        if (c == 0) atomicAdd(&dbh[kPer * eg + k], bacc[k]);
     }
+}
+
+// First of the n path entries whose row is >= row (rows ascend along a path).
+__device__ __forceinline__ int first_of_row(const int32_t* __restrict__ path, int n, int row) {
+    int lo = 0, hi = n;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (path[2 * mid] < row)
+            lo = mid + 1;
+        else
+            hi = mid;
+    }
+    return lo;
 }
 
 // Coarse column matched to every coarse row of A by the exact fine path:
 // the mean column of the path entries in the row's ds fine rows, divided by
-// ds.  Pass 1 sums (one thread per path entry), pass 2 divides.
-__global__ void k_targets_sum(const int32_t* __restrict__ path, const int* __restrict__ plen,
-                              int ds, unsigned long long* __restrict__ jsum,
-                              int* __restrict__ cnt) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= *plen) return;
-    const int i = path[2 * k] / ds;
-    atomicAdd(&jsum[i], (unsigned long long)path[2 * k + 1]);
-    atomicAdd(&cnt[i], 1);
-}
-__global__ void k_targets_fin(const unsigned long long* __restrict__ jsum,
-                              const int* __restrict__ cnt, int Lac, int Lbc, int ds,
-                              int* __restrict__ tgt) {
+// ds.  A row's entries are consecutive in the path.
+__global__ void k_targets(const int32_t* __restrict__ path, const int* __restrict__ plen, int cap,
+                          int ds, int Lac, int Lbc, int* __restrict__ tgt) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= Lac) return;
-    const int n = cnt[i];
+    const int len = min(*plen, cap);
+    unsigned long long jsum = 0;
+    int n = 0;
+    for (int k = first_of_row(path, len, i * ds); k < len && path[2 * k] < (i + 1) * ds; ++k) {
+        jsum += (unsigned long long)path[2 * k + 1];
+        ++n;
+    }
     // every fine row lies on a path except rows a (2,1) step skips; a coarse
     // row of ds >= 2 fine rows always holds one
-    const double m = n > 0 ? (double)jsum[i] / n : 0.0;
+    const double m = n > 0 ? (double)jsum / n : 0.0;
     tgt[i] = min((int)(m / ds), Lbc - 1);
 }
 
-// Contrastive loss, one thread per coarse row i of A (see the file comment).
-// gA[i] = dL/deA_i is written; dL/deB_j is added to gB with atomics.  The
-// loss is the mean over rows.
-__global__ void k_loss_emb(const float* __restrict__ eA, int Lac, const float* __restrict__ eB,
-                           int Lbc, const int* __restrict__ tgt, float* __restrict__ gA,
-                           float* __restrict__ gB, float* __restrict__ loss) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= Lac) return;
-    float a[kE];
-#pragma unroll
-    for (int e = 0; e < kE; ++e) a[e] = eA[(size_t)i * kE + e];
-    const int c = tgt[i];
-    const int j0 = max(c - kWin, 0), j1 = min(c + kWin, Lbc - 1);
-    float lg[2 * kWin + 1];
-    float mx = -INFINITY;
-    for (int j = j0; j <= j1; ++j) {
-        float d = 0.f;
-#pragma unroll
-        for (int e = 0; e < kE; ++e) d = fmaf(a[e], eB[(size_t)j * kE + e], d);
-        lg[j - j0] = d / kTau;
-        mx = fmaxf(mx, lg[j - j0]);
-    }
-    float se = 0.f;
-    for (int j = j0; j <= j1; ++j) se += expf(lg[j - j0] - mx);
-    const float lse = mx + logf(se);
+// Contrastive loss, one warp per coarse row i of A (see the file comment),
+// lane k at column j0 + k of its window (lane 0 also at j0 + 32).  gA[i] = dL/deA_i
+// is written; dL/deB_j is added to gB with atomics, 16 neighbouring floats at a
+// time.  The loss is the mean over rows.  (One thread per row took 75 us on 1500
+// rows: 528 atomics and three passes over its window each.)
+constexpr int kLossRows = 4;
+__global__ void __launch_bounds__(32 * kLossRows)
+    k_loss_emb(const float* __restrict__ eA, int Lac, const float* __restrict__ eB, int Lbc,
+               const int* __restrict__ tgt, float* __restrict__ gA, float* __restrict__ gB,
+               float* __restrict__ loss) {
+    constexpr int kWidth = 2 * kWin + 1;
+    static_assert(kWidth == 33, "a lane per column and one more");
+    __shared__ float s_w[kLossRows][kWidth], s_a[kLossRows][kE], s_loss[kLossRows];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.x * kLossRows + w;
+    float row_loss = 0.f;
     const float inv_n = 1.f / (float)Lac;
-    atomicAdd(loss, (lse - lg[c - j0]) * inv_n);
-    float ga[kE];
+    if (i < Lac) {
+        if (lane < kE) s_a[w][lane] = eA[(size_t)i * kE + lane];
+        __syncwarp();
+        const int c = tgt[i];
+        const int j0 = max(c - kWin, 0), j1 = min(c + kWin, Lbc - 1);
+        float lg[2] = {-INFINITY, -INFINITY};
 #pragma unroll
-    for (int e = 0; e < kE; ++e) ga[e] = 0.f;
-    for (int j = j0; j <= j1; ++j) {
-        const float pj = expf(lg[j - j0] - lse) - (j == c ? 1.f : 0.f);
-        const float w = pj * inv_n / kTau;
+        for (int h = 0; h < 2; ++h) {
+            const int j = j0 + lane + 32 * h;
+            if (j <= j1) {
+                const float4* b = reinterpret_cast<const float4*>(eB + (size_t)j * kE);
+                float d = 0.f;
 #pragma unroll
-        for (int e = 0; e < kE; ++e) {
-            ga[e] = fmaf(w, eB[(size_t)j * kE + e], ga[e]);
-            atomicAdd(&gB[(size_t)j * kE + e], w * a[e]);
+                for (int e4 = 0; e4 < kE / 4; ++e4) {
+                    const float4 v = b[e4];
+                    d = fmaf(s_a[w][4 * e4], v.x, d);
+                    d = fmaf(s_a[w][4 * e4 + 1], v.y, d);
+                    d = fmaf(s_a[w][4 * e4 + 2], v.z, d);
+                    d = fmaf(s_a[w][4 * e4 + 3], v.w, d);
+                }
+                lg[h] = d / kTau;
+            }
         }
-    }
+        float mx = fmaxf(lg[0], lg[1]);
 #pragma unroll
-    for (int e = 0; e < kE; ++e) gA[(size_t)i * kE + e] = ga[e];
+        for (int off = 16; off > 0; off >>= 1)
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+        float se = 0.f;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (j0 + lane + 32 * h <= j1) se += expf(lg[h] - mx);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) se += __shfl_xor_sync(0xffffffffu, se, off);
+        const float lse = mx + logf(se);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = j0 + lane + 32 * h;
+            if (j <= j1) {
+                const float pj = expf(lg[h] - lse) - (j == c ? 1.f : 0.f);
+                s_w[w][lane + 32 * h] = pj * inv_n / kTau;
+                if (j == c) s_loss[w] = (lse - lg[h]) * inv_n;
+            }
+        }
+        __syncwarp();
+        row_loss = s_loss[w];
+        const int n = j1 - j0 + 1;
+        // component lane % 16 over the even (lanes 0-15) and odd columns, then both
+        const int e = lane % kE;
+        float ga = 0.f;
+        for (int k = lane / kE; k < n; k += 2)
+            ga = fmaf(s_w[w][k], eB[(size_t)(j0 + k) * kE + e], ga);
+        ga += __shfl_xor_sync(0xffffffffu, ga, kE);
+        if (lane < kE) gA[(size_t)i * kE + e] = ga;
+        for (int k = lane; k < n * kE; k += 32)
+            atomicAdd(&gB[(size_t)j0 * kE + k], s_w[w][k / kE] * s_a[w][k % kE]);
+    }
+    __syncthreads();
+    if (lane == 0) s_loss[w] = row_loss;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float sum = 0.f;
+#pragma unroll
+        for (int k = 0; k < kLossRows; ++k) sum += s_loss[k];
+        atomicAdd(loss, sum);
+    }
 }
 
 // Width target of every coarse row i of A, in [0, 1] on the log scale of the
@@ -410,24 +606,14 @@ __global__ void k_width_target(const int32_t* __restrict__ cpath, const int* __r
     const int nc = *clen, nf = *plen;
     float need = 0.f;
     if (nc > 0) {
-        int lo = 0, hi = nc;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (cpath[2 * mid] < i - 1) lo = mid + 1; else hi = mid;
-        }
+        const int lo = first_of_row(cpath, nc, i - 1);
         int jmin = 0x7fffffff, jmax = -1;
         for (int k = lo; k < nc && cpath[2 * k] <= i + 1; ++k) {
             jmin = min(jmin, cpath[2 * k + 1]);
             jmax = max(jmax, cpath[2 * k + 1]);
         }
         const int f0 = jmin * ds, f1 = (jmax + 1) * ds - 1;
-        lo = 0;
-        hi = nf;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (path[2 * mid] < i * ds) lo = mid + 1; else hi = mid;
-        }
-        for (int k = lo; k < nf && path[2 * k] < (i + 1) * ds; ++k) {
+        for (int k = first_of_row(path, nf, i * ds); k < nf && path[2 * k] < (i + 1) * ds; ++k) {
             const int j = path[2 * k + 1];
             need = fmaxf(need, (float)max(max(f0 - j, j - f1), 0));
         }
@@ -467,29 +653,24 @@ __global__ void k_adam(int n, float* __restrict__ P, float* __restrict__ G, floa
     G[k] = 0.f;
 }
 
-template <bool kBwd, bool kBF16>
-cudaError_t conv_t(const float* X, const float* mask, int L, int Cin, const float* W,
-                   const float* b, int relu, float* Y, cudaStream_t s) {
-    const int smem = (Cin * kK * kC + (kTL + 2 * kPad) * Cin) * (int)sizeof(float);
-    static DeviceSlots raised;
-    const cudaError_t e = raise_smem_once(k_conv<kBwd, kBF16>,
-                                          (kC * kK * kC + (kTL + 2 * kPad) * kC) * 4, raised);
-    if (e != cudaSuccess) return e;
-    k_conv<kBwd, kBF16><<<(L + kTL - 1) / kTL, kConvThreads, smem, s>>>(X, mask, L, Cin, W, b,
-                                                                       relu, Y);
-    return cudaGetLastError();
+// Grid of both sequences of q in tiles of `rows` rows.
+template <class Q>
+dim3 enc_grid(const Q& q, int n, int rows, int y = 1) {
+    int L = 0;
+    for (int k = 0; k < n; ++k) L = q.s[k].L > L ? q.s[k].L : L;
+    return dim3((unsigned)((L + rows - 1) / rows), (unsigned)y, (unsigned)n);
 }
 
-template <int kCPT>
-cudaError_t wgrad_t(const float* X, int L, int Cin, const float* dY, const float* Yout, float* dW,
-                    float* db, cudaStream_t s) {
-    const int smem = (kTW * kC + (kTW + 2 * kPad) * Cin) * (int)sizeof(float);
-    static DeviceSlots raised;
-    const cudaError_t e = raise_smem_once(k_conv_wgrad<kCPT>,
-                                          (kTW * kC + (kTW + 2 * kPad) * kC) * 4, raised);
-    if (e != cudaSuccess) return e;
-    k_conv_wgrad<kCPT><<<(L + kTW - 1) / kTW, kConvThreads, smem, s>>>(X, L, Cin, dY, Yout, dW,
-                                                                      db);
+template <bool kBwd, bool kBF16>
+cudaError_t conv_t(const EncRows2& q, int n, int Cin, const float* W, const float* b, int relu,
+                   cudaStream_t s) {
+    static_assert((kC * kXS + kC * kK * kWS) * 4 <= 48 * 1024, "default shared memory");
+    const int smem = (Cin * kXS + Cin * kK * kWS) * (int)sizeof(float);
+    const dim3 grid = enc_grid(q, n, kTL, kC / kCO);
+    if (Cin == kC)
+        k_conv<kC, kBwd, kBF16><<<grid, kConvThreads, smem, s>>>(q, Cin, W, b, relu);
+    else
+        k_conv<0, kBwd, kBF16><<<grid, kConvThreads, smem, s>>>(q, Cin, W, b, relu);
     return cudaGetLastError();
 }
 
@@ -512,65 +693,65 @@ EncLayout enc_layout(int D) {
     return p;
 }
 
-cudaError_t launch_pool_norm(const float* X, int L, int D, int ds, float* Y, cudaStream_t s) {
-    const int Lc = (L + ds - 1) / ds;
-    k_pool_norm<<<(Lc + 127) / 128, 128, 0, s>>>(X, L, D, ds, Y);
+cudaError_t launch_pool_norm(const EncRows2& q, int n, int D, int ds, cudaStream_t s) {
+    if (D < 1 || D > kC) return cudaErrorInvalidValue;
+    EncRows2 c = q;  // coarse rows for the grid
+    for (int k = 0; k < n; ++k) c.s[k].L = (q.s[k].L + ds - 1) / ds;
+    if (D <= 16)
+        k_pool_norm<16><<<enc_grid(c, n, 8), 128, 0, s>>>(q, D, ds);
+    else
+        k_pool_norm<32><<<enc_grid(c, n, 4), 128, 0, s>>>(q, D, ds);
     return cudaGetLastError();
 }
 
-cudaError_t launch_conv(const float* X, const float* mask, int L, int Cin, const float* W,
-                        const float* b, int relu, int bwd, int bf16, float* Y, cudaStream_t s) {
+cudaError_t launch_conv(const EncRows2& q, int n, int Cin, const float* W, const float* b, int relu,
+                        int bwd, int bf16, cudaStream_t s) {
     if (Cin < 1 || Cin > kC) return cudaErrorInvalidValue;
-    if (bwd) return bf16 ? cudaErrorInvalidValue : conv_t<true, false>(X, mask, L, Cin, W, b, relu, Y, s);
-    return bf16 ? conv_t<false, true>(X, mask, L, Cin, W, b, relu, Y, s)
-                : conv_t<false, false>(X, mask, L, Cin, W, b, relu, Y, s);
+    if (bwd) return bf16 ? cudaErrorInvalidValue : conv_t<true, false>(q, n, Cin, W, b, relu, s);
+    return bf16 ? conv_t<false, true>(q, n, Cin, W, b, relu, s)
+                : conv_t<false, false>(q, n, Cin, W, b, relu, s);
 }
 
-cudaError_t launch_conv_wgrad(const float* X, int L, int Cin, const float* dY, const float* Yout,
-                              float* dW, float* db, cudaStream_t s) {
-    const int cpt = (Cin + 3) / 4;
-    if (cpt <= 4) return wgrad_t<4>(X, L, Cin, dY, Yout, dW, db, s);
-    if (cpt <= 8) return wgrad_t<8>(X, L, Cin, dY, Yout, dW, db, s);
-    if (cpt <= 16) return wgrad_t<16>(X, L, Cin, dY, Yout, dW, db, s);
-    return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_embed(const float* H, int L, const float* params, const EncLayout& p, int bf16,
-                         float wmin, float wmax, float* Emb, float* invn, float* S, float* HW,
-                         cudaStream_t s) {
-    k_embed<<<(L + 127) / 128, 128, 0, s>>>(H, L, params + p.W4, params + p.b4, params + p.W5,
-                                           params + p.b5, bf16, wmin, wmax, Emb, invn, S, HW);
+cudaError_t launch_conv_wgrad(const EncGrad2& q, int n, int Cin, float* dW, float* db,
+                              cudaStream_t s) {
+    if (Cin < 1 || Cin > kC) return cudaErrorInvalidValue;
+    k_conv_wgrad<<<enc_grid(q, n, kTW * kTiles, (Cin + kCI - 1) / kCI), kWgThreads, 0, s>>>(q, Cin, dW, db);
     return cudaGetLastError();
 }
 
-cudaError_t launch_embed_bwd(const float* Emb, const float* invn, int L, const float* W4,
-                             float* G, float* dH, cudaStream_t s) {
-    k_embed_bwd<<<(L + 127) / 128, 128, 0, s>>>(Emb, invn, L, W4, G, dH);
+cudaError_t launch_embed(const EncEmbed2& q, int n, const float* params, const EncLayout& p, int bf16,
+                         float wmin, float wmax, cudaStream_t s) {
+    k_embed<<<enc_grid(q, n, 32), 128, 0, s>>>(q, params + p.W4, params + p.b4, params + p.W5,
+                                              params + p.b5, bf16, wmin, wmax);
     return cudaGetLastError();
 }
 
-cudaError_t launch_outer(const float* U, int na, const float* V, int nb, int L, float* out,
-                         cudaStream_t s) {
-    if (na < 1 || na > kE || nb < 1 || nb > kC || na * nb > 1024) return cudaErrorInvalidValue;
-    k_outer<<<(L + 255) / 256, 256, 0, s>>>(U, na, V, nb, L, out);
+cudaError_t launch_embed_bwd(const EncEmbed2& q, int n, const float* W4, cudaStream_t s) {
+    k_embed_bwd<<<enc_grid(q, n, kBwdRows), 256, 0, s>>>(q, W4);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_head_grad(const EncHead2& q, int n, int outputs, float* dW, float* db,
+                             cudaStream_t s) {
+    if (outputs == kE)
+        k_head_grad<kE><<<enc_grid(q, n, kHeadRows), 256, 0, s>>>(q, dW, db);
+    else if (outputs == 1)
+        k_head_grad<1><<<enc_grid(q, n, kHeadRows), 256, 0, s>>>(q, dW, db);
+    else
+        return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
 
 cudaError_t launch_targets(const int32_t* path, const int* plen, int cap, int ds, int Lac, int Lbc,
-                           unsigned long long* jsum, int* cnt, int* tgt, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(jsum, 0, sizeof(unsigned long long) * Lac, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, sizeof(int) * Lac, s);
-    if (e != cudaSuccess) return e;
-    k_targets_sum<<<(cap + 255) / 256, 256, 0, s>>>(path, plen, ds, jsum, cnt);
-    k_targets_fin<<<(Lac + 255) / 256, 256, 0, s>>>(jsum, cnt, Lac, Lbc, ds, tgt);
+                           int* tgt, cudaStream_t s) {
+    k_targets<<<(Lac + 63) / 64, 64, 0, s>>>(path, plen, cap, ds, Lac, Lbc, tgt);
     return cudaGetLastError();
 }
 
 cudaError_t launch_loss_emb(const float* eA, int Lac, const float* eB, int Lbc, const int* tgt,
                             float* gA, float* gB, float* loss, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(gB, 0, sizeof(float) * (size_t)Lbc * kE, s);
-    if (e != cudaSuccess) return e;
-    k_loss_emb<<<(Lac + 127) / 128, 128, 0, s>>>(eA, Lac, eB, Lbc, tgt, gA, gB, loss);
+    k_loss_emb<<<(Lac + kLossRows - 1) / kLossRows, 32 * kLossRows, 0, s>>>(eA, Lac, eB, Lbc, tgt,
+                                                                           gA, gB, loss);
     return cudaGetLastError();
 }
 

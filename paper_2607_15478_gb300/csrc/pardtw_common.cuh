@@ -331,24 +331,49 @@ struct EncLayout {
     size_t W1, b1, W2, b2, W3, b3, W4, b4, W5, b5, count;
 };
 EncLayout enc_layout(int D);
-cudaError_t launch_pool_norm(const float* X, int L, int D, int ds, float* Y, cudaStream_t s);
+// A layer's rows of one or two sequences (n of them; one launch runs both).
+struct EncRows {
+    const float* X;  // input rows
+    const float* M;  // conv backward: rows of X count where M > 0 (may be null)
+    float* Y;        // output rows
+    int L;
+};
+struct EncGrad {
+    const float *X, *dY, *Yout;
+    int L;
+};
+struct EncEmbed {
+    const float* H;
+    float *Emb, *invn, *S, *HW, *G, *dH;  // see k_embed, k_embed_bwd
+    int L;
+};
+struct EncHead {
+    const float *U, *H;
+    int L;
+};
+struct EncRows2 { EncRows s[2]; };
+struct EncGrad2 { EncGrad s[2]; };
+struct EncEmbed2 { EncEmbed s[2]; };
+struct EncHead2 { EncHead s[2]; };
+// X: fine frames (L of them), Y: pooled, normalised frames.
+cudaError_t launch_pool_norm(const EncRows2& q, int n, int D, int ds, cudaStream_t s);
 // conv5 of L rows: forward (bwd = 0: W [64][Cin][5], bias, relu) or the
 // backward-data pass (bwd = 1: W the forward weight [64][64][5] read
-// transposed and flipped, X masked by mask > 0); bf16 rounds inputs and
+// transposed and flipped, X masked by M > 0); bf16 rounds inputs and
 // weights (forward only).
-cudaError_t launch_conv(const float* X, const float* mask, int L, int Cin, const float* W,
-                        const float* b, int relu, int bwd, int bf16, float* Y, cudaStream_t s);
-cudaError_t launch_conv_wgrad(const float* X, int L, int Cin, const float* dY, const float* Yout,
-                              float* dW, float* db, cudaStream_t s);
-cudaError_t launch_embed(const float* H, int L, const float* params, const EncLayout& p, int bf16,
-                         float wmin, float wmax, float* Emb, float* invn, float* S, float* HW,
-                         cudaStream_t s);
-cudaError_t launch_embed_bwd(const float* Emb, const float* invn, int L, const float* W4,
-                             float* G, float* dH, cudaStream_t s);
-cudaError_t launch_outer(const float* U, int na, const float* V, int nb, int L, float* out,
-                         cudaStream_t s);
+cudaError_t launch_conv(const EncRows2& q, int n, int Cin, const float* W, const float* b, int relu,
+                        int bwd, int bf16, cudaStream_t s);
+cudaError_t launch_conv_wgrad(const EncGrad2& q, int n, int Cin, float* dW, float* db,
+                              cudaStream_t s);
+cudaError_t launch_embed(const EncEmbed2& q, int n, const float* params, const EncLayout& p, int bf16,
+                         float wmin, float wmax, cudaStream_t s);
+cudaError_t launch_embed_bwd(const EncEmbed2& q, int n, const float* W4, cudaStream_t s);
+// outputs = 16 (embedding head) or 1 (half-width head).
+cudaError_t launch_head_grad(const EncHead2& q, int n, int outputs, float* dW, float* db,
+                             cudaStream_t s);
 cudaError_t launch_targets(const int32_t* path, const int* plen, int cap, int ds, int Lac, int Lbc,
-                           unsigned long long* jsum, int* cnt, int* tgt, cudaStream_t s);
+                           int* tgt, cudaStream_t s);
+// gB is added to (zeroed by launch_embed's G).
 cudaError_t launch_loss_emb(const float* eA, int Lac, const float* eB, int Lbc, const int* tgt,
                             float* gA, float* gB, float* loss, cudaStream_t s);
 cudaError_t launch_width_target(const int32_t* cpath, const int* clen, const int32_t* path,
