@@ -35,18 +35,21 @@
 namespace pardtw {
 namespace {
 
-constexpr int kSegCols = kSegThreads * kColsPerWord;  // 2048 columns computed per CTA
+constexpr int kMapWarps = 4;  // segments per CTA
 
 template <bool kMany, bool kBanded>
-__global__ void __launch_bounds__(kSegThreads) k_bandmap(const BtArgs one,
-                                                         const BtArgs* __restrict__ many) {
-    const BtArgs& a = kMany ? many[blockIdx.z] : one;
-    // left-neighbour exchange, double-buffered by row parity: columns 14, 15
-    // of row i-1 and column 15 of row i-2 of every thread
-    __shared__ int s_x[2][kSegThreads][3];
+__global__ void __launch_bounds__(32 * kMapWarps) k_bandmap(const BtArgs one,
+                                                            const BtArgs* __restrict__ many) {
+    const BtArgs a = kMany ? many[blockIdx.z] : one;
     // kMany: one pair per blockIdx.z (the grid covers the largest pair;
-    // blocks beyond a pair's bands or columns leave at once)
-    bandmap_segment<kSegThreads, kBanded>(a, blockIdx.y, blockIdx.x, s_x);
+    // warps beyond a pair's bands or columns leave at once)
+    bandmap_segment<kBanded>(a, blockIdx.y, blockIdx.x * kMapWarps + (threadIdx.x >> 5),
+                             threadIdx.x & 31);
+}
+// CTAs per band that cover the segments of all of a pair's columns.
+int map_ctas(int Lb) {
+    const int segs = (Lb + kSegWidth - 1) / kSegWidth;
+    return (segs + kMapWarps - 1) / kMapWarps;
 }
 
 }  // namespace
@@ -59,6 +62,15 @@ __device__ __forceinline__ int2 entry_cell(int e, int x) {
 // The entry of cell c of a band's last two rows from its exits word x (.x:
 // second-to-last row, .y: last row); last = the band's last row.
 __device__ __forceinline__ int pick_exit(int2 x, int ci, int last) { return ci == last ? x.y : x.x; }
+
+// Whether a path can cross rows r1-2, r1-1 at column j (see bandmap_segment; a
+// banded sweep's path lies in the ranges of those rows' strips).
+__device__ __forceinline__ bool map_column(const BtArgs& a, int r1, int j) {
+    const int lo = path_lo(r1 - 2, a.La, a.Lb), hi = path_hi(r1 - 1, a.La, a.Lb);
+    if (j < lo || j > hi) return false;
+    if (!a.ranges) return true;
+    return j >= a.ranges[(r1 - 2) / a.rps].x * 8 && j < a.ranges[(r1 - 1) / a.rps].y * 8;
+}
 
 // Two-band exit map: for band b = nbands-2-2m (m = blockIdx.y < n2) and
 // column j, the entries of the cells of band b's last two rows two bands up,
@@ -76,10 +88,7 @@ __global__ void __launch_bounds__(256) k_bt_compose(const BtArgs one,
     if (m >= sc.n2 || j >= Lb) return;
     const int b = sc.nbands - 2 - 2 * m;
     const int r1 = (b + 1) * kBand;  // b <= nbands-2: a whole band
-    // columns of rows r1-2, r1-1 that can lie on a path (see bandmap_segment)
-    const int lo = max((r1 - 1) / 2, Lb - 1 - 2 * (La - 1 - (r1 - 2)));
-    const int hi = min(2 * (r1 - 1), Lb - 1);
-    if (j < lo || j > hi) return;
+    if (!map_column(a, r1, j)) return;
     const int2* __restrict__ exits = sc.exits;
     const int2 x = exits[(size_t)b * Lb + j];
     auto hop = [&](int e) -> int {
@@ -106,9 +115,7 @@ __global__ void __launch_bounds__(256) k_bt_compose4(const BtArgs one,
     if (m >= sc.n4 || j >= Lb) return;
     const int b = sc.nbands - 2 - 4 * m;
     const int r1 = (b + 1) * kBand;
-    const int lo = max((r1 - 1) / 2, Lb - 1 - 2 * (La - 1 - (r1 - 2)));
-    const int hi = min(2 * (r1 - 1), Lb - 1);
-    if (j < lo || j > hi) return;
+    if (!map_column(a, r1, j)) return;
     const int2* __restrict__ exits2 = sc.exits2;
     const int2 x = exits2[(size_t)(2 * m) * Lb + j];  // into band b-2's last two rows
     auto hop = [&](int e) -> int {
@@ -191,10 +198,13 @@ __global__ void k_bt_chain(const BtArgs one, const BtArgs* __restrict__ many) {
 }
 
 // One warp per band: walk back from the path's last cell in band b while
-// inside the band (BlockWalker), writing the cells (descending) into
+// inside the band (WindowWalker), writing the cells (descending) into
 // seg + b * band; count[b] = cells written.
+constexpr int kWalkWarps = 4;  // bands per CTA
 template <bool kMany>
-__global__ void k_bt_walk(const BtArgs one, const BtArgs* __restrict__ many) {
+__global__ void __launch_bounds__(32 * kWalkWarps) k_bt_walk(const BtArgs one, const BtArgs* __restrict__ many) {
+    static_assert(kWalkRows >= kBand, "a band's rows fit the window");
+    __shared__ uint32_t s_win[kWalkWarps][kWalkWords];
     const BtArgs& a = kMany ? many[blockIdx.y] : one;
     const int band = kBand;
     DevCtl* ctl = a.ctl;
@@ -233,24 +243,24 @@ __global__ void k_bt_walk(const BtArgs one, const BtArgs* __restrict__ many) {
     }
     if (bad) c = make_int2(r0, 0);  // no walk; reported below
     int i = c.x, j = c.y;
-    BlockWalker w{a.bp, a.nchunk, a.rps, a.wpb, lane};
-    w.start(i, j);
+    WindowWalker w{a.bp, a.nchunk, a.rps, a.wpb, lane, s_win[threadIdx.x >> 5], 0, 0};
+    w.load(i, j);
     int n = 0;
     int2* out = seg + (size_t)b * band;
+    int2 mine = make_int2(0, 0);  // cell n of the walk for n % 32 = lane, stored 32 at a time
     while (!bad && i >= r0) {
-        if (n >= band || j < 0) {
+        if (n >= band || j < 0 || !w.inside(i, j)) {
             bad = 1;
             break;
         }
-        if (lane == 0) out[n] = make_int2(i, j);
-        ++n;
+        if ((n & 31) == lane) mine = make_int2(i, j);
+        if ((++n & 31) == 0) out[n - 32 + lane] = mine;
         if (i == 0 && j == 0) break;
-        const uint32_t f = w.field(j);
-        const int di = field_di(f);
-        i -= di;
+        const uint32_t f = w.field(i, j);
+        i -= field_di(f);
         j -= field_dj(f);
-        w.step(di, j, i >= r0);
     }
+    if (lane < (n & 31)) out[(n & ~31) + lane] = mine;
     // the walk must leave the band exactly at the cell its first cell's entry names
     if (b > 0 && !bad && (i != target.x || j != target.y)) bad = 1;
     if (lane == 0) {
@@ -347,12 +357,11 @@ size_t bandmap_scratch_bytes(int La, int Lb) {
 
 cudaError_t launch_backtrace_bands(const BtArgs& a, cudaStream_t s) {
     const int nbands = (a.La + kBand - 1) / kBand;
-    const int width = kSegCols - 2 * kBand;
-    dim3 grid((unsigned)((a.Lb + width - 1) / width), (unsigned)nbands, 1);
+    const dim3 grid((unsigned)map_ctas(a.Lb), (unsigned)nbands, 1);
     if (a.ranges)
-        k_bandmap<false, true><<<grid, kSegThreads, 0, s>>>(a, nullptr);
+        k_bandmap<false, true><<<grid, 32 * kMapWarps, 0, s>>>(a, nullptr);
     else
-        k_bandmap<false, false><<<grid, kSegThreads, 0, s>>>(a, nullptr);
+        k_bandmap<false, false><<<grid, 32 * kMapWarps, 0, s>>>(a, nullptr);
     const int n2 = nbands >= 4 ? (nbands - 2) / 2 : 0;
     if (n2 > 0)
         k_bt_compose<false><<<dim3((unsigned)((a.Lb + 255) / 256), (unsigned)n2, 1), 256, 0, s>>>(
@@ -362,7 +371,7 @@ cudaError_t launch_backtrace_bands(const BtArgs& a, cudaStream_t s) {
         k_bt_compose4<false><<<dim3((unsigned)((a.Lb + 255) / 256), (unsigned)n4, 1), 256, 0, s>>>(
             a, nullptr);
     k_bt_chain<false><<<1, 32, 0, s>>>(a, nullptr);
-    k_bt_walk<false><<<(nbands + 3) / 4, 128, 0, s>>>(a, nullptr);
+    k_bt_walk<false><<<(nbands + kWalkWarps - 1) / kWalkWarps, 32 * kWalkWarps, 0, s>>>(a, nullptr);
     k_bt_emit<false><<<dim3((unsigned)nbands, 1), kBand, 0, s>>>(a, nullptr);
     return cudaGetLastError();
 }
@@ -371,9 +380,8 @@ cudaError_t launch_backtrace_bands_many(const BtArgs* many, int n, int maxLa, in
                                         cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const int nbands = (maxLa + kBand - 1) / kBand;
-    const int width = kSegCols - 2 * kBand;
-    dim3 grid((unsigned)((maxLb + width - 1) / width), (unsigned)nbands, (unsigned)n);
-    k_bandmap<true, false><<<grid, kSegThreads, 0, s>>>(BtArgs{}, many);
+    const dim3 grid((unsigned)map_ctas(maxLb), (unsigned)nbands, (unsigned)n);
+    k_bandmap<true, false><<<grid, 32 * kMapWarps, 0, s>>>(BtArgs{}, many);
     const int n2 = nbands >= 4 ? (nbands - 2) / 2 : 0;
     if (n2 > 0)
         k_bt_compose<true><<<dim3((unsigned)((maxLb + 255) / 256), (unsigned)n2, (unsigned)n),
@@ -383,8 +391,8 @@ cudaError_t launch_backtrace_bands_many(const BtArgs* many, int n, int maxLa, in
         k_bt_compose4<true><<<dim3((unsigned)((maxLb + 255) / 256), (unsigned)n4, (unsigned)n),
                               256, 0, s>>>(BtArgs{}, many);
     k_bt_chain<true><<<n, 32, 0, s>>>(BtArgs{}, many);
-    k_bt_walk<true><<<dim3((unsigned)((nbands + 3) / 4), (unsigned)n), 128, 0, s>>>(BtArgs{},
-                                                                                     many);
+    k_bt_walk<true><<<dim3((unsigned)((nbands + kWalkWarps - 1) / kWalkWarps), (unsigned)n),
+                      32 * kWalkWarps, 0, s>>>(BtArgs{}, many);
     k_bt_emit<true><<<dim3((unsigned)nbands, (unsigned)n), kBand, 0, s>>>(BtArgs{}, many);
     return cudaGetLastError();
 }

@@ -7,7 +7,6 @@ namespace pardtw {
 
 namespace {
 
-constexpr int kSegThreads = 128;  // with 128-row bands: 64 +5%, 256 +5%, 512 +40% (backtrace time)
 constexpr int kNoPath = -2;
 constexpr int kOrigin = -1;
 constexpr int kBand = 128;  // rows per band
@@ -48,107 +47,76 @@ __host__ __device__ inline BtScratch bt_scratch(void* scratch, int La, int Lb) {
 }
 
 
-// A segment of a band is mapped by a block of NT threads: thread t owns the
-// 16 columns s0 + 16 t .. + 15 of the segment's computed range, where
-// s0 = c0 - halo; the segment stores columns c0 .. c0 + width - 1 with
-// width = NT * 16 - 2 * band (segments are width apart).  Two row buffers of
-// entries per thread live in registers; the left-neighbour columns a thread
-// needs come through shared memory.
+// A segment of a band is mapped by one warp: lane t owns the 32 columns
+// s0 + 32 t .. + 31 of the segment's computed range, where s0 = c0 - halo; the
+// segment stores columns c0 .. c0 + kSegWidth - 1 (segments are kSegWidth apart).
 //
-// One row of the band map for a thread's 16 columns.  kTop: the row is one
-// of the band's first two rows, whose predecessors may lie in the band above.
-template <int NT, bool kTop, bool kBanded>
-__device__ __forceinline__ void bandmap_row(int i, int r0, int r1, int La, int Lb, int jb, int c0,
-                                            int width, int b, uint32_t word, int t,
-                                            int (*s_x)[NT][3], int* e1, int* e2,
-                                            int2* __restrict__ exits, int* __restrict__ end_entry,
-                                            const int2* __restrict__ ranges, int rps) {
-    // banded DP: cells outside the row's strip range were never computed
-    int cx = 0, cy = 0;
-    if (kBanded) {
-        const int2 r = __ldg(ranges + i / rps);
-        cx = r.x * 8;
-        cy = r.y * 8;
-    }
-    const int par = i & 1;
-    s_x[par][t][0] = e1[kColsPerWord - 2];
-    s_x[par][t][1] = e1[kColsPerWord - 1];
-    s_x[par][t][2] = e2[kColsPerWord - 1];
-    __syncthreads();
-    // (i-1, jb-2), (i-1, jb-1), (i-2, jb-1) from the left neighbour
-    const int l1m2 = t > 0 ? s_x[par][t - 1][0] : kNoPath;
-    const int l1m1 = t > 0 ? s_x[par][t - 1][1] : kNoPath;
-    const int l2m1 = t > 0 ? s_x[par][t - 1][2] : kNoPath;
-    int en[kColsPerWord];
-#pragma unroll
-    for (int q = 0; q < kColsPerWord; ++q) {
-        // field bits of column q (see step_of_field): bit 0 -> (1,1), else
-        // bit 1 -> (1,2), else (2,1)
-        int p11 = (q >= 1) ? e1[q - 1] : l1m1;                    // (i-1, j-1)
-        int p12 = (q >= 2) ? e1[q - 2] : (q == 1 ? l1m1 : l1m2);  // (i-1, j-2)
-        int p21 = (q >= 1) ? e2[q - 1] : l2m1;                    // (i-2, j-1)
-        // the field's bits 0 and 1, each tested into a predicate
-        if (kTop) {
-            // predecessors in the band above are named 2 * column + (1 if in
-            // its last row)
-            const int j = jb + q;
-            if (i == r0) {
-                p11 = (i >= 1 && j >= 1) ? 2 * (j - 1) + 1 : kNoPath;
-                p12 = (i >= 1 && j >= 2) ? 2 * (j - 2) + 1 : kNoPath;
-                p21 = (i >= 2 && j >= 1) ? 2 * (j - 1) : kNoPath;
-            } else {  // i == r0 + 1: only (i-2, j-1) is above
-                p21 = (r0 >= 1 && j >= 1) ? 2 * (j - 1) + 1 : kNoPath;
-            }
-        }
-        int v = (word & (2u << (2 * q))) ? p12 : p21;  // bit 1: (1,2), else (2,1)
-        v = (word & (1u << (2 * q))) ? p11 : v;        // bit 0: (1,1)
-        if (kTop && i == 0 && jb + q == 0) v = kOrigin;
-        if (kBanded && (jb + q < cx || jb + q >= cy)) v = kNoPath;
-        en[q] = v;
-    }
-    // the band's last two rows are kept for the band below
-    if (i >= r1 - 2 && r1 < La) {
-        const int which = (i == r1 - 1) ? 1 : 0;
-#pragma unroll
-        for (int q = 0; q < kColsPerWord; ++q) {
-            const int j = jb + q;
-            if (j >= c0 && j < c0 + width && j < Lb)
-                reinterpret_cast<int*>(exits + (size_t)b * Lb + j)[which] = en[q];
-        }
-    }
-    if (i == La - 1) {
-        const int q = (Lb - 1) - jb;
-        if (q >= 0 && q < kColsPerWord && Lb - 1 >= c0 && Lb - 1 < c0 + width) {
-#pragma unroll
-            for (int u = 0; u < kColsPerWord; ++u)
-                if (u == q) *end_entry = en[u];
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < kColsPerWord; ++q) {
-        e2[q] = e1[q];
-        e1[q] = en[q];
+// Inside a segment an entry is 16 bits, 2 * (column - s0) + (1 if in the band
+// above's last row), or one of two codes; a register holds those of columns u
+// and u + 8 of a backpointer word, whose fields lie 16 bits apart, so the two
+// selects of a cell (bit 1: (1,2), else (2,1); bit 0: (1,1)) are two bitwise
+// selects for two cells, by masks that one shift and one byte permute (with sign
+// replication) make from the word.  The pairs of columns u-1 and u-2 are the
+// registers before; only u = 0, 1 need the neighbouring word (the left lane's by
+// two shuffles a row).  What bounds it: these ~108 instructions per row of 1024
+// columns, and the loads of the words: four rows at a time (16 bytes), since
+// every lane's word lies in a 32-byte sector of its own.  No barriers.  (One
+// entry per register, one word per load and a barrier per row of 128 threads
+// took 89 us on the 20000 x 25000 pair and 1.5 ms at 100000 x 126231; see
+// bandmap.cu for the times now.)
+constexpr int kSegCols = 1024;
+constexpr int kSegWidth = kSegCols - 2 * kBand;
+constexpr unsigned kNoPath2 = 0xFFFEFFFEu;  // two columns without a path
+constexpr unsigned kOrigin16 = 0xFFFFu;
+
+// 0xFFFF in the half whose field bit (bit 2u + k, and 16 above it) is set: the
+// bit shifted to its half's top, then each half filled with the sign of its
+// upper byte.
+template <int u, int k>
+__device__ __forceinline__ unsigned field_mask(unsigned w) {
+    unsigned m;
+    asm("prmt.b32 %0, %1, %1, 0xBB99;" : "=r"(m) : "r"(w << (15 - 2 * u - k)));
+    return m;
+}
+__device__ __forceinline__ unsigned bit_select(unsigned m, unsigned a, unsigned b) {
+    return (m & a) | (~m & b);
+}
+// The pair left of a word: (high half of l, low half of r).
+__device__ __forceinline__ unsigned left_pair(unsigned l, unsigned r) {
+    return __byte_perm(l, r, 0x5432u);
+}
+
+// Two words' entries of one row: columns u, u + 8 in w[0][u], 16 + u, 24 + u in w[1][u].
+struct RowEntries {
+    unsigned w[2][8];
+};
+
+// Row i from rows i-1 (e1) and i-2 (e2); l1a, l1b, l2a: registers 7 and 6 of the
+// left lane's second word in e1 and 7 in e2.
+template <int U = 0>
+__device__ __forceinline__ void bandmap_pairs(unsigned word, const unsigned* e1, const unsigned* e2,
+                                              unsigned q11, unsigned q12, unsigned q21,
+                                              unsigned* out) {
+    if constexpr (U < 8) {
+        // q11 = (column -1, 7), q12 = (-2, 6) of row i-1; q21 = (-1, 7) of row i-2
+        const unsigned p11 = U >= 1 ? e1[U >= 1 ? U - 1 : 0] : q11;
+        const unsigned p12 = U >= 2 ? e1[U >= 2 ? U - 2 : 0] : (U == 1 ? q11 : q12);
+        const unsigned p21 = U >= 1 ? e2[U >= 1 ? U - 1 : 0] : q21;
+        const unsigned v = bit_select(field_mask<U, 1>(word), p12, p21);
+        out[U] = bit_select(field_mask<U, 0>(word), p11, v);
+        bandmap_pairs<U + 1>(word, e1, e2, q11, q12, q21, out);
     }
 }
 
-constexpr int kRowsAhead = 8;  // backpointer rows loaded ahead of use
-
-// The band map of band b over segment segx of its columns, by the NT threads
-// of the calling block (all of them must call it; t = threadIdx.x < NT).
-// s_x: the block's left-neighbour exchange buffer.
-template <int NT, bool kBanded>
-__device__ __forceinline__ void bandmap_segment(const BtArgs& a, int b, int segx,
-                                                int (*s_x)[NT][3]) {
+// The band map of band b over segment segx of its columns, by one warp.
+template <bool kBanded>
+__device__ __forceinline__ void bandmap_segment(const BtArgs& a, int b, int segx, int lane) {
     const uint32_t* __restrict__ bp = a.bp;
     const int La = a.La, Lb = a.Lb, nchunk = a.nchunk, rps = a.rps, wpb = a.wpb;
-    const int band = kBand;
     const BtScratch sc = bt_scratch(a.scratch, La, Lb);
-    int2* __restrict__ exits = sc.exits;
-    int* __restrict__ end_entry = sc.end_entry;
-    const int width = NT * kColsPerWord - 2 * band;
-    if (b >= sc.nbands) return;  // CTA-uniform
-    const int r0 = b * band;
-    const int r1 = min(r0 + band, La);
+    if (b >= sc.nbands) return;  // warp-uniform, as are the returns below
+    const int r0 = b * kBand;
+    const int r1 = min(r0 + kBand, La);
     int c0, halo;  // first stored column; columns recomputed to its left (multiple of 16)
     if (kBanded) {
         // segments start at the band's first column over these rows (the
@@ -156,79 +124,133 @@ __device__ __forceinline__ void bandmap_segment(const BtArgs& a, int b, int segx
         // path, so the first segment needs no halo and the rest of the grid
         // covers only the band's columns
         const int xs = a.ranges[r0 / rps].x * 8, ys = a.ranges[(r1 - 1) / rps].y * 8;
-        c0 = (xs & ~(kColsPerWord - 1)) + segx * width;
-        if (c0 >= min(ys, Lb)) return;  // CTA-uniform
-        halo = segx == 0 ? 0 : 2 * band;
+        c0 = (xs & ~(kColsPerWord - 1)) + segx * kSegWidth;
+        if (c0 >= min(ys, Lb)) return;
     } else {
         // Only cells that can lie on a path (path_lo, path_hi): a path
         // cell's predecessors are path cells too, so segments start at
-        // path_lo(r0) (the first without a halo) and end at path_hi(r1-1);
+        // path_lo(r0), less the two columns a first step from the band above
+        // can come from, (the first without a halo) and end at path_hi(r1-1);
         // the cells left out are never asked for.
-        const int xs = max(0, path_lo(r0, La, Lb));
+        const int xs = max(0, path_lo(r0, La, Lb) - 2);
         const int ys = min(Lb, path_hi(r1 - 1, La, Lb) + 1);
-        c0 = (xs & ~(kColsPerWord - 1)) + segx * width;
-        if (c0 >= ys) return;  // CTA-uniform
-        halo = segx == 0 ? 0 : 2 * band;
+        c0 = (xs & ~(kColsPerWord - 1)) + segx * kSegWidth;
+        if (c0 >= ys) return;
     }
+    halo = segx == 0 ? 0 : 2 * kBand;
     const int s0 = c0 - halo;
-    const int t = threadIdx.x;
-    const int jb = s0 + kColsPerWord * t;  // first column of this thread
-    const bool have = jb < nchunk * kColsPerWord;
-    // rows are loaded in order r0, r0 + 1, ...: the word address of the next
-    // one (see bp_word_index) advances by one, and by a strip's stride less
-    // its rows where the next row starts a strip
-    int lrow = r0 % rps;
-    const uint32_t* lp =
-        have ? bp + bp_word_index(r0, jb, nchunk, rps, wpb) : bp;
-    const size_t wrap = (size_t)nchunk * wpb - rps;
-    auto load = [&](int i) -> uint32_t {
-        uint32_t w = 0u;
-        if (have && i < r1) w = __ldg(lp);
-        ++lp;
-        if (++lrow == rps) {
-            lrow = 0;
-            lp += wrap;
+    const int jb = s0 + 32 * lane;  // first column of this lane
+    // rows r0-2 and r0-1 name themselves: the entries of the cells below them
+    RowEntries e1, e2;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const unsigned v = 2u * (unsigned)(32 * lane + 16 * h + u);
+            const unsigned two = v | ((v + 16u) << 16);
+            e1.w[h][u] = b > 0 ? two + 0x00010001u : kNoPath2;
+            e2.w[h][u] = b > 0 ? two : kNoPath2;
         }
-        return w;
+    // groups of four rows of a strip, 16 bytes a word (a strip's block starts on
+    // 16 bytes: wpb is a multiple of 4), loaded two groups ahead
+    const int ca = min(jb >> 4, nchunk - 1), cb = min((jb >> 4) + 1, nchunk - 1);
+    struct Group {
+        uint4 a, b;
+        int i, k0, k1;  // row of its first word, words k0 .. k1-1 are rows of the band
     };
-
-    int e1[kColsPerWord], e2[kColsPerWord];  // entries of rows i-1 and i-2
+    int strip = r0 / rps, lr = r0 - strip * rps, next = r0;  // of the next group to load
+    auto load = [&](Group& g) {
+        if (next >= r1) {
+            g.k0 = g.k1 = 0;
+            return;
+        }
+        const int q = lr >> 2;
+        const uint32_t* src = bp + ((size_t)strip * nchunk) * wpb + 4 * q;
+        g.a = __ldg(reinterpret_cast<const uint4*>(src + (size_t)ca * wpb));
+        g.b = __ldg(reinterpret_cast<const uint4*>(src + (size_t)cb * wpb));
+        g.i = next - (lr & 3);
+        g.k0 = lr & 3;
+        g.k1 = min(4, min(rps - 4 * q, r1 - g.i));
+        next = g.i + g.k1;
+        lr = 4 * q + g.k1;
+        if (lr >= rps) {
+            lr = 0;
+            ++strip;
+        }
+    };
+    unsigned l2a = __shfl_up_sync(0xffffffffu, e2.w[1][7], 1);
+    if (lane == 0) l2a = kNoPath2;
+    auto row = [&](int i, unsigned wa, unsigned wb) {
+        unsigned l1a = __shfl_up_sync(0xffffffffu, e1.w[1][7], 1);
+        unsigned l1b = __shfl_up_sync(0xffffffffu, e1.w[1][6], 1);
+        if (lane == 0) l1a = l1b = kNoPath2;
+        RowEntries en;
+        bandmap_pairs(wa, e1.w[0], e2.w[0], left_pair(l1a, e1.w[0][7]), left_pair(l1b, e1.w[0][6]),
+                      left_pair(l2a, e2.w[0][7]), en.w[0]);
+        bandmap_pairs(wb, e1.w[1], e2.w[1], left_pair(e1.w[0][7], e1.w[1][7]),
+                      left_pair(e1.w[0][6], e1.w[1][6]), left_pair(e2.w[0][7], e2.w[1][7]),
+                      en.w[1]);
+        if (kBanded) {
+            // cells outside the row's strip range (whole sub-chunks) were never computed
+            const int2 rg = __ldg(a.ranges + i / rps);
+            const int n0 = jb >> 3;  // the lane's sub-chunks n0 .. n0 + 3
 #pragma unroll
-    for (int q = 0; q < kColsPerWord; ++q) e1[q] = e2[q] = kNoPath;
-
-    // the band's first two rows
-    const uint32_t top0 = load(r0), top1 = load(r0 + 1);
-    uint32_t wq[kRowsAhead];
+            for (int h = 0; h < 2; ++h) {
+                const int n = n0 + 2 * h;
+                const unsigned keep = (n >= rg.x && n < rg.y ? 0x0000FFFFu : 0u) |
+                                      (n + 1 >= rg.x && n + 1 < rg.y ? 0xFFFF0000u : 0u);
 #pragma unroll
-    for (int u = 0; u < kRowsAhead; ++u) wq[u] = load(r0 + 2 + u);
-    bandmap_row<NT, true, kBanded>(r0, r0, r1, La, Lb, jb, c0, width, b, top0, t, s_x, e1, e2,
-                               exits, end_entry, a.ranges, rps);
-    if (r0 + 1 < r1)
-        bandmap_row<NT, true, kBanded>(r0 + 1, r0, r1, La, Lb, jb, c0, width, b, top1, t, s_x, e1,
-                                   e2, exits, end_entry, a.ranges, rps);
-    // the rest, kRowsAhead at a time, loading the next group meanwhile; whole
-    // groups run without a per-row guard (so the two row buffers rotate by
-    // renaming, not by moves: -15%), then the last rows of the band
-    int i = r0 + 2;
-    for (; i + kRowsAhead <= r1; i += kRowsAhead) {
-        uint32_t wn[kRowsAhead];
+                for (int u = 0; u < 8; ++u) en.w[h][u] = bit_select(keep, en.w[h][u], kNoPath2);
+            }
+        }
+        if (i == 0 && jb == 0) en.w[0][0] = (en.w[0][0] & 0xFFFF0000u) | kOrigin16;
+        l2a = l1a;
+        e2 = e1;
+        e1 = en;
+    };
+    auto rows = [&](const Group& g) {
+        const unsigned ga[4] = {g.a.x, g.a.y, g.a.z, g.a.w}, gb[4] = {g.b.x, g.b.y, g.b.z, g.b.w};
+        if (g.k0 == 0 && g.k1 == 4) {
 #pragma unroll
-        for (int u = 0; u < kRowsAhead; ++u) wn[u] = load(i + kRowsAhead + u);
-#pragma unroll
-        for (int u = 0; u < kRowsAhead; ++u)
-            bandmap_row<NT, false, kBanded>(i + u, r0, r1, La, Lb, jb, c0, width, b, wq[u], t,
-                                        s_x, e1, e2, exits, end_entry, a.ranges, rps);
-#pragma unroll
-        for (int u = 0; u < kRowsAhead; ++u) wq[u] = wn[u];
-    }
+            for (int k = 0; k < 4; ++k) row(g.i + k, ga[k], gb[k]);
+        } else {
 #pragma unroll 1
-    for (int u = 0; i + u < r1; ++u) {
-        uint32_t w = 0;
+            for (int k = g.k0; k < g.k1; ++k)
+                row(g.i + k, k == 0 ? ga[0] : (k == 1 ? ga[1] : (k == 2 ? ga[2] : ga[3])),
+                    k == 0 ? gb[0] : (k == 1 ? gb[1] : (k == 2 ? gb[2] : gb[3])));
+        }
+    };
+    Group g0, g1;
+    load(g0);
+    load(g1);
+    while (g0.k1 > 0) {
+        const Group g = g0;
+        g0 = g1;
+        load(g1);
+        rows(g);
+    }
+    auto entry = [&](unsigned v) -> int {  // a 16-bit entry in the column numbers of the matrix
+        return v == (kNoPath2 & 0xFFFFu) ? kNoPath : (v == kOrigin16 ? kOrigin : 2 * s0 + (int)v);
+    };
+    auto half = [&](unsigned pair, int hi) -> unsigned { return hi ? pair >> 16 : pair & 0xFFFFu; };
+    if (r1 < La) {
+        // the band's last two rows are kept for the band below
+        int2* __restrict__ exits = sc.exits + (size_t)b * Lb;
 #pragma unroll
-        for (int v = 0; v < kRowsAhead; ++v)
-            if (v == u) w = wq[v];
-        bandmap_row<NT, false, kBanded>(i + u, r0, r1, La, Lb, jb, c0, width, b, w, t, s_x, e1, e2,
-                                    exits, end_entry, a.ranges, rps);
+        for (int q = 0; q < 32; ++q) {
+            const int h = q >> 4, u = q & 7, hi = (q >> 3) & 1;
+            const int j = jb + q;
+            if (j >= c0 && j < c0 + kSegWidth && j < Lb)
+                exits[j] = make_int2(entry(half(e2.w[h][u], hi)), entry(half(e1.w[h][u], hi)));
+        }
+    } else {
+        // the end cell's entry
+        const int q = (Lb - 1) - jb;
+        if (q >= 0 && q < 32 && Lb - 1 >= c0 && Lb - 1 < c0 + kSegWidth) {
+#pragma unroll
+            for (int v = 0; v < 32; ++v)
+                if (v == q) *sc.end_entry = entry(half(e1.w[v >> 4][v & 7], (v >> 3) & 1));
+        }
     }
 }
 

@@ -1,69 +1,65 @@
 // Walking a path back through a backtrace matrix with one warp (the band
 // walks of the parallel backtrace, bandmap.cu; the fragment walks of WSDTW,
-// wsdtw.cu).  Each step reads one 2-bit field (see step_of_field) whose
-// address depends on the step before, so the warp keeps the backpointer
-// block (one strip of rps rows x 16 columns, wpb words; see bp_word_index)
-// of the current cell in registers, lane l holding words l, l+32, l+64,
-// l+96, and reads a field with one shuffle.  A step moves at most two rows
-// and two columns up and left and a strip has more than two rows, so the
-// next block is the current one or its neighbour above, to the left or
-// above-left: the three are loaded when the path enters a block, while it
-// crosses it.  The row within the strip is tracked, not divided out.
+// wsdtw.cu).  Each step reads one 2-bit field (see step_of_field) whose address
+// depends on the step before, so the walk is a chain of loads: from shared
+// memory, where the warp first puts every word the next kWalkRows rows can
+// need.  From cell (i, j) a path moves at most two columns left per row, so the
+// rows i - kWalkRows + 1 .. i of the 17 chunks of 16 columns that end with j's
+// hold them (8.7 KB, 68 independent loads a lane).  (With the words in registers
+// and neighbouring blocks prefetched from global memory a step took 240 ns and
+// the walk of 128 rows 24 us.)
 #pragma once
 #include "pardtw_common.cuh"
 
 namespace pardtw {
 namespace {
 
-struct BlockWalker {
+constexpr int kWalkRows = 128;
+constexpr int kWalkChunks = (2 * (kWalkRows - 1) + 15) / 16 + 1;
+constexpr int kWalkWords = kWalkChunks * kWalkRows;
+
+struct WindowWalker {
     const uint32_t* __restrict__ bp;
     int nchunk, rps, wpb, lane;
-    int st, rr, ch;  // strip of the current row, row within it, chunk of the current column
-    uint32_t cur[4], up[4], lf[4], ul[4];
+    uint32_t* sm;   // kWalkWords words of this warp
+    int row0, ch1;  // first row and last chunk of the window
 
-    __device__ __forceinline__ void fetch(int bs, int bc, uint32_t (&w)[4]) const {
-        const bool ok = bs >= 0 && bc >= 0;
-        const uint32_t* src = bp + (ok ? ((size_t)bs * nchunk + bc) * wpb : 0);
+    // The window of cell (i, j): all lanes, warp-uniform arguments.
+    __device__ __forceinline__ void load(int i, int j) {
+        row0 = max(i - kWalkRows + 1, 0);
+        ch1 = j >> 4;
+        __syncwarp();  // the previous window has been read
+        const uint32_t* src[kWalkRows / 32];
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            w[k] = (ok && lane + 32 * k < wpb) ? __ldg(src + lane + 32 * k) : 0u;
-    }
-    __device__ __forceinline__ void fetch_next() {
-        fetch(st - 1, ch, up);
-        fetch(st, ch - 1, lf);
-        fetch(st - 1, ch - 1, ul);
-    }
-    // start at cell (i, j) (all lanes, warp-uniform arguments)
-    __device__ __forceinline__ void start(int i, int j) {
-        st = i / rps;
-        rr = i - st * rps;
-        ch = j >> 4;
-        fetch(st, ch, cur);
-        fetch_next();
-    }
-    // the 2-bit field of the current cell, whose column is j
-    __device__ __forceinline__ uint32_t field(int j) const {
-        const int slot = rr >> 5;
-        const uint32_t mine =
-            slot == 0 ? cur[0] : (slot == 1 ? cur[1] : (slot == 2 ? cur[2] : cur[3]));
-        return (__shfl_sync(0xffffffffu, mine, rr & 31) >> (2 * (j & 15))) & 3u;
-    }
-    // the step to the cell di rows up whose column is j_new; the new
-    // neighbours are loaded only if `more` (the walk goes on from there)
-    __device__ __forceinline__ void step(int di, int j_new, bool more) {
-        rr -= di;
-        const bool su = rr < 0;               // into the strip above
-        const bool sl = (j_new >> 4) != ch;   // into the chunk to the left
-        if (su || sl) {                       // warp-uniform
-#pragma unroll
-            for (int k = 0; k < 4; ++k) cur[k] = su ? (sl ? ul[k] : up[k]) : lf[k];
-            if (su) {
-                rr += rps;
-                --st;
-            }
-            if (sl) --ch;
-            if (more) fetch_next();
+        for (int m = 0; m < kWalkRows / 32; ++m) {
+            const int r = min(row0 + lane + 32 * m, i);
+            const int st = r / rps;
+            src[m] = bp + ((size_t)st * nchunk) * wpb + (r - st * rps);
         }
+#pragma unroll
+        for (int k0 = 0; k0 < kWalkChunks; k0 += 6) {
+            uint32_t v[6][kWalkRows / 32];
+#pragma unroll
+            for (int k = 0; k < 6; ++k)
+#pragma unroll
+                for (int m = 0; m < kWalkRows / 32; ++m)
+                    if (k0 + k < kWalkChunks)
+                        v[k][m] = __ldg(src[m] + (size_t)max(ch1 - k0 - k, 0) * wpb);
+#pragma unroll
+            for (int k = 0; k < 6; ++k)
+#pragma unroll
+                for (int m = 0; m < kWalkRows / 32; ++m)
+                    if (k0 + k < kWalkChunks) sm[(k0 + k) * kWalkRows + lane + 32 * m] = v[k][m];
+        }
+        __syncwarp();
+    }
+    // Whether cell (i, j) lies in the window (j >= 0).
+    __device__ __forceinline__ bool inside(int i, int j) const {
+        return i >= row0 && ch1 - (j >> 4) < kWalkChunks;
+    }
+    // The 2-bit field of cell (i, j) of the window.
+    __device__ __forceinline__ uint32_t field(int i, int j) const {
+        return (sm[(ch1 - (j >> 4)) * kWalkRows + (i - row0)] >> (2 * (j & 15))) & 3u;
     }
 };
 

@@ -24,7 +24,7 @@ namespace pardtw {
 
 namespace {
 
-constexpr int kSegThreads = 1024;
+constexpr int kCompactThreads = 256;
 
 // (value, index) minimum where the earlier index wins ties.
 struct MinArg {
@@ -161,13 +161,15 @@ __global__ void __launch_bounds__(kTile)
 }
 
 // One warp per fragment: the subsequence path from (len-1, e_k) to row 0
-// (BlockWalker), stored backwards (ascending once read from slot
+// (WindowWalker), stored backwards (ascending once read from slot
 // row0 + len - n) as global (row of A, frame of B) pairs.  A step that
 // leaves the fragment's cells raises DTW_ERR_CUDA (it cannot happen for a
 // finite end cell).
-__global__ void k_bt_subseq(const WsFrag* __restrict__ fr, int N, const int* __restrict__ ends,
-                            int32_t* __restrict__ scratch, int* __restrict__ count,
-                            DevCtl* ctl) {
+constexpr int kWalkWarps = 2;  // fragments per CTA
+__global__ void __launch_bounds__(32 * kWalkWarps)
+    k_bt_subseq(const WsFrag* __restrict__ fr, int N, const int* __restrict__ ends,
+                int32_t* __restrict__ scratch, int* __restrict__ count, DevCtl* ctl) {
+    __shared__ uint32_t s_win[kWalkWarps][kWalkWords];
     const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (k >= N) return;
@@ -178,19 +180,17 @@ __global__ void k_bt_subseq(const WsFrag* __restrict__ fr, int N, const int* __r
     const WsFrag f = fr[k];
     int i = f.len - 1, j = ends[k];
     int n = 0;
-    int32_t* out = scratch + 2 * (size_t)(f.row0 + f.len - 1);
-    BlockWalker w{f.bp, f.nchunk, f.rps, f.wpb, lane};
-    w.start(i, max(j, 0));
+    // cell n goes to pair row0 + len - 1 - n, 32 cells at a time
+    int2* out = reinterpret_cast<int2*>(scratch) + (f.row0 + f.len - 1);
+    int2 mine = make_int2(0, 0);
+    WindowWalker w{f.bp, f.nchunk, f.rps, f.wpb, lane, s_win[threadIdx.x >> 5], 0, 0};
+    w.load(i, max(j, 0));
     for (;;) {
-        if (lane == 0) {
-            out[-2 * n] = f.row0 + i;
-            out[-2 * n + 1] = j;
-        }
-        ++n;
+        if ((n & 31) == lane) mine = make_int2(f.row0 + i, j);
+        if ((++n & 31) == 0) out[-(n - 32 + lane)] = mine;
         if (i == 0) break;
-        const uint32_t fl = w.field(j);
-        const int di = field_di(fl);
-        i -= di;
+        const uint32_t fl = w.field(i, j);
+        i -= field_di(fl);
         j -= field_dj(fl);
         if (i < 0 || j < 0 || n >= f.len) {
             if (lane == 0) {
@@ -199,31 +199,40 @@ __global__ void k_bt_subseq(const WsFrag* __restrict__ fr, int N, const int* __r
             }
             return;
         }
-        w.step(di, j, i > 0);
+        if (!w.inside(i, j)) w.load(i, j);
     }
+    if (lane < (n & 31)) out[-((n & ~31) + lane)] = mine;
     if (lane == 0) count[k] = n;
 }
 
-// The fragment paths one after another: fragment k's n_k pairs sit at the
-// end of its slots [row0, row0 + len); *path_len = sum n_k (or -status).
-__global__ void __launch_bounds__(kSegThreads)
+// The fragment paths one after another, one CTA per fragment: fragment k's n_k
+// pairs sit at the end of its slots [row0, row0 + len), and go behind those of the
+// fragments before it; *path_len = sum n_k (or -status).
+__global__ void __launch_bounds__(kCompactThreads)
     k_compact(const WsFrag* __restrict__ fr, int N, const int* __restrict__ count,
               const int32_t* __restrict__ scratch, int32_t* __restrict__ path,
               int* __restrict__ path_len, const DevCtl* ctl) {
     const int st = ctl->status;
+    const int k = blockIdx.x;
     if (st != 0) {
-        if (threadIdx.x == 0) *path_len = -st;
+        if (k == 0 && threadIdx.x == 0) *path_len = -st;
         return;
     }
-    int base = 0;
-    for (int k = 0; k < N; ++k) {
-        const int n = count[k];
-        const WsFrag f = fr[k];
-        const int32_t* src = scratch + 2 * (size_t)(f.row0 + f.len - n);
-        for (int q = threadIdx.x; q < 2 * n; q += blockDim.x) path[2 * (size_t)base + q] = src[q];
-        base += n;
-    }
-    if (threadIdx.x == 0) *path_len = base;
+    __shared__ int s_before[kCompactThreads / 32];
+    int before = 0;
+    for (int q = threadIdx.x; q < k; q += blockDim.x) before += count[q];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) before += __shfl_xor_sync(0xffffffffu, before, off);
+    if ((threadIdx.x & 31) == 0) s_before[threadIdx.x >> 5] = before;
+    __syncthreads();
+    before = 0;
+#pragma unroll
+    for (int q = 0; q < kCompactThreads / 32; ++q) before += s_before[q];
+    const int n = count[k];
+    const WsFrag f = fr[k];
+    const int32_t* src = scratch + 2 * (size_t)(f.row0 + f.len - n);
+    for (int q = threadIdx.x; q < 2 * n; q += blockDim.x) path[2 * (size_t)before + q] = src[q];
+    if (k == N - 1 && threadIdx.x == 0) *path_len = before + n;
 }
 
 }  // namespace
@@ -404,8 +413,9 @@ size_t seg_dp_scratch_bytes(int Lb) { return sizeof(MinArg) * (size_t)((Lb + kTi
 cudaError_t launch_bt_subseq(const WsFrag* fr, int N, const int* ends, int32_t* scratch,
                              int* count, int32_t* path, int* path_len, DevCtl* ctl,
                              cudaStream_t s) {
-    k_bt_subseq<<<(N + 3) / 4, 128, 0, s>>>(fr, N, ends, scratch, count, ctl);
-    k_compact<<<1, kSegThreads, 0, s>>>(fr, N, count, scratch, path, path_len, ctl);
+    k_bt_subseq<<<(N + kWalkWarps - 1) / kWalkWarps, 32 * kWalkWarps, 0, s>>>(fr, N, ends, scratch,
+                                                                               count, ctl);
+    k_compact<<<N, kCompactThreads, 0, s>>>(fr, N, count, scratch, path, path_len, ctl);
     return cudaGetLastError();
 }
 
