@@ -82,16 +82,22 @@ constexpr int kBfBlkBytes = kColsPerWord * kBfStride * 2;
 // FP32 cost for D > 32 ("wide"): -a^ of the lane's R rows no longer fits in
 // registers, so the strip's rows of A^ sit in shared memory (rows padded by 4
 // floats: the 16-byte loads of rows 3l + k of a warp fall in distinct bank
-// groups), and two cost warps share a strip, taking alternate sub-chunks
-// (all 8 columns each).  Two cost warps also where one would be slower than
-// the DP warp (D > 8 and two strips per CTA).
+// groups), and several cost warps share a strip, taking sub-chunks in turn
+// (all 8 columns each).  So they do where one would be slower than the DP warp.
+// With two strips a CTA: two (two strips beside each other at D = 12: 83 cycles a
+// column, 126 with a third one, which shares the DP warp's SM sub-partition; 139
+// against 162 with two CTAs an SM; D = 16: 88 and 89), at D = 32 three (122, 151
+// with two).
 template <int DP, int NS, bool kBF>
 struct CostCfg {
     static constexpr bool kWide = DP > 32 && !kBF;
-        static constexpr int kNC = kWide ? (NS == 1 ? 4 : 2)
-                               : NS == 1                   ? 3
-                               : (!kBF && DP > 8 && NS == 2) ? 2
-                                                           : 1;  // cost warps a strip
+    // cost warps a strip
+    static constexpr int kNC = kWide           ? (NS == 1 ? 4 : 2)
+                               : NS == 1       ? 3
+                               : kBF || NS > 2 ? 1
+                               : DP > 16       ? 3
+                               : DP > 8        ? 2
+                                               : 1;
     static constexpr int kStride = DP + 4;   // floats per row of the A tile
     // each cost warp's ring of B: frames a block, blocks
     static constexpr int kBBlk = kWide ? kColsPerWord : (DP <= 16 ? 64 : 32);
@@ -1019,7 +1025,7 @@ __device__ __forceinline__ void run_link_reader(const DpArgs& p, int lane, unsig
 // a writer warp (their places: see `role`).  Persistent: a CTA takes strip
 // groups from the ticket counter until none are left, so a group only ever
 // waits on groups that started earlier.
-// kMany: the groups come from a work queue over many pairs (`many`, `item0`,
+// kMany: the groups come from a work queue over many pairs (`many`, `items`,
 // `ticket`; see launch_dp_split_many) instead of the pair `one`.
 // kCl (one pair): the kernel runs in clusters of cn CTAs that
 // take tickets together: ticket T gives CTA rank r the strip group
@@ -1032,8 +1038,8 @@ template <int DP, int R, int NS, bool kMany, bool kBF, bool kSubseq = false, boo
           bool kCl = false>
 __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
                                   (kCl ? 1 : split_ctas_per_sm(R, NS, DP, kBF)))
-    k_dp_split(const DpArgs one, const DpArgs* __restrict__ many, const int* __restrict__ item0,
-               int nmany, int* ticket) {
+    k_dp_split(const DpArgs one, const DpArgs* __restrict__ many, const int2* __restrict__ items,
+               int nitems, int* ticket) {
     static_assert(!kCl || (!kMany && !kSubseq), "clusters sweep one plain pair");
     constexpr int kThreads = split_threads<DP, NS, kBF>();
     using Cfg = CostCfg<DP, NS, kBF>;
@@ -1134,21 +1140,12 @@ __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
         }
         if (!kCl && threadIdx.x == 0) {
             if (kMany) {
-                // item t -> (pair, group): the last pair whose first item is <= t
                 const int t = atomicAdd(ticket, 1);
                 int pi = -1, gi = 0;
-                if (t < item0[nmany]) {
-                    int lo = 0, hi = nmany - 1;
-                    while (lo < hi) {
-                        const int mid = (lo + hi + 1) >> 1;
-                        if (item0[mid] <= t)
-                            lo = mid;
-                        else
-                            hi = mid - 1;
-                    }
-                    pi = lo;
-                    gi = t - item0[lo];
-                    if (read_status(many[pi].ctl) != 0) gi = -1;  // the pair has failed
+                if (t < nitems) {
+                    pi = items[t].x;
+                    // nothing of a failed pair runs
+                    gi = read_status(many[pi].ctl) != 0 ? -1 : items[t].y;
                 }
                 s_pair = pi;
                 s_group = gi;
@@ -1160,7 +1157,7 @@ __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
         }
         __syncthreads();
         if (kMany && s_pair < 0) return;
-        if (kMany && s_group < 0) continue;  // nothing of a failed pair runs
+        if (kMany && s_group < 0) continue;
         const DpArgs p = kMany ? many[s_pair] : one;
         const int g = s_group;
         if (kCl && g >= p.ngroups) continue;  // this CTA's group of the ticket does not exist
@@ -1268,8 +1265,8 @@ __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
 
 template <int DP, int R, int NS, bool kMany, bool kBF = false, bool kSubseq = false,
           bool kT = false>
-cudaError_t launch_t(const DpArgs& a, const DpArgs* many, const int* item0, int n, int items,
-                     int* ticket, int num_sms, cudaStream_t s) {
+cudaError_t launch_t(const DpArgs& a, const DpArgs* many, const int2* queue, int items, int* ticket,
+                     int num_sms, cudaStream_t s) {
     constexpr int kThreads = split_threads<DP, NS, kBF>();
     const int smem = NS * SplitSmem<DP, R, NS, kBF, false>::kStripBytes;
     auto* kern = k_dp_split<DP, R, NS, kMany, kBF, kSubseq, kT>;
@@ -1279,7 +1276,7 @@ cudaError_t launch_t(const DpArgs& a, const DpArgs* many, const int* item0, int 
     if (e != cudaSuccess) return e;
     int grid = blocks_per_sm * num_sms;
     if (grid > items) grid = items;
-    kern<<<grid, kThreads, smem, s>>>(a, many, item0, n, ticket);
+    kern<<<grid, kThreads, smem, s>>>(a, many, queue, items, ticket);
     return cudaGetLastError();
 }
 

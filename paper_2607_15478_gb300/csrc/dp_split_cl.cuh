@@ -141,7 +141,7 @@ cudaError_t launch_cl(const DpArgs& pair, cudaStream_t s, bool* used) {
         cl_config(dim3((unsigned)(nclusters * cn)), K::kThreads, K::smem(), s, at, cn);
     const cudaError_t e = cudaLaunchKernelEx(&cfg, K::kern(), a,
                                              static_cast<const DpArgs*>(nullptr),
-                                             static_cast<const int*>(nullptr), 1,
+                                             static_cast<const int2*>(nullptr), 0,
                                              static_cast<int*>(nullptr));
     if (e == cudaSuccess) *used = true;
     return e;

@@ -15,15 +15,11 @@ bool split_wide_supported(int dp) { return dp == 64 || dp == 128; }
 cudaError_t launch_dp_split_wide(const DpArgs& a, int dp, int num_sms, cudaStream_t s,
                                  bool transposed) {
     if (dp == 64)
-        return transposed ? launch_t<64, 3, 2, false, false, false, true>(
-                                a, nullptr, nullptr, 1, a.ngroups, nullptr, num_sms, s)
-                          : launch_t<64, 3, 2, false>(a, nullptr, nullptr, 1, a.ngroups, nullptr,
-                                                      num_sms, s);
+        return transposed ? launch_t<64, 3, 2, false, false, false, true>(a, nullptr, nullptr, a.ngroups, nullptr, num_sms, s)
+                          : launch_t<64, 3, 2, false>(a, nullptr, nullptr, a.ngroups, nullptr, num_sms, s);
     if (dp == 128)
-        return transposed ? launch_t<128, 3, 2, false, false, false, true>(
-                                a, nullptr, nullptr, 1, a.ngroups, nullptr, num_sms, s)
-                          : launch_t<128, 3, 2, false>(a, nullptr, nullptr, 1, a.ngroups, nullptr,
-                                                       num_sms, s);
+        return transposed ? launch_t<128, 3, 2, false, false, false, true>(a, nullptr, nullptr, a.ngroups, nullptr, num_sms, s)
+                          : launch_t<128, 3, 2, false>(a, nullptr, nullptr, a.ngroups, nullptr, num_sms, s);
     return cudaErrorInvalidValue;
 }
 

@@ -199,12 +199,12 @@ bool multirow_supported(int dp, int R);
 cudaError_t launch_dp_split(const DpArgs& a, int dp, int R, int ns, int num_sms, cudaStream_t s,
                             bool transposed = false);
 bool split4_supported(int dp, int R);
-cudaError_t launch_dp_split4(const DpArgs& a, const DpArgs* many, const int* item0, int n,
-                             int items, int* ticket, int dp, int R, int num_sms, cudaStream_t s,
+cudaError_t launch_dp_split4(const DpArgs& a, const DpArgs* many, const int2* queue, int items,
+                             int* ticket, int dp, int R, int num_sms, cudaStream_t s,
                              bool transposed);
 // The subsequence DP of WSDTW over a batch (R = 3, dp <= 32): weights 1, 1, 2,
 // free start in row 0, row La-1 of every pair into its DpArgs::lastrow.
-cudaError_t launch_dp_subseq_many(const DpArgs* many, const int* item0, int n, int total_items,
+cudaError_t launch_dp_subseq_many(const DpArgs* many, const int2* queue, int items,
                                   int* ticket, int dp, int num_sms, cudaStream_t s);
 // ns strips per CTA: 2 (every dp <= 32) or 4 (dp <= 16, R = 2, 3).
 bool split_supported(int dp, int R, int ns = 2);
@@ -232,13 +232,13 @@ bool split_bf16_supported(int dp);
 // kBfStride elements (features beyond D and frames beyond Lb are zero).
 cudaError_t launch_pack_b_bf16(const float* B, int Lb, int Lb_pad, int D, void* Bbf,
                                cudaStream_t s);
-// Many pairs in one persistent launch: `many` (device) holds n DpArgs, item0
-// (device, n + 1 ints) the prefix sums of their strip-group counts; CTAs take
-// (pair, group) items from *ticket in that order, so a group only waits on
-// groups of its own pair that were taken earlier.  Each pair's failures stay
-// in its own control block.
-cudaError_t launch_dp_split_many(const DpArgs* many, const int* item0, int n, int total_items,
-                                 int* ticket, int dp, int R, int ns, int num_sms, cudaStream_t s);
+// Many pairs in one persistent launch: `many` (device) holds the pairs' DpArgs,
+// queue (device) the `items` (pair, strip group) items in the order CTAs take
+// them from *ticket; a pair's groups stand in ascending order, so a group only
+// waits on groups of its own pair that were taken earlier.  Each pair's
+// failures stay in its own control block.
+cudaError_t launch_dp_split_many(const DpArgs* many, const int2* queue, int items, int* ticket,
+                                 int dp, int R, int ns, int num_sms, cudaStream_t s);
 
 // Which DP kernel runs a problem: kind 0 = one row per lane (dp_kernel.cu),
 // 1 = fused multi-row (dp_multirow.cu), 2 = cost/DP warp pairs (dp_split.cu);
