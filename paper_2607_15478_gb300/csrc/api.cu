@@ -289,10 +289,9 @@ int align_device(dtw_handle* h, const float* A, int La, const float* B, int Lb, 
         dB = st;
     }
     if (h->timing) CU(cudaEventRecord(h->ev[0], s));
-    CU(launch_normalise(dA, La, L.La_pad, dB, Lb, L.nchunk * kColsPerWord, D, L.dp, Ahat, Bhat,
-                        ctl, s));
     void* Bbf = L.plan.bf16 ? ws + L.off_bbf : nullptr;
-    if (Bbf) CU(launch_pack_b_bf16(dB, Lb, L.nchunk * kColsPerWord, D, Bbf, s));
+    CU(launch_normalise({dA, La, L.La_pad, dB, Lb, L.nchunk * kColsPerWord, Ahat, Bhat, ctl}, D,
+                        L.dp, Bbf, s));
     if (h->timing) CU(cudaEventRecord(h->ev[1], s));
 
     DpArgs a;
@@ -334,6 +333,7 @@ int align_device(dtw_handle* h, const float* A, int La, const float* B, int Lb, 
     bt.scratch = ws + L.off_bt;
     bt.ranges = ranges;
     bt.transposed = tr ? 1 : 0;
+    bt.band = band_rows(La, (double)La * Lb);
     CU(launch_plan(L.plan, a, L.dp, h->num_sms, s, tr));
     if (h->timing) CU(cudaEventRecord(h->ev[2], s));
     CU(launch_backtrace_bands(bt, s));
@@ -367,7 +367,8 @@ struct SubseqBatch {
 // control block per pair, then every pair's buffers; the border rows of all
 // pairs in another.
 struct BatchSetup {
-    int m = 0, D = 0, dp = 0, R = 3, NS = 2, maxLa = 0, maxLb = 0, max_frames = 0;
+    int m = 0, D = 0, dp = 0, R = 3, NS = 2, nbands = 0, maxLb = 0, norm_blocks = 0;
+    double cells = 0.0;
     std::vector<int> idx;  // pair indices, longest sweeps first
     std::vector<Layout> Ls;
     std::vector<size_t> off, boff;
@@ -451,9 +452,14 @@ BatchSetup batch_setup(std::vector<int> idx, const int* La, const int* Lb, int D
         o0 = align256(o0 + (L.off_stage_a - L.off_ahat));  // Ahat, Bhat, bp, band maps
         b.boff[q] = border_total;
         border_total += L.border_bytes;
-        b.maxLa = std::max(b.maxLa, La[k]);
         b.maxLb = std::max(b.maxLb, Lb[k]);
-        b.max_frames = std::max(b.max_frames, L.La_pad + L.nchunk * kColsPerWord);
+        b.norm_blocks =
+            std::max(b.norm_blocks, normalise_blocks(L.La_pad, L.nchunk * kColsPerWord));
+    }
+    for (int q = 0; q < m; ++q) b.cells += (double)La[idx[q]] * Lb[idx[q]];
+    for (int q = 0; q < m; ++q) {
+        const int band = band_rows(La[idx[q]], b.cells);
+        b.nbands = std::max(b.nbands, (La[idx[q]] + band - 1) / band);
     }
     b.ws_bytes = o0;
     b.border_bytes = border_total;
@@ -533,6 +539,8 @@ BatchDesc batch_descriptors(const BatchSetup& b, char* ws, unsigned long long* b
         bt.total = (cost && !sub) ? cost + k : nullptr;
         bt.scratch = base + L.off_bt;
         bt.ranges = nullptr;
+        bt.transposed = 0;
+        bt.band = band_rows(La[k], b.cells);
         if (sub) (*sub->bts_out)[k] = bt;
     }
     return d;
@@ -558,7 +566,7 @@ int batch_launch(const BatchSetup& b, char* ws, bool subseq, int num_sms, cudaSt
     const int items = (int)b.queue.size();
     int* ticket = reinterpret_cast<int*>(ws + b.off_item + sizeof(int2) * (size_t)items);
     if (ev) CU(cudaEventRecord(ev[0], s));
-    CU(launch_normalise_many(reinterpret_cast<const NormArgs*>(ws + b.off_norm), m, b.max_frames,
+    CU(launch_normalise_many(reinterpret_cast<const NormArgs*>(ws + b.off_norm), m, b.norm_blocks,
                              b.D, b.dp, ticket, s));
     if (ev) CU(cudaEventRecord(ev[1], s));
     const DpArgs* dps = reinterpret_cast<const DpArgs*>(ws + b.off_dp);
@@ -569,7 +577,7 @@ int batch_launch(const BatchSetup& b, char* ws, bool subseq, int num_sms, cudaSt
         CU(launch_dp_split_many(dps, queue, items, ticket, b.dp, b.R, b.NS, num_sms, s));
     if (ev) CU(cudaEventRecord(ev[2], s));
     if (!subseq)
-        CU(launch_backtrace_bands_many(reinterpret_cast<const BtArgs*>(ws + b.off_bt), m, b.maxLa,
+        CU(launch_backtrace_bands_many(reinterpret_cast<const BtArgs*>(ws + b.off_bt), m, b.nbands,
                                        b.maxLb, s));
     if (ev) CU(cudaEventRecord(ev[3], s));
     return DTW_OK;
@@ -735,8 +743,8 @@ int dtw_cost(dtw_handle* h, const float* A, int La, const float* B, int Lb, int 
     DevCtl* ctl = reinterpret_cast<DevCtl*>(ws + L.off_ctl);
     float* Ahat = reinterpret_cast<float*>(ws + L.off_ahat);
     float* Bhat = reinterpret_cast<float*>(ws + L.off_bhat);
-    CU(launch_normalise(dA, La, L.La_pad, dB, Lb, L.nchunk * kColsPerWord, D, dp, Ahat, Bhat,
-                        ctl, s));
+    CU(launch_normalise({dA, La, L.La_pad, dB, Lb, L.nchunk * kColsPerWord, Ahat, Bhat, ctl}, D,
+                        dp, nullptr, s));
     float* dC = c_dev ? C : reinterpret_cast<float*>(ws + L.total);
     CU(launch_cost(Ahat, La, Bhat, Lb, dp, dC, s));
     if (!c_dev) {

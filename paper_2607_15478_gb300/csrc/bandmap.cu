@@ -4,7 +4,7 @@
 // A serial walk costs one dependent memory access per path cell (~2e4 for
 // a 20000 x 25000 pair).  This file splits it:
 //
-//   1. k_bandmap: rows are cut into bands of 128 rows.  For every cell of
+//   1. k_bandmap: rows are cut into bands of 32 to 128 rows (band_rows).  For every cell of
 //      a band, "entry" = the cell of the band above where the optimal path
 //      to this cell last sat before entering the band, encoded as
 //      2 * column + (1 if that cell is in the band above's last row, 0 if in
@@ -14,7 +14,7 @@
 //                    = encode(predecessor)      predecessor in the band above
 //      All columns of a row are independent (the inputs are rows i-1, i-2),
 //      so bands and column segments run in parallel.  A segment recomputes
-//      2 * 128 columns to its left (dependencies move at most 2 columns
+//      two columns per row of the band to its left (dependencies move at most 2 columns
 //      left per row, so those halo values are exact when they are used).
 //      Only the entries of each band's last two rows are stored, and the
 //      end cell's entry.
@@ -47,8 +47,8 @@ __global__ void __launch_bounds__(32 * kMapWarps) k_bandmap(const BtArgs one,
                              threadIdx.x & 31);
 }
 // CTAs per band that cover the segments of all of a pair's columns.
-int map_ctas(int Lb) {
-    const int segs = (Lb + kSegWidth - 1) / kSegWidth;
+int map_ctas(int Lb, int band) {
+    const int segs = (Lb + seg_width(band) - 1) / seg_width(band);
     return (segs + kMapWarps - 1) / kMapWarps;
 }
 
@@ -56,8 +56,8 @@ int map_ctas(int Lb) {
 
 // The cell named by entry e of a cell of band x: a cell of band x-1's last
 // two rows.
-__device__ __forceinline__ int2 entry_cell(int e, int x) {
-    return make_int2((e & 1) ? x * kBand - 1 : x * kBand - 2, e >> 1);
+__device__ __forceinline__ int2 entry_cell(int e, int x, int band) {
+    return make_int2((e & 1) ? x * band - 1 : x * band - 2, e >> 1);
 }
 // The entry of cell c of a band's last two rows from its exits word x (.x:
 // second-to-last row, .y: last row); last = the band's last row.
@@ -82,20 +82,20 @@ __global__ void __launch_bounds__(256) k_bt_compose(const BtArgs one,
                                                     const BtArgs* __restrict__ many) {
     const BtArgs& a = kMany ? many[blockIdx.z] : one;
     const int La = a.La, Lb = a.Lb;
-    const BtScratch sc = bt_scratch(a.scratch, La, Lb);
+    const BtScratch sc = bt_scratch(a);
     const int m = blockIdx.y;
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= sc.n2 || j >= Lb) return;
     const int b = sc.nbands - 2 - 2 * m;
-    const int r1 = (b + 1) * kBand;  // b <= nbands-2: a whole band
+    const int r1 = (b + 1) * sc.band;  // b <= nbands-2: a whole band
     if (!map_column(a, r1, j)) return;
     const int2* __restrict__ exits = sc.exits;
     const int2 x = exits[(size_t)b * Lb + j];
     auto hop = [&](int e) -> int {
         if (e < 0) return kNoPath;
-        const int2 c = entry_cell(e, b);
+        const int2 c = entry_cell(e, b, sc.band);
         if (c.y < 0 || c.y >= Lb) return kNoPath;
-        return pick_exit(exits[(size_t)(b - 1) * Lb + c.y], c.x, b * kBand - 1);
+        return pick_exit(exits[(size_t)(b - 1) * Lb + c.y], c.x, b * sc.band - 1);
     };
     sc.exits2[(size_t)m * Lb + j] = make_int2(hop(x.x), hop(x.y));
 }
@@ -109,20 +109,20 @@ __global__ void __launch_bounds__(256) k_bt_compose4(const BtArgs one,
                                                      const BtArgs* __restrict__ many) {
     const BtArgs& a = kMany ? many[blockIdx.z] : one;
     const int La = a.La, Lb = a.Lb;
-    const BtScratch sc = bt_scratch(a.scratch, La, Lb);
+    const BtScratch sc = bt_scratch(a);
     const int m = blockIdx.y;
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= sc.n4 || j >= Lb) return;
     const int b = sc.nbands - 2 - 4 * m;
-    const int r1 = (b + 1) * kBand;
+    const int r1 = (b + 1) * sc.band;
     if (!map_column(a, r1, j)) return;
     const int2* __restrict__ exits2 = sc.exits2;
     const int2 x = exits2[(size_t)(2 * m) * Lb + j];  // into band b-2's last two rows
     auto hop = [&](int e) -> int {
         if (e < 0) return kNoPath;
-        const int2 c = entry_cell(e, b - 1);
+        const int2 c = entry_cell(e, b - 1, sc.band);
         if (c.y < 0 || c.y >= Lb) return kNoPath;
-        return pick_exit(exits2[(size_t)(2 * m + 1) * Lb + c.y], c.x, (b - 1) * kBand - 1);
+        return pick_exit(exits2[(size_t)(2 * m + 1) * Lb + c.y], c.x, (b - 1) * sc.band - 1);
     };
     sc.exits4[(size_t)m * Lb + j] = make_int2(hop(x.x), hop(x.y));
 }
@@ -136,9 +136,10 @@ template <bool kMany>
 __global__ void k_bt_chain(const BtArgs one, const BtArgs* __restrict__ many) {
     if (threadIdx.x != 0) return;
     const BtArgs& a = kMany ? many[blockIdx.x] : one;
-    const int La = a.La, Lb = a.Lb, band = kBand;
+    const int La = a.La, Lb = a.Lb;
     DevCtl* ctl = a.ctl;
-    const BtScratch sc = bt_scratch(a.scratch, La, Lb);
+    const BtScratch sc = bt_scratch(a);
+    const int band = sc.band;
     const int2* __restrict__ exits = sc.exits;
     const int2* __restrict__ exits2 = sc.exits2;
     const int nbands = sc.nbands;
@@ -150,7 +151,7 @@ __global__ void k_bt_chain(const BtArgs one, const BtArgs* __restrict__ many) {
     int2 c;
     auto take = [&](int x) -> bool {
         if (e < 0) return false;  // an entry must name a cell of the band above
-        c = entry_cell(e, x);
+        c = entry_cell(e, x, band);
         return c.x >= (x - 1) * band && c.y >= 0 && c.y < Lb;
     };
     bool ok = true;
@@ -203,12 +204,12 @@ __global__ void k_bt_chain(const BtArgs one, const BtArgs* __restrict__ many) {
 constexpr int kWalkWarps = 4;  // bands per CTA
 template <bool kMany>
 __global__ void __launch_bounds__(32 * kWalkWarps) k_bt_walk(const BtArgs one, const BtArgs* __restrict__ many) {
-    static_assert(kWalkRows >= kBand, "a band's rows fit the window");
+    static_assert(kWalkRows >= kMaxBand, "a band's rows fit the window");
     __shared__ uint32_t s_win[kWalkWarps][kWalkWords];
     const BtArgs& a = kMany ? many[blockIdx.y] : one;
-    const int band = kBand;
     DevCtl* ctl = a.ctl;
-    const BtScratch sc = bt_scratch(a.scratch, a.La, a.Lb);
+    const BtScratch sc = bt_scratch(a);
+    const int band = sc.band;
     const int nbands = sc.nbands;
     const int2* __restrict__ cross = sc.cross;
     int2* __restrict__ seg = sc.seg;
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(32 * kWalkWarps) k_bt_walk(const BtArgs one, c
     if (b < nbands - 1 && b > 0 && ((nbands - 2 - b) & 1)) {
         const int2 c1 = cross[b + 1];
         const int e = pick_exit(exits[(size_t)(b + 1) * Lb + c1.y], c1.x, (b + 2) * band - 1);
-        c = entry_cell(e, b + 1);
+        c = entry_cell(e, b + 1, sc.band);
         if (e < 0 || c.x < r0 || c.y < 0 || c.y >= Lb) bad = 1;
     }
     int2 target = make_int2(-1, -1);
@@ -239,28 +240,21 @@ __global__ void __launch_bounds__(32 * kWalkWarps) k_bt_walk(const BtArgs one, c
         const int e = b == nbands - 1
                           ? *sc.end_entry
                           : pick_exit(exits[(size_t)b * Lb + c.y], c.x, (b + 1) * band - 1);
-        target = e < 0 ? make_int2(-3, -3) : entry_cell(e, b);
+        target = e < 0 ? make_int2(-3, -3) : entry_cell(e, b, sc.band);
     }
     if (bad) c = make_int2(r0, 0);  // no walk; reported below
-    int i = c.x, j = c.y;
     WindowWalker w{a.bp, a.nchunk, a.rps, a.wpb, lane, s_win[threadIdx.x >> 5], 0, 0};
-    w.load(i, j);
-    int n = 0;
+    w.load(c.x, c.y);
+    int r = w.row(c.x), q = w.col(c.y);
+    const int rlo = w.row(r0);
     int2* out = seg + (size_t)b * band;
-    int2 mine = make_int2(0, 0);  // cell n of the walk for n % 32 = lane, stored 32 at a time
-    while (!bad && i >= r0) {
-        if (n >= band || j < 0 || !w.inside(i, j)) {
-            bad = 1;
-            break;
-        }
-        if ((n & 31) == lane) mine = make_int2(i, j);
-        if ((++n & 31) == 0) out[n - 32 + lane] = mine;
-        if (i == 0 && j == 0) break;
-        const uint32_t f = w.field(i, j);
-        i -= field_di(f);
-        j -= field_dj(f);
+    int n = 0, mr, mc;
+    for (int got = bad ? 0 : 32; got == 32 && n < band; n += got) {
+        got = w.steps32(r, q, rlo, mr, mc);
+        if (lane < got) out[n + lane] = make_int2(w.row0 + mr, w.col(mc));
     }
-    if (lane < (n & 31)) out[(n & ~31) + lane] = mine;
+    const int i = w.row0 + r, j = w.col(q);
+    if (r >= rlo) bad = 1;  // left the matrix on the left
     // the walk must leave the band exactly at the cell its first cell's entry names
     if (b > 0 && !bad && (i != target.x || j != target.y)) bad = 1;
     if (lane == 0) {
@@ -273,18 +267,19 @@ __global__ void __launch_bounds__(32 * kWalkWarps) k_bt_walk(const BtArgs one, c
 // of the bands before it) and the total, each by a block-wide sum, then the
 // band's cells in ascending order; the CTA of band 0 writes the length and
 // the total (or -status).
+constexpr int kEmitThreads = 128;
 template <bool kMany>
-__global__ void __launch_bounds__(kBand) k_bt_emit(const BtArgs one, const BtArgs* __restrict__ many) {
+__global__ void __launch_bounds__(kEmitThreads) k_bt_emit(const BtArgs one, const BtArgs* __restrict__ many) {
     const BtArgs& a = kMany ? many[blockIdx.y] : one;
-    const int La = a.La, Lb = a.Lb, band = kBand;
+    const int La = a.La, Lb = a.Lb;
     const int cap = La < Lb ? La : Lb;
-    const BtScratch sc = bt_scratch(a.scratch, La, Lb);
-    const int nbands = sc.nbands;
+    const BtScratch sc = bt_scratch(a);
+    const int nbands = sc.nbands, band = sc.band;
     const int b = blockIdx.x;
     if (b >= nbands) return;  // CTA-uniform (the grid covers the largest pair)
     const int2* __restrict__ seg = sc.seg;
     const int* __restrict__ count = sc.count;
-    __shared__ int s_red[2][kBand / 32];
+    __shared__ int s_red[2][kEmitThreads / 32];
     // this thread's share of the counts before band b and of all counts
     int before = 0, all = 0;
     for (int q = threadIdx.x; q < nbands; q += blockDim.x) {
@@ -341,23 +336,22 @@ __global__ void __launch_bounds__(kBand) k_bt_emit(const BtArgs one, const BtArg
     }
 }
 
-int bandmap_band_rows() { return kBand; }
-
 size_t bandmap_scratch_bytes(int La, int Lb) {
-    const int nbands = (La + kBand - 1) / kBand;
+    // the shortest bands a call may choose for these rows take the most
+    const int band = band_rows(La, 0.0), nbands = (La + band - 1) / band;
     const int n2 = nbands >= 4 ? (nbands - 2) / 2 : 0;
     const int n4 = nbands >= 6 ? (nbands - 6) / 4 + 1 : 0;
     return (size_t)nbands * Lb * sizeof(int2)        // exits
            + (size_t)n2 * Lb * sizeof(int2)           // exits2
            + (size_t)n4 * Lb * sizeof(int2)           // exits4
            + (size_t)nbands * sizeof(int2)            // cross
-           + (size_t)nbands * kBand * sizeof(int2)    // seg
+           + (size_t)nbands * band * sizeof(int2)     // seg
            + (size_t)nbands * sizeof(int) + 64;       // count, end entry
 }
 
 cudaError_t launch_backtrace_bands(const BtArgs& a, cudaStream_t s) {
-    const int nbands = (a.La + kBand - 1) / kBand;
-    const dim3 grid((unsigned)map_ctas(a.Lb), (unsigned)nbands, 1);
+    const int band = a.band, nbands = (a.La + band - 1) / band;
+    const dim3 grid((unsigned)map_ctas(a.Lb, band), (unsigned)nbands, 1);
     if (a.ranges)
         k_bandmap<false, true><<<grid, 32 * kMapWarps, 0, s>>>(a, nullptr);
     else
@@ -372,15 +366,14 @@ cudaError_t launch_backtrace_bands(const BtArgs& a, cudaStream_t s) {
             a, nullptr);
     k_bt_chain<false><<<1, 32, 0, s>>>(a, nullptr);
     k_bt_walk<false><<<(nbands + kWalkWarps - 1) / kWalkWarps, 32 * kWalkWarps, 0, s>>>(a, nullptr);
-    k_bt_emit<false><<<dim3((unsigned)nbands, 1), kBand, 0, s>>>(a, nullptr);
+    k_bt_emit<false><<<dim3((unsigned)nbands, 1), kEmitThreads, 0, s>>>(a, nullptr);
     return cudaGetLastError();
 }
 
-cudaError_t launch_backtrace_bands_many(const BtArgs* many, int n, int maxLa, int maxLb,
+cudaError_t launch_backtrace_bands_many(const BtArgs* many, int n, int nbands, int maxLb,
                                         cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    const int nbands = (maxLa + kBand - 1) / kBand;
-    const dim3 grid((unsigned)map_ctas(maxLb), (unsigned)nbands, (unsigned)n);
+    const dim3 grid((unsigned)map_ctas(maxLb, kMaxBand), (unsigned)nbands, (unsigned)n);
     k_bandmap<true, false><<<grid, 32 * kMapWarps, 0, s>>>(BtArgs{}, many);
     const int n2 = nbands >= 4 ? (nbands - 2) / 2 : 0;
     if (n2 > 0)
@@ -393,7 +386,7 @@ cudaError_t launch_backtrace_bands_many(const BtArgs* many, int n, int maxLa, in
     k_bt_chain<true><<<n, 32, 0, s>>>(BtArgs{}, many);
     k_bt_walk<true><<<dim3((unsigned)((nbands + kWalkWarps - 1) / kWalkWarps), (unsigned)n),
                       32 * kWalkWarps, 0, s>>>(BtArgs{}, many);
-    k_bt_emit<true><<<dim3((unsigned)nbands, (unsigned)n), kBand, 0, s>>>(BtArgs{}, many);
+    k_bt_emit<true><<<dim3((unsigned)nbands, (unsigned)n), kEmitThreads, 0, s>>>(BtArgs{}, many);
     return cudaGetLastError();
 }
 

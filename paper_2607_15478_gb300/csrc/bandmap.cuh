@@ -9,7 +9,7 @@ namespace {
 
 constexpr int kNoPath = -2;
 constexpr int kOrigin = -1;
-constexpr int kBand = 128;  // rows per band
+constexpr int kMaxBand = 128;
 
 // The backtrace scratch of one pair (bandmap_scratch_bytes(La, Lb) bytes).
 struct BtScratch {
@@ -22,14 +22,16 @@ struct BtScratch {
     int2* seg;       // nbands x band: each band's piece of the path, descending
     int* count;      // nbands: cells in each piece
     int* end_entry;  // the end cell's entry
-    int nbands, n2, n4;
+    int band, nbands, n2, n4;
 };
-__host__ __device__ inline BtScratch bt_scratch(void* scratch, int La, int Lb) {
+__host__ __device__ inline BtScratch bt_scratch(const BtArgs& a) {
+    const int La = a.La, Lb = a.Lb;
     BtScratch r;
-    r.nbands = (La + kBand - 1) / kBand;
+    r.band = a.band;
+    r.nbands = (La + r.band - 1) / r.band;
     r.n2 = r.nbands >= 4 ? (r.nbands - 2) / 2 : 0;
     r.n4 = r.nbands >= 6 ? (r.nbands - 6) / 4 + 1 : 0;
-    char* p = static_cast<char*>(scratch);
+    char* p = static_cast<char*>(a.scratch);
     r.exits = reinterpret_cast<int2*>(p);
     p += (size_t)r.nbands * Lb * sizeof(int2);
     r.exits2 = reinterpret_cast<int2*>(p);
@@ -39,7 +41,7 @@ __host__ __device__ inline BtScratch bt_scratch(void* scratch, int La, int Lb) {
     r.cross = reinterpret_cast<int2*>(p);
     p += (size_t)r.nbands * sizeof(int2);
     r.seg = reinterpret_cast<int2*>(p);
-    p += (size_t)r.nbands * kBand * sizeof(int2);
+    p += (size_t)r.nbands * r.band * sizeof(int2);
     r.count = reinterpret_cast<int*>(p);
     p += (size_t)r.nbands * sizeof(int);
     r.end_entry = reinterpret_cast<int*>(p);
@@ -49,7 +51,8 @@ __host__ __device__ inline BtScratch bt_scratch(void* scratch, int La, int Lb) {
 
 // A segment of a band is mapped by one warp: lane t owns the 32 columns
 // s0 + 32 t .. + 31 of the segment's computed range, where s0 = c0 - halo; the
-// segment stores columns c0 .. c0 + kSegWidth - 1 (segments are kSegWidth apart).
+// segment stores columns c0 .. c0 + width - 1 (segments are width apart, the halo
+// is twice the band's rows).
 //
 // Inside a segment an entry is 16 bits, 2 * (column - s0) + (1 if in the band
 // above's last row), or one of two codes; a register holds those of columns u
@@ -65,7 +68,7 @@ __host__ __device__ inline BtScratch bt_scratch(void* scratch, int La, int Lb) {
 // took 89 us on the 20000 x 25000 pair and 1.5 ms at 100000 x 126231; see
 // bandmap.cu for the times now.)
 constexpr int kSegCols = 1024;
-constexpr int kSegWidth = kSegCols - 2 * kBand;
+__host__ __device__ inline int seg_width(int band) { return kSegCols - 2 * band; }
 constexpr unsigned kNoPath2 = 0xFFFEFFFEu;  // two columns without a path
 constexpr unsigned kOrigin16 = 0xFFFFu;
 
@@ -113,10 +116,11 @@ template <bool kBanded>
 __device__ __forceinline__ void bandmap_segment(const BtArgs& a, int b, int segx, int lane) {
     const uint32_t* __restrict__ bp = a.bp;
     const int La = a.La, Lb = a.Lb, nchunk = a.nchunk, rps = a.rps, wpb = a.wpb;
-    const BtScratch sc = bt_scratch(a.scratch, La, Lb);
+    const BtScratch sc = bt_scratch(a);
     if (b >= sc.nbands) return;  // warp-uniform, as are the returns below
-    const int r0 = b * kBand;
-    const int r1 = min(r0 + kBand, La);
+    const int width = seg_width(sc.band);
+    const int r0 = b * sc.band;
+    const int r1 = min(r0 + sc.band, La);
     int c0, halo;  // first stored column; columns recomputed to its left (multiple of 16)
     if (kBanded) {
         // segments start at the band's first column over these rows (the
@@ -124,7 +128,7 @@ __device__ __forceinline__ void bandmap_segment(const BtArgs& a, int b, int segx
         // path, so the first segment needs no halo and the rest of the grid
         // covers only the band's columns
         const int xs = a.ranges[r0 / rps].x * 8, ys = a.ranges[(r1 - 1) / rps].y * 8;
-        c0 = (xs & ~(kColsPerWord - 1)) + segx * kSegWidth;
+        c0 = (xs & ~(kColsPerWord - 1)) + segx * width;
         if (c0 >= min(ys, Lb)) return;
     } else {
         // Only cells that can lie on a path (path_lo, path_hi): a path
@@ -134,10 +138,10 @@ __device__ __forceinline__ void bandmap_segment(const BtArgs& a, int b, int segx
         // the cells left out are never asked for.
         const int xs = max(0, path_lo(r0, La, Lb) - 2);
         const int ys = min(Lb, path_hi(r1 - 1, La, Lb) + 1);
-        c0 = (xs & ~(kColsPerWord - 1)) + segx * kSegWidth;
+        c0 = (xs & ~(kColsPerWord - 1)) + segx * width;
         if (c0 >= ys) return;
     }
-    halo = segx == 0 ? 0 : 2 * kBand;
+    halo = segx == 0 ? 0 : 2 * sc.band;
     const int s0 = c0 - halo;
     const int jb = s0 + 32 * lane;  // first column of this lane
     // rows r0-2 and r0-1 name themselves: the entries of the cells below them
@@ -240,13 +244,13 @@ __device__ __forceinline__ void bandmap_segment(const BtArgs& a, int b, int segx
         for (int q = 0; q < 32; ++q) {
             const int h = q >> 4, u = q & 7, hi = (q >> 3) & 1;
             const int j = jb + q;
-            if (j >= c0 && j < c0 + kSegWidth && j < Lb)
+            if (j >= c0 && j < c0 + width && j < Lb)
                 exits[j] = make_int2(entry(half(e2.w[h][u], hi)), entry(half(e1.w[h][u], hi)));
         }
     } else {
         // the end cell's entry
         const int q = (Lb - 1) - jb;
-        if (q >= 0 && q < 32 && Lb - 1 >= c0 && Lb - 1 < c0 + kSegWidth) {
+        if (q >= 0 && q < 32 && Lb - 1 >= c0 && Lb - 1 < c0 + width) {
 #pragma unroll
             for (int v = 0; v < 32; ++v)
                 if (v == q) *sc.end_entry = entry(half(e1.w[v >> 4][v & 7], (v >> 3) & 1));

@@ -53,20 +53,37 @@ struct WindowWalker {
         }
         __syncwarp();
     }
-    // Whether cell (i, j) lies in the window (j >= 0).
-    __device__ __forceinline__ bool inside(int i, int j) const {
-        return i >= row0 && ch1 - (j >> 4) < kWalkChunks;
-    }
-    // The 2-bit field of cell (i, j) of the window.
-    __device__ __forceinline__ uint32_t field(int i, int j) const {
-        return (sm[(ch1 - (j >> 4)) * kWalkRows + (i - row0)] >> (2 * (j & 15))) & 3u;
+    // A position in the window: r rows below row0, c columns left of its last one.
+    __device__ __forceinline__ int row(int i) const { return i - row0; }
+    __device__ __forceinline__ int col(int j) const { return 16 * ch1 + 15 - j; }
+
+    // Up to 32 cells of the walk from (r, c), while rows stay at or below rlo and
+    // columns in the window and the matrix; returns how many, the first of them in
+    // lane 0's (mr, mc), and (r, c) is the cell after the last.  No branch: a walk
+    // that has ended stays where it is (a step of a loop with tests and exits took
+    // 110 ns).
+    __device__ __forceinline__ int steps32(int& r, int& c, int rlo, int& mr, int& mc) const {
+        const int climit = min(16 * kWalkChunks, 16 * ch1 + 16);  // columns c of cells
+        int n = 0;
+#pragma unroll
+        for (int u = 0; u < 32; ++u) {
+            const bool on = r >= rlo && c < climit;
+            if (lane == u) {
+                mr = r;
+                mc = c;
+            }
+            const uint32_t w = sm[on ? (c >> 4) * kWalkRows + r : 0];
+            const uint32_t f = (w >> (2 * (15 - (c & 15)))) & 3u;
+            // moves by field: rows 2, 1, 1, 1, columns 1, 1, 2, 1 (see step_of_field)
+            if (on) {
+                r -= (0x56 >> (2 * f)) & 3;
+                c += (0x65 >> (2 * f)) & 3;
+                ++n;
+            }
+        }
+        return n;
     }
 };
-
-// step_of_field as row and column moves: bit 0 -> (1,1); field 2 -> (1,2);
-// field 0 -> (2,1).
-__device__ __forceinline__ int field_di(uint32_t f) { return f == 0u ? 2 : 1; }
-__device__ __forceinline__ int field_dj(uint32_t f) { return f == 2u ? 2 : 1; }
 
 }  // namespace
 }  // namespace pardtw

@@ -19,67 +19,123 @@ int padded_dim(int D) {
     return 0;
 }
 
-// One thread per frame.  A is written row-major (La_pad x dp), B
-// chunk-transposed (bt_index, Lb_pad frames).  Frames of A beyond La, frames
-// of B beyond Lb and feature slots beyond D are zero.  Thread 0 also clears
-// the control words of the call.
-__device__ __forceinline__ void normalise_frame(int t, const float* __restrict__ A, int La,
-                                                int La_pad, const float* __restrict__ B, int Lb,
-                                                int Lb_pad, int D, int dp,
-                                                float* __restrict__ Ahat, float* __restrict__ Bt,
-                                                DevCtl* ctl) {
-    if (t == 0) {
-        ctl->status = 0;
-        ctl->detail = 0;
-        ctl->ticket = 0;
+// kNormFrames frames of A or of B per block.  A is written row-major (La_pad x
+// dp), B chunk-transposed (bt_index, Lb_pad frames) or, for the BF16 cost, as
+// bf16 rows of kBfStride (Bbf).  Frames of A beyond La, frames of B beyond Lb and
+// feature slots beyond D are zero.  The first thread also clears the control
+// words of the call.
+// Bound by latency and the writes: the block's frames are one stretch of global
+// memory, staged as it lies (every load in flight before the first is used), the
+// sums of squares run one thread per frame in feature order from shared memory,
+// and the results leave in the order of their layout.  (One thread per frame
+// reading and writing its own row: 53 us for 51012 frames of D = 100, 5 now; one warp
+// per frame for the bf16 rows of 48000 x 128: 120 us.)
+constexpr int kNormFrames = 64;
+constexpr int kNormThreads = 256;
+__host__ __device__ inline int norm_blocks(int La_pad, int Lb_pad) {
+    return (La_pad + kNormFrames - 1) / kNormFrames + (Lb_pad + kNormFrames - 1) / kNormFrames;
+}
+
+__device__ __forceinline__ void normalise_block(int blk, const NormArgs& a, int D, int dp,
+                                                __nv_bfloat16* __restrict__ Bbf) {
+    extern __shared__ float sm[];  // kNormFrames rows of D + 1 floats (odd or even: read in order
+                                   // of d by one thread per row), then the reciprocal norms
+    const int tid = threadIdx.x;
+    if (blk == 0 && tid == 0) {
+        a.ctl->status = 0;
+        a.ctl->detail = 0;
+        a.ctl->ticket = 0;
     }
-    const float* src;
-    bool valid, is_a;
-    int k;
-    if (t < La_pad) {
-        k = t;
-        src = A + (size_t)t * D;
-        valid = t < La;
-        is_a = true;
-    } else if (t < La_pad + Lb_pad) {
-        k = t - La_pad;
-        src = B + (size_t)k * D;
-        valid = k < Lb;
-        is_a = false;
-    } else {
-        return;
-    }
-    float ss = 0.f;
-    if (valid)
-        for (int d = 0; d < D; ++d) {
-            const float v = src[d];
-            ss = fmaf(v, v, ss);
+    const int na = (a.La_pad + kNormFrames - 1) / kNormFrames;
+    const bool is_a = blk < na;
+    const int f0 = (is_a ? blk : blk - na) * kNormFrames;
+    const int L = is_a ? a.La : a.Lb, Lp = is_a ? a.La_pad : a.Lb_pad;
+    if (f0 >= Lp) return;  // CTA-uniform
+    const int S = D | 1;                                    // row stride: conflict-free
+    const int have = max(min(kNormFrames, L - f0), 0);      // frames that exist
+    const int rows = min(kNormFrames, Lp - f0);             // frames to write
+    const float* __restrict__ src = (is_a ? a.A : a.B) + (size_t)f0 * D;
+    float* rs = sm + kNormFrames * S;
+    {
+        // element k = frame k / D, feature k % D, advanced without divisions
+        int f = tid / D, d = tid - f * D;
+        const int df = kNormThreads / D, dd = kNormThreads - df * D;
+        const int n = have * D;
+#pragma unroll 8
+        for (int k = tid; k < n; k += kNormThreads) {
+            sm[f * S + d] = __ldg(src + k);
+            f += df;
+            d += dd;
+            if (d >= D) {
+                d -= D;
+                ++f;
+            }
         }
-    const float r = ss > 0.f ? 1.0f / sqrtf(ss) : 0.f;
-    for (int d = 0; d < dp; ++d) {
-        const float v = (valid && d < D) ? src[d] * r : 0.f;
-        if (is_a)
-            Ahat[(size_t)k * dp + d] = v;
-        else
-            Bt[bt_index(k, d, dp)] = v;
+    }
+    __syncthreads();
+    if (tid < kNormFrames) {
+        float ss = 0.f;
+        if (tid < have) {
+#pragma unroll 4
+            for (int d = 0; d < D; ++d) {
+                const float v = sm[tid * S + d];
+                ss = fmaf(v, v, ss);
+            }
+        }
+        rs[tid] = ss > 0.f ? 1.0f / sqrtf(ss) : 0.f;
+    }
+    __syncthreads();
+    auto value = [&](int f, int d) { return (f < have && d < D) ? sm[f * S + d] * rs[f] : 0.f; };
+    if (is_a) {
+        float* __restrict__ out = a.Ahat + (size_t)f0 * dp;
+        int f = tid / dp, d = tid - f * dp;
+        const int df = kNormThreads / dp, dd = kNormThreads - df * dp;
+        for (int k = tid; k < rows * dp; k += kNormThreads) {
+            out[k] = value(f, d);
+            f += df;
+            d += dd;
+            if (d >= dp) {
+                d -= dp;
+                ++f;
+            }
+        }
+    } else if (Bbf) {
+        __nv_bfloat16* __restrict__ out = Bbf + (size_t)f0 * kBfStride;
+        for (int k = tid; k < rows * kBfStride; k += kNormThreads) {
+            const int f = k / kBfStride;
+            out[k] = __float2bfloat16_rn(value(f, k - f * kBfStride));
+        }
+    } else {
+        // chunk c, feature d, frame 16 c + e at (c dp + d) 16 + e (bt_index)
+        float* __restrict__ out = a.Bt + (size_t)f0 * dp;
+        const int e = tid & 15;
+        int c = 0, d = tid >> 4;
+        for (int k = tid; k < rows * dp; k += kNormThreads) {
+            while (d >= dp) {
+                d -= dp;
+                ++c;
+            }
+            out[k] = value(16 * c + e, d);
+            d += kNormThreads / 16;
+        }
     }
 }
 
-__global__ void k_normalise(const float* __restrict__ A, int La, int La_pad,
-                            const float* __restrict__ B, int Lb, int Lb_pad, int D, int dp,
-                            float* __restrict__ Ahat, float* __restrict__ Bt, DevCtl* ctl) {
-    normalise_frame(blockIdx.x * blockDim.x + threadIdx.x, A, La, La_pad, B, Lb, Lb_pad, D, dp,
-                    Ahat, Bt, ctl);
+__global__ void __launch_bounds__(kNormThreads)
+    k_normalise(const NormArgs a, int D, int dp, __nv_bfloat16* __restrict__ Bbf) {
+    normalise_block(blockIdx.x, a, D, dp, Bbf);
 }
 
 // One pair per blockIdx.y (the grid covers the largest pair); also clears the
 // batch's work-queue ticket.
-__global__ void k_normalise_many(const NormArgs* __restrict__ many, int D, int dp, int* ticket) {
-    const NormArgs& a = many[blockIdx.y];
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t == 0 && blockIdx.y == 0) *ticket = 0;
-    normalise_frame(t, a.A, a.La, a.La_pad, a.B, a.Lb, a.Lb_pad, D, dp, a.Ahat, a.Bt, a.ctl);
+__global__ void __launch_bounds__(kNormThreads)
+    k_normalise_many(const NormArgs* __restrict__ many, int D, int dp, int* ticket) {
+    const NormArgs a = many[blockIdx.y];
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *ticket = 0;
+    if ((int)blockIdx.x < norm_blocks(a.La_pad, a.Lb_pad))
+        normalise_block(blockIdx.x, a, D, dp, nullptr);
 }
+int norm_smem(int D) { return (kNormFrames * (D | 1) + kNormFrames) * (int)sizeof(float); }
 
 // A replayed batch graph starts with this: a new tag for the border entries
 // of every pair (entries left by the previous replay carry the old one).
@@ -95,55 +151,20 @@ cudaError_t launch_bump_epoch(DpArgs* many, int n, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_normalise(const float* A, int La, int La_pad, const float* B, int Lb,
-                             int Lb_pad, int D, int dp, float* Ahat, float* Bt, DevCtl* ctl,
-                             cudaStream_t s) {
-    const int n = La_pad + Lb_pad;
-    const int threads = 256;
-    k_normalise<<<(n + threads - 1) / threads, threads, 0, s>>>(A, La, La_pad, B, Lb, Lb_pad, D,
-                                                                dp, Ahat, Bt, ctl);
+cudaError_t launch_normalise(const NormArgs& a, int D, int dp, void* Bbf, cudaStream_t s) {
+    k_normalise<<<norm_blocks(a.La_pad, a.Lb_pad), kNormThreads, norm_smem(D), s>>>(
+        a, D, dp, static_cast<__nv_bfloat16*>(Bbf));
     return cudaGetLastError();
 }
 
-// One warp per frame of B: normalise in FP32 (the same sum of squares and
-// reciprocal square root as k_normalise), round each feature to bf16.
-__global__ void k_pack_b_bf16(const float* __restrict__ B, int Lb, int Lb_pad, int D,
-                              __nv_bfloat16* __restrict__ Bbf) {
-    const int f = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (f >= Lb_pad) return;
-    float r = 0.f;
-    if (f < Lb && lane == 0) {
-        float ss = 0.f;
-        for (int d = 0; d < D; ++d) {
-            const float v = B[(size_t)f * D + d];
-            ss = fmaf(v, v, ss);
-        }
-        r = ss > 0.f ? 1.0f / sqrtf(ss) : 0.f;
-    }
-    r = __shfl_sync(0xffffffffu, r, 0);
-    for (int d = lane; d < kBfStride; d += 32) {
-        const float v = (f < Lb && d < D) ? B[(size_t)f * D + d] * r : 0.f;
-        Bbf[(size_t)f * kBfStride + d] = __float2bfloat16_rn(v);
-    }
-}
-
-cudaError_t launch_pack_b_bf16(const float* B, int Lb, int Lb_pad, int D, void* Bbf,
-                               cudaStream_t s) {
-    const int warps = 8;
-    k_pack_b_bf16<<<(Lb_pad + warps - 1) / warps, warps * 32, 0, s>>>(
-        B, Lb, Lb_pad, D, static_cast<__nv_bfloat16*>(Bbf));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_normalise_many(const NormArgs* many, int n, int max_frames, int D, int dp,
+cudaError_t launch_normalise_many(const NormArgs* many, int n, int max_blocks, int D, int dp,
                                   int* ticket, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    const int threads = 256;
-    dim3 grid((unsigned)((max_frames + threads - 1) / threads), (unsigned)n);
-    k_normalise_many<<<grid, threads, 0, s>>>(many, D, dp, ticket);
+    k_normalise_many<<<dim3((unsigned)max_blocks, (unsigned)n), kNormThreads, norm_smem(D), s>>>(
+        many, D, dp, ticket);
     return cudaGetLastError();
 }
+int normalise_blocks(int La_pad, int Lb_pad) { return norm_blocks(La_pad, Lb_pad); }
 
 // C[i][j] = 1 - sum_d a^_i[d] b^_j[d], accumulated as fma(-a, b, acc) from 1
 // in feature order -- bit-identical to the cost the DP kernel uses.

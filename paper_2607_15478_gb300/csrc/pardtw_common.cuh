@@ -165,7 +165,7 @@ __host__ __device__ inline size_t bt_index(int f, int d, int dp) {
     return ((size_t)(f >> 4) * (size_t)dp + (size_t)d) * 16u + (size_t)(f & 15);
 }
 
-// Normalisation of one pair of a batch (k_normalise_many).
+// Normalisation of one pair.
 struct NormArgs {
     const float* A;
     int La, La_pad;
@@ -177,15 +177,17 @@ struct NormArgs {
 };
 
 // Launchers (each returns a cudaError_t from the launch).
-cudaError_t launch_normalise(const float* A, int La, int La_pad, const float* B, int Lb,
-                             int Lb_pad, int D, int dp, float* Ahat, float* Bt, DevCtl* ctl,
-                             cudaStream_t s);
+// Bbf: null, or for the BF16 cost B normalised as bf16 instead of Bt: Lb_pad
+// frames of kBfStride elements (features beyond D and frames beyond Lb are zero).
+cudaError_t launch_normalise(const NormArgs& a, int D, int dp, void* Bbf, cudaStream_t s);
 cudaError_t launch_cost(const float* Ahat, int La, const float* Bt, int Lb, int dp, float* C,
                         cudaStream_t s);
-// n pairs at once (`many`: device array); max_frames = largest La_pad + Lb_pad;
-// also zeroes *ticket, the work queue of launch_dp_split_many.
-cudaError_t launch_normalise_many(const NormArgs* many, int n, int max_frames, int D, int dp,
+// n pairs at once (`many`: device array); max_blocks = the most
+// normalise_blocks(La_pad, Lb_pad) among them; also zeroes *ticket, the work
+// queue of launch_dp_split_many.
+cudaError_t launch_normalise_many(const NormArgs* many, int n, int max_blocks, int D, int dp,
                                   int* ticket, cudaStream_t s);
+int normalise_blocks(int La_pad, int Lb_pad);
 // Every DpArgs::epoch of a batch in device memory += 1 (0 skipped).
 cudaError_t launch_bump_epoch(DpArgs* many, int n, cudaStream_t s);
 cudaError_t launch_dp(const DpArgs& a, int dp, int num_sms, cudaStream_t s);           // R = 1
@@ -228,10 +230,6 @@ cudaError_t launch_dp_split_wide(const DpArgs& a, int dp, int num_sms, cudaStrea
 cudaError_t launch_dp_split_wide_cl(const DpArgs& a, int dp, bool transposed, cudaStream_t s,
                                     bool* used);
 bool split_bf16_supported(int dp);
-// B normalised and stored as bf16 for the BF16 cost: Lb_pad frames of
-// kBfStride elements (features beyond D and frames beyond Lb are zero).
-cudaError_t launch_pack_b_bf16(const float* B, int Lb, int Lb_pad, int D, void* Bbf,
-                               cudaStream_t s);
 // Many pairs in one persistent launch: `many` (device) holds the pairs' DpArgs,
 // queue (device) the `items` (pair, strip group) items in the order CTAs take
 // them from *ticket; a pair's groups stand in ascending order, so a group only
@@ -272,12 +270,24 @@ struct BtArgs {
     const int2* ranges;  // banded DP: the strips' sub-chunk ranges (cells outside have no
                          // path), else null
     int transposed;      // the matrix is the transposed problem's: emit (column, row)
+    int band;            // rows per band: band_rows(La, cells)
 };
+// Rows per band of a pair of La rows in a call over `cells` matrix cells in all:
+// the band map and the walks take time in proportion to a band's rows (~0.17 and
+// ~0.06 us a row, all bands at once), the chain in proportion to the number of
+// bands (~0.6 us for four), so short pairs take short bands (1000 x 1200: 117 us
+// with 128 rows, 99 with 32; 3001 x 3607: 237 and 226 with 64) unless the call
+// fills the GPU: a segment of the map recomputes two columns per row of its band (256
+// pairs of up to 8000 frames: 3.59 ms with 64 rows, 3.44 with 128).
+inline int band_rows(int La, double cells) {
+    if (cells > 1e9) return 128;
+    return La <= 1536 ? 32 : (La <= 6144 ? 64 : 128);
+}
 size_t bandmap_scratch_bytes(int La, int Lb);
 cudaError_t launch_backtrace_bands(const BtArgs& a, cudaStream_t s);
-// n pairs at once; `many` is a device array of n BtArgs, maxLa / maxLb the
-// largest sizes among them.
-cudaError_t launch_backtrace_bands_many(const BtArgs* many, int n, int maxLa, int maxLb,
+// n pairs at once; `many` is a device array of n BtArgs, nbands and maxLb the
+// most bands and columns among them.
+cudaError_t launch_backtrace_bands_many(const BtArgs* many, int n, int nbands, int maxLb,
                                         cudaStream_t s);
 
 // Padded feature width used by the kernels for a given D (0 = unsupported).

@@ -142,8 +142,8 @@ extern "C" int dtw_align_static(const float* A, int La, const float* B, int Lb, 
         (void)cudaGetLastError();
         return DTW_ERR_CUDA;
     }
-    if (launch_normalise(A, La, La_pad, B, Lb, nchunk * kColsPerWord, D, dp, Ahat, Bt, ctl, s) !=
-        cudaSuccess) {
+    if (launch_normalise({A, La, La_pad, B, Lb, nchunk * kColsPerWord, Ahat, Bt, ctl}, D, dp,
+                         nullptr, s) != cudaSuccess) {
         (void)cudaGetLastError();
         return DTW_ERR_CUDA;
     }
@@ -185,6 +185,7 @@ extern "C" int dtw_align_static(const float* A, int La, const float* B, int Lb, 
     bt.scratch = base + off_map;
     bt.ranges = nullptr;
     bt.transposed = 0;
+    bt.band = band_rows(La, (double)La * Lb);
     const cudaError_t e = launch_plan(plan, a, dp, num_sms, s);
     if (e != cudaSuccess || launch_backtrace_bands(bt, s) != cudaSuccess) {
         (void)cudaGetLastError();

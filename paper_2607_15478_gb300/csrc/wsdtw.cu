@@ -178,31 +178,29 @@ __global__ void __launch_bounds__(32 * kWalkWarps)
         return;
     }
     const WsFrag f = fr[k];
-    int i = f.len - 1, j = ends[k];
-    int n = 0;
-    // cell n goes to pair row0 + len - 1 - n, 32 cells at a time
+    int i = f.len - 1, j = max(ends[k], 0);
+    // cell n goes to pair row0 + len - 1 - n
     int2* out = reinterpret_cast<int2*>(scratch) + (f.row0 + f.len - 1);
-    int2 mine = make_int2(0, 0);
     WindowWalker w{f.bp, f.nchunk, f.rps, f.wpb, lane, s_win[threadIdx.x >> 5], 0, 0};
-    w.load(i, max(j, 0));
-    for (;;) {
-        if ((n & 31) == lane) mine = make_int2(f.row0 + i, j);
-        if ((++n & 31) == 0) out[-(n - 32 + lane)] = mine;
-        if (i == 0) break;
-        const uint32_t fl = w.field(i, j);
-        i -= field_di(fl);
-        j -= field_dj(fl);
-        if (i < 0 || j < 0 || n >= f.len) {
-            if (lane == 0) {
-                raise_status(ctl, DTW_ERR_CUDA, 22);
-                count[k] = 0;
-            }
-            return;
-        }
-        if (!w.inside(i, j)) w.load(i, j);
+    int n = 0, last = -1;  // cells so far, row of the last one
+    while (i >= 0 && j >= 0) {
+        w.load(i, j);
+        int r = w.row(i), c = w.col(j), got;
+        do {
+            int mr, mc;
+            got = w.steps32(r, c, 0, mr, mc);
+            if (lane < got) out[-(n + lane)] = make_int2(f.row0 + w.row0 + mr, w.col(mc));
+            if (got > 0) last = w.row0 + __shfl_sync(0xffffffffu, mr, got - 1);
+            n += got;
+        } while (got == 32);
+        i = w.row0 + r;
+        j = w.col(c);
     }
-    if (lane < (n & 31)) out[-((n & ~31) + lane)] = mine;
-    if (lane == 0) count[k] = n;
+    const bool bad = last != 0;  // the walk has to end in the fragment's row 0
+    if (lane == 0) {
+        if (bad) raise_status(ctl, DTW_ERR_CUDA, 22);
+        count[k] = bad ? 0 : n;
+    }
 }
 
 // The fragment paths one after another, one CTA per fragment: fragment k's n_k
