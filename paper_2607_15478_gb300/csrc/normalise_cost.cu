@@ -8,6 +8,8 @@
 // matrix is never stored); dtw_cost materialises it for inspection.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "pardtw_common.cuh"
 
 namespace pardtw {
@@ -168,127 +170,114 @@ int normalise_blocks(int La_pad, int Lb_pad) { return norm_blocks(La_pad, Lb_pad
 
 // C[i][j] = 1 - sum_d a^_i[d] b^_j[d], accumulated as fma(-a, b, acc) from 1
 // in feature order -- bit-identical to the cost the DP kernel uses.
-// Writing the matrix is the whole cost of this kernel (4 bytes a cell against
-// (La + Lb) * D * 4 bytes read), so it is laid out for the HBM write: a block
-// of 256 threads covers kCostCols columns and takes tiles of kCostRows rows
-// (about 8192 blocks, each over several tiles); thread (tx, ty) makes the 4 x 4
-// cells of columns 4 tx .. 4 tx + 3 and rows 4 ty .. 4 ty + 3 of each tile.
-// b^ comes as one 16-byte word per feature (bt_index puts 16 consecutive frames
-// of a feature side by side), a^ as 16-byte broadcast loads (a warp holds one
-// ty), and each row of 4 results is one 16-byte store when the rows are
-// 16-byte aligned (Lb % 4 == 0), else four 4-byte stores.  Loading b^ per tile
-// from the chunk layout costs ~8 L1 wavefronts per warp load (a warp's 128
-// columns span 8 chunks): that, not HBM, bounded the first form of this kernel
-// (3.3 TB/s against 7.6 for a plain write), hence the registers below.
-constexpr int kCostRows = 16, kCostCols = 256, kCostMaxDp = 128;
+// Writing the matrix is most of the cost of this kernel (4 bytes a cell against
+// (La + Lb) * D * 4 bytes read), so it is laid out for the HBM write: a warp covers
+// 128 columns, lane l columns l, l + 32, l + 64, l + 96 of them, so every store of
+// a row is 128 neighbouring bytes whatever Lb and C's alignment are (4 neighbouring
+// columns a lane needed 16-byte stores, and fell to strided ones where a row
+// did not start on 16 bytes); the 8 warps of a block write 4 KB of each row.  a^
+// comes as 16-byte broadcast loads; the FMAs are paired (two columns each, each
+// rounded once).  Blocks take kRows rows at a time, grid-stride; about 16 of them
+// per SM, two resident (more registers, for loads in flight, were worth more than
+// more warps).  Measured, the whole call (TB/s written; before / now): 12000 x 15000,
+// D = 12, 4.06 / 5.7; 11999 x 14999 2.7 / 5.5; D = 16 2.9 / 4.3; D = 20 1.4 / 2.0; 6001 x
+// 7003, D = 64, 0.55 / 0.95 (a plain write of such a buffer: 7.3).
+constexpr int kCostWarps = 8, kCostCols = 128 * kCostWarps, kCostMaxDp = 128;
 
-// The rows i0 .. i0+3 of a thread's tile against its 4 columns, features
-// d0 .. d0+3 (b[u]: the 4 columns' values of feature d0 + u).
-__device__ __forceinline__ void cost_fma4(float (&acc)[4][4], const float4 (&a)[4],
-                                          const float4 (&b)[4]) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const float av[4] = {a[r].x, a[r].y, a[r].z, a[r].w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            acc[r][0] = fmaf(-av[u], b[u].x, acc[r][0]);
-            acc[r][1] = fmaf(-av[u], b[u].y, acc[r][1]);
-            acc[r][2] = fmaf(-av[u], b[u].z, acc[r][2]);
-            acc[r][3] = fmaf(-av[u], b[u].w, acc[r][3]);
-        }
-    }
-}
-
-__device__ __forceinline__ void cost_store4(const float (&acc)[4][4], int i0, int La, int j,
-                                            int Lb, float* __restrict__ C, int vec) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int i = i0 + r;
-        if (i >= La) continue;
-        float* out = C + (size_t)i * Lb + j;
-        if (vec && j + 3 < Lb) {
-            __stcs(reinterpret_cast<float4*>(out),
-                   make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]));
-        } else {
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (j + c < Lb) __stcs(out + c, acc[r][c]);
-        }
-    }
-}
-
-// DP <= 16: the thread's 4 columns of b^ stay in registers over all its row
-// tiles (DP float4 words), so a tile costs only the 4 rows' values of a^ (one
-// broadcast load per 4 features and row) and the stores.  Other widths load
-// b^ per tile (L1 hits).
-template <int DP>
-__global__ void __launch_bounds__(256) k_cost(const float* __restrict__ Ahat, int La,
-                                              const float* __restrict__ Bt, int Lb, int dp,
-                                              float* __restrict__ C, int vec) {
-    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
-    const int j = blockIdx.x * kCostCols + 4 * tx;
-    if (j >= Lb) return;  // Bt holds whole chunks of 16 frames: j .. j+3 exist
+// DP <= 16: the lane's 4 columns of b^ stay in registers over all its rows.
+// Other widths (DP = 0) load b^ per tile of rows (L1 hits).
+template <int DP, int kRows>
+__global__ void __launch_bounds__(32 * kCostWarps, 2)
+    k_cost(const float* __restrict__ Ahat, int La, const float* __restrict__ Bt, int Lb, int dp,
+           float* __restrict__ C) {
+    const int lane = threadIdx.x & 31;
+    const int jw = blockIdx.x * kCostCols + 128 * (threadIdx.x >> 5);  // the warp's first column
+    if (jw >= Lb) return;
     if (DP > 0) dp = DP;
-    const float* bcol = Bt + bt_index(j, 0, dp);  // feature d at bcol + 16 d
-    constexpr int kRegD = DP > 0 ? DP : 4;
-    float4 breg[kRegD];
+    const float* bcol[4];  // feature d of column c at bcol[c] + 16 d
+#pragma unroll
+    for (int c = 0; c < 4; ++c) bcol[c] = Bt + bt_index(min(jw + lane + 32 * c, Lb - 1), 0, dp);
+    constexpr int kRegD = DP > 0 ? DP : 1;
+    float2 b[kRegD][2];
     if constexpr (DP > 0) {
 #pragma unroll
-        for (int d = 0; d < DP; ++d)
-            breg[d] = __ldg(reinterpret_cast<const float4*>(bcol + (size_t)d * 16));
+        for (int d = 0; d < DP; ++d) {
+            b[d][0] = make_float2(__ldg(bcol[0] + 16 * d), __ldg(bcol[1] + 16 * d));
+            b[d][1] = make_float2(__ldg(bcol[2] + 16 * d), __ldg(bcol[3] + 16 * d));
+        }
     }
-    for (int i0 = blockIdx.y * kCostRows + 4 * ty; i0 < La; i0 += gridDim.y * kCostRows) {
-        float acc[4][4];
+    const bool whole = jw + 128 <= Lb;
+    for (int i0 = blockIdx.y * kRows; i0 < La; i0 += gridDim.y * kRows) {
+        float2 acc[kRows][2];
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < kRows; ++r) acc[r][0] = acc[r][1] = make_float2(1.0f, 1.0f);
+        // features d0 .. d0 + 3 of the rows (those beyond La read row La - 1 and are
+        // never stored)
+        auto features = [&](int d0, const float2 (*bb)[2]) {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[r][c] = 1.0f;
-        const float* arow[4];  // rows beyond La read row La - 1 (never stored)
+            for (int r = 0; r < kRows; ++r) {
+                const float4 a = __ldg(reinterpret_cast<const float4*>(
+                    Ahat + (size_t)min(i0 + r, La - 1) * dp + d0));
+                const float av[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
-        for (int r = 0; r < 4; ++r) arow[r] = Ahat + (size_t)min(i0 + r, La - 1) * dp;
+                for (int u = 0; u < 4; ++u) {
+                    const float2 x = make_float2(-av[u], -av[u]);
+                    acc[r][0] = __ffma2_rn(x, bb[u][0], acc[r][0]);
+                    acc[r][1] = __ffma2_rn(x, bb[u][1], acc[r][1]);
+                }
+            }
+        };
         if constexpr (DP > 0) {
 #pragma unroll
-            for (int d0 = 0; d0 < DP; d0 += 4) {
-                float4 a[4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-                    a[r] = __ldg(reinterpret_cast<const float4*>(arow[r] + d0));
-                const float4 b[4] = {breg[d0], breg[d0 + 1], breg[d0 + 2], breg[d0 + 3]};
-                cost_fma4(acc, a, b);
-            }
+            for (int d0 = 0; d0 < DP; d0 += 4) features(d0, b + d0);
         } else {
             for (int d0 = 0; d0 < dp; d0 += 4) {
-                float4 a[4], b[4];
+                float2 t[4][2];
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    b[u] = __ldg(reinterpret_cast<const float4*>(bcol + (size_t)(d0 + u) * 16));
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-                    a[r] = __ldg(reinterpret_cast<const float4*>(arow[r] + d0));
-                cost_fma4(acc, a, b);
+                for (int u = 0; u < 4; ++u) {
+                    t[u][0] = make_float2(__ldg(bcol[0] + 16 * (d0 + u)), __ldg(bcol[1] + 16 * (d0 + u)));
+                    t[u][1] = make_float2(__ldg(bcol[2] + 16 * (d0 + u)), __ldg(bcol[3] + 16 * (d0 + u)));
+                }
+                features(d0, t);
             }
         }
-        cost_store4(acc, i0, La, j, Lb, C, vec);
+        float* out = C + (size_t)i0 * Lb + jw + lane;
+        if (whole && i0 + kRows <= La) {
+#pragma unroll
+            for (int r = 0; r < kRows; ++r, out += Lb) {
+                __stcs(out, acc[r][0].x);
+                __stcs(out + 32, acc[r][0].y);
+                __stcs(out + 64, acc[r][1].x);
+                __stcs(out + 96, acc[r][1].y);
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < kRows; ++r, out += Lb) {
+                const float v[4] = {acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y};
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (i0 + r < La && jw + lane + 32 * c < Lb) __stcs(out + 32 * c, v[c]);
+            }
+        }
     }
 }
 
 cudaError_t launch_cost(const float* Ahat, int La, const float* Bt, int Lb, int dp, float* C,
                         cudaStream_t s) {
     if (dp > kCostMaxDp || dp % 4 != 0) return cudaErrorInvalidValue;
+    constexpr int kFew = 4, kMany = 8;  // rows a tile with b^ in registers, with b^ loaded per tile
+    const int rows = dp <= 16 ? kFew : kMany;
     const int gx = (Lb + kCostCols - 1) / kCostCols;
-    const int ty = (La + kCostRows - 1) / kCostRows;
-    // about 8192 blocks: each takes several row tiles, reusing its columns
-    int gy = (8192 + gx - 1) / gx;
-    if (gy > ty) gy = ty;
-    if (gy > 65535) gy = 65535;
+    const int ty = (La + rows - 1) / rows;
+    const int gy = std::min(std::min((2432 + gx - 1) / gx, ty), 65535);
     const dim3 grid((unsigned)gx, (unsigned)gy);
-    const int vec = (Lb % 4 == 0 && reinterpret_cast<uintptr_t>(C) % 16 == 0) ? 1 : 0;
+    const int threads = 32 * kCostWarps;
     switch (dp) {
-        case 4: k_cost<4><<<grid, 256, 0, s>>>(Ahat, La, Bt, Lb, dp, C, vec); break;
-        case 8: k_cost<8><<<grid, 256, 0, s>>>(Ahat, La, Bt, Lb, dp, C, vec); break;
-        case 12: k_cost<12><<<grid, 256, 0, s>>>(Ahat, La, Bt, Lb, dp, C, vec); break;
-        case 16: k_cost<16><<<grid, 256, 0, s>>>(Ahat, La, Bt, Lb, dp, C, vec); break;
-        default: k_cost<0><<<grid, 256, 0, s>>>(Ahat, La, Bt, Lb, dp, C, vec); break;
+        case 4: k_cost<4, kFew><<<grid, threads, 0, s>>>(Ahat, La, Bt, Lb, dp, C); break;
+        case 8: k_cost<8, kFew><<<grid, threads, 0, s>>>(Ahat, La, Bt, Lb, dp, C); break;
+        case 12: k_cost<12, kFew><<<grid, threads, 0, s>>>(Ahat, La, Bt, Lb, dp, C); break;
+        case 16: k_cost<16, kFew><<<grid, threads, 0, s>>>(Ahat, La, Bt, Lb, dp, C); break;
+        default: k_cost<0, kMany><<<grid, threads, 0, s>>>(Ahat, La, Bt, Lb, dp, C); break;
     }
     return cudaGetLastError();
 }
