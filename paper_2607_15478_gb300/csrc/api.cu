@@ -86,8 +86,8 @@ bool reachable(int La, int Lb) {
 struct Layout {
     DpPlan plan;
     int dp, R, rps, wpb, nstrips, nchunk, ngroups, La_pad, cap;
-    size_t off_ctl, off_ahat, off_bhat, off_bbf, off_bp, off_bt, off_stage_a, off_stage_b,
-        total;
+    size_t off_ctl, off_ahat, off_bhat, off_bbf, off_bp, off_bt, off_bt_end, off_stage_a,
+        off_stage_b, total;
     size_t border_bytes;
 };
 
@@ -179,15 +179,19 @@ Layout make_layout(int La, int Lb, int D, const DpPlan& plan) {
     L.off_bp = o;
     o = align256(o + (size_t)L.nstrips * L.nchunk * L.wpb * sizeof(uint32_t));
     L.off_bt = o;
-    o = align256(o + bandmap_scratch_bytes(La, Lb));
+    L.off_bt_end = align256(o + bandmap_scratch_bytes(La, Lb));
+    // host inputs are staged where the backtrace's scratch lies: they have been
+    // read when it is first written
     L.off_stage_a = o;
     o = align256(o + (size_t)La * D * sizeof(float));
     L.off_stage_b = o;
     o = align256(o + (size_t)Lb * D * sizeof(float));
-    L.total = o;
+    L.total = std::max(o, L.off_bt_end);
     L.border_bytes = (size_t)L.ngroups * Lb * 2 * sizeof(unsigned long long);
     return L;
 }
+
+constexpr size_t kGrowRoomFrom = size_t(4) << 20;
 
 int ensure_workspace(dtw_handle* h, size_t bytes, size_t border_bytes) {
     if (bytes > h->ws_cap) {
@@ -195,7 +199,9 @@ int ensure_workspace(dtw_handle* h, size_t bytes, size_t border_bytes) {
         if (h->ws) cudaFree(h->ws);
         h->ws = nullptr;
         h->ws_cap = 0;
-        size_t want = bytes + bytes / 8;
+        // room to grow, but not where it would cost a mapping of its own (small
+        // allocations share one)
+        size_t want = bytes + (bytes > kGrowRoomFrom ? bytes / 8 : 0);
         if (cudaMalloc(&h->ws, want) != cudaSuccess) {
             (void)cudaGetLastError();
             if (cudaMalloc(&h->ws, bytes) != cudaSuccess) {
@@ -212,7 +218,7 @@ int ensure_workspace(dtw_handle* h, size_t bytes, size_t border_bytes) {
         if (h->border) cudaFree(h->border);
         h->border = nullptr;
         h->border_cap = 0;
-        size_t want = border_bytes + border_bytes / 8;
+        size_t want = border_bytes + (border_bytes > kGrowRoomFrom ? border_bytes / 8 : 0);
         if (cudaMalloc(&h->border, want) != cudaSuccess) {
             (void)cudaGetLastError();
             h->border = nullptr;
@@ -449,7 +455,7 @@ BatchSetup batch_setup(std::vector<int> idx, const int* La, const int* Lb, int D
         const int k = idx[q];
         const Layout& L = b.Ls[q];
         b.off[q] = o0;
-        o0 = align256(o0 + (L.off_stage_a - L.off_ahat));  // Ahat, Bhat, bp, band maps
+        o0 = align256(o0 + (L.off_bt_end - L.off_ahat));  // Ahat, Bhat, bp, band maps
         b.boff[q] = border_total;
         border_total += L.border_bytes;
         b.maxLb = std::max(b.maxLb, Lb[k]);
