@@ -36,10 +36,21 @@ namespace pardtw {
 namespace {
 
 constexpr int kMapWarps = 4;  // segments per CTA
+// CTAs of the band map up to which a pair's backtrace kernels form a chain
+// (launch_chained): the next kernel's CTAs are placed while one runs, which hides
+// ~2 us of each launch (with the DP kernel's: 1000 x 1200 frames 99.0 -> 85.6 us, 3001 x
+// 3607 230 -> 215, 20000 x 25000 (1565 CTAs) 1.129 -> 1.120 ms), but the wait
+// costs every CTA of a grid of many waves (3756 CTAs: 2.781 and 2.784 ms; 24490: 7.698
+// ms, 7.764 chained; a batch of 256 pairs 3.49, 3.65 chained).
+constexpr int kChainCtas = 2048;
 
 template <bool kMany, bool kBanded>
 __global__ void __launch_bounds__(32 * kMapWarps) k_bandmap(const BtArgs one,
                                                             const BtArgs* __restrict__ many) {
+    if (!kMany && one.chained) {
+        chain_wait();
+        chain_next();
+    }
     const BtArgs a = kMany ? many[blockIdx.z] : one;
     // kMany: one pair per blockIdx.z (the grid covers the largest pair;
     // warps beyond a pair's bands or columns leave at once)
@@ -80,6 +91,10 @@ __device__ __forceinline__ bool map_column(const BtArgs& a, int r1, int j) {
 template <bool kMany>
 __global__ void __launch_bounds__(256) k_bt_compose(const BtArgs one,
                                                     const BtArgs* __restrict__ many) {
+    if (!kMany && one.chained) {
+        chain_wait();
+        chain_next();
+    }
     const BtArgs& a = kMany ? many[blockIdx.z] : one;
     const int La = a.La, Lb = a.Lb;
     const BtScratch sc = bt_scratch(a);
@@ -107,6 +122,10 @@ __global__ void __launch_bounds__(256) k_bt_compose(const BtArgs one,
 template <bool kMany>
 __global__ void __launch_bounds__(256) k_bt_compose4(const BtArgs one,
                                                      const BtArgs* __restrict__ many) {
+    if (!kMany && one.chained) {
+        chain_wait();
+        chain_next();
+    }
     const BtArgs& a = kMany ? many[blockIdx.z] : one;
     const int La = a.La, Lb = a.Lb;
     const BtScratch sc = bt_scratch(a);
@@ -134,6 +153,10 @@ __global__ void __launch_bounds__(256) k_bt_compose4(const BtArgs one,
 // cross[b] = (i, j) of that cell; status on failure.
 template <bool kMany>
 __global__ void k_bt_chain(const BtArgs one, const BtArgs* __restrict__ many) {
+    if (!kMany && one.chained) {
+        chain_wait();
+        chain_next();
+    }
     if (threadIdx.x != 0) return;
     const BtArgs& a = kMany ? many[blockIdx.x] : one;
     const int La = a.La, Lb = a.Lb;
@@ -206,6 +229,10 @@ template <bool kMany>
 __global__ void __launch_bounds__(32 * kWalkWarps) k_bt_walk(const BtArgs one, const BtArgs* __restrict__ many) {
     static_assert(kWalkRows >= kMaxBand, "a band's rows fit the window");
     __shared__ uint32_t s_win[kWalkWarps][kWalkWords];
+    if (!kMany && one.chained) {
+        chain_wait();
+        chain_next();
+    }
     const BtArgs& a = kMany ? many[blockIdx.y] : one;
     DevCtl* ctl = a.ctl;
     const BtScratch sc = bt_scratch(a);
@@ -270,6 +297,7 @@ __global__ void __launch_bounds__(32 * kWalkWarps) k_bt_walk(const BtArgs one, c
 constexpr int kEmitThreads = 128;
 template <bool kMany>
 __global__ void __launch_bounds__(kEmitThreads) k_bt_emit(const BtArgs one, const BtArgs* __restrict__ many) {
+    if (!kMany && one.chained) chain_wait();
     const BtArgs& a = kMany ? many[blockIdx.y] : one;
     const int La = a.La, Lb = a.Lb;
     const int cap = La < Lb ? La : Lb;
@@ -349,25 +377,32 @@ size_t bandmap_scratch_bytes(int La, int Lb) {
            + (size_t)nbands * sizeof(int) + 64;       // count, end entry
 }
 
-cudaError_t launch_backtrace_bands(const BtArgs& a, cudaStream_t s) {
+cudaError_t launch_backtrace_bands(const BtArgs& pair, cudaStream_t s) {
+    BtArgs a = pair;
     const int band = a.band, nbands = (a.La + band - 1) / band;
     const dim3 grid((unsigned)map_ctas(a.Lb, band), (unsigned)nbands, 1);
-    if (a.ranges)
-        k_bandmap<false, true><<<grid, 32 * kMapWarps, 0, s>>>(a, nullptr);
-    else
-        k_bandmap<false, false><<<grid, 32 * kMapWarps, 0, s>>>(a, nullptr);
+    a.chained = !a.ranges && (long long)grid.x * grid.y <= kChainCtas;
+    const bool ch = a.chained != 0;
+    const BtArgs* none = nullptr;
+    cudaError_t e = launch_chained(ch, a.ranges ? k_bandmap<false, true> : k_bandmap<false, false>,
+                                   grid, 32 * kMapWarps, 0, s, a, none);
     const int n2 = nbands >= 4 ? (nbands - 2) / 2 : 0;
-    if (n2 > 0)
-        k_bt_compose<false><<<dim3((unsigned)((a.Lb + 255) / 256), (unsigned)n2, 1), 256, 0, s>>>(
-            a, nullptr);
+    const unsigned cols = (unsigned)((a.Lb + 255) / 256);
+    if (e == cudaSuccess && n2 > 0)
+        e = launch_chained(ch, k_bt_compose<false>, dim3(cols, (unsigned)n2, 1), 256, 0, s, a, none);
     const int n4 = nbands >= 6 ? (nbands - 6) / 4 + 1 : 0;
-    if (n4 > 0)
-        k_bt_compose4<false><<<dim3((unsigned)((a.Lb + 255) / 256), (unsigned)n4, 1), 256, 0, s>>>(
-            a, nullptr);
-    k_bt_chain<false><<<1, 32, 0, s>>>(a, nullptr);
-    k_bt_walk<false><<<(nbands + kWalkWarps - 1) / kWalkWarps, 32 * kWalkWarps, 0, s>>>(a, nullptr);
-    k_bt_emit<false><<<dim3((unsigned)nbands, 1), kEmitThreads, 0, s>>>(a, nullptr);
-    return cudaGetLastError();
+    if (e == cudaSuccess && n4 > 0)
+        e = launch_chained(ch, k_bt_compose4<false>, dim3(cols, (unsigned)n4, 1), 256, 0, s, a, none);
+    if (e == cudaSuccess)
+        e = launch_chained(ch, k_bt_chain<false>, dim3(1), 32, 0, s, a, none);
+    if (e == cudaSuccess)
+        e = launch_chained(ch, k_bt_walk<false>,
+                           dim3((unsigned)((nbands + kWalkWarps - 1) / kWalkWarps)), 32 * kWalkWarps,
+                           0, s, a, none);
+    if (e == cudaSuccess)
+        e = launch_chained(ch, k_bt_emit<false>, dim3((unsigned)nbands, 1), kEmitThreads, 0, s, a,
+                           none);
+    return e;
 }
 
 cudaError_t launch_backtrace_bands_many(const BtArgs* many, int n, int nbands, int maxLb,

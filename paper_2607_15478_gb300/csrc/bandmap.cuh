@@ -170,8 +170,8 @@ __device__ __forceinline__ void bandmap_segment(const BtArgs& a, int b, int segx
         }
         const int q = lr >> 2;
         const uint32_t* src = bp + ((size_t)strip * nchunk) * wpb + 4 * q;
-        g.a = __ldg(reinterpret_cast<const uint4*>(src + (size_t)ca * wpb));
-        g.b = __ldg(reinterpret_cast<const uint4*>(src + (size_t)cb * wpb));
+        g.a = *reinterpret_cast<const uint4*>(src + (size_t)ca * wpb);
+        g.b = *reinterpret_cast<const uint4*>(src + (size_t)cb * wpb);
         g.i = next - (lr & 3);
         g.k0 = lr & 3;
         g.k1 = min(4, min(rps - 4 * q, r1 - g.i));

@@ -202,7 +202,7 @@ __device__ __forceinline__ void run_cost(const DpArgs& p, int strip, int half, i
         const float4* s = reinterpret_cast<const float4*>(p.Ahat + (size_t)(i0 + k) * DP);
 #pragma unroll
         for (int q = 0; q < DP / 4; ++q) {
-            const float4 v = ghost ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(s + q);
+            const float4 v = ghost ? make_float4(0.f, 0.f, 0.f, 0.f) : s[q];
             na[k][4 * q] = -v.x;
             na[k][4 * q + 1] = -v.y;
             na[k][4 * q + 2] = -v.z;
@@ -317,7 +317,7 @@ __device__ __forceinline__ void run_cost_wide(const DpArgs& p, int strip, int w,
             const int r = e / (DP / 4), q = e - r * (DP / 4);
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
             if (r < kRows)
-                v = __ldg(reinterpret_cast<const float4*>(p.Ahat + (size_t)(strip * kRows + r) * DP) + q);
+                v = reinterpret_cast<const float4*>(p.Ahat + (size_t)(strip * kRows + r) * DP)[q];
             *reinterpret_cast<float4*>(tile + r * kS + 4 * q) = v;
         }
         asm volatile("bar.sync %0, %1;" ::"r"(1 + w), "r"(kT) : "memory");
@@ -457,8 +457,8 @@ __device__ __forceinline__ void run_cost_bf16(const DpArgs& p, int strip, int w,
         for (int d = 0; d < DP; d += 8) {
             float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
             if (r < kRows) {
-                v0 = __ldg(reinterpret_cast<const float4*>(src + d));
-                v1 = __ldg(reinterpret_cast<const float4*>(src + d + 4));
+                v0 = *reinterpret_cast<const float4*>(src + d);
+                v1 = *reinterpret_cast<const float4*>(src + d + 4);
             }
             const uint32_t w0 = pack_bf16x2(v0.x, v0.y), w1 = pack_bf16x2(v0.z, v0.w);
             const uint32_t w2 = pack_bf16x2(v1.x, v1.y), w3 = pack_bf16x2(v1.z, v1.w);
@@ -1112,7 +1112,12 @@ __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if constexpr (kCl) cluster_sync_all();  // every CTA's barriers before any remote access
+    if constexpr (kCl) {
+        chain_wait();  // for the normalised sequences and ctl
+        asm volatile("fence.proxy.async;" ::: "memory");  // the bulk copies read them, too
+        chain_next();
+        cluster_sync_all();  // every CTA's barriers before any remote access
+    }
     // Lifetime sub-chunk counts of the slots and of the writer's ring, and (in
     // a cluster) of the slots of the first strip of the CTA below and of the
     // links into and out of this CTA.

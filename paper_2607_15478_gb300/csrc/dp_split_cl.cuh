@@ -60,8 +60,9 @@ cudaLaunchConfig_t cl_config(dim3 grid, int threads, int smem, cudaStream_t s,
     at[0].val.clusterDim.x = (unsigned)cn;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1] = chained_attr(true);
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cfg;
 }
 
@@ -82,7 +83,7 @@ const ClInfo& cl_info(int dev) {
         return ci;
     }
     for (int k = 0; k < kNClSizes; ++k) {
-        cudaLaunchAttribute at[1];
+        cudaLaunchAttribute at[2];
         cudaLaunchConfig_t cfg =
             cl_config(dim3((unsigned)kClSizes[k]), K::kThreads, K::smem(), nullptr, at, kClSizes[k]);
         int n = 0;
@@ -136,7 +137,7 @@ cudaError_t launch_cl(const DpArgs& pair, cudaStream_t s, bool* used) {
     }
     if (cn == 0) return cudaSuccess;
     using K = ClKernel<DP, kBF, kT, NS>;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     cudaLaunchConfig_t cfg =
         cl_config(dim3((unsigned)(nclusters * cn)), K::kThreads, K::smem(), s, at, cn);
     const cudaError_t e = cudaLaunchKernelEx(&cfg, K::kern(), a,

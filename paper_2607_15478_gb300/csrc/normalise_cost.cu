@@ -125,6 +125,7 @@ __device__ __forceinline__ void normalise_block(int blk, const NormArgs& a, int 
 
 __global__ void __launch_bounds__(kNormThreads)
     k_normalise(const NormArgs a, int D, int dp, __nv_bfloat16* __restrict__ Bbf) {
+    chain_next();
     normalise_block(blockIdx.x, a, D, dp, Bbf);
 }
 

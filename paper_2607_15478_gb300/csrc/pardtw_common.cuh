@@ -62,6 +62,45 @@ cudaError_t blocks_per_sm_once(K* kern, int threads, int smem, DeviceSlots& cach
     return cudaSuccess;
 }
 
+// Kernels of one call in a chain: each is launched with launch_chained, so that
+// its CTAs are placed while the kernel before it in the stream still runs, and
+// starts with chain_wait (all its threads, before the first access to global
+// memory), which returns when that kernel has completed and its writes can be
+// seen; chain_next then lets the kernel behind it be placed.  As it comes after
+// the wait, a kernel that runs has only its direct predecessor in flight beside
+// it: what older kernels of the chain wrote may be read through the read-only
+// path, the direct predecessor's results may not (a plain load).  The first kernel
+// of a call is launched plainly, behind everything in its stream, and only
+// calls chain_next.
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void chain_next() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+inline cudaLaunchAttribute chained_attr(bool chained) {
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = chained ? 1 : 0;
+    return at;
+}
+// (chained false: an ordinary launch)
+template <class... P, class... A>
+cudaError_t launch_chained(bool chained, void (*kern)(P...), dim3 grid, int threads, int smem,
+                           cudaStream_t s, const A&... args) {
+    cudaLaunchAttribute at = chained_attr(chained);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
+}
+
 constexpr int kWarp = 32;
 constexpr long long kDefaultTimeoutNs = 2000000000LL;  // bounded device waits: 2 s
 constexpr int kRowsPerStrip = 30;   // rows of A per warp: lanes 0..29 (lanes 30, 31 carry
@@ -271,6 +310,7 @@ struct BtArgs {
                          // path), else null
     int transposed;      // the matrix is the transposed problem's: emit (column, row)
     int band;            // rows per band: band_rows(La, cells)
+    int chained;         // set by launch_backtrace_bands: its kernels form a chain
 };
 // Rows per band of a pair of La rows in a call over `cells` matrix cells in all:
 // the band map and the walks take time in proportion to a band's rows (~0.17 and
