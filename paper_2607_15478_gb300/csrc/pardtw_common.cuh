@@ -360,7 +360,7 @@ struct WsFrag {
 // Segment-level DP over the fragments' last rows (stride floats apart) with
 // shortest matches delta[k]; end frames, total (D_seg[N-1][Lb-1]) and status.
 // agg: seg_dp_scratch_bytes(Lb) bytes; done: two counters (zeroed here);
-// timeout_ns bounds each wait of the one-launch form.
+// timeout_ns bounds each wait of the one-grid form.
 cudaError_t launch_seg_dp(const WsFrag* fr, const float* lastrow, size_t stride, int N, int Lb,
                           const int* delta, float* Dseg, int* arg, void* agg, unsigned* done,
                           int* ends, float* total, DevCtl* ctl, long long timeout_ns,

@@ -11,6 +11,7 @@
 //                  arg[k][j]   = the first j' attaining it,
 //                as a tiled prefix scan; then the end frames
 //                e_{N-1} = arg[N-1][Lb-1], e_{k-1} = arg[k-1][e_k - delta_k].
+//   k_seg_cluster, k_seg_all   the same in one launch: in one cluster, or in one grid
 //   k_bt_subseq  step 5, one warp per fragment: the walk from (last row,
 //                e_k) back to row 0 through the fragment's backtrace matrix,
 //                written backwards into the fragment's slots of a scratch path.
@@ -358,12 +359,186 @@ __global__ void __launch_bounds__(kTile)
     }
 }
 
+// The whole segment DP in one thread-block cluster, for a B of up to 131072
+// columns: CTA r has the columns [r kCols, (r + 1) kCols) and keeps their D_seg in
+// shared memory, where the next fragment's matches read it, from the CTAs to the
+// left where delta reaches that far.  What bounds it is the chain of fragments, each
+// two exchanges long (the CTAs' minima; D_seg before fragment k+1 reads it): a
+// barrier of the grid costs a round trip through L2 and its poll, one of the cluster
+// less than half of that, and eight SMs hold the columns of a few minutes to an hour
+// of frames.  A thread loads and stores columns kSegThreads apart, and scans
+// kPer neighbouring ones (shared memory, one word of padding in 32, no bank
+// conflicts).  Same values and columns as k_seg_tile + k_seg_fix.  32 fragments x
+// 50021 columns: 140 us, 248 with k_seg_all (the whole call 4.40 -> 4.28 ms).
+constexpr int kSegThreads = 1024;
+__device__ __forceinline__ int seg_slot(int p) { return p + (p >> 5); }
+template <int kPer>
+constexpr int seg_smem() {
+    return 2 * (kSegThreads * kPer + kSegThreads * kPer / 32) * (int)sizeof(float);
+}
+
+template <int kPer>
+__global__ void __launch_bounds__(kSegThreads)
+    k_seg_cluster(const WsFrag* __restrict__ fr, const float* __restrict__ lastrow, size_t stride,
+                  int N, int Lb, const int* __restrict__ delta, int* arg, int* ends, float* total,
+                  DevCtl* ctl) {
+    constexpr int kCols = kSegThreads * kPer;
+    extern __shared__ float s_seg[];
+    float* Ds = s_seg;                              // D_seg of the fragment before
+    float* Ms = s_seg + kCols + kCols / 32;         // its matches, then its arg
+    __shared__ MinArg s_warp[kSegThreads / 32], s_cta[8];
+    __shared__ int s_bad;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const unsigned rank = cluster_rank(), cn = cluster_size();
+    const int c0 = (int)rank * kCols;
+    const unsigned ds = smem_u32(Ds);
+    // a fragment whose DP failed (a bounded wait expired) fails the call
+    if (rank == 0) {
+        if (tid == 0) s_bad = N;
+        __syncthreads();
+        for (int q = tid; q < N; q += kSegThreads)
+            if (fr[q].pctl->status != 0) atomicMin(&s_bad, q);
+        __syncthreads();
+        if (tid == 0 && s_bad < N) raise_status(ctl, fr[s_bad].pctl->status, 20);
+    }
+    float cs[kPer];  // C_seg of fragment k at columns c0 + tid + i kSegThreads
+    auto load = [&](int k) {
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int col = c0 + tid + i * kSegThreads;
+            cs[i] = col < Lb ? lastrow[(size_t)k * stride + col] : INFINITY;
+        }
+    };
+    load(0);
+    for (int k = 0; k < N; ++k) {
+        const int dk = k > 0 ? delta[k] : 0;
+        float m[kPer];
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int src = c0 + tid + i * kSegThreads - dk;
+            m[i] = k == 0 ? 0.f : INFINITY;
+            if (k > 0 && src >= 0)
+                m[i] = ld_cluster_f32(map_rank(ds + 4u * (unsigned)seg_slot(src % kCols), src / kCols));
+        }
+#pragma unroll
+        for (int i = 0; i < kPer; ++i)
+            Ms[seg_slot(tid + i * kSegThreads)] = k == 0 ? cs[i] : m[i] + cs[i];
+        if (k + 1 < N) load(k + 1);
+        __syncthreads();
+        // the minimum of the thread's columns, of the lanes and warps before it
+        MinArg x{INFINITY, -1};
+#pragma unroll
+        for (int i = 0; i < kPer; ++i)
+            x = better(x, MinArg{Ms[seg_slot(tid * kPer + i)], c0 + tid * kPer + i});
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            MinArg o;
+            o.v = __shfl_up_sync(0xffffffffu, x.v, off);
+            o.j = __shfl_up_sync(0xffffffffu, x.j, off);
+            if (lane >= off) x = better(o, x);
+        }
+        if (lane == 31) s_warp[w] = x;
+        MinArg run;
+        run.v = __shfl_up_sync(0xffffffffu, x.v, 1);
+        run.j = __shfl_up_sync(0xffffffffu, x.j, 1);
+        if (lane == 0) run = MinArg{INFINITY, -1};
+        __syncthreads();
+        MinArg c = lane < w ? s_warp[lane] : MinArg{INFINITY, -1};
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            MinArg o;
+            o.v = __shfl_xor_sync(0xffffffffu, c.v, off);
+            o.j = __shfl_xor_sync(0xffffffffu, c.j, off);
+            c = lex_min(c, o);
+        }
+        if (w == kSegThreads / 32 - 1) {  // the CTA's minimum, to every CTA
+            const MinArg all = better(c, s_warp[w]);
+            if (lane < (int)cn) {
+                const unsigned at = map_rank(smem_u32(&s_cta[rank]), (unsigned)lane);
+                st_cluster_u32(at, __float_as_uint(all.v));
+                st_cluster_u32(at + 4, (unsigned)all.j);
+            }
+        }
+        run = better(c, run);
+        cluster_sync_all();
+        c = MinArg{INFINITY, -1};
+        for (unsigned r = 0; r < rank; ++r) c = better(c, s_cta[r]);
+        run = better(c, run);
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int p = seg_slot(tid * kPer + i);
+            run = better(run, MinArg{Ms[p], c0 + tid * kPer + i});
+            Ds[p] = run.v;
+            Ms[p] = __int_as_float(run.j);
+        }
+        cluster_sync_all();
+        // (the same thread stores the next fragment's matches there)
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int p = tid + i * kSegThreads;
+            if (c0 + p < Lb) arg[(size_t)k * Lb + c0 + p] = __float_as_int(Ms[seg_slot(p)]);
+        }
+    }
+    // the last fragment's last column: the total and the end frames
+    const int last = Lb - 1 - c0;
+    if (tid == 0 && last >= 0 && last < kCols) {
+        if (read_status(ctl) != 0) return;
+        const float v = Ds[seg_slot(last)];
+        if (!(v < INFINITY)) {
+            raise_status(ctl, DTW_ERR_UNREACHABLE, 21);
+            return;
+        }
+        *total = v;
+        int e = __float_as_int(Ms[seg_slot(last)]);
+        ends[N - 1] = e;
+        for (int q = N - 1; q > 0; --q) {
+            e = __ldcg(arg + (size_t)(q - 1) * Lb + (e - delta[q]));
+            ends[q - 1] = e;
+        }
+    }
+}
+
+template <int kPer>
+cudaError_t launch_seg_cluster(const WsFrag* fr, const float* lastrow, size_t stride, int N, int Lb,
+                               const int* delta, int* arg, int* ends, float* total, DevCtl* ctl,
+                               cudaStream_t s) {
+    static DeviceSlots done;
+    cudaError_t e = raise_smem_once(k_seg_cluster<kPer>, seg_smem<kPer>(), done);
+    if (e != cudaSuccess) return e;
+    const int cn = (Lb + kSegThreads * kPer - 1) / (kSegThreads * kPer);
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)cn;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)cn);
+    cfg.blockDim = dim3(kSegThreads);
+    cfg.dynamicSmemBytes = (size_t)seg_smem<kPer>();
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_seg_cluster<kPer>, fr, lastrow, stride, N, Lb, delta, arg,
+                              ends, total, ctl);
+}
+
 cudaError_t launch_seg_dp(const WsFrag* fr, const float* lastrow, size_t stride, int N, int Lb,
                           const int* delta, float* Dseg, int* arg, void* agg, unsigned* done,
                           int* ends, float* total, DevCtl* ctl, long long timeout_ns,
                           cudaStream_t s) {
+    // one cluster where its eight CTAs hold the columns (131072 of them)
+    cudaError_t e = cudaErrorInvalidValue;
+    const int per = (Lb + 8 * kSegThreads - 1) / (8 * kSegThreads);
+    if (per <= 4)
+        e = launch_seg_cluster<4>(fr, lastrow, stride, N, Lb, delta, arg, ends, total, ctl, s);
+    else if (per <= 8)
+        e = launch_seg_cluster<8>(fr, lastrow, stride, N, Lb, delta, arg, ends, total, ctl, s);
+    else if (per <= 16)
+        e = launch_seg_cluster<16>(fr, lastrow, stride, N, Lb, delta, arg, ends, total, ctl, s);
+    if (e == cudaSuccess) return e;
+    (void)cudaGetLastError();
     const int ntile = (Lb + kTile - 1) / kTile;
-    cudaError_t e = cudaMemsetAsync(done, 0, 2 * sizeof(unsigned), s);
+    e = cudaMemsetAsync(done, 0, 2 * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     // one cooperative launch when every tile's CTA can be resident at once
     // (CTAs resident on the current device, looked up once per device)
