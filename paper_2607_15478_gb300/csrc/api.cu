@@ -86,7 +86,7 @@ bool reachable(int La, int Lb) {
 struct Layout {
     DpPlan plan;
     int dp, R, rps, wpb, nstrips, nchunk, ngroups, La_pad, cap;
-    size_t off_ctl, off_ahat, off_bhat, off_bbf, off_bp, off_bt, off_bt_end, off_stage_a,
+    size_t off_ctl, off_ahat, off_bhat, off_bbf, off_bp, off_bt, off_stage_a,
         off_stage_b, total;
     size_t border_bytes;
 };
@@ -153,7 +153,7 @@ bool pardtw::transpose_pair(int La, int Lb, int dp, const dtw_options& o, int nu
 
 namespace {
 
-Layout make_layout(int La, int Lb, int D, const DpPlan& plan) {
+Layout make_layout(int La, int Lb, int D, const DpPlan& plan, bool staged = true) {
     Layout L;
     L.plan = plan;
     // the BF16 cost runs its tensor-core products over 64 or 128 features
@@ -176,17 +176,20 @@ Layout make_layout(int La, int Lb, int D, const DpPlan& plan) {
     o = align256(o + (size_t)L.nchunk * kColsPerWord * L.dp * sizeof(float));
     L.off_bbf = o;
     if (plan.bf16) o = align256(o + (size_t)L.nchunk * kColsPerWord * kBfStride * 2);
+    // host inputs are staged behind them (one pair; a batch's are on the device)
+    L.off_stage_a = o;
+    if (staged) o = align256(o + (size_t)La * D * sizeof(float));
+    L.off_stage_b = o;
+    if (staged) o = align256(o + (size_t)Lb * D * sizeof(float));
+    // the backtrace's scratch lies where the normalised and staged sequences do:
+    // the DP, which reads them last, has finished when it is first written (a
+    // workspace of less than 1 MB shares its mapping with others: 1000 x 1200 frames,
+    // 1.07 to 0.97 MB)
+    L.off_bt = L.off_ahat;
+    o = std::max(o, align256(L.off_bt + bandmap_scratch_bytes(La, Lb)));
     L.off_bp = o;
     o = align256(o + (size_t)L.nstrips * L.nchunk * L.wpb * sizeof(uint32_t));
-    L.off_bt = o;
-    L.off_bt_end = align256(o + bandmap_scratch_bytes(La, Lb));
-    // host inputs are staged where the backtrace's scratch lies: they have been
-    // read when it is first written
-    L.off_stage_a = o;
-    o = align256(o + (size_t)La * D * sizeof(float));
-    L.off_stage_b = o;
-    o = align256(o + (size_t)Lb * D * sizeof(float));
-    L.total = std::max(o, L.off_bt_end);
+    L.total = o;
     L.border_bytes = (size_t)L.ngroups * Lb * 2 * sizeof(unsigned long long);
     return L;
 }
@@ -446,7 +449,7 @@ BatchSetup batch_setup(std::vector<int> idx, const int* La, const int* Lb, int D
     b.Ls.resize(m);
     b.off.resize(m);
     b.boff.resize(m);
-    for (int q = 0; q < m; ++q) b.Ls[q] = make_layout(La[idx[q]], Lb[idx[q]], D, plan);
+    for (int q = 0; q < m; ++q) b.Ls[q] = make_layout(La[idx[q]], Lb[idx[q]], D, plan, false);
     b.queue = batch_queue(b.Ls, idx, La, Lb, subseq);
     size_t o0 = 0;
     b.off_dp = o0;
@@ -464,7 +467,7 @@ BatchSetup batch_setup(std::vector<int> idx, const int* La, const int* Lb, int D
         const int k = idx[q];
         const Layout& L = b.Ls[q];
         b.off[q] = o0;
-        o0 = align256(o0 + (L.off_bt_end - L.off_ahat));  // Ahat, Bhat, bp, band maps
+        o0 = align256(o0 + (L.total - L.off_ahat));  // Ahat, Bhat (band maps), bp
         b.boff[q] = border_total;
         border_total += L.border_bytes;
         b.maxLb = std::max(b.maxLb, Lb[k]);
