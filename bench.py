@@ -47,23 +47,39 @@ L2_FLUSH_BYTES = 512 << 20
 
 def backtrace_kernels(rows):
     """Launches of the parallel backtrace of a sweep with `rows` rows: band
-    map, two-band map (at least 4 bands of 128 rows), four-band map (at least
-    6), chain, walks, emission.  Every workload here has at least 768 frames on
-    each side, so both sweep directions give the same count."""
+    map, two-band map (at least 4 bands of at most 128 rows), four-band map (at
+    least 6), chain, walks, emission.  Every workload here has at least 768
+    frames on each side, so both sweep directions give the same count."""
     nb = -(-rows // 128)
     return 4 + (nb >= 4) + (nb >= 6)
 
 
+def swept_cells(La, Lb):
+    """Cells that the DP of one pair computes: per strip of 93 rows (along the
+    longer sequence) the columns that a path can cross there, in words of 16.
+    The others (about two thirds of a square matrix) hold no path."""
+    rows, cols = max(La, Lb), min(La, Lb)
+    total = 0
+    for r0 in range(0, rows, 93):
+        r1 = min(r0 + 93, rows) - 1
+        lo = max((r0 + 1) // 2, cols - 1 - 2 * (rows - 1 - r0))
+        hi = min(2 * r1, cols - 1 - (rows - r1) // 2)
+        x = max(lo - 2, 0) // 16 * 16
+        y = min((max(hi, 0) // 8 + 1) * 8, cols)
+        total += (r1 - r0 + 1) * max(y - x, 0)
+    return total
+
+
 # normalise, DP, backtrace
 KERNELS_PER_STEP = 2 + backtrace_kernels(20000)
-# learned band: 2 x (pool, 3 convolutions, heads), coarse alignment of the
-# 8x pooled sequences (normalise, DP, backtrace), band ranges (2), banded
+# learned band: pool, 3 convolutions, heads (both sequences in each launch), coarse
+# alignment of the 8x pooled sequences (normalise, DP, backtrace), band ranges (2), banded
 # alignment (normalise, DP, backtrace), band-side test (1)
-KERNELS_PER_LEARNED_STEP = 10 + (2 + backtrace_kernels(100000 // 8)) + 2 + (2 + backtrace_kernels(100000)) + 1
-# WSDTW: batched normalisation, subsequence DP, segment DP (one cooperative
-# launch while every column tile's CTA fits on the GPU at once, as at this
-# size; else a tile pass and a fix-up pass per fragment), fragment
-# backtraces, compaction
+KERNELS_PER_LEARNED_STEP = 5 + (2 + backtrace_kernels(100000 // 8)) + 2 + (2 + backtrace_kernels(100000)) + 1
+# WSDTW: batched normalisation, subsequence DP, segment DP (one launch, in one
+# cluster up to 131072 columns, else in one grid while every column tile's CTA
+# fits on the GPU at once; else a tile pass and a fix-up pass per fragment),
+# fragment backtraces, compaction
 def kernels_per_wsdtw_step(nfrag, Lb):
     return 5 if (Lb + 1023) // 1024 <= 2 * SM_COUNT else 4 + 2 * nfrag
 SM_COUNT = 152
@@ -399,7 +415,8 @@ def run_ours(args):
             pclk.mark_end()
         ops_per_cell = D + 6
         dp_avg = statistics.mean(dp_ms) / 1e3
-        achieved = cells * ops_per_cell / dp_avg
+        swept = swept_cells(La, Lb)
+        achieved = swept * ops_per_cell / dp_avg
         traffic = dp_traffic_from_profiles()
         cpu = None
         if not args.no_cpu_baseline:
@@ -417,12 +434,16 @@ def run_ours(args):
             "data": "synthetic",
             "config": {"workload": workload_name(La, Lb), "La": La, "Lb": Lb, "D": D,
                        "l2": "flushed between steps (512 MiB write)",
+                       "value_definition": "La x Lb cells over the step time; the DP computes "
+                                           "cells_swept of them (no path crosses the others)",
+                       "cells_swept": swept,
                        "parallelism": "replicas" if ws > 1 else "single GPU"},
             "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12,
                          "unit": "T FP32 lane-ops/s", "frac": achieved / peak_ops,
+                         "basis": "cells_swept",
                          "traffic": traffic,
-                         "kernel": "k_dp_split (column-sweep DP: per strip a cost warp and a DP "
-                                   "warp, cost on the fly; thread-block clusters, the strip "
+                         "kernel": "k_dp_split (column-sweep DP: per strip two cost warps and a "
+                                   "DP warp, cost on the fly; thread-block clusters, the strip "
                                    "border between CTAs of a cluster in distributed shared "
                                    "memory)",
                          "ops_per_cell": ops_per_cell, "dp_ms": 1e3 * dp_avg,
@@ -503,7 +524,7 @@ def measure_cost(dev, steps, warmup):
         "bytes_written": written, "gbs": gbs, "peak_gbs": peaks["hbm_gbs"],
         "frac_of_hbm": gbs / peaks["hbm_gbs"],
         "peak_basis": f"HBM copy bandwidth ({basis})",
-        "kernels": "k_normalise + k_cost (4 x 4 cells a thread, b^ of its 4 columns in registers over its row tiles, one 16-byte store per row of 4)",
+        "kernels": "k_normalise + k_cost (4 x 4 cells a thread, columns 32 apart, b^ of its 4 columns in registers over its row tiles)",
         "timing": "CUDA events on the aligner's stream, device buffers",
     }
     del C
@@ -822,7 +843,8 @@ def run_batch(args):
         peaks, src = measured_peaks()
         peak_ops, basis = nominal_peak(peaks, src)
         dp_avg = statistics.mean(ex["dp_ms"]) / 1e3
-        achieved = cells * 18 / dp_avg
+        swept = sum(swept_cells(p.A.shape[0], p.B.shape[0]) for p in pairs)
+        achieved = swept * 18 / dp_avg
         cpu = None
         if not args.no_cpu_baseline:
             import oracle
@@ -859,7 +881,8 @@ def run_batch(args):
                          "traffic": None,
                          "kernel": "k_dp_split, batch mode (work queue over pairs), timed "
                                    "through dtw_align_many",
-                         "ops_per_cell": 18, "dp_ms": 1e3 * dp_avg, "peak_basis": basis},
+                         "ops_per_cell": 18, "cells_swept": swept, "dp_ms": 1e3 * dp_avg,
+                         "peak_basis": basis},
             "cpu_baseline": cpu,
             "e2e": {"value": sum(cells_all) * args.steps / t_e2e / 1e9, "unit": UNIT,
                     "h2d_bytes_per_step": ex["h2d"], "d2h_bytes_per_step": ex["d2h"]},
@@ -904,7 +927,7 @@ def run_precision(args):
     t_e2e = sum(e2e_t[args.warmup:])
     peaks, src = measured_peaks()
     dp_avg = statistics.mean(ex["dp_ms"]) / 1e3
-    tflops = cells * 2 * 128 / dp_avg / 1e12
+    tflops = swept_cells(La, Lb) * 2 * 128 / dp_avg / 1e12
     peak_tf = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops", 1900.0))
     _rank0_line({
         "metric": METRIC, "value": cells * args.steps / t / 1e9, "unit": UNIT, "n_gpus": 1,
@@ -918,14 +941,14 @@ def run_precision(args):
                      "unit": "TFLOP/s", "frac": tflops / peak_tf, "traffic": None,
                      "kernel": "k_dp_split BF16 (cost warps: mma.sync m16n8k16; DP warps FP32)",
                      "dp_ms": 1e3 * dp_avg,
-                     "note": "cost contraction flops (2 x 128 per cell) over the DP launch; the "
+                     "note": "cost contraction flops (2 x 128 per swept cell) over the DP launch; the "
                              "launch is bound by the DP recurrence, not the tensor pipe"},
         "bf16": block,
         "cpu_baseline": None,
         "e2e": {"value": cells * args.steps / t_e2e / 1e9, "unit": UNIT,
                 "h2d_bytes_per_step": (La + Lb) * D * 4, "d2h_bytes_per_step": cap * 8 + 8},
-        # normalisation, bf16 packing of B, DP, backtrace
-        "gpu_launches": (3 + backtrace_kernels(min(La, Lb))) * args.steps,
+        # normalisation (with the bf16 rows of B), DP, backtrace
+        "gpu_launches": (2 + backtrace_kernels(min(La, Lb))) * args.steps,
         "clocks": ex["clocks"],
     })
     al.close()

@@ -108,13 +108,11 @@ DpPlan pardtw::choose_plan(int La, int dp, const dtw_options& o, int num_sms) {
         return one;
     }
     const int R = req == 0 ? 3 : req;
-    // D = 64, 128: the warp pairs with two cost warps per strip, 3 rows per lane
+    // D = 64, 128: several cost warps per strip, 3 rows per lane
     if (split_wide_supported(dp)) return R == 3 ? DpPlan{2, 3, kSplitStrips, 0, nocl} : one;
     if (!split_supported(dp, R)) return one;
-    // two strips per CTA unless asked for four: with the DP warp's costs
-    // loaded at the start of each sub-chunk, two beat four on single pairs
-    // of every size measured (1e5 x 1.26e5: 30.3 vs 31.5 ms; 5e4 x 6.25e4:
-    // 8.32 vs 8.45 ms); batches pick theirs with the autotuner
+    // two strips per CTA (in clusters, or one: launch_dp_split_cl) unless asked
+    // for four; batches pick theirs with the autotuner
     if (o.strips_per_cta == 4 && split_supported(dp, R, 4)) return {2, R, 4};
     return {2, R, kSplitStrips, 0, nocl};
 }

@@ -1,7 +1,8 @@
 // Warp-pair DP with two strips per CTA (k_dp_split<..., NS = 2, ...>, see
 // dp_split.cuh): each DP warp has an SM sub-partition of its own, which keeps
-// the per-column step of a strip short; the choice for a chain of strips
-// that does not fill the GPU (one pair of up to ~2 x 152 strips, a band).
+// the per-column step of a strip short; the choice for
+// single pairs without clusters, for batches at D > 16 and for the fragments of a
+// segmental alignment.
 #include "dp_split.cuh"
 
 namespace pardtw {

@@ -289,7 +289,7 @@ __device__ __forceinline__ void run_cost(const DpArgs& p, int strip, int half, i
 // 8 columns, C' = (1 - mu) - a^_i . b^_j with one FMA per feature in feature
 // order (the values of every other decomposition).  A^ of the strip comes
 // from the A tile in shared memory (`tile`, 32 R rows of kStride floats),
-// which the two cost warps of the strip load together at the strip's start
+// which the cost warps of the strip load together at the strip's start
 // (named barrier 1 + w), and is reused for 8 columns per load; B^ from the
 // warp's own ring of two 16-frame chunks in shared memory, filled by bulk
 // copies one chunk ahead (B^ through L1 instead ran at L2 latency, ~1100

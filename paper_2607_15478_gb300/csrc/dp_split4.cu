@@ -1,7 +1,7 @@
 // Warp-pair DP with four strips per CTA (k_dp_split<..., NS = 4, ...>, see
 // dp_split.cuh): ten warps, one DP warp and one cost warp on every SM
 // sub-partition, twice the DP warps of the two-strip CTA per SM.  The choice
-// when there are more strip groups than SMs (a long pair, a batch): the
+// for batches at D <= 16, unless a plan measures two to be faster: the
 // per-column step of a strip is longer (the DP warp shares its
 // sub-partition) but twice as many strips advance at once, and three of four
 // strip-to-strip handoffs stay in shared memory.  Register budget: at ten
