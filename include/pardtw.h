@@ -81,7 +81,7 @@ typedef struct dtw_options {
     int debug_skip_publish;
     /* Rows of A each GPU lane sweeps (1, 2, 3 or 4); 0 = chosen from La, D
      * and the SM count.  Results do not depend on it (it only changes the
-     * work decomposition); 32 < D <= 128 runs with 3 (two cost warps per
+     * work decomposition); 32 < D <= 128 runs with 3 (several cost warps per
      * strip) or 1, and a value the chosen schedule does not support falls
      * back to 1. */
     int rows_per_lane;
@@ -91,22 +91,20 @@ typedef struct dtw_options {
      * or DTW_SCHEDULE_SPLIT (2: a cost warp and a DP warp per strip;
      * rows_per_lane 2, 3 or 4).  Results do not depend on it. */
     int dp_schedule;
-    /* Strips per CTA of the cost/DP warp-pair DP: 0 (default: four when a
-     * pair has more two-strip groups than the GPU has SMs and the kernel has
-     * the four-strip form for D and rows_per_lane, else two), 2 or 4 (D <= 16,
-     * rows_per_lane 2 or 3; else two).  Results do not depend on it. */
+    /* Strips per CTA of the cost/DP warp-pair DP: 0 (default: a single pair two,
+     * or one in clusters at D > 16 and with the BF16 cost; dtw_align_many four
+     * where the kernel has that form), 2 or 4 (D <= 16, rows_per_lane 2 or 3;
+     * else two).  Results do not depend on it. */
     int strips_per_cta;
     /* DTW_TRANSPOSE_AUTO (0, default): the DP sweeps the transposed pair
-     * (B's frames as rows) when a model of the sweep's time (waves of strip
-     * groups x columns + the chain of strips) says it is faster, e.g. a pair
-     * with B longer that fits one wave of strip groups; DTW_TRANSPOSE_NEVER
-     * (1); DTW_TRANSPOSE_ALWAYS (2).
+     * (B's frames as rows) when B is longer than A, so that the sweep runs along
+     * the shorter sequence (20000 x 25000: 20000 columns instead of 25000);
+     * DTW_TRANSPOSE_NEVER (1); DTW_TRANSPOSE_ALWAYS (2).
      * Applies to the default warp-pair DP at 3 rows per lane (FP32 or BF16
      * cost); the tie order is mapped so that results do not depend on it. */
     int transpose;
     /* DTW_CLUSTERS_AUTO (0, default): the default DP of one pair (warp pairs
-     * at 3 rows per lane, two strips per CTA) runs in thread-block clusters
-     * of up to 8 CTAs, which hand the strip border from CTA to CTA through
+     * at 3 rows per lane) runs in persistent thread-block clusters of 2 to 8 CTAs, which hand the strip border from CTA to CTA through
      * distributed shared memory instead of global memory, when the device
      * has room for them; DTW_CLUSTERS_NEVER (1): never.  Results do not
      * depend on it. */

@@ -87,12 +87,14 @@ constexpr int kBfBlkBytes = kColsPerWord * kBfStride * 2;
 // With two strips a CTA: two (two strips beside each other at D = 12: 83 cycles a
 // column, 126 with a third one, which shares the DP warp's SM sub-partition; 139
 // against 162 with two CTAs an SM; D = 16: 88 and 89), at D = 32 three (122, 151
-// with two).
+// with two).  With one strip, six of the wide ones, which wait for their own loads
+// and FMAs (24001 x 27011, D = 100: 3.58 ms with four, 2.69 with six, 2.77 with eight),
+// and three otherwise (40000 x 48000 with the BF16 cost: 2.78, 2.77 with four).
 template <int DP, int NS, bool kBF>
 struct CostCfg {
     static constexpr bool kWide = DP > 32 && !kBF;
     // cost warps a strip
-    static constexpr int kNC = kWide           ? (NS == 1 ? 4 : 2)
+    static constexpr int kNC = kWide           ? (NS == 1 ? 6 : 2)
                                : NS == 1       ? 3
                                : kBF || NS > 2 ? 1
                                : DP > 16       ? 3
