@@ -319,6 +319,7 @@ int align_device(dtw_handle* h, const float* A, int La, const float* B, int Lb, 
     a.rps = L.rps;
     a.wpb = L.wpb;
     a.mu = o.cost_shift;
+    a.feats = D;
     a.kcost = 1.0f - o.cost_shift;
     a.epoch = ++h->epoch;
     if (a.epoch == 0) a.epoch = ++h->epoch;
@@ -545,6 +546,7 @@ BatchDesc batch_descriptors(const BatchSetup& b, char* ws, unsigned long long* b
         a.rps = L.rps;
         a.wpb = L.wpb;
         a.mu = o.cost_shift;
+        a.feats = b.D;
         a.kcost = 1.0f - o.cost_shift;
         a.epoch = epoch;
         a.timeout_ns = o.wait_limit > 0 ? (long long)o.wait_limit * 1000LL : kDefaultTimeoutNs;

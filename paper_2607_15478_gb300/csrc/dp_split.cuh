@@ -249,6 +249,11 @@ __device__ __forceinline__ void run_cost(const DpArgs& p, int strip, int half, i
         }
 #pragma unroll
         for (int gi = 0; gi < kNG; ++gi) {
+            // D = 17 .. 20: the groups beyond are zero in both frames, and an FMA with a
+            // zero product leaves every bit of the sum (48 pairs of up to 2500 frames at
+            // D = 20: DP 204 us, 181 so).  One test: one per group costs D = 32 more (3%);
+            // with one strip a CTA the cost warps don't set the pace (D = 32 would lose 1%)
+            if (DP > 16 && NS > 1 && gi == 5 && p.feats <= gi * kFG) break;
             if (gi + 1 < kNG) {
 #pragma unroll
                 for (int e = 0; e < kFG; ++e) {
@@ -331,6 +336,10 @@ __device__ __forceinline__ void run_cost_wide(const DpArgs& p, int strip, int w,
     // this warp's sub-chunks n0, n0 + kNC, ...: one in every kNC / 2 chunks of B
     // (kNC is even), which are the blocks 0, 1, ... of its ring
     static_assert(W::kNC % 2 == 0, "a warp keeps to one half of its chunks");
+    // groups of 4 features, in whole trips of four: beyond them both frames are
+    // zero, and an FMA with a zero product leaves every bit of the sum (24001 x 27011 at
+    // D = 100: 2.69 ms, 2.51 so)
+    const int ng = min((p.feats + 15) / 16 * 4, DP / 4);
     const int n0 = rg.x + half;
     br.stride = W::kNC / 2;
     br.off = n0 / 2;
@@ -388,14 +397,14 @@ __device__ __forceinline__ void run_cost_wide(const DpArgs& p, int strip, int w,
         static_assert((DP / 4) % 4 == 0, "whole trips of four feature groups");
         load(0, a0, b0);
 #pragma unroll 1
-        for (int g = 0; g < DP / 4; g += 4) {
+        for (int g = 0; g < ng; g += 4) {
             load(g + 1, a1, b1);
             fmas(a0, b0);
             load(g + 2, a0, b0);
             fmas(a1, b1);
             load(g + 3, a1, b1);
             fmas(a0, b0);
-            if (g + 4 < DP / 4) load(g + 4, a0, b0);
+            if (g + 4 < ng) load(g + 4, a0, b0);
             fmas(a1, b1);
         }
         const unsigned sbase = cring + slot * CR::kSlotBytes;

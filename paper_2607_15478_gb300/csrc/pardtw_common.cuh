@@ -147,6 +147,7 @@ struct DpArgs {
     unsigned epoch;                 // call tag for global border entries
     long long timeout_ns;
     int skip_publish;               // group that never publishes (fault injection), -1 off
+    int feats;                      // features of a frame; those up to the padded width are zero
     const int2* ranges;             // banded DP (warp-pair kernel): per strip the sub-chunks
                                     // [x, y) of 8 columns it sweeps (x even; x and y
                                     // non-decreasing in the strip); null = every column

@@ -165,6 +165,7 @@ extern "C" int dtw_align_static(const float* A, int La, const float* B, int Lb, 
     a.rps = rps;
     a.wpb = wpb;
     a.mu = o.cost_shift;
+    a.feats = D;
     a.kcost = 1.0f - o.cost_shift;
     a.epoch = 1u;
     a.timeout_ns = o.wait_limit > 0 ? (long long)o.wait_limit * 1000LL : kDefaultTimeoutNs;
