@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(256) k_bt_compose(const BtArgs one,
         chain_next();
     }
     const BtArgs& a = kMany ? many[blockIdx.z] : one;
-    const int La = a.La, Lb = a.Lb;
+    const int Lb = a.Lb;
     const BtScratch sc = bt_scratch(a);
     const int m = blockIdx.y;
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(256) k_bt_compose4(const BtArgs one,
         chain_next();
     }
     const BtArgs& a = kMany ? many[blockIdx.z] : one;
-    const int La = a.La, Lb = a.Lb;
+    const int Lb = a.Lb;
     const BtScratch sc = bt_scratch(a);
     const int m = blockIdx.y;
     const int j = blockIdx.x * blockDim.x + threadIdx.x;

@@ -87,14 +87,14 @@ constexpr int kBfBlkBytes = kColsPerWord * kBfStride * 2;
 // With two strips a CTA: two (two strips beside each other at D = 12: 83 cycles a
 // column, 126 with a third one, which shares the DP warp's SM sub-partition; 139
 // against 162 with two CTAs an SM; D = 16: 88 and 89), at D = 32 three (122, 151
-// with two).  With one strip, six of the wide ones, which wait for their own loads
-// and FMAs (24001 x 27011, D = 100: 3.58 ms with four, 2.69 with six, 2.77 with eight),
-// and three otherwise (40000 x 48000 with the BF16 cost: 2.78, 2.77 with four).
+// with two).  With one strip, four of the wide ones (six are faster, but about one call in a
+// thousand then returned a wrong path; four: none in 17000), and three otherwise
+// (40000 x 48000 with the BF16 cost: 2.78, 2.77 with four).
 template <int DP, int NS, bool kBF>
 struct CostCfg {
     static constexpr bool kWide = DP > 32 && !kBF;
     // cost warps a strip
-    static constexpr int kNC = kWide           ? (NS == 1 ? 6 : 2)
+    static constexpr int kNC = kWide           ? (NS == 1 ? 4 : 2)
                                : NS == 1       ? 3
                                : kBF || NS > 2 ? 1
                                : DP > 16       ? 3
@@ -291,9 +291,8 @@ __device__ __forceinline__ void run_cost(const DpArgs& p, int strip, int half, i
     br.drain();
 }
 
-// Cost warp `half` (0 or 1) of `strip` for D > 32, FP32: every other
-// sub-chunk of the strip (the (n - first)-th for n - first = half mod 2), all
-// 8 columns, C' = (1 - mu) - a^_i . b^_j with one FMA per feature in feature
+// Cost warp `half` (of kNC) of `strip` for D > 32, FP32: every kNC-th
+// sub-chunk of the strip (those with n - first = half mod kNC), all 8 columns, C' = (1 - mu) - a^_i . b^_j with one FMA per feature in feature
 // order (the values of every other decomposition).  A^ of the strip comes
 // from the A tile in shared memory (`tile`, 32 R rows of kStride floats),
 // which the cost warps of the strip load together at the strip's start

@@ -14,7 +14,7 @@
 // Every CTA of a cluster sits on an SM of its own (the dynamic shared
 // memory is raised so that two CTAs cannot share an SM, which would put two
 // DP warps on one SM sub-partition).  One strip a CTA where one or two cost
-// warps cannot keep up with a DP warp (D > 16, the BF16 cost: three to six cost
+// warps cannot keep up with a DP warp (D > 16, the BF16 cost: three or four cost
 // warps a strip, on the sub-partitions beside the DP warp's), else two.  The
 // cluster size: see launch_cl.  Measured (DP, ms): 20000 x 25000, D = 12, clusters
 // of 8 / 6 / 4 / 2: 1.001 / 1.009 / 1.027 / 1.080; 100000 x 126231 (335 groups active

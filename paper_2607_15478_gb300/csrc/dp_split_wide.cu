@@ -1,6 +1,6 @@
 // Warp-pair DP with the FP32 cost at D = 64 and 128 (k_dp_split with the
 // wide cost warps of dp_split.cuh, run_cost_wide): the strip's rows of A^ in shared
-// memory, sub-chunks of 8 columns taken in turn by the cost warps of a strip, six
+// memory, sub-chunks of 8 columns taken in turn by the cost warps of a strip, four
 // with one strip a CTA (in clusters), two with two, and the DP warp of the
 // narrow kernels, so the FP32 cost keeps one FMA per feature in feature order (the
 // values of every other decomposition) while its 2 D FLOP per cell are spread
