@@ -337,7 +337,7 @@ __device__ __forceinline__ void run_cost_wide(const DpArgs& p, int strip, int w,
     static_assert(W::kNC % 2 == 0, "a warp keeps to one half of its chunks");
     // groups of 4 features, in whole trips of four: beyond them both frames are
     // zero, and an FMA with a zero product leaves every bit of the sum (24001 x 27011 at
-    // D = 100: 2.69 ms, 2.51 so)
+    // D = 100: 3.58 ms, 3.26 so)
     const int ng = min((p.feats + 15) / 16 * 4, DP / 4);
     const int n0 = rg.x + half;
     br.stride = W::kNC / 2;
