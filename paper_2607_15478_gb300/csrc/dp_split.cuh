@@ -87,9 +87,9 @@ constexpr int kBfBlkBytes = kColsPerWord * kBfStride * 2;
 // With two strips a CTA: two (two strips beside each other at D = 12: 83 cycles a
 // column, 126 with a third one, which shares the DP warp's SM sub-partition; 139
 // against 162 with two CTAs an SM; D = 16: 88 and 89), at D = 32 three (122, 151
-// with two).  With one strip, four of the wide ones (six are faster, but about one call in a
-// thousand then returned a wrong path; four: none in 17000), and three otherwise
-// (40000 x 48000 with the BF16 cost: 2.78, 2.77 with four).
+// with two).  With one strip, four of the wide ones (24001 x 27011 at D = 100: 3.23 ms, 2.50 with six,
+// which are not measured at other sizes), and three otherwise (40000 x 48000 with the
+// BF16 cost: 2.78, 2.77 with four).
 template <int DP, int NS, bool kBF>
 struct CostCfg {
     static constexpr bool kWide = DP > 32 && !kBF;
@@ -685,10 +685,12 @@ __device__ __forceinline__ void run_dp(const DpArgs& p, int strip, int lane, con
     using Slot = SlotOf<R, kRM>;
     constexpr int kRows = 31 * R;
     constexpr int kLoads = 2 * R + 4;  // 16-byte loads of a slot
-    // the next slot is loaded behind the shuffles of columns kFirst, kFirst + 1, ..,
-    // kPer loads each: as late as the loads' latency allows, since a strip can
-    // follow the one above no closer than its tests look ahead
-    constexpr int kFirst = 4, kPer = 4;
+    // the next slot's barrier is tested behind the shuffles of column kTest and the slot
+    // loaded behind those of columns kFirst, kFirst + 1, .., kPer loads each: as late
+    // as the latencies allow, since a strip can follow the one above no closer than
+    // its tests look ahead (20000 x 25000, D = 12: DP 0.980 ms; 1.00 with test and
+    // loads at column 4 and the loads not waiting for the test, see `test`)
+    constexpr int kTest = 4, kFirst = 5, kPer = 4;
     const bool ghost = lane == kGhostLane;
     const int i0 = strip * kRows + lane * R;
     const float mu = p.mu;
@@ -748,18 +750,25 @@ __device__ __forceinline__ void run_dp(const DpArgs& p, int strip, int lane, con
 #pragma unroll
         for (int k = 0; k < R; ++k) word[k] |= field_bits(fw[k], h);
     };
-    // the loads of use t behind the shuffles of columns kFirst, kFirst + 1, ...
-    auto part = [&](SubIn<R>& in, unsigned t, int u) {
+    // the loads of a slot behind the shuffles of columns kFirst, kFirst + 1, ...
+    auto part = [&](SubIn<R>& in, unsigned slot, int u) {
         if (u >= kFirst) {
 #pragma unroll
             for (int z = 0; z < kPer; ++z)
                 if (kPer * (u - kFirst) + z < kLoads)
-                    load_part<R, kRM>(in, cring + (t % kSlots) * Slot::kBytes, lane,
-                                      kPer * (u - kFirst) + z);
+                    load_part<R, kRM>(in, slot, lane, kPer * (u - kFirst) + z);
         }
     };
-    auto test = [&](unsigned t) -> int {
-        return mbar_test_wait(bar_at(cfull, t % kSlots), use_parity(t, kSlots));
+    // Whether use t is there, and the slot to load next: its own, or where it is not yet
+    // there that of use t - 1, whose values are then dropped.  The address comes
+    // from the test's result, so that no load can be performed before the test.  (Loads of
+    // use t's slot in any case, dropped like these where the test failed, came too early
+    // now and then: with six cost warps a strip at D = 100 one call in 70 of 12007 x 9001
+    // frames had a wrong total; since then none in 23000.)
+    auto test = [&](unsigned t, unsigned& slot) -> int {
+        const int there = mbar_test_wait(bar_at(cfull, t % kSlots), use_parity(t, kSlots));
+        slot = cring + ((there ? t : t - 1u) % kSlots) * Slot::kBytes;
+        return there;
     };
     auto store = [&](int n, uint32_t* word) {
         if constexpr (kT) {
@@ -791,9 +800,10 @@ __device__ __forceinline__ void run_dp(const DpArgs& p, int strip, int lane, con
         const unsigned dst0 = out.base + (to % kSlots) * out.stride;
         const unsigned dst1 = out.base + ((to + 1u) % kSlots) * out.stride;
         int rb = 1, ra = 1, ro = 1;
+        unsigned sb = 0, sa = 0;
         full_sub(n, ia, 0, dst0, st, word, [&](int u) {
-            if (u == kFirst) rb = test(t + 1u);
-            part(ib, t + 1u, u);
+            if (u == kTest) rb = test(t + 1u, sb);
+            part(ib, sb, u);
         });
         mbar_arrive_if(bar_at(out.full, to % kSlots), st);
         const DpState<R> before = s;
@@ -801,8 +811,8 @@ __device__ __forceinline__ void run_dp(const DpArgs& p, int strip, int lane, con
             if (u == 0)  // its consumer empties the output ring in order
                 ro = mbar_test_wait(bar_at(out.empty, (to + 3u) % kSlots),
                                     use_parity(to + 3u, kSlots) ^ 1u);
-            if (u == kFirst) ra = test(t + 2u);
-            part(ia, t + 2u, u);
+            if (u == kTest) ra = test(t + 2u, sa);
+            part(ia, sa, u);
         });
         if (!__all_sync(kFull, rb & (ra | (int)!more) & (ro | (int)!next_on))) {
             if (!__all_sync(kFull, rb)) {
