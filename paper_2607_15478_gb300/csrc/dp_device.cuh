@@ -343,11 +343,15 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(unsigned bar, unsigned byt
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                  : "memory");
 }
-// Relaxed arrival on an mbarrier of another CTA of the cluster (a release at
-// cluster scope costs a fence: measured 1.68 against 1.32 ms of DP on the
-// 20000 x 25000 pair).
-__device__ __forceinline__ void mbar_arrive_remote_relaxed(unsigned remote_bar) {
-    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote_bar)
+// Arrival on an mbarrier of another CTA of the cluster, which hands memory of this CTA
+// back to it: a release, so that the reads of that memory (this thread's, and those it
+// has learned of by a wait) are done before the arrival is sent.  At the default scope,
+// as in the waits: what is handed over is shared memory, of which there is one
+// copy, and a release at cluster scope would wait for the SM's stores to global memory, too
+// (20000 x 25000, D = 12: DP 0.958 ms, 0.907 so; 1.066 with that scope in the waits as well
+// and each use by itself).
+__device__ __forceinline__ void mbar_arrive_remote(unsigned remote_bar) {
+    asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(remote_bar)
                  : "memory");
 }
 

@@ -47,6 +47,10 @@ template <bool kCl>
 constexpr int slots_of() {
     return kCl ? 16 : 8;
 }
+// Uses of the slots between two CTAs of a cluster that are handed back together (20000 x
+// 25000, D = 12: DP 0.996 ms with every use handed back by itself, 0.919 by 4, 0.907 by
+// 8, half of the slots).
+constexpr int kLinkPage = 8;
 constexpr int kBorderBytes = 2 * kSub * 4;  // 8 columns of (row top-2, row top-1) pairs
 
 // One slot holds the 8 costs of each of a lane's R rows: float4 q of lane l
@@ -688,8 +692,8 @@ __device__ __forceinline__ void run_dp(const DpArgs& p, int strip, int lane, con
     // the next slot's barrier is tested behind the shuffles of column kTest and the slot
     // loaded behind those of columns kFirst, kFirst + 1, .., kPer loads each: as late
     // as the latencies allow, since a strip can follow the one above no closer than
-    // its tests look ahead (20000 x 25000, D = 12: DP 0.980 ms; 1.00 with test and
-    // loads at column 4 and the loads not waiting for the test, see `test`)
+    // its tests look ahead (20000 x 25000, D = 12: DP 0.907 ms, 0.947 a column
+    // earlier; 40000 x 48000 with the BF16 cost 2.527, 2.519)
     constexpr int kTest = 4, kFirst = 5, kPer = 4;
     const bool ghost = lane == kGhostLane;
     const int i0 = strip * kRows + lane * R;
@@ -980,9 +984,11 @@ __device__ __forceinline__ void run_writer(const DpArgs& p, int grow, int lane,
 // of the first strip of CTA crank + 1, whose range starts at block bfirst with
 // lifetime use bsub of its slots; each of the 16 values an asynchronous store
 // completing 4 of the 64 bytes the slot's full barrier expects.  (Blocks before
-// bfirst are not needed below.)  Use lv of the link, counted from lsub, waits
-// until the reader warp below has handed use lv - kSlots back on `lempty`: the slot's
-// previous use in this ticket (those of earlier tickets are all released).
+// bfirst are not needed below.)  The reader warp below hands the slots back in pages
+// of kLinkPage uses on `lempty`: page q of the ticket is page lsub + q of the link, and
+// its first store waits until page lsub + q - kSlots / kLinkPage is back, which holds
+// its slots' previous uses where they lie in this ticket (those of earlier
+// tickets are all released).
 template <int kSlots>
 __device__ __forceinline__ void run_link_writer(const DpArgs& p, int lane,
                                                 const float (*ringo)[2 * kSub], unsigned bfullo,
@@ -996,12 +1002,15 @@ __device__ __forceinline__ void run_link_writer(const DpArgs& p, int lane,
     for (int n = nfirst; n < nsub; ++n) {
         const unsigned t = rbase + (unsigned)(n - nfirst);  // use of the writer's ring
         const unsigned u = bsub + (unsigned)(n - bfirst);   // use of the slots below
-        const unsigned lv = lsub + (unsigned)(n - bfirst);  // use of the link
         const bool send = n >= bfirst;
-        // the slot below is normally free long before the block is there
-        if (send && !mbar_wait(bar_at(lempty, lv % kSlots), use_parity(lv, kSlots) ^ 1u, p.ctl,
-                               p.timeout_ns, 10))
-            return;
+        if (send && (n - bfirst) % kLinkPage == 0) {
+            constexpr unsigned kPages = kSlots / kLinkPage;
+            const unsigned pg = lsub + (unsigned)(n - bfirst) / kLinkPage;
+            // the slots below are normally free long before the block is there
+            if (!mbar_wait(bar_at(lempty, pg % kPages), use_parity(pg, kPages) ^ 1u, p.ctl,
+                           p.timeout_ns, 10))
+                return;
+        }
         if (!mbar_wait(bar_at(bfullo, t % kSlots), use_parity(t, kSlots), p.ctl, p.timeout_ns, 9))
             return;
         const float v = ringo[t % kSlots][lane & (2 * kSub - 1)];
@@ -1014,8 +1023,8 @@ __device__ __forceinline__ void run_link_writer(const DpArgs& p, int lane,
 
 // Reader warp of a CTA with another CTA of its cluster above: the first
 // strip's blocks [nfirst, nsub), uses csub .. of its slots.  Those the CTA above
-// sends (before nsent; uses lsub .. of the link) it hands back once the DP warp
-// has released their slot; the later ones read +inf.  (It also stores those,
+// sends (before nsent; pages lsub .. of the link) it hands back, kLinkPage at a time,
+// once the DP warp has released their slots; the later ones read +inf.  (It also stores those,
 // rather than the cost warp, so that no slot can be released twice before
 // this warp has seen the first release.)
 template <int kSlots>
@@ -1028,9 +1037,12 @@ __device__ __forceinline__ void run_link_reader(const DpArgs& p, int lane, unsig
         if (n < nsent) {
             if (!mbar_wait(bar_at(empty, slot), use_parity(t, kSlots), p.ctl, p.timeout_ns, 11))
                 return;
-            const unsigned v = lsub + (unsigned)(n - nfirst);
-            if (lane == 0) mbar_arrive_remote_relaxed(map_rank(bar_at(lempty, v % kSlots), crank - 1));
-            __syncwarp();
+            if ((n - nfirst) % kLinkPage == kLinkPage - 1 || n + 1 == nsent) {
+                const unsigned pg = lsub + (unsigned)(n - nfirst) / kLinkPage;
+                if (lane == 0)
+                    mbar_arrive_remote(map_rank(bar_at(lempty, pg % (kSlots / kLinkPage)), crank - 1));
+                __syncwarp();
+            }
         } else {
             if (!mbar_wait(bar_at(empty, slot), use_parity(t, kSlots) ^ 1u, p.ctl, p.timeout_ns, 8))
                 return;
@@ -1075,7 +1087,7 @@ __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
     __shared__ __align__(8) unsigned long long ofull[kSlots];
     __shared__ __align__(8) unsigned long long oempty[kSlots];
     // releases of the slots of the CTA below, in a cluster
-    __shared__ __align__(8) unsigned long long lempty[kCl ? kSlots : 1];
+    __shared__ __align__(8) unsigned long long lempty[kSlots / kLinkPage];
     __shared__ int s_group, s_pair;
     extern __shared__ __align__(128) unsigned char dyn[];  // NS * M::kStripBytes
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1128,7 +1140,8 @@ __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
             }
             mbar_init(smem_u32(&ofull[k]), 1);   // lane 30 of the last strip's DP warp
             mbar_init(smem_u32(&oempty[k]), 1);  // the writer
-            if (kCl) mbar_init(smem_u32(&lempty[k]), 1);  // the reader of the CTA below
+            if (kCl && k < kSlots / kLinkPage)
+                mbar_init(smem_u32(&lempty[k]), 1);  // the reader of the CTA below
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -1139,7 +1152,7 @@ __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
         cluster_sync_all();  // every CTA's barriers before any remote access
     }
     // Lifetime sub-chunk counts of the slots and of the writer's ring, and (in
-    // a cluster) of the slots of the first strip of the CTA below and of the
+    // a cluster) of the slots of the first strip of the CTA below; page counts of the
     // links into and out of this CTA.
     unsigned csub[NS], osub = 0, lsub = 0, lin = 0, lout = 0;
 #pragma unroll
@@ -1279,10 +1292,11 @@ __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
 #pragma unroll
         for (int q = 0; q < NS; ++q) csub[q] += (unsigned)(rgs[q].y - rgs[q].x);
         if (gr.writer) osub += (unsigned)(rgs[NS - 1].y - rgs[NS - 1].x);
-        if (link_in) lin += (unsigned)max(above.y - rgs[0].x, 0);
+        auto pages = [](int uses) { return (unsigned)((max(uses, 0) + kLinkPage - 1) / kLinkPage); };
+        if (link_in) lin += pages(above.y - rgs[0].x);
         if (link_out) {
             lsub += (unsigned)(below.y - below.x);
-            lout += (unsigned)max(rgs[NS - 1].y - below.x, 0);
+            lout += pages(rgs[NS - 1].y - below.x);
         }
     }
     if constexpr (kCl) cluster_sync_all();  // no peer reaches this CTA's shared memory any more
