@@ -410,6 +410,7 @@ __global__ void __launch_bounds__(kSegThreads)
         }
     };
     load(0);
+    cluster_sync_all();  // every CTA runs before any is stored into
     for (int k = 0; k < N; ++k) {
         const int dk = k > 0 ? delta[k] : 0;
         float m[kPer];
