@@ -29,6 +29,8 @@
 //   4. k_bt_emit: the pieces are concatenated in ascending order.
 //
 // Entry codes: -1 = the origin (0, 0); -2 = no path (unreachable cell).
+#include <algorithm>
+
 #include "bandmap.cuh"
 #include "block_walk.cuh"
 
@@ -365,16 +367,10 @@ __global__ void __launch_bounds__(kEmitThreads) k_bt_emit(const BtArgs one, cons
 }
 
 size_t bandmap_scratch_bytes(int La, int Lb) {
-    // the shortest bands a call may choose for these rows take the most
-    const int band = band_rows(La, 0.0), nbands = (La + band - 1) / band;
-    const int n2 = nbands >= 4 ? (nbands - 2) / 2 : 0;
-    const int n4 = nbands >= 6 ? (nbands - 6) / 4 + 1 : 0;
-    return (size_t)nbands * Lb * sizeof(int2)        // exits
-           + (size_t)n2 * Lb * sizeof(int2)           // exits2
-           + (size_t)n4 * Lb * sizeof(int2)           // exits4
-           + (size_t)nbands * sizeof(int2)            // cross
-           + (size_t)nbands * band * sizeof(int2)     // seg
-           + (size_t)nbands * sizeof(int) + 64;       // count, end entry
+    // a call takes short bands or, where it fills the GPU, the longest: short ones have the
+    // more exits, the longest the more cells (a pair's pieces are whole bands)
+    return std::max(bt_scratch_bytes(La, Lb, band_rows(La, 0.0)),
+                    bt_scratch_bytes(La, Lb, kMaxBand));
 }
 
 cudaError_t launch_backtrace_bands(const BtArgs& pair, cudaStream_t s) {
@@ -386,11 +382,10 @@ cudaError_t launch_backtrace_bands(const BtArgs& pair, cudaStream_t s) {
     const BtArgs* none = nullptr;
     cudaError_t e = launch_chained(ch, a.ranges ? k_bandmap<false, true> : k_bandmap<false, false>,
                                    grid, 32 * kMapWarps, 0, s, a, none);
-    const int n2 = nbands >= 4 ? (nbands - 2) / 2 : 0;
+    const int n2 = bt_bands(a.La, band).n2, n4 = bt_bands(a.La, band).n4;
     const unsigned cols = (unsigned)((a.Lb + 255) / 256);
     if (e == cudaSuccess && n2 > 0)
         e = launch_chained(ch, k_bt_compose<false>, dim3(cols, (unsigned)n2, 1), 256, 0, s, a, none);
-    const int n4 = nbands >= 6 ? (nbands - 6) / 4 + 1 : 0;
     if (e == cudaSuccess && n4 > 0)
         e = launch_chained(ch, k_bt_compose4<false>, dim3(cols, (unsigned)n4, 1), 256, 0, s, a, none);
     if (e == cudaSuccess)

@@ -24,13 +24,32 @@ struct BtScratch {
     int* end_entry;  // the end cell's entry
     int band, nbands, n2, n4;
 };
-__host__ __device__ inline BtScratch bt_scratch(const BtArgs& a) {
-    const int La = a.La, Lb = a.Lb;
-    BtScratch r;
-    r.band = a.band;
-    r.nbands = (La + r.band - 1) / r.band;
+// Bands of La rows, and how many of them have a two-band and a four-band map.
+struct BtBands {
+    int nbands, n2, n4;
+};
+__host__ __device__ inline BtBands bt_bands(int La, int band) {
+    BtBands r;
+    r.nbands = (La + band - 1) / band;
     r.n2 = r.nbands >= 4 ? (r.nbands - 2) / 2 : 0;
     r.n4 = r.nbands >= 6 ? (r.nbands - 6) / 4 + 1 : 0;
+    return r;
+}
+// Bytes of the scratch with bands of `band` rows.
+inline size_t bt_scratch_bytes(int La, int Lb, int band) {
+    const BtBands r = bt_bands(La, band);
+    return (size_t)(r.nbands + r.n2 + r.n4) * Lb * sizeof(int2)  // exits, exits2, exits4
+           + (size_t)r.nbands * (1 + band) * sizeof(int2)        // cross, seg
+           + (size_t)(r.nbands + 1) * sizeof(int);               // count, end entry
+}
+__host__ __device__ inline BtScratch bt_scratch(const BtArgs& a) {
+    const int La = a.La, Lb = a.Lb;
+    const BtBands n = bt_bands(La, a.band);
+    BtScratch r;
+    r.band = a.band;
+    r.nbands = n.nbands;
+    r.n2 = n.n2;
+    r.n4 = n.n4;
     char* p = static_cast<char*>(a.scratch);
     r.exits = reinterpret_cast<int2*>(p);
     p += (size_t)r.nbands * Lb * sizeof(int2);
