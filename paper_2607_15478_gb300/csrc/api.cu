@@ -192,17 +192,22 @@ Layout make_layout(int La, int Lb, int D, const DpPlan& plan, bool staged = true
     return L;
 }
 
-constexpr size_t kGrowRoomFrom = size_t(4) << 20;
+}  // namespace
+
+size_t pardtw::grown_bytes(size_t need, size_t had) {
+    constexpr size_t kShared = size_t(4) << 20;
+    return had == 0 && need <= kShared ? need : need + need / 8;
+}
+
+namespace {
 
 int ensure_workspace(dtw_handle* h, size_t bytes, size_t border_bytes) {
     if (bytes > h->ws_cap) {
         CU(cudaStreamSynchronize(h->stream));
+        size_t want = grown_bytes(bytes, h->ws_cap);
         if (h->ws) cudaFree(h->ws);
         h->ws = nullptr;
         h->ws_cap = 0;
-        // room to grow, but not where it would cost a mapping of its own (small
-        // allocations share one)
-        size_t want = bytes + (bytes > kGrowRoomFrom ? bytes / 8 : 0);
         if (cudaMalloc(&h->ws, want) != cudaSuccess) {
             (void)cudaGetLastError();
             if (cudaMalloc(&h->ws, bytes) != cudaSuccess) {
@@ -216,10 +221,10 @@ int ensure_workspace(dtw_handle* h, size_t bytes, size_t border_bytes) {
     }
     if (border_bytes > h->border_cap) {
         CU(cudaStreamSynchronize(h->stream));
+        const size_t want = grown_bytes(border_bytes, h->border_cap);
         if (h->border) cudaFree(h->border);
         h->border = nullptr;
         h->border_cap = 0;
-        size_t want = border_bytes + (border_bytes > kGrowRoomFrom ? border_bytes / 8 : 0);
         if (cudaMalloc(&h->border, want) != cudaSuccess) {
             (void)cudaGetLastError();
             h->border = nullptr;

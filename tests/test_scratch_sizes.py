@@ -53,3 +53,21 @@ def test_short_pairs_in_a_large_call():
             for k, path in enumerate(paths):
                 ref, total = aligner.align(A[k], B[k], rows_per_lane=1)
                 assert status[k] == 0 and float(cost[k]) == total and torch.equal(path, ref), k
+
+
+def test_growing_pairs_allocate_seldom():
+    """A handle fed pairs whose needs grow by 1% a call allocates once per eighth, and a
+    first small allocation has no spare room."""
+    pbuild.build()
+    grown = ctypes.CDLL(pbuild.LIB)["_ZN6pardtw11grown_bytesEmm"]
+    grown.restype = ctypes.c_size_t
+    grown.argtypes = [ctypes.c_size_t, ctypes.c_size_t]
+    assert grown(1 << 20, 0) == 1 << 20
+    for start in (100 << 10, 1 << 20, 3 << 20, 64 << 20):
+        need, cap, allocations = float(start), 0, 0
+        while need < 4 * start:
+            if need > cap:
+                cap = grown(int(need) + 1, cap)
+                allocations += 1
+            need *= 1.01
+        assert allocations <= 14  # ln 4 / ln 1.125 = 11.8, the first, one of rounding
