@@ -1072,18 +1072,19 @@ EncSeq enc_seq(size_t base, int Lc, int D) {
     q.total = o;
     return q;
 }
-// Both sequences, then the per-row training data of A: targets (int), width
-// targets, width-logit gradients.
+// Both sequences, then the per-row training data of A: the targets' sums and counts,
+// width targets, width-logit gradients.
 struct EncBuf {
     EncSeq a, b;
-    size_t tgt, wt, dS, total;
+    size_t jsum, cnt, wt, dS, total;
 };
 EncBuf enc_buf(int Lac, int Lbc, int D) {
     EncBuf e;
     e.a = enc_seq(0, Lac, D);
     e.b = enc_seq(e.a.total, Lbc, D);
     size_t o = e.b.total;
-    e.tgt = o; o = align256(o + (size_t)Lac * sizeof(int));
+    e.jsum = o; o = align256(o + (size_t)Lac * sizeof(unsigned long long));
+    e.cnt = o; o = align256(o + (size_t)Lac * sizeof(int));
     e.wt = o; o = align256(o + (size_t)Lac * sizeof(float));
     e.dS = o; o = align256(o + (size_t)Lac * sizeof(float));
     e.total = o;
@@ -1100,10 +1101,10 @@ struct EncIn {
 };
 
 // Encoder forward of n (1 or 2) sequences: pooled input, the three conv layers
-// and the heads, into the buffers of each.  train: also zeroes the embedding
-// gradients.
+// and the heads, into the buffers of each.  train (may be null): also zeroes the
+// embedding gradients and the sums of A's targets.
 int enc_forward(dtw_handle* h, const float* P, const EncLayout& pl, int D, const EncIn* in, int n,
-                int ds, int bf16, bool train) {
+                int ds, int bf16, const EncBuf* train) {
     cudaStream_t s = h->stream;
     EncRows2 r{};
     auto rows = [&](size_t EncSeq::*x, size_t EncSeq::*y) {
@@ -1122,7 +1123,12 @@ int enc_forward(dtw_handle* h, const float* P, const EncLayout& pl, int D, const
     for (int k = 0; k < n; ++k) {
         const EncSeq& q = in[k].q;
         e.s[k] = {ef(h, q.H3), ef(h, q.E),  ef(h, q.invn),                 ef(h, q.S),
-                  ef(h, q.HW), train ? ef(h, q.G) : nullptr, nullptr, (in[k].L + ds - 1) / ds};
+                  ef(h, q.HW), train ? ef(h, q.G) : nullptr, nullptr, (in[k].L + ds - 1) / ds,
+                  nullptr, nullptr};
+    }
+    if (train) {
+        e.s[0].jsum = reinterpret_cast<unsigned long long*>(h->enc + train->jsum);
+        e.s[0].cnt = reinterpret_cast<int*>(h->enc + train->cnt);
     }
     CU(launch_embed(e, n, P, pl, bf16, (float)DTW_BAND_WMIN, (float)DTW_BAND_WMAX, s));
     return DTW_OK;
@@ -1223,7 +1229,7 @@ int dtw_encode(dtw_handle* h, const float* params, int D, const float* X, int L,
     if (rc != DTW_OK) return rc;
     const EncLayout pl = enc_layout(D);
     const EncIn in = {X, L, q};
-    rc = enc_forward(h, params, pl, D, &in, 1, downsample, bf16 != 0, false);
+    rc = enc_forward(h, params, pl, D, &in, 1, downsample, bf16 != 0, nullptr);
     if (rc != DTW_OK) return rc;
     CU(cudaMemcpyAsync(emb, ef(h, q.E), sizeof(float) * (size_t)Lc * kEncEmbed,
                        cudaMemcpyDeviceToDevice, h->stream));
@@ -1254,13 +1260,14 @@ int dtw_encoder_grad(dtw_handle* h, const float* params, int D, int downsample, 
     if (rc != DTW_OK) return rc;
     const EncLayout pl = enc_layout(D);
     const EncIn in[2] = {{A, La, eb.a}, {B, Lb, eb.b}};
-    rc = enc_forward(h, params, pl, D, in, 2, downsample, 0, mode == 0);
+    rc = enc_forward(h, params, pl, D, in, 2, downsample, 0, mode == 0 ? &eb : nullptr);
     if (rc != DTW_OK) return rc;
     if (mode == 0) {
-        int* tgt = reinterpret_cast<int*>(h->enc + eb.tgt);
-        CU(launch_targets(path, path_len, std::min(La, Lb), downsample, Lac, Lbc, tgt, s));
-        CU(launch_loss_emb(ef(h, eb.a.E), Lac, ef(h, eb.b.E), Lbc, tgt, ef(h, eb.a.G),
-                           ef(h, eb.b.G), loss, s));
+        unsigned long long* jsum = reinterpret_cast<unsigned long long*>(h->enc + eb.jsum);
+        int* cnt = reinterpret_cast<int*>(h->enc + eb.cnt);
+        CU(launch_targets(path, path_len, std::min(La, Lb), downsample, Lac, jsum, cnt, s));
+        CU(launch_loss_emb(ef(h, eb.a.E), Lac, ef(h, eb.b.E), Lbc, jsum, cnt, downsample,
+                           ef(h, eb.a.G), ef(h, eb.b.G), loss, s));
         return enc_backward(h, params, pl, D, in, 2, downsample, grad);
     }
     // mode 1: the coarse path on the current embeddings, the half-width each
@@ -1320,7 +1327,7 @@ int dtw_align_learned(dtw_handle* h, const float* A, int La, const float* B, int
     if (rc != DTW_OK) return rc;
     const EncLayout pl = enc_layout(D);
     const EncIn in[2] = {{A, La, eb.a}, {B, Lb, eb.b}};
-    rc = enc_forward(h, params, pl, D, in, 2, downsample, bf16 != 0, false);
+    rc = enc_forward(h, params, pl, D, in, 2, downsample, bf16 != 0, nullptr);
     if (rc != DTW_OK) return rc;
     return band_align(h, A, La, B, Lb, D, o, downsample, ef(h, eb.a.E), Lac, ef(h, eb.b.E), Lbc,
                       kEncEmbed, 0, ef(h, eb.a.HW), ef(h, eb.b.HW), bb, path, path_len,

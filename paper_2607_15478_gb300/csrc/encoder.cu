@@ -336,7 +336,8 @@ __global__ void __launch_bounds__(kWgThreads)
 // Heads, four threads per row (four embedding components each): z = W4 h3 + b4,
 // e = z / |z| (invn = 1/|z|, 0 for z = 0), s = W5 . h3 + b5 and the half-width in
 // fine frames.  Sums run over the channels, and the norm over the components,
-// in order.  G (may be null): zeroed, the embedding gradient of a training step.
+// in order.  G, jsum, cnt (may be null): zeroed, a training step's embedding gradient and
+// the sums of its targets.
 __global__ void __launch_bounds__(128) k_embed(const EncEmbed2 q, const float* __restrict__ W4,
                         const float* __restrict__ b4, const float* __restrict__ W5,
                         const float* __restrict__ b5, int bf16, float wmin, float wmax) {
@@ -391,6 +392,10 @@ __global__ void __launch_bounds__(128) k_embed(const EncEmbed2 q, const float* _
         make_float4(z[0] * r, z[1] * r, z[2] * r, z[3] * r);
     if (a.G) reinterpret_cast<float4*>(a.G + (size_t)l * kE)[eg] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (eg != 0) return;
+    if (a.jsum) {
+        a.jsum[l] = 0ull;
+        a.cnt[l] = 0;
+    }
     if (a.invn) a.invn[l] = r;
     s += bb[kE];
     if (a.S) a.S[l] = s;
@@ -491,22 +496,28 @@ __device__ __forceinline__ int first_of_row(const int32_t* __restrict__ path, in
 
 // Coarse column matched to every coarse row of A by the exact fine path:
 // the mean column of the path entries in the row's ds fine rows, divided by
-// ds.  A row's entries are consecutive in the path.
+// ds.  One thread per path entry, in whatever order they come, adds to its row's
+// sum and count (zeroed by k_embed); k_loss_emb divides.
 __global__ void k_targets(const int32_t* __restrict__ path, const int* __restrict__ plen, int cap,
-                          int ds, int Lac, int Lbc, int* __restrict__ tgt) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= Lac) return;
-    const int len = min(*plen, cap);
-    unsigned long long jsum = 0;
-    int n = 0;
-    for (int k = first_of_row(path, len, i * ds); k < len && path[2 * k] < (i + 1) * ds; ++k) {
-        jsum += (unsigned long long)path[2 * k + 1];
-        ++n;
-    }
+                          int ds, int Lac, unsigned long long* __restrict__ jsum,
+                          int* __restrict__ cnt) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= min(*plen, cap)) return;
+    const int2 c = make_int2(path[2 * k], path[2 * k + 1]);
+    const int i = c.x / ds;
+    if (c.x < 0 || i >= Lac) return;
+    atomicAdd(&jsum[i], (unsigned long long)c.y);
+    atomicAdd(&cnt[i], 1);
+}
+__device__ __forceinline__ int target_column(unsigned long long jsum, int n, int ds, int Lbc) {
     // every fine row lies on a path except rows a (2,1) step skips; a coarse
     // row of ds >= 2 fine rows always holds one
-    const double m = n > 0 ? (double)jsum / n : 0.0;
-    tgt[i] = min((int)(m / ds), Lbc - 1);
+    if (n == 0) return min(0, Lbc - 1);
+    // (the same whole number in 32 bits: below 2^52 no rounding reaches the next one)
+    const unsigned long long rows = (unsigned long long)n * (unsigned)ds;
+    if (((jsum | rows) >> 32) == 0) return min((int)((unsigned)jsum / (unsigned)rows), Lbc - 1);
+    const double m = (double)jsum / n;
+    return min((int)(m / ds), Lbc - 1);
 }
 
 // Contrastive loss, one warp per coarse row i of A (see the file comment),
@@ -517,8 +528,8 @@ __global__ void k_targets(const int32_t* __restrict__ path, const int* __restric
 constexpr int kLossRows = 4;
 __global__ void __launch_bounds__(32 * kLossRows)
     k_loss_emb(const float* __restrict__ eA, int Lac, const float* __restrict__ eB, int Lbc,
-               const int* __restrict__ tgt, float* __restrict__ gA, float* __restrict__ gB,
-               float* __restrict__ loss) {
+               const unsigned long long* __restrict__ jsum, const int* __restrict__ cnt, int ds,
+               float* __restrict__ gA, float* __restrict__ gB, float* __restrict__ loss) {
     constexpr int kWidth = 2 * kWin + 1;
     static_assert(kWidth == 33, "a lane per column and one more");
     __shared__ float s_w[kLossRows][kWidth], s_a[kLossRows][kE], s_loss[kLossRows];
@@ -529,7 +540,7 @@ __global__ void __launch_bounds__(32 * kLossRows)
     if (i < Lac) {
         if (lane < kE) s_a[w][lane] = eA[(size_t)i * kE + lane];
         __syncwarp();
-        const int c = tgt[i];
+        const int c = target_column(jsum[i], cnt[i], ds, Lbc);
         const int j0 = max(c - kWin, 0), j1 = min(c + kWin, Lbc - 1);
         float lg[2] = {-INFINITY, -INFINITY};
 #pragma unroll
@@ -742,16 +753,17 @@ cudaError_t launch_head_grad(const EncHead2& q, int n, int outputs, float* dW, f
     return cudaGetLastError();
 }
 
-cudaError_t launch_targets(const int32_t* path, const int* plen, int cap, int ds, int Lac, int Lbc,
-                           int* tgt, cudaStream_t s) {
-    k_targets<<<(Lac + 63) / 64, 64, 0, s>>>(path, plen, cap, ds, Lac, Lbc, tgt);
+cudaError_t launch_targets(const int32_t* path, const int* plen, int cap, int ds, int Lac,
+                           unsigned long long* jsum, int* cnt, cudaStream_t s) {
+    k_targets<<<(cap + 127) / 128, 128, 0, s>>>(path, plen, cap, ds, Lac, jsum, cnt);
     return cudaGetLastError();
 }
 
-cudaError_t launch_loss_emb(const float* eA, int Lac, const float* eB, int Lbc, const int* tgt,
-                            float* gA, float* gB, float* loss, cudaStream_t s) {
-    k_loss_emb<<<(Lac + kLossRows - 1) / kLossRows, 32 * kLossRows, 0, s>>>(eA, Lac, eB, Lbc, tgt,
-                                                                           gA, gB, loss);
+cudaError_t launch_loss_emb(const float* eA, int Lac, const float* eB, int Lbc,
+                            const unsigned long long* jsum, const int* cnt, int ds, float* gA,
+                            float* gB, float* loss, cudaStream_t s) {
+    k_loss_emb<<<(Lac + kLossRows - 1) / kLossRows, 32 * kLossRows, 0, s>>>(
+        eA, Lac, eB, Lbc, jsum, cnt, ds, gA, gB, loss);
     return cudaGetLastError();
 }
 

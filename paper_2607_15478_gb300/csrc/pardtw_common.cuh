@@ -403,6 +403,8 @@ struct EncEmbed {
     const float* H;
     float *Emb, *invn, *S, *HW, *G, *dH;  // see k_embed, k_embed_bwd
     int L;
+    unsigned long long* jsum;  // see k_targets
+    int* cnt;
 };
 struct EncHead {
     const float *U, *H;
@@ -428,11 +430,13 @@ cudaError_t launch_embed_bwd(const EncEmbed2& q, int n, const float* W4, cudaStr
 // outputs = 16 (embedding head) or 1 (half-width head).
 cudaError_t launch_head_grad(const EncHead2& q, int n, int outputs, float* dW, float* db,
                              cudaStream_t s);
-cudaError_t launch_targets(const int32_t* path, const int* plen, int cap, int ds, int Lac, int Lbc,
-                           int* tgt, cudaStream_t s);
+// jsum, cnt: Lac each, added to (zeroed by launch_embed).
+cudaError_t launch_targets(const int32_t* path, const int* plen, int cap, int ds, int Lac,
+                           unsigned long long* jsum, int* cnt, cudaStream_t s);
 // gB is added to (zeroed by launch_embed's G).
-cudaError_t launch_loss_emb(const float* eA, int Lac, const float* eB, int Lbc, const int* tgt,
-                            float* gA, float* gB, float* loss, cudaStream_t s);
+cudaError_t launch_loss_emb(const float* eA, int Lac, const float* eB, int Lbc,
+                            const unsigned long long* jsum, const int* cnt, int ds, float* gA,
+                            float* gB, float* loss, cudaStream_t s);
 cudaError_t launch_width_target(const int32_t* cpath, const int* clen, const int32_t* path,
                                 const int* plen, int ds, int Lac, float wmin, float wmax,
                                 float* wt, cudaStream_t s);
