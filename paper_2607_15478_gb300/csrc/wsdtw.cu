@@ -46,10 +46,13 @@ __device__ __forceinline__ MinArg better(MinArg a, MinArg b) {  // a is earlier
 //                from its carry, written as D_seg[k][*] and arg[k][*].
 constexpr int kTile = 1024;
 
+// A match that is NaN (a frame that is) is never attained: +inf, in every form of this DP.
+__device__ __forceinline__ float attainable(float match) { return fminf(match, INFINITY); }
+
 __device__ __forceinline__ float seg_match(const float* cs, const float* prev, int k, int dk,
                                            int j) {
-    if (k == 0) return cs[j];
-    return j - dk >= 0 ? prev[j - dk] + cs[j] : INFINITY;
+    if (k == 0) return attainable(cs[j]);
+    return j - dk >= 0 ? attainable(prev[j - dk] + cs[j]) : INFINITY;
 }
 
 // Block-wide inclusive scan of one (value, column) per thread, earlier wins.
@@ -311,7 +314,7 @@ __global__ void __launch_bounds__(kTile)
         if (j < Lb) {
             // D_seg[k-1] was written by other CTAs of this launch: read through L2
             const float m = k == 0 ? cs[j] : (j - dk >= 0 ? __ldcg(prev + j - dk) + cs[j] : INFINITY);
-            v = MinArg{m, j};
+            v = MinArg{attainable(m), j};
         }
         v = block_scan_min(v, s_warp);
         if (threadIdx.x == blockDim.x - 1) {
@@ -423,7 +426,7 @@ __global__ void __launch_bounds__(kSegThreads)
         }
 #pragma unroll
         for (int i = 0; i < kPer; ++i)
-            Ms[seg_slot(tid + i * kSegThreads)] = k == 0 ? cs[i] : m[i] + cs[i];
+            Ms[seg_slot(tid + i * kSegThreads)] = attainable(k == 0 ? cs[i] : m[i] + cs[i]);
         if (k + 1 < N) load(k + 1);
         __syncthreads();
         // the minimum of the thread's columns, of the lanes and warps before it
