@@ -187,7 +187,7 @@ __device__ __forceinline__ void cost_arrive(unsigned full, unsigned border, int 
 // on its SM sub-partition and 52 with two, scalar ones 64 and 60.  (A pass over
 // 16 columns takes 49 and 47 but fills its slots in bursts: no faster in the
 // kernel, and slower at D = 32 and where two CTAs share an SM's registers.)
-template <int DP, int R, int NS, int kSlots, bool kAllCols>
+template <int DP, int R, int NS, int kSlots, bool kAllCols, int kNG = DP / 4>
 __device__ __forceinline__ void run_cost(const DpArgs& p, int strip, int half, int lane,
                                          unsigned cring, unsigned cfull, unsigned cempty,
                                          unsigned csub, const BorderSrc& bs,
@@ -197,8 +197,7 @@ __device__ __forceinline__ void run_cost(const DpArgs& p, int strip, int half, i
     using S = BStage<DP, Cfg::kBSlots, Cfg::kBBlk>;
     using CR = CostRing<R>;
     constexpr int kRows = 31 * R;
-    constexpr int kFG = 4;            // features per group of loads
-    constexpr int kNG = DP / kFG;     // DP is a multiple of 4
+    constexpr int kFG = 4;            // features per group of loads; kNG groups have some
     static_assert(S::kBlk >= kSub * Cfg::kNC, "a warp reads some of every block of B");
     const bool ghost = lane == kGhostLane;
     const int i0 = strip * kRows + lane * R;
@@ -253,11 +252,6 @@ __device__ __forceinline__ void run_cost(const DpArgs& p, int strip, int half, i
         }
 #pragma unroll
         for (int gi = 0; gi < kNG; ++gi) {
-            // D = 17 .. 20: the groups beyond are zero in both frames, and an FMA with a
-            // zero product leaves every bit of the sum (48 pairs of up to 2500 frames at
-            // D = 20: DP 204 us, 181 so).  One test: one per group costs D = 32 more (3%);
-            // with one strip a CTA the cost warps don't set the pace (D = 32 would lose 1%)
-            if (DP > 16 && NS > 1 && gi == 5 && p.feats <= gi * kFG) break;
             if (gi + 1 < kNG) {
 #pragma unroll
                 for (int e = 0; e < kFG; ++e) {
@@ -1238,7 +1232,25 @@ __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
                 else if constexpr (Cfg::kWide)
                     run_cost_wide<DP, R, NS, kSlots>(p, strip, w, half, lane, reinterpret_cast<float*>(mine),
                                          cring_s, cfull_s, cempty_s, cs, bs, br);
-                else
+                else if constexpr (DP > 16 && NS > 1) {
+                    // groups of four features that are padding in both frames are left out:
+                    // an FMA with a zero product leaves every bit of the sum.  A loop for each
+                    // number of groups, as a test in one loop costs D = 32 3%: DP of 48 pairs of up
+                    // to 2500 frames, 5 to 8 groups: 177, 185, 192, 205 us, all as 8 before.
+                    // With one strip a CTA the cost warps don't set the pace.
+                    if (p.feats > 28)
+                        run_cost<DP, R, NS, kSlots, kSubseq, 8>(p, strip, half, lane, cring_s, cfull_s,
+                                                                cempty_s, cs, bs, br);
+                    else if (p.feats > 24)
+                        run_cost<DP, R, NS, kSlots, kSubseq, 7>(p, strip, half, lane, cring_s, cfull_s,
+                                                                cempty_s, cs, bs, br);
+                    else if (p.feats > 20)
+                        run_cost<DP, R, NS, kSlots, kSubseq, 6>(p, strip, half, lane, cring_s, cfull_s,
+                                                                cempty_s, cs, bs, br);
+                    else
+                        run_cost<DP, R, NS, kSlots, kSubseq, 5>(p, strip, half, lane, cring_s, cfull_s,
+                                                                cempty_s, cs, bs, br);
+                } else
                     run_cost<DP, R, NS, kSlots, kSubseq>(p, strip, half, lane, cring_s,
                                                                 cfull_s, cempty_s, cs, bs, br);
             }
