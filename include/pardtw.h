@@ -104,10 +104,10 @@ typedef struct dtw_options {
      * cost); the tie order is mapped so that results do not depend on it. */
     int transpose;
     /* DTW_CLUSTERS_AUTO (0, default): the default DP of one pair (warp pairs
-     * at 3 rows per lane) runs in persistent thread-block clusters of 2 to 8 CTAs, which hand the strip border from CTA to CTA through
-     * distributed shared memory instead of global memory, when the device
-     * has room for them; DTW_CLUSTERS_NEVER (1): never.  Results do not
-     * depend on it. */
+     * at 3 rows per lane) runs in persistent thread-block clusters of 2 to 8
+     * CTAs, which hand the strip border from CTA to CTA through distributed
+     * shared memory instead of global memory, when the device has room for
+     * them; DTW_CLUSTERS_NEVER (1): never.  Results do not depend on it. */
     int clusters;
 } dtw_options;
 
@@ -329,8 +329,9 @@ int dtw_encode(dtw_handle* h, const float* params, int D, const float* X, int L,
 
 /* Training: adds to grad (device, dtw_encoder_param_count(D) floats) the
  * gradient of the loss of one pair and adds the loss to *loss (device).
- * path / path_len (device) is the exact alignment of (A, B) (as dtw_align
- * writes it).  Per coarse row i of A the exact path matches coarse column
+ * path / path_len (device) is the exact alignment of (A, B), its pairs in
+ * ascending order as dtw_align writes them (mode 0 takes them in any order).
+ * Per coarse row i of A the exact path matches coarse column
  * c_i (its mean column in the row's frames / downsample).
  *   mode 0: embedding loss, mean over i of -log softmax_j(eA_i . eB_j / 0.1)
  *           at j = c_i, j over the coarse columns within 16 of c_i; gradient

@@ -53,8 +53,7 @@ __device__ __forceinline__ unsigned long long ldg1(const unsigned long long* p) 
 __device__ __forceinline__ void stg1(unsigned long long* p, unsigned long long a) {
     asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(a) : "memory");
 }
-// Per-strip completion flags in global memory: released by the DP warp that
-// finished the strip, acquired by the band-map items that read its words.
+// The generation counter of a barrier over a grid (wsdtw.cu) in global memory.
 __device__ __forceinline__ void st_release_g(unsigned* p, unsigned v) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }

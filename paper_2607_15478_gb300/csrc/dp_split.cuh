@@ -88,12 +88,12 @@ constexpr int kBfBlkBytes = kColsPerWord * kBfStride * 2;
 // floats: the 16-byte loads of rows 3l + k of a warp fall in distinct bank
 // groups), and several cost warps share a strip, taking sub-chunks in turn
 // (all 8 columns each).  So they do where one would be slower than the DP warp.
-// With two strips a CTA: two (two strips beside each other at D = 12: 83 cycles a
-// column, 126 with a third one, which shares the DP warp's SM sub-partition; 139
-// against 162 with two CTAs an SM; D = 16: 88 and 89), at D = 32 three (122, 151
-// with two).  With one strip, four of the wide ones (24001 x 27011 at D = 100: 3.23 ms, 2.50 with six,
-// which are not measured at other sizes), and three otherwise (40000 x 48000 with the
-// BF16 cost: 2.78, 2.77 with four).
+// With two strips a CTA: two (20000 x 25000 at D = 12: DP 0.907 ms, 1.056 with a third one,
+// which shares the DP warp's SM sub-partition; a plan of 256 pairs 3.53 and 3.78), at
+// D = 32 three (256 pairs of up to 4000 frames: 1.43 ms, 1.60 with two).  With one strip, four
+// of the wide ones (24001 x 27011 at D = 100: 3.23 ms, 2.50 with six, which are not
+// measured at other sizes), and three otherwise (40000 x 48000 with the BF16 cost: 2.80,
+// and with four).
 template <int DP, int NS, bool kBF>
 struct CostCfg {
     static constexpr bool kWide = DP > 32 && !kBF;

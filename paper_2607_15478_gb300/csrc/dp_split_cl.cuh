@@ -7,8 +7,8 @@
 // the writer warp of the CTA above stores it, the reader warp of the CTA
 // below polls it.  In a cluster the writer warp stores it straight into the
 // slots of the CTA below, so only one hop in cn stays global.  From strip to
-// strip of a 4000-column chain at D = 12, two strips a CTA: 1.5 us without
-// clusters, 0.81 in them (one strip a CTA: 2.6 and 1.0), of which the 31 lanes'
+// strip of a 4000-column chain at D = 12, two strips a CTA: 1.55 us without
+// clusters, 0.75 in them (one strip a CTA: 2.4 and 0.9), of which the 31 lanes'
 // skew alone is 0.66.
 //
 // Every CTA of a cluster sits on an SM of its own (the dynamic shared
@@ -17,9 +17,9 @@
 // warps cannot keep up with a DP warp (D > 16, the BF16 cost: three or four cost
 // warps a strip, on the sub-partitions beside the DP warp's), else two.  The
 // cluster size: see launch_cl.  Measured (DP, ms): 20000 x 25000, D = 12, clusters
-// of 8 / 6 / 4 / 2: 1.001 / 1.009 / 1.027 / 1.080; 100000 x 126231 (335 groups active
-// at once, 152 SMs): 7.66 / 7.18 / 6.94 / 6.59; 40000 x 48000, D = 128, BF16: 2.65 / 2.55
-// / 2.52 / 2.50 with one strip a CTA, 3.16 without clusters and two.
+// of 8 / 6 / 4 / 2: 0.906 / 0.916 / 0.928 / 0.976; 100000 x 126231 (335 groups active
+// at once, 152 SMs): 6.87 / 6.38 / 6.19 / 5.88; 40000 x 48000, D = 128, BF16: 2.70 / 2.59
+// / 2.57 / 2.52 with one strip a CTA, 3.18 without clusters and two.
 #pragma once
 #include <algorithm>
 #include <mutex>

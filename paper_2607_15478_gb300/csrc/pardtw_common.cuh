@@ -150,7 +150,8 @@ struct DpArgs {
     int feats;                      // features of a frame; those up to the padded width are zero
     const int2* ranges;             // banded DP (warp-pair kernel): per strip the sub-chunks
                                     // [x, y) of 8 columns it sweeps (x even; x and y
-                                    // non-decreasing in the strip); null = every column
+                                    // non-decreasing in the strip); null = the columns
+                                    // that a path can cross (subsequence DP: every column)
     float* lastrow;                 // subsequence DP (WSDTW): the cumulative cost of row
                                     // La-1 at every column (nchunk * 16 floats), else null
 };
@@ -254,16 +255,16 @@ bool split_supported(int dp, int R, int ns = 2);
 // tensor cores (mma.sync m16n8k16): D padded to 64 or 128, R = 3.
 cudaError_t launch_dp_split_bf16(const DpArgs& a, int dp, int num_sms, cudaStream_t s,
                                  bool transposed = false);
-// The warp-pair DP of one pair at 3 rows per lane and two strips per CTA,
-// run in thread-block clusters whose CTAs pass the strip border through
-// distributed shared memory (dp_split_cl.cu; dp <= 32, or 64 / 128 with
-// bf16).  *used = false (and nothing launched) when no cluster
-// configuration fits this device.
+// The warp-pair DP of one pair at 3 rows per lane, run in thread-block clusters whose
+// CTAs pass the strip border through distributed shared memory (dp_split_cl.cu; two
+// strips per CTA at dp <= 16, one at 32 and, FP32 or bf16, at 64 and 128).
+// *used = false (and nothing launched) when no cluster configuration fits
+// this device.
 cudaError_t launch_dp_split_cl(const DpArgs& a, int dp, bool bf16, bool transposed,
                                cudaStream_t s, bool* used);
-// The warp-pair DP with the FP32 cost at D = 64, 128 (dp_split_wide.cu): two
-// cost warps per strip, 3 rows per lane, two strips per CTA; the same in
-// thread-block clusters.
+// The warp-pair DP with the FP32 cost at D = 64, 128 (dp_split_wide.cu), 3 rows per
+// lane: two strips per CTA with two cost warps each; in thread-block clusters one
+// with four.
 bool split_wide_supported(int dp);
 cudaError_t launch_dp_split_wide(const DpArgs& a, int dp, int num_sms, cudaStream_t s,
                                  bool transposed = false);
@@ -322,10 +323,10 @@ struct BtArgs {
 // Rows per band of a pair of La rows in a call over `cells` matrix cells in all:
 // the band map and the walks take time in proportion to a band's rows (~0.17 and
 // ~0.06 us a row, all bands at once), the chain in proportion to the number of
-// bands (~0.6 us for four), so short pairs take short bands (1000 x 1200: 117 us
-// with 128 rows, 99 with 32; 3001 x 3607: 237 and 226 with 64) unless the call
+// bands (~0.6 us for four), so short pairs take short bands (1000 x 1200: 96.9 us
+// with 128 rows, 82.6 with 32; 3001 x 3607: 216 and 206 with 64) unless the call
 // fills the GPU: a segment of the map recomputes two columns per row of its band (256
-// pairs of up to 8000 frames: 3.59 ms with 64 rows, 3.44 with 128).
+// pairs of up to 8000 frames: 3.69 ms with 64 rows, 3.53 with 128).
 inline int band_rows(int La, double cells) {
     if (cells > 1e9) return 128;
     return La <= 1536 ? 32 : (La <= 6144 ? 64 : 128);

@@ -66,6 +66,7 @@ def test_queued_pairs(D, opts):
 
 
 @pytest.mark.parametrize("D,opts", [(8, {}), (12, {}), (12, {"strips_per_cta": 2}), (20, {}),
+                                    (24, {}), (25, {}), (28, {}), (29, {}),
                                     (12, {"rows_per_lane": 2})])
 def test_repeated_batches(D, opts):
     from paper_2607_15478_gb300 import build, pardtw
