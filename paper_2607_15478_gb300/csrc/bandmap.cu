@@ -42,7 +42,7 @@ constexpr int kMapWarps = 4;  // segments per CTA
 // (launch_chained): the next kernel's CTAs are placed while one runs, which hides
 // ~2 us of each launch (1000 x 1200 frames 96.9 -> 82.6 us, 3001 x 3607 221 -> 206, 20000 x
 // 25000 (1565 CTAs) 1.038 -> 1.027 ms), but the wait costs every CTA of a grid of many
-// waves (3756 CTAs: 2.80 ms, 2.82 chained; 24490: 7.01 and 7.08; a batch of 256
+// waves (3756 CTAs: 2.72 ms, 2.74 chained; 24490: 7.01 and 7.08; a batch of 256
 // pairs, when it took 3.49 ms, 3.65).
 constexpr int kChainCtas = 2048;
 

@@ -89,11 +89,11 @@ constexpr int kBfBlkBytes = kColsPerWord * kBfStride * 2;
 // groups), and several cost warps share a strip, taking sub-chunks in turn
 // (all 8 columns each).  So they do where one would be slower than the DP warp.
 // With two strips a CTA: two (20000 x 25000 at D = 12: DP 0.907 ms, 1.056 with a third one,
-// which shares the DP warp's SM sub-partition; a plan of 256 pairs 3.53 and 3.78), at
+// which shares the DP warp's SM sub-partition; a plan of 256 pairs 3.51 and 3.73), at
 // D = 32 three (256 pairs of up to 4000 frames: 1.43 ms, 1.60 with two).  With one strip, four
 // of the wide ones (24001 x 27011 at D = 100: 3.23 ms, 2.50 with six, which are not
-// measured at other sizes), and three otherwise (40000 x 48000 with the BF16 cost: 2.80,
-// and with four).
+// measured at other sizes), and three otherwise (40000 x 48000 with the BF16 cost: 2.72,
+// 2.73 with four).
 template <int DP, int NS, bool kBF>
 struct CostCfg {
     static constexpr bool kWide = DP > 32 && !kBF;
@@ -687,7 +687,7 @@ __device__ __forceinline__ void run_dp(const DpArgs& p, int strip, int lane, con
     // loaded behind those of columns kFirst, kFirst + 1, .., kPer loads each: as late
     // as the latencies allow, since a strip can follow the one above no closer than
     // its tests look ahead (20000 x 25000, D = 12: DP 0.907 ms, 0.947 a column
-    // earlier; 40000 x 48000 with the BF16 cost 2.527, 2.519)
+    // earlier; 40000 x 48000 with the BF16 cost 2.445, 2.437)
     constexpr int kTest = 4, kFirst = 5, kPer = 4;
     const bool ghost = lane == kGhostLane;
     const int i0 = strip * kRows + lane * R;
@@ -763,11 +763,17 @@ __device__ __forceinline__ void run_dp(const DpArgs& p, int strip, int lane, con
     // use t's slot in any case, dropped like these where the test failed, came too early
     // now and then: with six cost warps a strip at D = 100 one call in 70 of 12007 x 9001
     // frames had a wrong total; since then none in 23000.)
-    auto test = [&](unsigned t, unsigned& slot) -> int {
-        const int there = mbar_test_wait(bar_at(cfull, t % kSlots), use_parity(t, kSlots));
-        slot = cring + ((there ? t : t - 1u) % kSlots) * Slot::kBytes;
-        return there;
+    auto slot_of = [&](unsigned t) { return cring + (t % kSlots) * Slot::kBytes; };
+    auto test = [&](unsigned t, int& there) -> unsigned {
+        there = mbar_test_wait(bar_at(cfull, t % kSlots), use_parity(t, kSlots));
+        return slot_of(there ? t : t - 1u);
     };
+    // The trip's end takes the outcomes from the tests in the FP32 cluster kernels, and
+    // elsewhere from the slots that were loaded, which keeps two registers less (DP of 20000
+    // x 25000 at D = 12, in clusters: 0.907 ms, 0.950 from the slots; the whole call of
+    // 40000 x 48000 with the BF16 cost 2.80 and 2.72, of 256 planned pairs 3.53 and 3.51, of
+    // 32 fragments of 40003 x 50021 frames 4.27 and 4.11).
+    constexpr bool kKeepTests = kSlots > 8 && !kRM;
     auto store = [&](int n, uint32_t* word) {
         if constexpr (kT) {
 #pragma unroll
@@ -798,9 +804,9 @@ __device__ __forceinline__ void run_dp(const DpArgs& p, int strip, int lane, con
         const unsigned dst0 = out.base + (to % kSlots) * out.stride;
         const unsigned dst1 = out.base + ((to + 1u) % kSlots) * out.stride;
         int rb = 1, ra = 1, ro = 1;
-        unsigned sb = 0, sa = 0;
+        unsigned sb = 0, sa = 0;  // the slots loaded
         full_sub(n, ia, 0, dst0, st, word, [&](int u) {
-            if (u == kTest) rb = test(t + 1u, sb);
+            if (u == kTest) sb = test(t + 1u, rb);
             part(ib, sb, u);
         });
         mbar_arrive_if(bar_at(out.full, to % kSlots), st);
@@ -809,11 +815,17 @@ __device__ __forceinline__ void run_dp(const DpArgs& p, int strip, int lane, con
             if (u == 0)  // its consumer empties the output ring in order
                 ro = mbar_test_wait(bar_at(out.empty, (to + 3u) % kSlots),
                                     use_parity(to + 3u, kSlots) ^ 1u);
-            if (u == kTest) ra = test(t + 2u, sa);
+            if (u == kTest) sa = test(t + 2u, ra);
             part(ia, sa, u);
         });
-        if (!__all_sync(kFull, rb & (ra | (int)!more) & (ro | (int)!next_on))) {
-            if (!__all_sync(kFull, rb)) {
+        int go;  // (a vote on whole numbers, or on predicates: 0.907 and 1.009 ms in clusters)
+        if constexpr (kKeepTests)
+            go = __all_sync(kFull, rb & (ra | (int)!more) & (ro | (int)!next_on));
+        else
+            go = __all_sync(kFull, (sb == slot_of(t + 1u)) & ((sa == slot_of(t + 2u)) | !more) &
+                                       ((bool)ro | !next_on));
+        if (!go) {
+            if (!__all_sync(kFull, kKeepTests ? rb : (int)(sb == slot_of(t + 1u)))) {
                 if (!wait_load(t + 1u, ib)) return;
                 s = before;
 #pragma unroll

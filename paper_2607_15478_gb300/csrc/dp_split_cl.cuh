@@ -18,8 +18,8 @@
 // warps a strip, on the sub-partitions beside the DP warp's), else two.  The
 // cluster size: see launch_cl.  Measured (DP, ms): 20000 x 25000, D = 12, clusters
 // of 8 / 6 / 4 / 2: 0.906 / 0.916 / 0.928 / 0.976; 100000 x 126231 (335 groups active
-// at once, 152 SMs): 6.87 / 6.38 / 6.19 / 5.88; 40000 x 48000, D = 128, BF16: 2.70 / 2.59
-// / 2.57 / 2.52 with one strip a CTA, 3.18 without clusters and two.
+// at once, 152 SMs): 6.87 / 6.38 / 6.19 / 5.88; 40000 x 48000, D = 128, BF16: 2.59 / 2.48
+// / 2.46 / 2.45 with one strip a CTA, 3.16 without clusters and two.
 #pragma once
 #include <algorithm>
 #include <mutex>

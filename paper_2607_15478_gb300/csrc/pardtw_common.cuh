@@ -326,7 +326,7 @@ struct BtArgs {
 // bands (~0.6 us for four), so short pairs take short bands (1000 x 1200: 96.9 us
 // with 128 rows, 82.6 with 32; 3001 x 3607: 216 and 206 with 64) unless the call
 // fills the GPU: a segment of the map recomputes two columns per row of its band (256
-// pairs of up to 8000 frames: 3.69 ms with 64 rows, 3.53 with 128).
+// pairs of up to 8000 frames: 3.66 ms with 64 rows, 3.51 with 128).
 inline int band_rows(int La, double cells) {
     if (cells > 1e9) return 128;
     return La <= 1536 ? 32 : (La <= 6144 ? 64 : 128);
