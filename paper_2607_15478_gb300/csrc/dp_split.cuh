@@ -676,7 +676,7 @@ __device__ __forceinline__ void sweep_col(const SubIn<R>& in, int u, bool origin
 // end.  Where they were not, the state before n + 1 is put back, the barrier is
 // waited for and n + 1 is swept again: in a chain that is on time this is
 // rare, and a strip that is early has time to lose.
-template <int R, int kSlots, bool kRM, bool kSubseq, bool kT>
+template <int R, int NS, int kSlots, bool kRM, bool kSubseq, bool kT>
 __device__ __forceinline__ void run_dp(const DpArgs& p, int strip, int lane, const int2 rg,
                                        const OutRing& out, unsigned cring, unsigned cfull,
                                        unsigned cempty, unsigned csub) {
@@ -768,12 +768,13 @@ __device__ __forceinline__ void run_dp(const DpArgs& p, int strip, int lane, con
         there = mbar_test_wait(bar_at(cfull, t % kSlots), use_parity(t, kSlots));
         return slot_of(there ? t : t - 1u);
     };
-    // The trip's end takes the outcomes from the tests in the FP32 cluster kernels, and
-    // elsewhere from the slots that were loaded, which keeps two registers less (DP of 20000
-    // x 25000 at D = 12, in clusters: 0.907 ms, 0.950 from the slots; the whole call of
-    // 40000 x 48000 with the BF16 cost 2.80 and 2.72, of 256 planned pairs 3.53 and 3.51, of
-    // 32 fragments of 40003 x 50021 frames 4.27 and 4.11).
-    constexpr bool kKeepTests = kSlots > 8 && !kRM;
+    // The trip's end takes the outcomes from the tests in the FP32 cluster kernels and with
+    // four strips a CTA, and elsewhere from the slots that were loaded, which keeps two
+    // registers less (DP of 20000 x 25000 at D = 12, in clusters: 0.907 ms, 0.950 from the
+    // slots; of 256 pairs, four strips a CTA, 3.225 and 3.254; the whole call of 40000 x 48000
+    // with the BF16 cost 2.80 and 2.72, of 256 planned pairs 3.53 and 3.51, of 32 fragments of
+    // 40003 x 50021 frames 4.27 and 4.11).
+    constexpr bool kKeepTests = (kSlots > 8 && !kRM) || NS == 4;
     auto store = [&](int n, uint32_t* word) {
         if constexpr (kT) {
 #pragma unroll
@@ -1287,7 +1288,7 @@ __global__ void __launch_bounds__(split_threads<DP, NS, kBF>(),
                     out.first = rg.x;
                     out.end = w == NS - 1 && gr.writer ? rg.y : rg.x;
                 }
-                run_dp<R, kSlots, kBF, kSubseq, kT>(p, strip, lane, rg, out, cring_s, cfull_s,
+                run_dp<R, NS, kSlots, kBF, kSubseq, kT>(p, strip, lane, rg, out, cring_s, cfull_s,
                                                     cempty_s, cs);
             }
         } else if (role == 2) {
